@@ -228,6 +228,11 @@ StepParams make_params(const rhi_ctx* h, double dt, double a, double adot) {
     P.inv_a2dx2 = P.inv_adx * P.inv_adx;
     const int nmax = std::max(h->grid.nx, std::max(h->grid.ny, h->grid.nz));
     P.R_min = 1.0 / (a * nmax * h->grid.dx);
+    P.quart_adx = 0.5 * P.half_adx;
+    P.R_min2 = 2.0 * P.R_min;
+    P.cF = 2.0 * C_LIGHT * P.inv_a2dx2;
+    P.cK = -0.5 / (C_LIGHT * P.inv_a2dx2);
+    P.cV = C_LIGHT * P.inv_a2dx2 * P.half_adx;
     P.kappa_floor = h->prm.kappa_floor;
     P.m_grey = (double)h->prm.m_grey;
     P.isothermal = h->prm.isothermal; P.limiter = h->prm.limiter;
@@ -235,13 +240,26 @@ StepParams make_params(const rhi_ctx* h, double dt, double a, double adot) {
     P.y_he = h->prm.y_he;
     P.u_e = h->prm.u_e; P.u_n = h->prm.u_n; P.u_E = h->prm.u_E;
     P.iu_e = 1.0 / P.u_e; P.iu_n = 1.0 / P.u_n; P.iu_E = 1.0 / P.u_E;
-    P.sc_ne = P.dth * P.u_n * P.iu_e;
-    P.sc_en = P.dth * P.u_e * P.iu_n;
-    P.sc_Ee = P.dth * P.u_E * P.iu_e;
-    P.sc_En = P.dth * P.u_E * P.iu_n;
-    P.sc_eE = P.dth * P.u_e * P.iu_E;
-    P.sc_nE = P.dth * P.u_n * P.iu_E;
     for (int X = 0; X < 3; ++X) { P.sk[X] = h->prm.sk[X]; P.pg[X] = h->prm.pgam[X]; P.ph[X] = h->prm.ph[X]; }
+    P.cR = M_H * (1.0 + 4.0 * P.y_he);
+    P.cN = 1.0 + P.y_he;
+    P.cT = (GAMMA - 1.0) * P.cR / K_BOLTZ;
+    P.cTR = (GAMMA - 1.0) / K_BOLTZ;
+    P.i3 = P.dth * P.ia3;
+    P.cdth = C_LIGHT * P.dth;
+    P.cE3 = P.cdth * P.ia3;
+    P.madot_dth = P.m_grey * P.adot_a * P.dth;
+    P.adot2_dth = 2.0 * P.adot_a * P.dth;
+    P.one_adot2 = 1.0 + P.adot2_dth;
+    P.r_ne = P.u_n * P.iu_e;
+    P.r_en = P.u_e * P.iu_n;
+    P.cz0 = -P.cE3 * P.u_E * P.iu_e;
+    for (int X = 0; X < 3; ++X) {
+        P.cz[X] = P.cE3 * P.u_E * P.iu_n * P.pg[X];
+        P.ksk[X] = P.sk[X] * P.ia3 * P.u_n * P.iu_E;
+    }
+    P.dtm1_dth = (h->prm.theta - 1.0) / h->prm.theta;
+    P.dt_dth = 1.0 / h->prm.theta;
     P.tau = h->prm.tau;
     P.lte = h->prm.model == RHI_MODEL_LTE;
     P.kappa_total = h->prm.kappa_total;

@@ -53,15 +53,22 @@ struct StepParams {
     double inv_adx;                   // 1 / (a dx)
     double half_adx;                  // a dx / 2
     double R_min;                     // limiter floor 1 / (a L)
+    // face formulas: a dx / 4, 2 R_min, 2 c / (a dx)^2, -(a dx)^2 / (2 c), c / (2 a dx)
+    double quart_adx, R_min2, cF, cK, cV;
     double kappa_floor;
     double m_grey;
     int isothermal, limiter;
     int limiter_newton;               // 1: keep dD/dE in the Newton matrix (non-symmetric S)
     double y_he;
     double u_e, u_n, u_E, iu_e, iu_n, iu_E;
-    // dt theta times ratios of scalings for the scaled local blocks: M[0][s>0] (u_n / u_e),
-    // M[r>0][0] (u_e / u_n), U column (u_E / u_e, u_E / u_n), L row (u_e / u_E, u_n / u_E)
-    double sc_ne, sc_en, sc_Ee, sc_En, sc_eE, sc_nE;
+    // constants of the local model: rho = cR n_H, n_tot = cN n_H + n_e, dT/de = cT n_H / n_tot,
+    // cTR = cT / cR; with dt theta folded in: i3 = dth / a^3, cE3 = c dth / a^3, cdth = c dth,
+    // madot_dth = m adot/a dth, adot2_dth = 2 adot/a dth, one_adot2 = 1 + adot2_dth; and with
+    // the ratios of scalings: r_ne = u_n / u_e, r_en = u_e / u_n, the U column's cz0 (times heating
+    // / rho) and cz[X] (times n_X), ksk[X] = d kappa / d n_X in scaled unknowns
+    double cR, cN, cT, cTR, i3, cE3, cdth, madot_dth, adot2_dth, one_adot2, r_ne, r_en, cz0;
+    double cz[3], ksk[3];
+    double dtm1_dth, dt_dth;          // (theta - 1) / theta, 1 / theta
     double sk[3], pg[3], ph[3];
     double tau;
     // LTE coupling (eq. LTE_coupling; no species): constant opacities, T = lte_cT e
@@ -69,6 +76,20 @@ struct StepParams {
     double kappa_total, kappa_planck, lte_cT;
     const double2* __restrict__ table;
 };
+
+// ---------------------------------------------------------------------------------------------
+// arithmetic
+
+// Reciprocal to within one unit in the last place: the hardware's reciprocal seed (PTX
+// rcp.approx.ftz.f64, about 20 bits) and one third-order Householder step r (1 + e + e^2) with
+// e = 1 - d r, whose error is e^3 < 2^-55: three FP64 instructions where the IEEE division takes
+// about ten.  For normal d with a normal reciprocal.
+__device__ __forceinline__ double fast_rcp(double d) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+    const double e = fma(-d, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
 
 // ---------------------------------------------------------------------------------------------
 // grid helpers
