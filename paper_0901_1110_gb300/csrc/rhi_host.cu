@@ -110,15 +110,23 @@ struct rhi_ctx {
     double *E_p = nullptr, *e_p = nullptr, *n_p = nullptr;
     double dt_prev = 0.0;
     bool have_prev = false;
-    // two work iterates, contiguous (e_c | n_1 .. | E), their opacity and face coefficients
+    // two work iterates, contiguous (e_c | n_1 .. | E), their opacity and face arrays (times
+    // dt theta): W (limiter_jacobian 0) or the fluxes W (E_c - E_lower), and with dD/dE kept the
+    // Newton-matrix entries PQ and the exact matrix's opacity terms Kf
     double* U[2] = {nullptr, nullptr};
     double* kap[2] = {nullptr, nullptr};
     double* W[2] = {nullptr, nullptr};
-    double* PQ[2] = {nullptr, nullptr};         // Newton-matrix face entries (dD/dE kept)
-    double* Kf[2] = {nullptr, nullptr};         // exact matrix: (1/2) dW/dkappa dE per face
+    double* PQ[2] = {nullptr, nullptr};
+    double* Kf[2] = {nullptr, nullptr};
     double* Upred = nullptr;                    // explicit predictor of the step (dt_norm)
-    double* diag_ns[2] = {nullptr, nullptr};
     double* g = nullptr;
+    // Schur sets: the diagonal (limiter_jacobian 0) or its local part, right-hand side, opacity
+    // responses (exact matrix), elimination
+    double *rho[2] = {nullptr, nullptr}, *phi[2] = {nullptr, nullptr};
+    // the assembled Newton matrix and right-hand side of the current system (dD/dE kept), and the
+    // lagged-D matrix's W and diagonal where such a solver needs them (allocated on first use)
+    double *sysPQ = nullptr, *sysdiag = nullptr, *sysrhs = nullptr;
+    double *lagW = nullptr, *lagdiag = nullptr;
     double *diag[2] = {nullptr, nullptr}, *rhs[2] = {nullptr, nullptr};
     double *fMt[2] = {nullptr, nullptr}, *MiU[2] = {nullptr, nullptr};
     double* f_tmp = nullptr;
@@ -148,18 +156,16 @@ struct rhi_ctx {
         cudaGraphExec_t exec = nullptr;
         cudaStream_t st = nullptr;
         cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-        double scale = 0.0;
         bool nonsym = false;
         std::vector<float*> post;       // level buffers (x, xt) after the captured cycle
         int kernels = 0;
         bool failed = false;
     } vg;
 
-    // the BiCGStab solve as one CUDA graph (a while node whose body is one iteration),
-    // cached per set of buffers and operator scale
+    // the BiCGStab solve as one CUDA graph (a while node whose body is one iteration); the
+    // assembled system and the hierarchy live in fixed buffers and hold dt theta, so one capture
+    // serves every solve of the handle, whatever the step size (two with the lagged-D hierarchy)
     struct KGraph {
-        const void* key[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-        double scale = 0.0;
         bool nonsym = false;
         cudaGraphExec_t exec = nullptr;
         int k_init = 0, k_body = 0;
@@ -230,9 +236,11 @@ StepParams make_params(const rhi_ctx* h, double dt, double a, double adot) {
     P.R_min = 1.0 / (a * nmax * h->grid.dx);
     P.quart_adx = 0.5 * P.half_adx;
     P.R_min2 = 2.0 * P.R_min;
-    P.cF = 2.0 * C_LIGHT * P.inv_a2dx2;
-    P.cK = -0.5 / (C_LIGHT * P.inv_a2dx2);
-    P.cV = C_LIGHT * P.inv_a2dx2 * P.half_adx;
+    const double d = C_LIGHT * P.dth * P.inv_a2dx2;
+    P.cF = 2.0 * d;
+    P.cK = -0.5 / d;
+    P.cV = d * P.half_adx;
+    P.cD = d / 3.0;
     P.kappa_floor = h->prm.kappa_floor;
     P.m_grey = (double)h->prm.m_grey;
     P.isothermal = h->prm.isothermal; P.limiter = h->prm.limiter;
@@ -367,7 +375,6 @@ Op<T> level_op(const rhi_ctx* h, const Level<T>& v) {
     A.diag = v.diag;
     A.wid = v.wid;
     A.loc = v.loc;
-    A.scale = T(1);
     return A;
 }
 
@@ -379,12 +386,12 @@ Op<double> newton_op(const rhi_ctx* h) {
     A.fd_nx = B.fd_nx; A.fd_nxy = B.fd_nxy;
     for (int a = 0; a < 3; ++a) { A.per[a] = B.per[a]; A.W[a] = B.Q[a]; A.Wp[a] = B.P[a]; }
     A.diag = B.diag;
-    A.scale = B.scale;
     return A;
 }
 
 // coarse operators for the finest operator A0 (the lagged-D matrix h->op0, or the Newton matrix
-// when nonsym); A0 becomes the preconditioner's finest operator h->pc0
+// when nonsym, whose finest level the assembly has written); A0 becomes the preconditioner's
+// finest operator h->pc0
 int precond_setup(rhi_ctx* h, const Op<double>& A0, bool nonsym) {
     LinLaunch L(h->st, &h->prof);
     const double om = h->prm.mg_omega;
@@ -396,7 +403,7 @@ int precond_setup(rhi_ctx* h, const Op<double>& A0, bool nonsym) {
             return fail(h, RHI_ERR_ARG, "multigrid of the Newton matrix needs params.mg_matrix = 1");
         h->pc0.wid = lv[0].wid;
         h->pc0.loc = lv[0].loc;
-        CK((L.level_prep<double, double>(h->pc0, om, lv[0].wid, lv[0].loc)));
+        if (!nonsym) CK((L.level_prep<double, double>(h->pc0, om, lv[0].wid, lv[0].loc)));
         for (size_t l = 0; l + 1 < lv.size(); ++l) {
             Op<double> A = (l == 0) ? h->pc0 : level_op(h, lv[l]);
             auto& c = lv[l + 1];
@@ -408,10 +415,12 @@ int precond_setup(rhi_ctx* h, const Op<double>& A0, bool nonsym) {
         auto& lv = h->mg32;
         if (nonsym && !lv[0].Wp[0])
             return fail(h, RHI_ERR_ARG, "multigrid of the Newton matrix needs params.mg_matrix = 1");
-        CK(L.cast_op(h->pc0, lv[0].diag, lv[0].W, nonsym ? lv[0].Wp : nullptr));
-        // the finest level's omega / diag from the FP64 operator (the FP32 restriction takes
-        // each child's full row and needs no local part)
-        CK((L.level_prep<double, float>(h->pc0, om, lv[0].wid, nullptr)));
+        if (!nonsym) {
+            CK(L.cast_op(h->pc0, lv[0].diag, lv[0].W));
+            // the finest level's omega / diag from the FP64 operator (the FP32 restriction takes
+            // each child's full row and needs no local part)
+            CK((L.level_prep<double, float>(h->pc0, om, lv[0].wid, nullptr)));
+        }
         for (size_t l = 0; l + 1 < lv.size(); ++l) {
             auto& c = lv[l + 1];
             if (l == 0)
@@ -425,11 +434,16 @@ int precond_setup(rhi_ctx* h, const Op<double>& A0, bool nonsym) {
     return RHI_OK;
 }
 
+// the hierarchy is built from the Newton matrix itself
+bool newton_hierarchy(const rhi_ctx* h) {
+    return h->prm.mg_matrix == 1 && h->prm.limiter_jacobian != 0 &&
+           h->prm.precond != RHI_PRECOND_JACOBI;
+}
+
 // the preconditioner of the system the Krylov method solves: the Newton matrix's own
 // hierarchy when params.mg_matrix = 1 and the matrix keeps dD/dE, else the lagged-D matrix's
 int precond_setup_newton(rhi_ctx* h) {
-    const bool nonsym = h->prm.mg_matrix == 1 && h->prm.limiter_jacobian != 0 &&
-                        h->prm.precond != RHI_PRECOND_JACOBI;
+    const bool nonsym = newton_hierarchy(h);
     return precond_setup(h, nonsym ? newton_op(h) : h->op0, nonsym);
 }
 
@@ -482,9 +496,8 @@ int vcycle(rhi_ctx* h, std::vector<Level<T>>& lv, size_t l, const Op<T>& A0,
 // One V-cycle is about 45 launches, most of them on grids of 64^3 cells and below, where the
 // launch gap is longer than the kernel.  The cycle is captured once (on a private stream) and
 // replayed as one graph launch ordered after / before the handle's stream by events.  The
-// graph binds the level buffers and the operator's scale (dt theta) at capture; it is
-// captured again when the scale changes or the host's view of the ping-pong buffers no longer
-// matches the state after capture (a direct V-cycle ran in between).
+// graph binds the level buffers at capture; it is captured again when the host's view of the
+// ping-pong buffers no longer matches the state after capture (a direct V-cycle ran in between).
 
 struct Counter : LaunchHook {
     int n = 0;
@@ -505,7 +518,7 @@ bool vcycle_graph_usable(const rhi_ctx* h) {
 int vcycle_graph(rhi_ctx* h, const Op<float>& A0) {
     auto& lv = h->mg32;
     auto& g = h->vg;
-    bool valid = g.exec && g.scale == (double)A0.scale && g.nonsym == h->pc_nonsym &&
+    bool valid = g.exec && g.nonsym == h->pc_nonsym &&
                  g.post.size() == 2 * lv.size();
     for (size_t l = 0; valid && l < lv.size(); ++l)
         valid = g.post[2 * l] == lv[l].x && g.post[2 * l + 1] == lv[l].xt;
@@ -534,7 +547,6 @@ int vcycle_graph(rhi_ctx* h, const Op<float>& A0) {
             return fail(h, RHI_ERR_CUDA, std::string("V-cycle graph: ") + cudaGetErrorString(e));
         }
         g.kernels = cnt.n;
-        g.scale = (double)A0.scale;
         g.nonsym = h->pc_nonsym;
         g.post.clear();
         for (auto& v : lv) { g.post.push_back(v.x); g.post.push_back(v.xt); }
@@ -767,14 +779,14 @@ int bicg_outcome(rhi_ctx* h, int* its_out) {
     return RHI_OK;
 }
 
-// Right-preconditioned BiCGStab on the non-symmetric Schur matrix h->opns (dD/dE kept), to
+// Right-preconditioned BiCGStab on the assembled Newton matrix and right-hand side (dD/dE kept), to
 // ||r||_RMS <= tol (counted over the N (N_s + 2) unknowns of eq. rmsnorm); solution in h->x.
 // The iteration's control runs on the device: as one CUDA graph launch per solve, or, while
 // per-launch timing is on, as direct launches with one host read per iteration.  With
 // `deferred` and the graph, the call only enqueues the solve (*its_out = -1): the next host
 // read of the scalars brings its outcome back for bicg_outcome.  Otherwise the outcome is read
 // here; RHI_ERR_NONPHYSICAL on a breakdown.
-int bicgstab(rhi_ctx* h, const double* rhs, double tol, int* its_out, bool deferred = false) {
+int bicgstab(rhi_ctx* h, double tol, int* its_out, bool deferred = false) {
     const long long N = h->N;
     h->h_ctl[0] = tol * tol * (double)N * h->nv;                   // S_THR: bound on r.r
     h->h_ctl[1] = (double)h->prm.max_pcg;                           // S_MAXIT
@@ -787,22 +799,13 @@ int bicgstab(rhi_ctx* h, const double* rhs, double tol, int* its_out, bool defer
     CK(cudaMemcpyAsync(h->scal + S_THR, h->h_ctl, 3 * sizeof(double), cudaMemcpyHostToDevice, h->st));
     int rc = RHI_OK;
     if (krylov_graph_usable(h)) {
-        const void* key[6] = {rhs, h->opns.diag, h->opns.P[0], h->pc0.diag, h->pc0.W[0],
-                              (const void*)(long long)h->prm.precond};
         rhi_ctx::KGraph* g = nullptr;
         for (auto& c : h->kg)
-            if (std::equal(key, key + 6, c.key) && c.scale == h->opns.scale && c.nonsym == h->pc_nonsym)
-                g = &c;
+            if (c.nonsym == h->pc_nonsym) g = &c;
         if (!g) {
-            if (h->kg.size() >= 8) {
-                for (auto& c : h->kg) if (c.exec) cudaGraphExecDestroy(c.exec);
-                h->kg.clear();
-            }
             rhi_ctx::KGraph ng;
-            std::copy(key, key + 6, ng.key);
-            ng.scale = h->opns.scale;
             ng.nonsym = h->pc_nonsym;
-            if ((rc = krylov_graph_build(h, rhs, ng))) return rc;
+            if ((rc = krylov_graph_build(h, h->sysrhs, ng))) return rc;
             h->kg.push_back(ng);
             g = &h->kg.back();
         }
@@ -823,7 +826,7 @@ int bicgstab(rhi_ctx* h, const double* rhs, double tol, int* its_out, bool defer
         h->kg_body_kernels = 0;                         // direct launches count themselves
         LinLaunch L(h->st, &h->prof);
         L.fine_N = N;
-        if ((rc = bicg_start(h, L, rhs, 0))) return rc;
+        if ((rc = bicg_start(h, L, h->sysrhs, 0))) return rc;
         double cont = 0.0;
         if ((rc = read_scalar(h, S_CONT, &cont))) return rc;
         while (cont != 0.0) {
@@ -842,7 +845,15 @@ PhysBuffers state_buffers(rhi_ctx* h) {
     B.E_n = h->E_s; B.n_n = h->n_s; B.eh = h->e_s; B.nH = h->nH; B.src = h->src; B.Tiso = h->Tiso;
     B.g = h->g;
     B.partials = h->partials;
+    B.flux = h->prm.limiter_jacobian != 0;
     return B;
+}
+
+// the face arrays `b` and the Schur set `set` an evaluation works with
+void with_set(rhi_ctx* h, PhysBuffers& B, int b, int set) {
+    B.W = h->W[b];
+    B.diag = h->diag[set]; B.rhs = h->rhs[set]; B.rho = h->rho[set]; B.phi = h->phi[set];
+    B.fMt = h->fMt[set]; B.MiU = h->MiU[set];
 }
 
 int cell(rhi_ctx* h, const StepParams& P, int mode, PhysBuffers B) {
@@ -857,21 +868,13 @@ int ncell_blocks(const rhi_ctx* h) { return (int)((h->N + cell_block_size() - 1)
 
 int faces(rhi_ctx* h, const StepParams& P, const double* E, const double* kap, int b) {
     Scope s(h->prof, "faces_limiter");
-    CK(launch_faces(P, E, kap, h->W[b], h->PQ[b], h->Kf[b], h->st));
+    CK(launch_faces(P, h->prm.limiter_jacobian, 0, E, kap, h->W[b], h->PQ[b], h->Kf[b], h->st));
     return RHI_OK;
 }
-// W alone (an iterate evaluated for its residual only)
+// what the residual needs alone (an iterate evaluated for its residual only)
 int faces_w(rhi_ctx* h, const StepParams& P, const double* E, const double* kap, int b) {
     Scope s(h->prof, "faces_w");
-    CK(launch_faces_w(P, h->prm.limiter_jacobian, E, kap, h->W[b], h->st));
-    return RHI_OK;
-}
-// exact Newton matrix: fold the opacity coupling into Schur set `set` built from buffer b
-int schur_kappa(rhi_ctx* h, const StepParams& P, int b, int set) {
-    if (h->prm.limiter_jacobian != 2) return RHI_OK;
-    Scope s(h->prof, "schur_kappa");
-    CK(launch_schur_kappa(P, h->ns, h->Kf[b], h->fMt[set], h->MiU[set], h->PQ[b], h->diag_ns[set],
-                          h->rhs[set], h->st));
+    CK(launch_faces(P, h->prm.limiter_jacobian, 1, E, kap, h->W[b], nullptr, nullptr, h->st));
     return RHI_OK;
 }
 int kappa(rhi_ctx* h, const StepParams& P, const double* n, double* kap) {
@@ -880,28 +883,71 @@ int kappa(rhi_ctx* h, const StepParams& P, const double* n, double* kap) {
     return RHI_OK;
 }
 
-void set_op0(rhi_ctx* h, const StepParams& P, int set, const double* W) {
+// the lagged-D matrix: coefficients W and diagonal
+void set_op0(rhi_ctx* h, const double* W, const double* diag) {
     Op<double>& A = h->op0;
     A.nx = h->grid.nx; A.ny = h->grid.ny; A.nz = h->grid.nz; A.N = h->N;
     A.fd_nx = make_fastdiv((unsigned)A.nx);
     A.fd_nxy = make_fastdiv((unsigned)A.nx * (unsigned)A.ny);
     for (int a = 0; a < 3; ++a) { A.per[a] = h->per[a]; A.W[a] = A.Wp[a] = W + a * h->N; }
-    A.diag = h->diag[set];
-    A.scale = P.dth;
+    A.diag = diag;
 }
 
-void set_opns(rhi_ctx* h, const StepParams& P, int set, const double* PQ) {
+// the lagged-D matrix of an iterate of a solver that keeps dD/dE
+int lagged_system(rhi_ctx* h, const StepParams& P, const double* E, const double* kap, int set) {
+    int rc;
+    if (!h->lagW && (rc = dalloc(h, &h->lagW, 3 * (size_t)h->N))) return rc;
+    if (!h->lagdiag && (rc = dalloc(h, &h->lagdiag, (size_t)h->N))) return rc;
+    {
+        Scope s(h->prof, "faces_lagged");
+        CK(launch_faces(P, 0, 0, E, kap, h->lagW, nullptr, nullptr, h->st));
+    }
+    Scope s(h->prof, "lagged_diag");
+    CK(launch_lagged_diag(P, h->lagW, h->diag[set], E, kap, h->lagdiag, h->st));
+    set_op0(h, h->lagW, h->lagdiag);
+    return RHI_OK;
+}
+
+// The system of an evaluated iterate (face arrays b, Schur set `set`, at E and kap): the lagged-D
+// matrix, or the assembled Newton matrix with the finest level of its hierarchy
+int build_system(rhi_ctx* h, const StepParams& P, int b, int set, const double* E, const double* kap) {
+    if (!h->prm.limiter_jacobian) {
+        set_op0(h, h->W[b], h->diag[set]);
+        return RHI_OK;
+    }
+    SchurIn I{};
+    I.PQ = h->PQ[b]; I.K = h->Kf[b]; I.dloc = h->diag[set]; I.rhs = h->rhs[set];
+    I.rho = h->rho[set]; I.phi = h->phi[set];
+    SchurOut O{};
+    O.PQ = h->sysPQ; O.diag = h->sysdiag; O.rhs = h->sysrhs;
+    O.omega = h->prm.mg_omega;
+    if (newton_hierarchy(h)) {
+        if (h->prm.precond == RHI_PRECOND_MG_FP32) {
+            auto& v = h->mg32[0];
+            O.d32 = v.diag;
+            O.wid32 = v.wid;
+            for (int a = 0; a < 3; ++a) { O.W32[a] = v.W[a]; O.Wp32[a] = v.Wp[a]; }
+        } else {
+            O.wid64 = h->mg64[0].wid;
+        }
+    }
+    {
+        Scope s(h->prof, "schur_assemble");
+        CK(launch_schur_assemble(P, I, O, h->st));
+    }
     OpNS& A = h->opns;
     A.nx = h->grid.nx; A.ny = h->grid.ny; A.nz = h->grid.nz; A.N = h->N;
     A.fd_nx = make_fastdiv((unsigned)A.nx);
     A.fd_nxy = make_fastdiv((unsigned)A.nx * (unsigned)A.ny);
     for (int a = 0; a < 3; ++a) {
         A.per[a] = h->per[a];
-        A.P[a] = PQ + a * h->N;
-        A.Q[a] = PQ + (3 + a) * h->N;
+        A.P[a] = h->sysPQ + a * h->N;
+        A.Q[a] = h->sysPQ + (3 + a) * h->N;
     }
-    A.diag = h->diag_ns[set];
-    A.scale = P.dth;
+    A.diag = h->sysdiag;
+    // the hierarchy of the lagged-D matrix, or its diagonal for Jacobi
+    if (!newton_hierarchy(h)) return lagged_system(h, P, E, kap, set);
+    return RHI_OK;
 }
 
 // U views of a work buffer
@@ -1102,10 +1148,14 @@ int rhi_create(const rhi_grid* grid, const rhi_bc* bc, const rhi_params* params,
         A(&h->U[b], (size_t)h->nv * N); A(&h->kap[b], N); A(&h->W[b], 3 * (size_t)N);
         A(&h->diag[b], N); A(&h->rhs[b], N); A(&h->fMt[b], (size_t)h->nm * N);
         A(&h->MiU[b], (size_t)h->nm * N);
-        if (params->limiter_jacobian) { A(&h->PQ[b], 6 * (size_t)N); A(&h->diag_ns[b], N); }
-        if (params->limiter_jacobian == 2) A(&h->Kf[b], 3 * (size_t)N);
+        if (params->limiter_jacobian) A(&h->PQ[b], 6 * (size_t)N);
+        // (with a constant opacity, n_species = 0, the exact matrix has no opacity terms)
+        if (params->limiter_jacobian == 2 && h->ns > 0) {
+            A(&h->Kf[b], 3 * (size_t)N); A(&h->rho[b], N); A(&h->phi[b], N);
+        }
     }
     if (params->limiter_jacobian) {
+        A(&h->sysPQ, 6 * (size_t)N); A(&h->sysdiag, N); A(&h->sysrhs, N);
         A(&h->rh, N); A(&h->v, N); A(&h->s, N); A(&h->t, N); A(&h->ph, N); A(&h->sh, N);
     }
     A(&h->g, (size_t)h->nv * N);
@@ -1306,36 +1356,37 @@ int rhi_linearize(rhi_handle h, double dt, double a, double adot, double* f, dou
     if ((rc = kappa(h, P, h->n_s, h->kap[0]))) return rc;
     if ((rc = faces(h, P, h->E_s, h->kap[0], 0))) return rc;
     PhysBuffers B = state_buffers(h);
-    B.W = h->W[0];
-    B.PQ = h->PQ[0]; B.diag_ns = h->diag_ns[0];
-    B.diag = h->diag[0]; B.rhs = h->rhs[0]; B.fMt = h->fMt[0]; B.MiU = h->MiU[0];
+    with_set(h, B, 0, 0);
     // the residual goes straight to a device destination, or via a free work buffer
     if (f) B.f_out = on_device ? f : h->U[1];
     if ((rc = cell(h, P, MODE_PREP, B))) return rc;
-    if ((rc = schur_kappa(h, P, 0, 0))) return rc;
-    set_op0(h, P, 0, h->W[0]);
-    if (h->prm.limiter_jacobian) set_opns(h, P, 0, h->PQ[0]);
+    if ((rc = build_system(h, P, 0, 0, h->E_s, h->kap[0]))) return rc;
     if ((rc = precond_setup_newton(h))) return rc;
     const long long N = h->N;
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     if (f && !on_device) CK(cudaMemcpyAsync(f, h->U[1], (size_t)h->nv * N * sizeof(double), kind, h->st));
-    const double* dsrc = h->prm.limiter_jacobian ? h->diag_ns[0] : h->diag[0];
-    if (S_diag) CK(cudaMemcpyAsync(S_diag, dsrc, N * sizeof(double), kind, h->st));
-    if (rhs) CK(cudaMemcpyAsync(rhs, h->rhs[0], N * sizeof(double), kind, h->st));
+    const bool nonsym = h->prm.limiter_jacobian != 0;
+    if (S_diag) CK(cudaMemcpyAsync(S_diag, nonsym ? h->sysdiag : h->diag[0], N * sizeof(double), kind, h->st));
+    if (rhs) CK(cudaMemcpyAsync(rhs, nonsym ? h->sysrhs : h->rhs[0], N * sizeof(double), kind, h->st));
     if (S_lo || S_hi) {
-        // face entries of the Newton matrix (an inspection path: a temporary buffer)
-        double* tmp = nullptr;
-        CK(cudaMalloc(&tmp, 6 * N * sizeof(double)));
-        cudaError_t e = cudaSuccess;
-        {
+        // face entries of the Newton matrix: straight to a device destination, or by way of the
+        // face arrays of the second work iterate and g^n, which every call writes anew
+        const double* Q = nonsym ? h->opns.Q[0] : h->W[0];
+        const double* Pf = nonsym ? h->opns.P[0] : h->W[0];
+        if (on_device) {
             Scope s(h->prof, "export_faces");
-            e = launch_export_faces(P, h->W[0], h->PQ[0], tmp, tmp + 3 * N, h->st);
+            CK(launch_export_faces(P, Q, Pf, S_lo, S_hi, h->st));
+        } else {
+            for (int q = 0; q < 2; ++q) {
+                double* dst = q ? S_hi : S_lo;
+                if (!dst) continue;
+                {
+                    Scope s(h->prof, "export_faces");
+                    CK(launch_export_faces(P, Q, Pf, q ? nullptr : h->W[1], q ? h->W[1] : nullptr, h->st));
+                }
+                CK(cudaMemcpyAsync(dst, h->W[1], 3 * N * sizeof(double), kind, h->st));
+            }
         }
-        if (e == cudaSuccess && S_lo) e = cudaMemcpyAsync(S_lo, tmp, 3 * N * sizeof(double), kind, h->st);
-        if (e == cudaSuccess && S_hi) e = cudaMemcpyAsync(S_hi, tmp + 3 * N, 3 * N * sizeof(double), kind, h->st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
-        cudaFree(tmp);
-        if (e != cudaSuccess) return fail(h, RHI_ERR_CUDA, std::string("rhi_linearize: ") + cudaGetErrorString(e));
     }
     CK(cudaStreamSynchronize(h->st));
     h->prof.resolve();
@@ -1357,16 +1408,14 @@ int rhi_residual(rhi_handle h, double dt, double a, double adot, const double* U
     if ((rc = kappa(h, P, h->n_s, h->kap[0]))) return rc;
     if ((rc = faces(h, P, h->E_s, h->kap[0], 0))) return rc;
     PhysBuffers B = state_buffers(h);
-    B.W = h->W[0]; B.PQ = h->PQ[0]; B.diag_ns = h->diag_ns[0];
-    B.diag = h->diag[0]; B.rhs = h->rhs[0]; B.fMt = h->fMt[0]; B.MiU = h->MiU[0];
+    with_set(h, B, 0, 0);
     if ((rc = cell(h, P, MODE_PREP, B))) return rc;
     CK(cudaMemcpyAsync(h->U[1], U, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->st));
     if ((rc = kappa(h, P, U_n(h, 1), h->kap[1]))) return rc;
     if ((rc = faces(h, P, U_E(h, 1), h->kap[1], 1))) return rc;
     PhysBuffers C = state_buffers(h);
-    C.ec = U_ec(h, 1); C.n = U_n(h, 1); C.E = U_E(h, 1); C.W = h->W[1];
-    C.PQ = h->PQ[1]; C.diag_ns = h->diag_ns[1];
-    C.diag = h->diag[1]; C.rhs = h->rhs[1]; C.fMt = h->fMt[1]; C.MiU = h->MiU[1];
+    C.ec = U_ec(h, 1); C.n = U_n(h, 1); C.E = U_E(h, 1);
+    with_set(h, C, 1, 1);
     if (f) C.f_out = on_device ? f : h->U[0];
     if ((rc = cell(h, P, MODE_ITER, C))) return rc;
     double r = 0.0;
@@ -1449,14 +1498,12 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
     if ((rc = kappa(h, P, h->n_s, h->kap[0]))) return rc;
     if ((rc = faces(h, P, h->E_s, h->kap[0], 0))) return rc;
     PhysBuffers B = state_buffers(h);
-    B.W = h->W[0];
-    B.PQ = h->PQ[0]; B.diag_ns = h->diag_ns[0];
+    with_set(h, B, 0, 0);
     int cur = -1;            // -1: U_k is the state U^n (e_c = 0); 0 / 1: work buffer
     int set = 0;             // Schur set of U_k
     double res = 0.0;
     S.guess_used = h->prm.guess;
     if (h->prm.guess == RHI_GUESS_PREVIOUS || h->prm.guess == RHI_GUESS_LEARNED) {
-        B.diag = h->diag[0]; B.rhs = h->rhs[0]; B.fMt = h->fMt[0]; B.MiU = h->MiU[0];
         B.U0 = h->Upred;                    // the explicit predictor, for the error estimate
         if ((rc = cell(h, P, MODE_PREP, B))) return rc;
         B.U0 = nullptr;
@@ -1476,9 +1523,8 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
             if ((rc = kappa(h, P, U_n(h, 1), h->kap[1]))) return rc;
             if ((rc = faces(h, P, U_E(h, 1), h->kap[1], 1))) return rc;
             PhysBuffers C = state_buffers(h);
-            C.ec = U_ec(h, 1); C.n = U_n(h, 1); C.E = U_E(h, 1); C.W = h->W[1];
-            C.PQ = h->PQ[1]; C.diag_ns = h->diag_ns[1];
-            C.diag = h->diag[1]; C.rhs = h->rhs[1]; C.fMt = h->fMt[1]; C.MiU = h->MiU[1];
+            C.ec = U_ec(h, 1); C.n = U_n(h, 1); C.E = U_E(h, 1);
+            with_set(h, C, 1, 1);
             if ((rc = cell(h, P, MODE_ITER, C))) return rc;
             double rg = 0.0;
             if ((rc = residual_norm(h, ncell_blocks(h), &rg))) return rc;
@@ -1502,9 +1548,8 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
         if ((rc = kappa(h, P, U_n(h, 0), h->kap[0]))) return rc;
         if ((rc = faces(h, P, U_E(h, 0), h->kap[0], 0))) return rc;
         PhysBuffers C = state_buffers(h);
-        C.ec = U_ec(h, 0); C.n = U_n(h, 0); C.E = U_E(h, 0); C.W = h->W[0];
-        C.PQ = h->PQ[0]; C.diag_ns = h->diag_ns[0];
-        C.diag = h->diag[0]; C.rhs = h->rhs[0]; C.fMt = h->fMt[0]; C.MiU = h->MiU[0];
+        C.ec = U_ec(h, 0); C.n = U_n(h, 0); C.E = U_E(h, 0);
+        with_set(h, C, 0, 0);
         if ((rc = cell(h, P, MODE_ITER, C))) return rc;
         if ((rc = residual_norm(h, ncell_blocks(h), &res))) return rc;
     }
@@ -1527,8 +1572,7 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
             if ((rc = kappa(h, P, h->n_s, h->kap[0]))) return rc;
             if ((rc = faces(h, P, h->E_s, h->kap[0], 0))) return rc;
             PhysBuffers C = state_buffers(h);
-            C.W = h->W[0]; C.PQ = h->PQ[0]; C.diag_ns = h->diag_ns[0];
-            C.diag = h->diag[0]; C.rhs = h->rhs[0]; C.fMt = h->fMt[0]; C.MiU = h->MiU[0];
+            with_set(h, C, 0, 0);
             if ((rc = cell(h, P, MODE_PREP, C))) return rc;
             if ((rc = residual_norm(h, ncell_blocks(h), &res))) return rc;
             cur = -1;
@@ -1541,10 +1585,9 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
             S.guess_restarts = 1;
             if (res < newton_tol) break;
         }
-        const double* Wk = h->W[cur < 0 ? 0 : cur];
-        if ((rc = schur_kappa(h, P, cur < 0 ? 0 : cur, set))) return rc;
-        set_op0(h, P, set, Wk);
-        if (h->prm.limiter_jacobian) set_opns(h, P, set, h->PQ[cur < 0 ? 0 : cur]);
+        const int fb = cur < 0 ? 0 : cur;
+        const double* Ek = cur < 0 ? h->E_s : U_E(h, cur);
+        if ((rc = build_system(h, P, fb, set, Ek, h->kap[fb]))) return rc;
         if ((rc = precond_setup_newton(h))) return rc;
         int its = 0;
         // BiCGStab broke down (where free streaming makes the advective part of the matrix
@@ -1554,12 +1597,15 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
             S.krylov_fallbacks += 1;
             S.pcg_its += its;
             int r2;
+            // (from U^n, a trial evaluated meanwhile has overwritten the opacity in kap[0])
+            if (cur < 0 && (r2 = kappa(h, P, h->n_s, h->kap[0]))) return r2;
+            if ((r2 = lagged_system(h, P, Ek, h->kap[fb], set))) return r2;
             if (h->pc_nonsym && (r2 = precond_setup(h, h->op0, false))) return r2;
-            return pcg(h, h->rhs[set], lin_tol * res, &its);
+            return pcg(h, h->sysrhs, lin_tol * res, &its);
         };
         bool deferred = false;
         if (h->prm.limiter_jacobian) {
-            rc = bicgstab(h, h->rhs[set], lin_tol * res, &its, true);
+            rc = bicgstab(h, lin_tol * res, &its, true);
             deferred = rc == RHI_OK && its < 0;
             if (rc == RHI_ERR_NONPHYSICAL) rc = krylov_fallback();
             if (rc) { S.status = rc; return rc; }
@@ -1580,10 +1626,8 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
                 return r2;
             }
             PhysBuffers C = state_buffers(h);
-            C.ec = U_ec(h, t); C.n = U_n(h, t); C.E = U_E(h, t); C.W = h->W[t];
-            C.PQ = h->PQ[t]; C.diag_ns = h->diag_ns[1 - set];
-            C.diag = h->diag[1 - set]; C.rhs = h->rhs[1 - set];
-            C.fMt = h->fMt[1 - set]; C.MiU = h->MiU[1 - set];
+            C.ec = U_ec(h, t); C.n = U_n(h, t); C.E = U_E(h, t);
+            with_set(h, C, t, 1 - set);
             if ((r2 = cell(h, P, resid_only ? MODE_RESID : MODE_ITER, C))) return r2;
             return residual_norm(h, ncell_blocks(h), rt);
         };

@@ -53,8 +53,9 @@ struct StepParams {
     double inv_adx;                   // 1 / (a dx)
     double half_adx;                  // a dx / 2
     double R_min;                     // limiter floor 1 / (a L)
-    // face formulas: a dx / 4, 2 R_min, 2 c / (a dx)^2, -(a dx)^2 / (2 c), c / (2 a dx)
-    double quart_adx, R_min2, cF, cK, cV;
+    // face formulas, whose results come multiplied by dt theta: a dx / 4, 2 R_min, and with
+    // d = c dth / (a dx)^2: 2 d, -1 / (2 d), d a dx / 2, d (a dx)^2 / 3 (no limiter) over (a dx)^2
+    double quart_adx, R_min2, cF, cK, cV, cD;
     double kappa_floor;
     double m_grey;
     int isothermal, limiter;
@@ -164,13 +165,20 @@ struct PhysBuffers {
     const double* n;
     const double* E;
     const double* kap;
-    const double* W;        // 3 * N lower-face coefficients (per unit time)
-    const double* PQ;       // 6 * N Newton-matrix face entries (P then Q) or null
+    // per lower face, times dt theta (3 * N): the coefficients W (limiter_jacobian 0), or with
+    // `flux` the fluxes W (E_c - E_lower), all the residual needs
+    const double* W;
+    int flux;
     double* g;              // (ns + 2) * N
     // outputs of the cell kernel
-    double* diag;           // Schur diagonal with D lagged (scaled; the preconditioner's)
-    double* diag_ns;        // Schur diagonal with dD/dE kept (when PQ is given)
-    double* rhs;            // Schur right-hand side (scaled)
+    // Schur diagonal (scaled): complete (D lagged), or with `flux` its local part, which
+    // launch_schur_assemble completes
+    double* diag;
+    double* rhs;            // Schur right-hand side (scaled), without the faces' opacity terms
+    // exact matrix: the cell's opacity response to its E and to its residual,
+    // (d kappa / d n) M^-1 U and (d kappa / d n) M^-1 f_M (scaled; null: not needed)
+    double* rho;
+    double* phi;
     double* fMt;            // (ns + 1) * N   M^-1 f_M (scaled)
     double* MiU;            // (ns + 1) * N   M^-1 U  (scaled)
     double* f_out;          // optional (ns + 2) * N scaled residual
@@ -182,16 +190,30 @@ enum CellMode { MODE_PREP = 0, MODE_ITER = 1, MODE_PREP_PREDICT = 2, MODE_RESID 
 
 cudaError_t launch_kappa(const StepParams& P, int ns, const double* n, double* kap,
                          cudaStream_t st);
-cudaError_t launch_faces(const StepParams& P, const double* E, const double* kap, double* W,
-                         double* PQ, double* K, cudaStream_t st);
-// the face coefficients W alone, with the arithmetic of launch_faces for Newton matrix jm
-// (limiter_jacobian), so that W is the same to the bit
-cudaError_t launch_faces_w(const StepParams& P, int jm, const double* E, const double* kap,
-                           double* W, cudaStream_t st);
-cudaError_t launch_schur_kappa(const StepParams& P, int ns, const double* K, const double* fMt,
-                               const double* MiU, double* PQ, double* diag_ns, double* rhs,
-                               cudaStream_t st);
-cudaError_t launch_export_faces(const StepParams& P, const double* W, const double* PQ,
+// Face arrays, times dt theta.  jm (limiter_jacobian) 0: the coefficients W.  1, 2: the fluxes
+// W (E_c - E_lower) into W, the Newton-matrix entries P and Q into PQ (6 N) and, for 2, the opacity
+// terms K.  resid_only: W (fluxes) alone, with the same arithmetic.
+cudaError_t launch_faces(const StepParams& P, int jm, int resid_only, const double* E,
+                         const double* kap, double* W, double* PQ, double* K, cudaStream_t st);
+// The Newton matrix in E of limiter_jacobian 1 or 2 from an evaluated iterate: entries PQ (P then
+// Q per lower face, times dt theta), diagonal and right-hand side, and the finest level of the
+// multigrid hierarchy built from it (f32: the FP32 operator; wid64: omega / diagonal; or neither).
+struct SchurIn {
+    const double *PQ, *K, *dloc, *rhs, *rho, *phi;   // K, rho, phi null: limiter_jacobian 1
+};
+struct SchurOut {
+    double *PQ, *diag, *rhs;
+    float *d32, *wid32, *W32[3], *Wp32[3];
+    double* wid64;
+    double omega;
+};
+cudaError_t launch_schur_assemble(const StepParams& P, const SchurIn& I, const SchurOut& O,
+                                  cudaStream_t st);
+// Schur diagonal of the lagged-D matrix (coefficients W) from the local part dloc of the Newton
+// matrix's
+cudaError_t launch_lagged_diag(const StepParams& P, const double* W, const double* dloc,
+                               const double* E, const double* kap, double* diag, cudaStream_t st);
+cudaError_t launch_export_faces(const StepParams& P, const double* Q, const double* Pf,
                                 double* S_lo, double* S_hi, cudaStream_t st);
 cudaError_t launch_cell(const StepParams& P, int ns, int mode, const PhysBuffers& B,
                         int nblocks, cudaStream_t st);

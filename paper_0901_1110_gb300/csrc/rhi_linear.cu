@@ -3,7 +3,7 @@
 // precision form) or by Jacobi.  Reductions are deterministic: per-block partial sums are
 // added in a fixed order by a single block.
 //
-// Operator of a level: (A x)_c = diag_c x_c - scale * sum_ax (W[ax]_c x_lo + Wp[ax]_hi x_hi),
+// Operator of a level: (A x)_c = diag_c x_c - sum_ax (W[ax]_c x_lo + Wp[ax]_hi x_hi),
 // stored per lower face (0 on zero-flux boundary faces): W couples the upper cell's row to the
 // lower cell, Wp the lower cell's row to the upper cell.  Symmetric levels pass Wp = W.
 #include "rhi_linear.cuh"
@@ -47,8 +47,7 @@ __device__ __forceinline__ void coords_fd(long long c, const FastDiv& fx, const 
     i = (int)(r - jj * fx.d);
 }
 
-// sum over the six neighbours of c of W_face x_neighbour (the off-diagonal part of row c
-// before the scale)
+// sum over the six neighbours of c of W_face x_neighbour (the off-diagonal part of row c)
 template <typename T, typename TX>
 __device__ __forceinline__ T off_row(const Op<T>& A, const TX* __restrict__ x, long long c,
                                      int i, int j, int k) {
@@ -78,14 +77,14 @@ __device__ __forceinline__ T off_row(const Op<T>& A, const TX* __restrict__ x, l
 template <typename T, typename TX>
 __device__ __forceinline__ T apply_row(const Op<T>& A, const TX* __restrict__ x, long long c,
                                        int i, int j, int k, T xc) {
-    return A.diag[c] * xc - A.scale * off_row(A, x, c, i, j, k);
+    return A.diag[c] * xc - off_row(A, x, c, i, j, k);
 }
 
 // one weighted-Jacobi update of cell c from the off-diagonal sum:
-// x + omega (b - A x) / diag = (1 - omega) x + (omega / diag) (b + scale off)
+// x + omega (b - A x) / diag = (1 - omega) x + (omega / diag) (b + off)
 template <typename T>
-__device__ __forceinline__ T jacobi_update(T xc, T b, T wi, T scale, T off, T omega) {
-    return (T(1) - omega) * xc + wi * (b + scale * off);
+__device__ __forceinline__ T jacobi_update(T xc, T b, T wi, T off, T omega) {
+    return (T(1) - omega) * xc + wi * (b + off);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -277,7 +276,7 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_matvec_ns(const OpNS A, const dou
             else if (A.per[ax]) hi = c - (long long)(n[ax] - 1) * s[ax];
             if (hi >= 0) off += A.P[ax][hi] * x[hi];
         }
-        const double v = A.diag[c] * x[c] - A.scale * off;
+        const double v = A.diag[c] * x[c] - off;
         y[c] = v;
         d1 += w1[c] * v;
         if (TWO) d2 += v * v;
@@ -539,7 +538,7 @@ __global__ void __launch_bounds__(RED_BLOCK) k_reduce_loop(const double* __restr
 // multigrid kernels (templated on the level precision)
 
 // weighted Jacobi with wid = omega / diag: first sweep from x = 0: x_out = wid b; else
-// x_out = x_in + omega (b - A x_in) / diag, written as (1 - omega) x_in + wid (b + scale off)
+// x_out = x_in + omega (b - A x_in) / diag, written as (1 - omega) x_in + wid (b + off)
 template <typename T>
 __global__ void __launch_bounds__(LIN_BLOCK) k_mg_smooth(const Op<T> A, const T* __restrict__ b,
                                                          const T* __restrict__ xin,
@@ -555,7 +554,7 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_smooth(const Op<T> A, const T*
             int i, j, k;
             coords3(A, c, i, j, k);
             const T off = off_row(A, xin, c, i, j, k);
-            xout[c] = jacobi_update(xin[c], b[c], wi, A.scale, off, omega);
+            xout[c] = jacobi_update(xin[c], b[c], wi, off, omega);
         }
     }
 }
@@ -658,7 +657,7 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_smooth_zm(const Op<T> A, const
         if (hhi1) off += w1h[kk] * x1h[kk];
         off += wz[kk] * xz[kk];
         if (hz) off += pz[kk] * xz[kk + 2];
-        xout[c0 + (long long)kk * nxy] = jacobi_update(xz[kk + 1], bb[kk], dd[kk], A.scale, off, omega);
+        xout[c0 + (long long)kk * nxy] = jacobi_update(xz[kk + 1], bb[kk], dd[kk], off, omega);
     }
 }
 
@@ -799,7 +798,7 @@ __global__ void __launch_bounds__(BULK_MAX_NX) k_mg_smooth_bulk(const Op<float> 
             off += R2[i] * xlo;
             if (hz) off += Q2[i] * XU[i];
             xout[(long long)j * nx + (long long)k * nxy + i] =
-                jacobi_update(xcen, BB[i], WD[i], A.scale, off, omega);
+                jacobi_update(xcen, BB[i], WD[i], off, omega);
         }
         xlo = xcen;
         __syncthreads();                                    // stage st is free again
@@ -849,7 +848,7 @@ __global__ void __launch_bounds__(COARSE_BLOCK) k_mg_coarse(const Op<T> A, const
                 int i, j, k;
                 coords3(A, c, i, j, k);
                 const T off = off_row(A, xin, c, i, j, k);
-                xout[c] = jacobi_update(xin[c], b[c], wi, A.scale, off, omega);
+                xout[c] = jacobi_update(xin[c], b[c], wi, off, omega);
             }
         }
         __syncthreads();
@@ -860,7 +859,7 @@ __global__ void __launch_bounds__(COARSE_BLOCK) k_mg_coarse(const Op<T> A, const
 // transpose of the injection prolongation scaled by 1/8 (a parent with fewer than 8 children,
 // at an odd extent, keeps the factor, so that the cycle stays symmetric).
 //
-// FP64 and symmetric: with (A x)_c = loc_c x_c + scale sum_faces W (x_c - x_nb), the faces
+// FP64 and symmetric: with (A x)_c = loc_c x_c + sum_faces W (x_c - x_nb), the faces
 // between two children of the parent cancel in the sum, so only the faces to cells outside the
 // parent are evaluated; this halves the FP64 arithmetic that bounds the FP64 instance.  (For a
 // non-symmetric operator the two rows of an inner face carry W and Wp, which do not cancel.)
@@ -911,7 +910,7 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_restrict(const Op<T> A, const 
                                 if (hi >= 0) fl += A.W[ax][hi] * (xc - x[hi]);
                             }
                         }
-                        acc += b[c] - A.loc[c] * xc - A.scale * fl;
+                        acc += b[c] - A.loc[c] * xc - fl;
                     }
                 }
             }
@@ -983,7 +982,7 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_prolong(int nx, int ny, int nz
 }
 
 // Coarse operator by re-discretisation: local diagonal = mean of the children's local
-// diagonals (diag - scale * the six couplings of their rows); each face array of the coarse
+// diagonals (diag - the six couplings of their rows); each face array of the coarse
 // cell's lower face = (mean of that array over the existing fine lower faces of its first-layer
 // children) / 4, W from W and, for a non-symmetric operator, Wp from Wp (wpc null: symmetric).
 // Writes diag_c = local part only; k_mg_diag_faces adds the row's couplings.
@@ -1032,12 +1031,12 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_coarsen(const Op<TF> A, int cn
                             ++nf[ax];
                         }
                     }
-                    dl += (double)A.diag[c] - (double)A.scale * fsum;
+                    dl += (double)A.diag[c] - fsum;
                     ++cnt;
                 }
             }
         }
-        const double sc = (double)A.scale * 0.25;
+        const double sc = 0.25;
         dc[cc] = (TC)(dl / cnt);
         wcx[cc] = (TC)(sc * wl[0] / nf[0]);
         wcy[cc] = (TC)(sc * wl[1] / nf[1]);
@@ -1050,7 +1049,7 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_coarsen(const Op<TF> A, int cn
     }
 }
 
-// diag += sum of the six couplings of the row (scale 1 on coarse levels)
+// diag += sum of the six couplings of the row
 template <typename T>
 __global__ void __launch_bounds__(LIN_BLOCK) k_mg_diag_faces(Op<T> A, T* __restrict__ diag) {
     const long long sz = (long long)A.nx * A.ny;
@@ -1072,30 +1071,21 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_diag_faces(Op<T> A, T* __restr
     }
 }
 
-// FP32 copy of the finest operator with the scale folded into the faces (W and, when the
-// operator is non-symmetric, Wp)
+// FP32 copy of a symmetric finest operator
 __global__ void __launch_bounds__(LIN_BLOCK) k_cast_op(const Op<double> A, float* __restrict__ d,
                                                        float* __restrict__ wx,
                                                        float* __restrict__ wy,
-                                                       float* __restrict__ wz,
-                                                       float* __restrict__ px,
-                                                       float* __restrict__ py,
-                                                       float* __restrict__ pz) {
+                                                       float* __restrict__ wz) {
     for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < A.N;
          c += (long long)gridDim.x * LIN_BLOCK) {
         d[c] = (float)A.diag[c];
-        wx[c] = (float)(A.scale * A.W[0][c]);
-        wy[c] = (float)(A.scale * A.W[1][c]);
-        wz[c] = (float)(A.scale * A.W[2][c]);
-        if (px) {
-            px[c] = (float)(A.scale * A.Wp[0][c]);
-            py[c] = (float)(A.scale * A.Wp[1][c]);
-            pz[c] = (float)(A.scale * A.Wp[2][c]);
-        }
+        wx[c] = (float)A.W[0][c];
+        wy[c] = (float)A.W[1][c];
+        wz[c] = (float)A.W[2][c];
     }
 }
 
-// wid = omega / diag and, where loc is given, loc = diag - scale * (sum of the six couplings of
+// wid = omega / diag and, where loc is given, loc = diag - (sum of the six couplings of
 // the row), in TF
 template <typename TF, typename TO>
 __global__ void __launch_bounds__(LIN_BLOCK) k_mg_level_prep(const Op<TF> A, double omega,
@@ -1119,7 +1109,7 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_level_prep(const Op<TF> A, dou
                 if (q[ax] < n[ax] - 1) f += A.Wp[ax][c + s[ax]];
                 else if (A.per[ax]) f += A.Wp[ax][c - (long long)(n[ax] - 1) * s[ax]];
             }
-            loc[c] = (TO)(d - A.scale * f);
+            loc[c] = (TO)(d - f);
         }
     }
 }
@@ -1387,12 +1377,9 @@ cudaError_t LinLaunch::level_prep(const Op<TF>& A, double omega, TO* wid, TO* lo
     k_mg_level_prep<TF, TO><<<stream_blocks(A.N), LIN_BLOCK, 0, st>>>(A, omega, wid, loc);
     return end();
 }
-cudaError_t LinLaunch::cast_op(const Op<double>& A, float* d, float* const* w, float* const* wp) {
+cudaError_t LinLaunch::cast_op(const Op<double>& A, float* d, float* const* w) {
     begin("mg_cast_op");
-    k_cast_op<<<stream_blocks(A.N), LIN_BLOCK, 0, st>>>(A, d, w[0], w[1], w[2],
-                                                        wp ? wp[0] : nullptr,
-                                                        wp ? wp[1] : nullptr,
-                                                        wp ? wp[2] : nullptr);
+    k_cast_op<<<stream_blocks(A.N), LIN_BLOCK, 0, st>>>(A, d, w[0], w[1], w[2]);
     return end();
 }
 cudaError_t LinLaunch::to_f32(long long N, const double* a, float* b) {

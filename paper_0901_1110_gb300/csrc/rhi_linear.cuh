@@ -8,7 +8,7 @@ namespace rhi {
 // One level's 7-point operator, stored per face: the face below cell c along axis ax carries
 // W[ax][c], the coupling of row c to its lower neighbour, and Wp[ax][c], the coupling of the
 // lower neighbour's row to c:
-//   (A x)_c = diag_c x_c - scale * sum_ax (W[ax]_c x_lo(ax) + Wp[ax]_hi(ax) x_hi(ax)).
+//   (A x)_c = diag_c x_c - sum_ax (W[ax]_c x_lo(ax) + Wp[ax]_hi(ax) x_hi(ax)).
 // A symmetric operator has Wp = W (the same arrays); the Newton matrix that keeps dD/dE has
 // Wp != W.  Both are 0 on zero-flux boundary faces.
 template <typename T>
@@ -20,15 +20,14 @@ struct Op {
     const T* diag;
     const T* W[3];       // per lower face: the coupling of the upper cell's row
     const T* Wp[3];      // per lower face: the coupling of the lower cell's row (= W: symmetric)
-    T scale;
     const T* wid;        // omega / diag, read by the multigrid smoothers
-    const T* loc;        // diag - scale * (sum of the row's six couplings); FP64 levels only
+    const T* loc;        // diag - the sum of the row's six couplings; symmetric FP64 levels only
     const double* skip;  // when not null and *skip != 0 the kernel returns at once (the second
                          // half of a BiCGStab iteration after the solve converged at its middle)
 };
 
 // Non-symmetric 7-point operator (the Schur matrix with dD/dE kept):
-// (A x)_c = diag_c x_c - scale * sum_ax (Q[ax]_c x_lo + P[ax]_hi x_hi), P and Q per lower face.
+// (A x)_c = diag_c x_c - sum_ax (Q[ax]_c x_lo + P[ax]_hi x_hi), P and Q per lower face.
 struct OpNS {
     int nx, ny, nz;
     long long N;
@@ -37,7 +36,6 @@ struct OpNS {
     const double* diag;
     const double* P[3];
     const double* Q[3];
-    double scale;
     const double* skip;  // as Op::skip
 };
 
@@ -148,11 +146,11 @@ struct LinLaunch {
     template <typename T>
     cudaError_t diag_faces(const Op<T>& A, T* diag);
     // per cell of a level: wid = omega / diag (smoothers) and, if loc is not null,
-    // loc = diag - scale * (six faces) (FP64 restriction), evaluated in TF and rounded to TO
+    // loc = diag - (six faces) (FP64 restriction), evaluated in TF and rounded to TO
     template <typename TF, typename TO>
     cudaError_t level_prep(const Op<TF>& A, double omega, TO* wid, TO* loc);
-    // FP32 copy of an FP64 operator with the scale folded into the faces (wp null: symmetric)
-    cudaError_t cast_op(const Op<double>& A, float* d, float* const* w, float* const* wp);
+    // FP32 copy of a symmetric FP64 operator
+    cudaError_t cast_op(const Op<double>& A, float* d, float* const* w);
     cudaError_t to_f32(long long N, const double* a, float* b);
     cudaError_t from_f32_dot(long long N, const float* x, const double* r, double* z,
                              double* part, int& nparts);

@@ -105,7 +105,7 @@ __device__ __forceinline__ FaceCoef face_coef(const StepParams& P, double Ea, do
         r.Q = fma(-v, G, u);
         return r;
     }
-    r.W = C_LIGHT / (3.0 * fmax(0.5 * (ka + kb), P.kappa_floor)) * P.inv_a2dx2;
+    r.W = P.cD / fmax(0.5 * (ka + kb), P.kappa_floor);
     r.P = r.Q = r.W;
     if (JM == 2 && 0.5 * (ka + kb) > P.kappa_floor) r.K = -0.5 * r.W / (0.5 * (ka + kb)) * (Eb - Ea);
     return r;
@@ -115,7 +115,7 @@ __device__ __forceinline__ FaceCoef face_coef(const StepParams& P, double Ea, do
 // the face's opacity is the cell's.  The coefficient is D / (a^2 dx dx/2) with R over that
 // half-cell distance (s = a (dx/2) Ebar); Qd is the cell's Newton-diagonal entry
 // W - dW/dE_c (E_b - E_c) and dWdk = dW/dkappa (exact matrix).
-struct BoundaryFace { double W, Qd, dWdk; };
+struct BoundaryFace { double W, Qd, dWdk; };         // times dt theta
 
 __device__ __forceinline__ BoundaryFace boundary_face(const StepParams& P, double E, double Eb,
                                                       double kap) {
@@ -130,24 +130,24 @@ __device__ __forceinline__ BoundaryFace boundary_face(const StepParams& P, doubl
         const double ks = kap * s;
         const double den = 6.0 * ks * ks + 3.0 * ks * q + q * q;
         const double iden = 1.0 / den;
-        r.W = 2.0 * C_LIGHT * s * (2.0 * ks + q) * iden * P.inv_a2dx2;
+        r.W = s * (2.0 * ks + q) * iden * P.cF;
         r.Qd = r.W;
         if (P.limiter_newton >= 1 && qraw > P.R_min * s) {
-            const double X = -2.0 * C_LIGHT * q * q * (4.0 * ks + q) * iden * iden * P.inv_a2dx2;
+            const double X = -q * q * (4.0 * ks + q) * iden * iden * P.cF;
             r.Qd = r.W + X * s + X * dE * 0.5 * P.half_adx;
         }
-        r.dWdk = -2.0 * C_LIGHT * s * s * (12.0 * ks * ks + 12.0 * ks * q + q * q) * iden * iden *
-                 P.inv_a2dx2;
+        r.dWdk = -s * s * (12.0 * ks * ks + 12.0 * ks * q + q * q) * iden * iden * P.cF;
         return r;
     }
-    r.W = 2.0 * C_LIGHT / (3.0 * fmax(kap, P.kappa_floor)) * P.inv_a2dx2;
+    r.W = 2.0 * P.cD / fmax(kap, P.kappa_floor);
     r.Qd = r.W;
     r.dWdk = kap > P.kappa_floor ? -r.W / kap : 0.0;
     return r;
 }
 
-// WONLY: the coefficients W alone (a trial iterate evaluated for its residual only), by the
-// same arithmetic as the JM kernel's W
+// JM 0: the coefficients W.  JM 1, 2: the fluxes W (E_c - E_lower), which are all the residual
+// needs (each computed once per face instead of by both cells of it), P, Q and K; WONLY: the fluxes
+// alone (a trial iterate evaluated for its residual), by the same arithmetic.
 template <int JM, bool WONLY = false>
 __global__ void __launch_bounds__(256) k_faces(const StepParams P, const double* __restrict__ E,
                                                const double* __restrict__ kap,
@@ -163,8 +163,9 @@ __global__ void __launch_bounds__(256) k_faces(const StepParams P, const double*
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
         FaceCoef f{0.0, 0.0, 0.0, 0.0};
-        if (b.has_lo[ax]) f = face_coef<JM, WONLY>(P, E[b.lo[ax]], Ec, kap[b.lo[ax]], kc);
-        W[ax * P.N + c] = f.W;
+        const double El = E[b.lo[ax]];
+        if (b.has_lo[ax]) f = face_coef<JM, WONLY>(P, El, Ec, kap[b.lo[ax]], kc);
+        W[ax * P.N + c] = JM == 0 ? f.W : f.W * (Ec - El);
         if (PQ) {
             PQv[ax * P.N + c] = f.P;
             PQv[(3 + ax) * P.N + c] = f.Q;
@@ -173,100 +174,148 @@ __global__ void __launch_bounds__(256) k_faces(const StepParams P, const double*
     }
 }
 
-cudaError_t launch_faces(const StepParams& P, const double* E, const double* kap, double* W,
-                         double* PQ, double* K, cudaStream_t st) {
+cudaError_t launch_faces(const StepParams& P, int jm, int resid_only, const double* E,
+                         const double* kap, double* W, double* PQ, double* K, cudaStream_t st) {
     const int b = 256;
     const unsigned g = (unsigned)((P.N + b - 1) / b);
-    if (PQ && K) k_faces<2><<<g, b, 0, st>>>(P, E, kap, W, PQ, K);
-    else if (PQ) k_faces<1><<<g, b, 0, st>>>(P, E, kap, W, PQ, nullptr);
-    else k_faces<0><<<g, b, 0, st>>>(P, E, kap, W, nullptr, nullptr);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_faces_w(const StepParams& P, int jm, const double* E, const double* kap,
-                           double* W, cudaStream_t st) {
-    const int b = 256;
-    const unsigned g = (unsigned)((P.N + b - 1) / b);
+    if (jm == 2 && !resid_only && !K) jm = 1;          // constant opacity: no opacity terms
     if (jm == 0) k_faces<0><<<g, b, 0, st>>>(P, E, kap, W, nullptr, nullptr);
-    else if (jm == 1) k_faces<1, true><<<g, b, 0, st>>>(P, E, kap, W, nullptr, nullptr);
-    else k_faces<2, true><<<g, b, 0, st>>>(P, E, kap, W, nullptr, nullptr);
+    else if (jm == 1 && resid_only) k_faces<1, true><<<g, b, 0, st>>>(P, E, kap, W, nullptr, nullptr);
+    else if (jm == 1) k_faces<1><<<g, b, 0, st>>>(P, E, kap, W, PQ, nullptr);
+    else if (resid_only) k_faces<2, true><<<g, b, 0, st>>>(P, E, kap, W, nullptr, nullptr);
+    else k_faces<2><<<g, b, 0, st>>>(P, E, kap, W, PQ, K);
     return cudaGetLastError();
 }
 
-// Exact Newton matrix: the E row of a cell couples to the species of the cell and of its
-// face neighbours through D's opacity.  After the cell-local elimination
-// dn_j = -M_j^-1 f_M,j - M_j^-1 U_j dE_j, face f (lower cell l, upper cell u, stored at u) adds,
-// with rho_j = sum_X (dkappa/dn_X) (M^-1 U)_j,X and phi_j likewise with M^-1 f_M (scaled),
+// Newton matrix in E.  The diagonal is the local part plus the row's own face entries, P of its
+// lower faces and Q of its upper ones.  In the exact matrix the E row of a cell also couples to the
+// species of the cell and of its face neighbours through D's opacity: after the cell-local
+// elimination dn_j = -M_j^-1 f_M,j - M_j^-1 U_j dE_j, face f (lower cell l, upper cell u, stored at
+// u) adds, with rho_j = sum_X (dkappa/dn_X) (M^-1 U)_j,X and phi_j likewise with M^-1 f_M (scaled),
 //   P_f -= K_f rho_u,  Q_f += K_f rho_l,
-//   diag_u -= dt theta K_f rho_u,  diag_l += dt theta K_f rho_l,
-//   rhs_u += dt theta K_f (phi_l + phi_u),  rhs_l -= dt theta K_f (phi_l + phi_u).
-// Each thread owns its cell's three lower faces, so every write has one writer.
-template <int NS>
-__global__ void __launch_bounds__(256) k_schur_kappa(const StepParams P,
-                                                     const double* __restrict__ K,
-                                                     const double* __restrict__ fMt,
-                                                     const double* __restrict__ MiU,
-                                                     double* __restrict__ PQ,
-                                                     double* __restrict__ diag_ns,
-                                                     double* __restrict__ rhs) {
+//   rhs_u += K_f (phi_l + phi_u),  rhs_l -= K_f (phi_l + phi_u),
+// and the diagonal follows from the changed P and Q.  The cell kernel hands over rho and phi, so a
+// face costs four FMAs here.  Each thread writes its cell's three lower faces, out of place: the
+// cell below reads this cell's original Q and K.  The finest multigrid level, copied from the same
+// entries, is written in the same pass.
+//
+// Bound by the FP64 pipe, with HBM close behind (200 B per cell with the FP32 level).  Measured at
+// 256^3, H + He: 1.21 ms, against 2.68 ms for the in-place opacity coupling that formed rho and phi of
+// every neighbour, the FP32 copy and the omega / diagonal pass that this replaces; the cell
+// kernel without the diagonal's face sums and with one flux per face 7.39 against 8.09 ms.
+template <bool KAPPA, int PC>
+__global__ void __launch_bounds__(256) k_schur_assemble(const StepParams P, const SchurIn I,
+                                                        const SchurOut O) {
     const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const long long N = P.N;
     if (c >= N) return;
     int i, j, k;
     cell_coords(P, c, i, j, k);
     const Nbr b = neighbours(P, c, i, j, k);
-    const double kfac = P.u_n * P.iu_E * P.ia3;     // d kappa / d n_X = sk_X / a^3, scaled
-    auto rho = [&](long long q) {
-        double s = 0.0;
-#pragma unroll
-        for (int X = 0; X < NS; ++X) s += P.sk[X] * MiU[(1 + X) * N + q];
-        return kfac * s;
-    };
-    auto phi = [&](long long q) {
-        double s = 0.0;
-#pragma unroll
-        for (int X = 0; X < NS; ++X) s += P.sk[X] * fMt[(1 + X) * N + q];
-        return kfac * s;
-    };
-    const double rc = rho(c), pc = phi(c);
-    double dd = 0.0, dr = 0.0;
+    double rc = 0.0, pc = 0.0;
+    if (KAPPA) { rc = __ldg(I.rho + c); pc = __ldg(I.phi + c); }
+    double diag = __ldg(I.dloc + c), dr = 0.0;
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
+        double p = 0.0, q = 0.0;
         if (b.has_lo[ax]) {
             const long long l = b.lo[ax];
-            const double Kf = K[ax * N + c];
-            PQ[ax * N + c] -= Kf * rc;
-            PQ[(3 + ax) * N + c] += Kf * rho(l);
-            dd -= Kf * rc;
-            dr += Kf * (phi(l) + pc);
+            p = __ldg(I.PQ + ax * N + c);
+            q = __ldg(I.PQ + (3 + ax) * N + c);
+            if (KAPPA) {
+                const double K = __ldg(I.K + ax * N + c);
+                p = fma(-K, rc, p);
+                q = fma(K, __ldg(I.rho + l), q);
+                dr = fma(K, __ldg(I.phi + l) + pc, dr);
+            }
+            diag += p;
         }
         if (b.has_hi[ax]) {
             const long long h = b.hi[ax];
-            const double Kh = K[ax * N + h];
-            dd += Kh * rc;
-            dr -= Kh * (pc + phi(h));
+            double qh = __ldg(I.PQ + (3 + ax) * N + h);
+            if (KAPPA) {
+                const double K = __ldg(I.K + ax * N + h);
+                qh = fma(K, rc, qh);
+                dr = fma(-K, pc + __ldg(I.phi + h), dr);
+            }
+            diag += qh;
+        }
+        O.PQ[ax * N + c] = p;
+        O.PQ[(3 + ax) * N + c] = q;
+        if (PC == 1) {
+            O.W32[ax][c] = (float)q;
+            O.Wp32[ax][c] = (float)p;
         }
     }
-    diag_ns[c] += P.dth * dd;
-    rhs[c] += P.dth * dr;
+    O.diag[c] = diag;
+    O.rhs[c] = __ldg(I.rhs + c) + dr;
+    if (PC == 1) {
+        O.d32[c] = (float)diag;
+        O.wid32[c] = (float)(O.omega * fast_rcp(diag));
+    }
+    if (PC == 2) O.wid64[c] = O.omega * fast_rcp(diag);
 }
 
-cudaError_t launch_schur_kappa(const StepParams& P, int ns, const double* K, const double* fMt,
-                               const double* MiU, double* PQ, double* diag_ns, double* rhs,
-                               cudaStream_t st) {
+cudaError_t launch_schur_assemble(const StepParams& P, const SchurIn& I, const SchurOut& O,
+                                  cudaStream_t st) {
     const int b = 256;
     const unsigned g = (unsigned)((P.N + b - 1) / b);
-    if (ns == 0) return cudaSuccess;                  // constant opacity: no coupling
-    if (ns == 1) k_schur_kappa<1><<<g, b, 0, st>>>(P, K, fMt, MiU, PQ, diag_ns, rhs);
-    else k_schur_kappa<3><<<g, b, 0, st>>>(P, K, fMt, MiU, PQ, diag_ns, rhs);
+    const int pc = O.d32 ? 1 : (O.wid64 ? 2 : 0);
+    if (I.K) {
+        if (pc == 1) k_schur_assemble<true, 1><<<g, b, 0, st>>>(P, I, O);
+        else if (pc == 2) k_schur_assemble<true, 2><<<g, b, 0, st>>>(P, I, O);
+        else k_schur_assemble<true, 0><<<g, b, 0, st>>>(P, I, O);
+    } else {
+        if (pc == 1) k_schur_assemble<false, 1><<<g, b, 0, st>>>(P, I, O);
+        else if (pc == 2) k_schur_assemble<false, 2><<<g, b, 0, st>>>(P, I, O);
+        else k_schur_assemble<false, 0><<<g, b, 0, st>>>(P, I, O);
+    }
+    return cudaGetLastError();
+}
+
+// Diagonal of the lagged-D matrix (the breakdown fallback, the mg_matrix = 0 hierarchy and the
+// Jacobi preconditioner of a solver that keeps dD/dE): the local part, whose Dirichlet faces carry
+// the Newton entry, plus the coefficients W of the six faces.
+__global__ void k_lagged_diag(const StepParams P, const double* __restrict__ W,
+                              const double* __restrict__ dloc, const double* __restrict__ E,
+                              const double* __restrict__ kap, double* __restrict__ diag) {
+    const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (c >= P.N) return;
+    int i, j, k;
+    cell_coords(P, c, i, j, k);
+    const Nbr b = neighbours(P, c, i, j, k);
+    double d = dloc[c];
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        d += W[ax * P.N + c];
+        if (b.has_hi[ax]) d += W[ax * P.N + b.hi[ax]];
+    }
+    if (P.dir_mask) {
+        const int q[3] = {i, j, k};
+        const int ext[3] = {P.nx, P.ny, P.nz};
+        for (int f = 0; f < 6; ++f) {
+            const int ax = f >> 1;
+            if ((P.dir_mask >> f & 1) && q[ax] == ((f & 1) ? ext[ax] - 1 : 0)) {
+                const BoundaryFace bf = boundary_face(P, E[c], P.Eb[f], kap[c]);
+                d += bf.W - bf.Qd;
+            }
+        }
+    }
+    diag[c] = d;
+}
+
+cudaError_t launch_lagged_diag(const StepParams& P, const double* W, const double* dloc,
+                               const double* E, const double* kap, double* diag, cudaStream_t st) {
+    const int b = 256;
+    k_lagged_diag<<<(unsigned)((P.N + b - 1) / b), b, 0, st>>>(P, W, dloc, E, kap, diag);
     return cudaGetLastError();
 }
 
 // Newton-matrix face entries of each cell for inspection: S_lo[ax] couples a cell to its
 // lower neighbour, S_hi[ax] to its upper neighbour (positive numbers; the matrix entries are
 // their negatives; 0 where the face carries no flux).
-__global__ void k_export_faces(const StepParams P, const double* __restrict__ W,
-                               const double* __restrict__ PQ, double* __restrict__ lo,
+__global__ void k_export_faces(const StepParams P, const double* __restrict__ Q,
+                               const double* __restrict__ Pf, double* __restrict__ lo,
                                double* __restrict__ hi) {
     const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (c >= P.N) return;
@@ -275,17 +324,17 @@ __global__ void k_export_faces(const StepParams P, const double* __restrict__ W,
     const Nbr b = neighbours(P, c, i, j, k);
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
-        const double* Qa = PQ ? PQ + (3 + ax) * P.N : W + ax * P.N;
-        const double* Pa = PQ ? PQ + ax * P.N : W + ax * P.N;
-        lo[ax * P.N + c] = P.dth * Qa[c];
-        hi[ax * P.N + c] = b.has_hi[ax] ? P.dth * Pa[b.hi[ax]] : 0.0;
+        if (lo) lo[ax * P.N + c] = Q[ax * P.N + c];
+        if (hi) hi[ax * P.N + c] = b.has_hi[ax] ? Pf[ax * P.N + b.hi[ax]] : 0.0;
     }
 }
 
-cudaError_t launch_export_faces(const StepParams& P, const double* W, const double* PQ,
+// Q, Pf: the rows' couplings to the lower and from the lower cell per lower face (equal for the
+// lagged-D matrix); S_lo or S_hi may be null
+cudaError_t launch_export_faces(const StepParams& P, const double* Q, const double* Pf,
                                 double* S_lo, double* S_hi, cudaStream_t st) {
     const int b = 256;
-    k_export_faces<<<(unsigned)((P.N + b - 1) / b), b, 0, st>>>(P, W, PQ, S_lo, S_hi);
+    k_export_faces<<<(unsigned)((P.N + b - 1) / b), b, 0, st>>>(P, Q, Pf, S_lo, S_hi);
     return cudaGetLastError();
 }
 
@@ -517,7 +566,10 @@ __device__ __forceinline__ void lu_solve2(double (&A)[NM][NM], double (&y)[NM], 
 // MODE_PREP_PREDICT: writes g^n and the explicit predictor U^n - dt L(U^n) (capped).
 // MODE_RESID:        U given; reads g; writes f(U) only (the same arithmetic as MODE_ITER).
 
-template <int NS, int MODE>
+// FLUX (limiter_jacobian 1, 2): B.W holds the face fluxes, and the Schur diagonal's face entries
+// are left to k_schur_assemble; else B.W holds the coefficients.
+
+template <int NS, int MODE, bool FLUX>
 __global__ void __launch_bounds__(CELL_BLOCK) k_cell(const StepParams P, const PhysBuffers B) {
     constexpr int NM = NS + 1, NV = NS + 2;
     const long long c = blockIdx.x * (long long)CELL_BLOCK + threadIdx.x;
@@ -539,18 +591,17 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_cell(const StepParams P, const P
         const double eh = B.eh[c], nH = B.nH[c], src = B.src[c];
         const double Tfix = P.isothermal ? B.Tiso[c] : 0.0;
 
-        // diffusion: sum over faces W (E_c - E_nb); W sum for the lagged-D diagonal and, with
-        // dD/dE kept, the Newton-matrix diagonal sum (P of own lower faces, Q of upper faces)
-        double Dterm = 0.0, Wsum = 0.0, PQsum = 0.0;
+        // diffusion, times dt theta: sum over faces W (E_c - E_nb); face part of the diagonal
+        double Dterm = 0.0, Wsum = 0.0;
 #pragma unroll
         for (int ax = 0; ax < 3; ++ax) {
             const double wlo = B.W[ax * N + c];
             const double whi = nb.has_hi[ax] ? B.W[ax * N + nb.hi[ax]] : 0.0;
-            Dterm += wlo * (E - En[nb.lo[ax]]) + whi * (E - En[nb.hi[ax]]);
-            Wsum += wlo + whi;
-            if (JAC && B.PQ) {
-                PQsum += B.PQ[ax * N + c];
-                if (nb.has_hi[ax]) PQsum += B.PQ[(3 + ax) * N + nb.hi[ax]];
+            if constexpr (FLUX) {
+                Dterm += wlo - whi;
+            } else {
+                Dterm += wlo * (E - En[nb.lo[ax]]) + whi * (E - En[nb.hi[ax]]);
+                Wsum += wlo + whi;
             }
         }
         // Dirichlet faces of boundary cells (they carry no entry in the face arrays)
@@ -574,8 +625,7 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_cell(const StepParams P, const P
                     const double Eb = P.Eb[d];
                     const BoundaryFace bf = boundary_face(P, E, Eb, kc);
                     Dterm += bf.W * (E - Eb);
-                    Wsum += bf.W;
-                    PQsum += bf.Qd;
+                    Wsum += FLUX ? bf.Qd : bf.W;
                     kb_term += bf.dWdk * (E - Eb);
                 }
             }
@@ -586,7 +636,7 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_cell(const StepParams P, const P
         double Lf[NV];                                      // dt theta L(U)
 #pragma unroll
         for (int v = 0; v <= NS; ++v) Lf[v] = lo.L[v];
-        Lf[NV - 1] = fma(P.dth, Dterm, lo.LE);
+        Lf[NV - 1] = Dterm + lo.LE;
         double U[NV];
         U[0] = ec;
 #pragma unroll
@@ -657,13 +707,15 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_cell(const StepParams P, const P
                     phi = fma(P.ksk[1], y[2], fma(P.ksk[2], y[3], phi));
                 }
                 double cE = P.cdth * E;
-                if (P.limiter_newton == 2) cE = fma(P.dth, kb_term, cE);
+                if (P.limiter_newton == 2) cE += kb_term;
                 LMU = cE * rho;
                 LMf = cE * phi;
+                if (FLUX && B.rho) {
+                    B.rho[c] = rho;
+                    B.phi[c] = phi;
+                }
             }
-            const double Dloc = 1.0 + lo.dLEE;
-            B.diag[c] = Dloc - LMU + P.dth * Wsum;
-            if (B.PQ) B.diag_ns[c] = Dloc - LMU + P.dth * PQsum;
+            B.diag[c] = (1.0 + lo.dLEE) - LMU + Wsum;
             B.rhs[c] = LMf - fs[NV - 1];
 #pragma unroll
             for (int r = 0; r < NM; ++r) {
@@ -679,24 +731,27 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_cell(const StepParams P, const P
     }
 }
 
+template <int NS, bool FLUX>
+static void launch_cell_mode(const StepParams& P, int mode, const PhysBuffers& B, int nblocks,
+                             cudaStream_t st) {
+    const dim3 g(nblocks), b(CELL_BLOCK);
+    if (mode == MODE_PREP) k_cell<NS, MODE_PREP, FLUX><<<g, b, 0, st>>>(P, B);
+    else if (mode == MODE_ITER) k_cell<NS, MODE_ITER, FLUX><<<g, b, 0, st>>>(P, B);
+    else if (mode == MODE_RESID) k_cell<NS, MODE_RESID, FLUX><<<g, b, 0, st>>>(P, B);
+    else k_cell<NS, MODE_PREP_PREDICT, FLUX><<<g, b, 0, st>>>(P, B);
+}
+
 cudaError_t launch_cell(const StepParams& P, int ns, int mode, const PhysBuffers& B,
                         int nblocks, cudaStream_t st) {
-    const dim3 g(nblocks), b(CELL_BLOCK);
     if (ns == 0) {
-        if (mode == MODE_PREP) k_cell<0, MODE_PREP><<<g, b, 0, st>>>(P, B);
-        else if (mode == MODE_ITER) k_cell<0, MODE_ITER><<<g, b, 0, st>>>(P, B);
-        else if (mode == MODE_RESID) k_cell<0, MODE_RESID><<<g, b, 0, st>>>(P, B);
-        else k_cell<0, MODE_PREP_PREDICT><<<g, b, 0, st>>>(P, B);
+        if (B.flux) launch_cell_mode<0, true>(P, mode, B, nblocks, st);
+        else launch_cell_mode<0, false>(P, mode, B, nblocks, st);
     } else if (ns == 1) {
-        if (mode == MODE_PREP) k_cell<1, MODE_PREP><<<g, b, 0, st>>>(P, B);
-        else if (mode == MODE_ITER) k_cell<1, MODE_ITER><<<g, b, 0, st>>>(P, B);
-        else if (mode == MODE_RESID) k_cell<1, MODE_RESID><<<g, b, 0, st>>>(P, B);
-        else k_cell<1, MODE_PREP_PREDICT><<<g, b, 0, st>>>(P, B);
+        if (B.flux) launch_cell_mode<1, true>(P, mode, B, nblocks, st);
+        else launch_cell_mode<1, false>(P, mode, B, nblocks, st);
     } else {
-        if (mode == MODE_PREP) k_cell<3, MODE_PREP><<<g, b, 0, st>>>(P, B);
-        else if (mode == MODE_ITER) k_cell<3, MODE_ITER><<<g, b, 0, st>>>(P, B);
-        else if (mode == MODE_RESID) k_cell<3, MODE_RESID><<<g, b, 0, st>>>(P, B);
-        else k_cell<3, MODE_PREP_PREDICT><<<g, b, 0, st>>>(P, B);
+        if (B.flux) launch_cell_mode<3, true>(P, mode, B, nblocks, st);
+        else launch_cell_mode<3, false>(P, mode, B, nblocks, st);
     }
     return cudaGetLastError();
 }
