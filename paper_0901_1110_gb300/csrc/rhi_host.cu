@@ -269,6 +269,7 @@ StepParams make_params(const rhi_ctx* h, double dt, double a, double adot) {
     P.dtm1_dth = (h->prm.theta - 1.0) / h->prm.theta;
     P.dt_dth = 1.0 / h->prm.theta;
     P.tau = h->prm.tau;
+    P.tau_tiny = 1e-13 * P.tau;
     P.lte = h->prm.model == RHI_MODEL_LTE;
     P.kappa_total = h->prm.kappa_total;
     P.kappa_planck = h->prm.kappa_planck;

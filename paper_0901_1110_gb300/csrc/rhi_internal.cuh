@@ -71,7 +71,7 @@ struct StepParams {
     double cz[3], ksk[3];
     double dtm1_dth, dt_dth;          // (theta - 1) / theta, 1 / theta
     double sk[3], pg[3], ph[3];
-    double tau;
+    double tau, tau_tiny;             // positivity cap: tau, 1e-13 tau
     // LTE coupling (eq. LTE_coupling; no species): constant opacities, T = lte_cT e
     int lte;
     double kappa_total, kappa_planck, lte_cT;
