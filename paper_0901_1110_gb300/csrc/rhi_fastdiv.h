@@ -3,9 +3,9 @@
 // Granlund & Montgomery, "Division by invariant integers using multiplication" (PLDI 1994),
 // Theorem 4.2: for N-bit numerators and a divisor d >= 1, with l = ceil(log2 d),
 // s = N + l and m = ceil(2^s / d), floor(n / d) = floor(n m / 2^s) for every 0 <= n < 2^N.
-// Cell indices are below 2^31 (N = 31), so m <= 2^32 and n m < 2^63: one 64-bit multiply and a
-// shift replace the ~70-instruction 64-bit integer division of the stencil kernels' index
-// arithmetic.
+// Cell indices are below 2^31 (N = 31), and d > 2^(l-1) puts m below 2^32: one 32 x 32 -> 64-bit
+// multiply and a shift replace the ~70-instruction 64-bit integer division of the stencil kernels'
+// index arithmetic.
 #pragma once
 
 #ifdef __CUDACC__
@@ -17,7 +17,7 @@
 namespace rhi {
 
 struct FastDiv {
-    unsigned long long m;   // ceil(2^s / d)
+    unsigned m;             // ceil(2^s / d)
     unsigned s;             // 31 + ceil(log2 d)
     unsigned d;
 };
@@ -28,7 +28,7 @@ inline FastDiv make_fastdiv(unsigned d) {
     FastDiv f;
     f.d = d;
     f.s = 31 + l;
-    f.m = ((1ULL << f.s) + d - 1) / d;
+    f.m = (unsigned)(((1ULL << f.s) + d - 1) / d);
     return f;
 }
 

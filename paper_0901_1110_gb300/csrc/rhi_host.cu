@@ -142,6 +142,7 @@ struct rhi_ctx {
     // multigrid
     std::vector<Level<double>> mg64;
     std::vector<Level<float>> mg32;
+    int tail_blocks[2] = {0, 0};          // cluster size of the coarse-end kernel, FP32 and FP64
     // the lagged-D Schur matrix, the Newton matrix when dD/dE is kept, and the finest operator
     // the preconditioner was last set up from (one of the two; pc_nonsym: the Newton matrix)
     Op<double> op0{};
@@ -448,6 +449,27 @@ int precond_setup_newton(rhi_ctx* h) {
     return precond_setup(h, nonsym ? newton_op(h) : h->op0, nonsym);
 }
 
+// the levels from l on run as one launch: few enough cells for one cluster
+template <typename T>
+bool tail_at(const rhi_ctx* h, const std::vector<Level<T>>& lv, size_t l) {
+    return mg_tail_fits<T>(lv[l].N, l + 1 < lv.size() ? lv[l + 1].N : 0, h->tail_blocks[sizeof(T) == 8]) &&
+           lv.size() - l <= (size_t)MG_TAIL_LEVELS;
+}
+template <typename T>
+MgTail<T> tail_from(const rhi_ctx* h, const std::vector<Level<T>>& lv, size_t l, const Op<T>& A0,
+                    const T* b, const double* b64, T* x, double* x64) {
+    MgTail<T> M{};
+    M.n = (int)(lv.size() - l);
+    M.blocks = h->tail_blocks[sizeof(T) == 8];
+    for (int q = 0; q < M.n; ++q) M.op[q] = l + q == 0 ? A0 : level_op(h, lv[l + q]);
+    M.pre = h->prm.mg_pre;
+    M.post = h->prm.mg_post;
+    M.coarse = h->prm.mg_coarse_sweeps;
+    M.omega = (T)h->prm.mg_omega;
+    M.b = b; M.b64 = b64; M.x = x; M.x64 = x64;
+    return M;
+}
+
 // one V-cycle on levels l.. with right-hand side lv[l].b; result in lv[l].x
 template <typename T>
 int vcycle(rhi_ctx* h, std::vector<Level<T>>& lv, size_t l, const Op<T>& A0,
@@ -459,13 +481,12 @@ int vcycle(rhi_ctx* h, std::vector<Level<T>>& lv, size_t l, const Op<T>& A0,
     Level<T>& v = lv[l];
     const Op<T> A = (l == 0) ? A0 : level_op(h, v);
     const T om = (T)h->prm.mg_omega;
+    if (tail_at(h, lv, l)) {
+        // this level and all below it in one launch
+        CK(L.mg_tail<T>(tail_from(h, lv, l, A0, v.b, nullptr, v.x, nullptr)));
+        return RHI_OK;
+    }
     if (l + 1 == lv.size()) {
-        if (v.N <= COARSE_MAX) {
-            // all sweeps in one launch; x and xt alternate as in the loop below
-            CK(L.coarse_solve<T>(A, v.b, v.x, v.xt, om, h->prm.mg_coarse_sweeps));
-            if ((h->prm.mg_coarse_sweeps - 1) % 2) std::swap(v.x, v.xt);
-            return RHI_OK;
-        }
         CK(L.smooth<T>(A, v.b, v.x, v.x, om, 1));
         for (int s = 1; s < h->prm.mg_coarse_sweeps; ++s) {
             CK(L.smooth<T>(A, v.b, v.x, v.xt, om, 0));
@@ -583,8 +604,15 @@ int precond_apply(rhi_ctx* h, const double* r, double** zout, int& nparts) {
         CK(L.dot(N, r, h->z, h->partials, nparts));
     } else {
         auto& lv = h->mg32;
-        CK(L.to_f32(N, r, lv[0].b));
         Op<float> A0 = level_op(h, lv[0]);
+        if (tail_at(h, lv, 0)) {                         // the whole cycle and its conversions
+            CK(L.mg_tail<float>(tail_from<float>(h, lv, 0, A0, nullptr, r, nullptr, h->z)));
+            CK(L.dot(N, r, h->z, h->partials, nparts));
+            *zout = h->z;
+            h->stats.vcycles += 1;
+            return RHI_OK;
+        }
+        CK(L.to_f32(N, r, lv[0].b));
         int rc = vcycle_graph_usable(h) ? vcycle_graph(h, A0) : vcycle<float>(h, lv, 0, A0);
         if (rc) return rc;
         CK(L.from_f32_dot(N, lv[0].x, r, h->z, h->partials, nparts));
@@ -651,6 +679,10 @@ int precond_into(rhi_ctx* h, LinLaunch& L, const double* r, double* dest) {
         lv[0].xt = xt0;
     } else {
         auto& lv = h->mg32;
+        if (tail_at(h, lv, 0)) {                         // the whole cycle and its conversions
+            CK(L.mg_tail<float>(tail_from<float>(h, lv, 0, level_op(h, lv[0]), nullptr, r, nullptr, dest)));
+            return RHI_OK;
+        }
         CK(L.to_f32(N, r, lv[0].b));
         int rc = vcycle<float>(h, lv, 0, level_op(h, lv[0]), L.st, L.hook, L.skip);
         if (rc) return rc;
@@ -1177,6 +1209,7 @@ int rhi_create(const rhi_grid* grid, const rhi_bc* bc, const rhi_params* params,
         if (!rc) {
             *h->h_kerr = 0;
             e = linear_kernels_init();
+            if (e == cudaSuccess) e = mg_tail_init(&h->tail_blocks[0], &h->tail_blocks[1]);
             if (e != cudaSuccess) rc = fail(h, RHI_ERR_CUDA, std::string("multigrid kernels: ") + cudaGetErrorString(e));
         }
     }

@@ -828,33 +828,6 @@ cudaError_t bulk_wait_flag_clear(cudaStream_t st) {
     return cudaMemcpyToSymbolAsync(g_bulk_wait_error, &zero, sizeof(int), 0, cudaMemcpyHostToDevice, st);
 }
 
-// all Jacobi sweeps of the coarsest level in one CTA: the same arithmetic as that many
-// k_mg_smooth launches (first sweep from x = 0 into x, then x and xt alternate), with a block
-// barrier in place of each kernel boundary
-constexpr int COARSE_BLOCK = 1024;
-template <typename T>
-__global__ void __launch_bounds__(COARSE_BLOCK) k_mg_coarse(const Op<T> A, const T* __restrict__ b,
-                                                            T* x, T* xt, T omega, int sweeps) {
-    if (skipped(A.skip)) return;
-    T* buf[2] = {x, xt};
-    for (int s = 0; s < sweeps; ++s) {
-        const T* xin = buf[(s + 1) & 1];
-        T* xout = buf[s & 1];
-        for (long long c = threadIdx.x; c < A.N; c += COARSE_BLOCK) {
-            const T wi = A.wid[c];
-            if (s == 0) {
-                xout[c] = wi * b[c];
-            } else {
-                int i, j, k;
-                coords3(A, c, i, j, k);
-                const T off = off_row(A, xin, c, i, j, k);
-                xout[c] = jacobi_update(xin[c], b[c], wi, off, omega);
-            }
-        }
-        __syncthreads();
-    }
-}
-
 // coarse right-hand side: (sum over the children of the fine residual b - A x) / 8, the
 // transpose of the injection prolongation scaled by 1/8 (a parent with fewer than 8 children,
 // at an odd extent, keeps the factor, so that the cycle stays symmetric).
@@ -1318,14 +1291,6 @@ cudaError_t LinLaunch::smooth(const Op<T>& A, const T* b, const T* xin, T* xout,
     return end();
 }
 template <typename T>
-cudaError_t LinLaunch::coarse_solve(const Op<T>& A, const T* b, T* x, T* xt, T omega, int sweeps) {
-    begin(sizeof(T) == 4 ? "mg_coarse_f32" : "mg_coarse_f64");
-    Op<T> B = A;
-    B.skip = skip;
-    k_mg_coarse<T><<<1, COARSE_BLOCK, 0, st>>>(B, b, x, xt, omega, sweeps);
-    return end();
-}
-template <typename T>
 cudaError_t LinLaunch::restrict_res(const Op<T>& A, const T* b, const T* x, int cnx, int cny,
                                     int cnz, T* bc) {
     if (A.N == fine_N) begin(sizeof(T) == 4 ? "mg_restrict_f32_fine" : "mg_restrict_f64_fine");
@@ -1402,10 +1367,6 @@ template cudaError_t LinLaunch::smooth<double>(const Op<double>&, const double*,
                                                double*, double, int);
 template cudaError_t LinLaunch::smooth<float>(const Op<float>&, const float*, const float*,
                                               float*, float, int);
-template cudaError_t LinLaunch::coarse_solve<double>(const Op<double>&, const double*, double*,
-                                                     double*, double, int);
-template cudaError_t LinLaunch::coarse_solve<float>(const Op<float>&, const float*, float*, float*,
-                                                    float, int);
 template cudaError_t LinLaunch::restrict_res<double>(const Op<double>&, const double*,
                                                      const double*, int, int, int, double*);
 template cudaError_t LinLaunch::restrict_res<float>(const Op<float>&, const float*, const float*,

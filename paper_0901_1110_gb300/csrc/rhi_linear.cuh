@@ -39,8 +39,25 @@ struct OpNS {
     const double* skip;  // as Op::skip
 };
 
-// largest level solved by one single-CTA launch (all coarse sweeps)
-constexpr long long COARSE_MAX = 8192;
+// The coarse end of a V-cycle as one launch (rhi_mgtail.cu): up to MG_TAIL_LEVELS levels within
+// MG_TAIL_SMEM bytes of shared memory per block (at most 3 values of 2048 + 512 x 16 levels).
+// mg_tail_fits: a level of N cells, the next of N_next (0: none), can start it.  mg_tail_init: the
+// blocks of the cluster on the current device; called for every handle.
+constexpr int MG_TAIL_LEVELS = 18;
+constexpr int MG_TAIL_SMEM = 128 * 1024;
+template <typename T> bool mg_tail_fits(long long N, long long N_next, int blocks);
+template <typename T>
+struct MgTail {
+    Op<T> op[MG_TAIL_LEVELS];
+    int n, blocks;
+    int pre, post, coarse;      // sweeps
+    T omega;
+    const T* b;                 // right-hand side of the first level, or in FP64 (b64)
+    const double* b64;
+    T* x;                       // result, in T and / or FP64
+    double* x64;
+};
+cudaError_t mg_tail_init(int* blocks32, int* blocks64);
 
 // device scalar slots of the Krylov iterations.  The BiCGStab loop keeps its control state
 // on the device: S_THR (converged when r.r <= S_THR), S_MAXIT, the iteration count S_ITS, S_DONE
@@ -129,10 +146,8 @@ struct LinLaunch {
 
     template <typename T>
     cudaError_t smooth(const Op<T>& A, const T* b, const T* xin, T* xout, T omega, int first);
-    // every sweep of a level of at most COARSE_MAX cells in one single-CTA launch; the result
-    // ends in x when sweeps is odd, else in xt
     template <typename T>
-    cudaError_t coarse_solve(const Op<T>& A, const T* b, T* x, T* xt, T omega, int sweeps);
+    cudaError_t mg_tail(const MgTail<T>& M);
     template <typename T>
     cudaError_t restrict_res(const Op<T>& A, const T* b, const T* x, int cnx, int cny, int cnz,
                              T* bc);
