@@ -409,9 +409,8 @@ int precond_setup(rhi_ctx* h, const Op<double>& A0, bool nonsym) {
         for (size_t l = 0; l + 1 < lv.size(); ++l) {
             Op<double> A = (l == 0) ? h->pc0 : level_op(h, lv[l]);
             auto& c = lv[l + 1];
-            CK((L.coarsen<double, double>(A, c.nx, c.ny, c.nz, c.diag, c.W, nonsym ? c.Wp : nullptr)));
-            CK(L.diag_faces<double>(level_op(h, c), c.diag));
-            CK((L.level_prep<double, double>(level_op(h, c), om, c.wid, c.loc)));
+            CK((L.build_level<double, double>(A, c.nx, c.ny, c.nz, om, c.diag, c.wid, nonsym ? nullptr : c.loc,
+                                              c.W, nonsym ? c.Wp : nullptr)));
         }
     } else if (h->prm.precond == RHI_PRECOND_MG_FP32) {
         auto& lv = h->mg32;
@@ -425,12 +424,11 @@ int precond_setup(rhi_ctx* h, const Op<double>& A0, bool nonsym) {
         }
         for (size_t l = 0; l + 1 < lv.size(); ++l) {
             auto& c = lv[l + 1];
+            float* const* wp = nonsym ? c.Wp : nullptr;
             if (l == 0)
-                CK((L.coarsen<double, float>(h->pc0, c.nx, c.ny, c.nz, c.diag, c.W, nonsym ? c.Wp : nullptr)));
+                CK((L.build_level<double, float>(h->pc0, c.nx, c.ny, c.nz, om, c.diag, c.wid, nullptr, c.W, wp)));
             else
-                CK((L.coarsen<float, float>(level_op(h, lv[l]), c.nx, c.ny, c.nz, c.diag, c.W, nonsym ? c.Wp : nullptr)));
-            CK(L.diag_faces<float>(level_op(h, c), c.diag));
-            CK((L.level_prep<float, float>(level_op(h, c), om, c.wid, nullptr)));
+                CK((L.build_level<float, float>(level_op(h, lv[l]), c.nx, c.ny, c.nz, om, c.diag, c.wid, nullptr, c.W, wp)));
         }
     }
     return RHI_OK;

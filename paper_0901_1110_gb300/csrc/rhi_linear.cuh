@@ -153,14 +153,12 @@ struct LinLaunch {
                              T* bc);
     template <typename T>
     cudaError_t prolong(int nx, int ny, int nz, int cnx, int cny, const T* xc, T* xf);
-    // coarse operator of A: diagonal dc (local part; diag_faces adds the couplings), W-type
-    // face arrays wc[3] and, for a non-symmetric A, Wp-type face arrays wpc[3] (else null)
+    // coarse level of A: diagonal dc, wid = omega / diagonal, loc (may be null) the diagonal's local
+    // part, W-type face arrays wc[3] and, for a non-symmetric A, Wp-type face arrays wpc[3] (else null)
     template <typename TF, typename TC>
-    cudaError_t coarsen(const Op<TF>& A, int cnx, int cny, int cnz, TC* dc, TC* const* wc,
-                        TC* const* wpc);
-    template <typename T>
-    cudaError_t diag_faces(const Op<T>& A, T* diag);
-    // per cell of a level: wid = omega / diag (smoothers) and, if loc is not null,
+    cudaError_t build_level(const Op<TF>& A, int cnx, int cny, int cnz, double omega, TC* dc, TC* wid,
+                            TC* loc, TC* const* wc, TC* const* wpc);
+    // finest level of a symmetric operator: wid = omega / diag (smoothers) and, if loc is not null,
     // loc = diag - (six faces) (FP64 restriction), evaluated in TF and rounded to TO
     template <typename TF, typename TO>
     cudaError_t level_prep(const Op<TF>& A, double omega, TO* wid, TO* loc);
