@@ -122,6 +122,9 @@ def alg_bytes(nonsym):
         "bicg_update_xr": 8 * 6 + 8 * 2,
         "bicg_update_p": 8 * 3 + 8,
         "bicg_update_s": 8 * 2 + 8,
+        # with the FP32 multigrid p and s are also written in FP32
+        "bicg_update_p_f32": 8 * 3 + 8 + 4,
+        "bicg_update_s_f32": 8 * 2 + 8 + 4,
         "kappa": 8 * 3 + 8,
         # weighted-Jacobi sweep on the finest level: x, b, omega / diag and the face arrays
         # read, x written; the first sweep of a cycle starts from x = 0: b, omega / diag read
@@ -147,7 +150,8 @@ def alg_bytes(nonsym):
 # the stencil / vector kernels of the Krylov solver and the multigrid preconditioner whose HBM
 # fraction is reported per form
 LINEAR_KERNELS = ("cg_matvec_dot", "cg_update_xr", "cg_update_p", "bicg_matvec",
-                  "bicg_update_xr", "bicg_update_p", "bicg_update_s", "mg_smooth_f32_fine",
+                  "bicg_update_xr", "bicg_update_p", "bicg_update_s", "bicg_update_p_f32",
+                  "bicg_update_s_f32", "mg_smooth_f32_fine",
                   "mg_smooth_f32_fine_first", "mg_smooth_f64_fine", "mg_smooth_f64_fine_first",
                   "mg_restrict_f32_fine", "mg_restrict_f64_fine", "mg_prolong_f32_fine",
                   "mg_prolong_f64_fine", "mg_to_f32", "mg_from_f32", "mg_from_f32_dot")

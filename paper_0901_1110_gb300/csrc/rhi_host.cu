@@ -136,6 +136,7 @@ struct rhi_ctx {
     double *rh = nullptr, *v = nullptr, *s = nullptr, *t = nullptr, *ph = nullptr, *sh = nullptr;
     double* partials = nullptr;
     double* scal = nullptr;
+    unsigned* red_count = nullptr;        // tickets of the kernels that end with a sum
     double* h_scal = nullptr;   // pinned
     int* d_flag = nullptr;
     double2* table = nullptr;
@@ -294,10 +295,14 @@ int read_scalar(rhi_ctx* h, int slot, double* out) {
     return RHI_OK;
 }
 
-// ||f||_RMS from the cell kernel's partials
+// The cell kernel's last block sums its partials up to this many blocks (10^6 cells); beyond, one
+// block of 1024 threads does it faster in a launch of its own (15 us at 256^3).
+constexpr int CELL_SUM_BLOCKS = 8192;
+
+// ||f||_RMS from the cell kernel's sum or partials
 int residual_norm(rhi_ctx* h, int nparts, double* out) {
     LinLaunch L(h->st, &h->prof);
-    CK(L.reduce(h->partials, nparts, h->scal, RED_SUM, S_TMP));
+    if (nparts > CELL_SUM_BLOCKS) CK(L.reduce(h->partials, nparts, h->scal, RED_SUM, S_TMP));
     double s;
     int rc = read_scalar(h, S_TMP, &s);
     if (rc) return rc;
@@ -468,10 +473,12 @@ MgTail<T> tail_from(const rhi_ctx* h, const std::vector<Level<T>>& lv, size_t l,
     return M;
 }
 
-// one V-cycle on levels l.. with right-hand side lv[l].b; result in lv[l].x
+// one V-cycle on levels l.. with right-hand side lv[l].b; result in lv[l].x, or with out64 in that
+// vector (by the last sweep)
 template <typename T>
 int vcycle(rhi_ctx* h, std::vector<Level<T>>& lv, size_t l, const Op<T>& A0,
-           cudaStream_t st = nullptr, LaunchHook* hook = nullptr, const double* skip = nullptr) {
+           cudaStream_t st = nullptr, LaunchHook* hook = nullptr, const double* skip = nullptr,
+           double* out64 = nullptr) {
     if (!hook) { st = h->st; hook = &h->prof; }
     LinLaunch L(st, hook);
     L.fine_N = h->N;
@@ -490,6 +497,8 @@ int vcycle(rhi_ctx* h, std::vector<Level<T>>& lv, size_t l, const Op<T>& A0,
             CK(L.smooth<T>(A, v.b, v.x, v.xt, om, 0));
             std::swap(v.x, v.xt);
         }
+        if constexpr (sizeof(T) == 4)
+            if (out64) CK(L.from_f32(v.N, v.x, out64));
         return RHI_OK;
     }
     CK(L.smooth<T>(A, v.b, v.x, v.x, om, 1));
@@ -505,9 +514,11 @@ int vcycle(rhi_ctx* h, std::vector<Level<T>>& lv, size_t l, const Op<T>& A0,
     // separate prolongation and sweep at 256^3, so the two stay separate)
     CK(L.prolong<T>(v.nx, v.ny, v.nz, c.nx, c.ny, c.x, v.x));
     for (int s = 0; s < h->prm.mg_post; ++s) {
-        CK(L.smooth<T>(A, v.b, v.x, v.xt, om, 0));
+        CK(L.smooth<T>(A, v.b, v.x, v.xt, om, 0, s == h->prm.mg_post - 1 ? out64 : nullptr));
         std::swap(v.x, v.xt);
     }
+    if constexpr (sizeof(T) == 4)
+        if (out64 && !h->prm.mg_post) CK(L.from_f32(v.N, v.x, out64));
     return RHI_OK;
 }
 
@@ -581,12 +592,20 @@ int vcycle_graph(rhi_ctx* h, const Op<float>& A0) {
     return RHI_OK;
 }
 
-// z = M^-1 r, and r.z into the partials; returns the partial count
-int precond_apply(rhi_ctx* h, const double* r, double** zout, int& nparts) {
+// what the last block of a kernel with a sum does with it
+Finish fin(const rhi_ctx* h, int op, int slot = 0, unsigned long long cond = 0) {
+    Finish F;
+    F.partials = h->partials; F.count = h->red_count; F.scal = h->scal;
+    F.op = op; F.slot = slot; F.cond = cond;
+    return F;
+}
+
+// z = M^-1 r, and the scalar update of r.z
+int precond_apply(rhi_ctx* h, const double* r, double** zout, const Finish& F) {
     LinLaunch L(h->st, &h->prof);
     const long long N = h->N;
     if (h->prm.precond == RHI_PRECOND_JACOBI) {
-        CK(L.jacobi_dot(N, r, h->pc0.diag, h->z, h->partials, nparts));
+        CK(L.jacobi_dot(N, r, h->pc0.diag, h->z, F));
         *zout = h->z;
     } else if (h->prm.precond == RHI_PRECOND_MG_FP64) {
         auto& lv = h->mg64;
@@ -599,13 +618,13 @@ int precond_apply(rhi_ctx* h, const double* r, double** zout, int& nparts) {
         if (R != h->z) { lv[0].xt = h->z; h->z = R; }
         *zout = h->z;
         lv[0].x = nullptr;
-        CK(L.dot(N, r, h->z, h->partials, nparts));
+        CK(L.dot(N, r, h->z, F));
     } else {
         auto& lv = h->mg32;
         Op<float> A0 = level_op(h, lv[0]);
         if (tail_at(h, lv, 0)) {                         // the whole cycle and its conversions
             CK(L.mg_tail<float>(tail_from<float>(h, lv, 0, A0, nullptr, r, nullptr, h->z)));
-            CK(L.dot(N, r, h->z, h->partials, nparts));
+            CK(L.dot(N, r, h->z, F));
             *zout = h->z;
             h->stats.vcycles += 1;
             return RHI_OK;
@@ -613,7 +632,7 @@ int precond_apply(rhi_ctx* h, const double* r, double** zout, int& nparts) {
         CK(L.to_f32(N, r, lv[0].b));
         int rc = vcycle_graph_usable(h) ? vcycle_graph(h, A0) : vcycle<float>(h, lv, 0, A0);
         if (rc) return rc;
-        CK(L.from_f32_dot(N, lv[0].x, r, h->z, h->partials, nparts));
+        CK(L.from_f32_dot(N, lv[0].x, r, h->z, F));
         *zout = h->z;
     }
     h->stats.vcycles += 1;
@@ -625,30 +644,24 @@ int pcg(rhi_ctx* h, const double* rhs, double tol, int* its_out) {
     LinLaunch L(h->st, &h->prof);
     const long long N = h->N;
     const double norm = 1.0 / ((double)N * h->nv);
-    int np = 0;
     CK(cudaMemsetAsync(h->scal + S_BREAK, 0, sizeof(double), h->st));     // clear an old breakdown
-    CK(L.cg_init(N, rhs, h->r, h->x, h->partials, np));
-    CK(L.reduce(h->partials, np, h->scal, RED_SUM, S_RR));
+    CK(L.cg_init(N, rhs, h->r, h->x, fin(h, RED_SUM, S_RR)));
     double rr;
     int rc = read_scalar(h, S_RR, &rr);
     if (rc) return rc;
     int its = 0;
     if (std::sqrt(rr * norm) > tol) {
         double* z = nullptr;
-        if ((rc = precond_apply(h, h->r, &z, np))) return rc;
-        CK(L.reduce(h->partials, np, h->scal, RED_SUM, S_RZ));
+        if ((rc = precond_apply(h, h->r, &z, fin(h, RED_SUM, S_RZ)))) return rc;
         CK(L.cg_p(N, h->scal, z, h->p, 1));
         for (its = 1; its <= h->prm.max_pcg; ++its) {
-            CK(L.matvec_dot(h->op0, h->p, h->q, h->partials, np));
-            CK(L.reduce(h->partials, np, h->scal, RED_ALPHA, 0));
-            CK(L.cg_xr(N, h->scal, h->x, h->r, h->p, h->q, h->partials, np));
-            CK(L.reduce(h->partials, np, h->scal, RED_SUM, S_RR));
+            CK(L.matvec_dot(h->op0, h->p, h->q, fin(h, RED_ALPHA)));
+            CK(L.cg_xr(N, h->scal, h->x, h->r, h->p, h->q, fin(h, RED_SUM, S_RR)));
             if ((rc = read_scalar(h, S_RR, &rr))) return rc;
             if (h->h_scal[S_BREAK] != 0.0 || !std::isfinite(rr))
                 return fail(h, RHI_ERR_NONPHYSICAL, "CG breakdown: p.Sp <= 0 or non-finite residual");
             if (std::sqrt(rr * norm) <= tol) break;
-            if ((rc = precond_apply(h, h->r, &z, np))) return rc;
-            CK(L.reduce(h->partials, np, h->scal, RED_BETA, 0));
+            if ((rc = precond_apply(h, h->r, &z, fin(h, RED_BETA)))) return rc;
             CK(L.cg_p(N, h->scal, z, h->p, 0));
         }
         if (its > h->prm.max_pcg) its = h->prm.max_pcg;
@@ -657,14 +670,19 @@ int pcg(rhi_ctx* h, const double* rhs, double tol, int* its_out) {
     return RHI_OK;
 }
 
-// M^-1 r into dest with the launcher's stream, hook and skip flag (the second half of a
-// BiCGStab iteration); the V-cycle's kernels are launched one by one (also while a graph is
-// being captured)
+// the FP32 copy of a vector the FP32 cycle takes as its right-hand side (null: none; a cycle that is
+// one launch reads the FP64 vector)
+float* cycle_rhs(const rhi_ctx* h) {
+    if (h->prm.precond != RHI_PRECOND_MG_FP32 || tail_at(h, h->mg32, 0)) return nullptr;
+    return h->mg32[0].b;
+}
+
+// M^-1 r into dest with the launcher's stream, hook and skip flag (an iteration of BiCGStab; the
+// FP32 copy of r is in place where cycle_rhs names one); the V-cycle's kernels are launched one by one (also while a graph is being captured)
 int precond_into(rhi_ctx* h, LinLaunch& L, const double* r, double* dest) {
     const long long N = h->N;
     if (h->prm.precond == RHI_PRECOND_JACOBI) {
-        int np = 0;
-        CK(L.jacobi_dot(N, r, h->pc0.diag, dest, h->partials, np));
+        CK(L.jacobi_dot(N, r, h->pc0.diag, dest, fin(h, RED_NONE)));
     } else if (h->prm.precond == RHI_PRECOND_MG_FP64) {
         auto& lv = h->mg64;
         double* xt0 = lv[0].xt;
@@ -677,24 +695,23 @@ int precond_into(rhi_ctx* h, LinLaunch& L, const double* r, double* dest) {
         lv[0].xt = xt0;
     } else {
         auto& lv = h->mg32;
-        if (tail_at(h, lv, 0)) {                         // the whole cycle and its conversions
+        if (!cycle_rhs(h)) {
             CK(L.mg_tail<float>(tail_from<float>(h, lv, 0, level_op(h, lv[0]), nullptr, r, nullptr, dest)));
             return RHI_OK;
         }
-        CK(L.to_f32(N, r, lv[0].b));
-        int rc = vcycle<float>(h, lv, 0, level_op(h, lv[0]), L.st, L.hook, L.skip);
+        float *x0 = lv[0].x, *xt0 = lv[0].xt;
+        int rc = vcycle<float>(h, lv, 0, level_op(h, lv[0]), L.st, L.hook, L.skip, dest);
+        lv[0].x = x0;
+        lv[0].xt = xt0;
         if (rc) return rc;
-        CK(L.from_f32(N, lv[0].x, dest));
     }
     return RHI_OK;
 }
 
 // r = b, rh = b, x = 0 and the loop's start (S_RR = S_RHO = r.r, counters cleared)
 int bicg_start(rhi_ctx* h, LinLaunch& L, const double* rhs, unsigned long long cond) {
-    int np = 0;
     L.skip = nullptr;
-    CK(L.bicg_init(h->N, rhs, h->r, h->rh, h->x, h->partials, np));
-    CK(L.reduce_loop(h->partials, np, h->scal, RED_BICG_START, cond));
+    CK(L.bicg_init(h->N, rhs, h->r, h->rh, h->x, fin(h, RED_BICG_START, 0, cond)));
     return RHI_OK;
 }
 
@@ -704,21 +721,20 @@ int bicg_start(rhi_ctx* h, LinLaunch& L, const double* rhs, unsigned long long c
 // r update; the next rho, beta and the continue flag (cond: the graph's while handle, or 0).
 int bicg_iteration(rhi_ctx* h, LinLaunch& L, unsigned long long cond) {
     const long long N = h->N;
-    int np = 0, rc;
+    const Finish fa = fin(h, RED_BICG_ALPHA), fs = fin(h, RED_BICG_SS), fo = fin(h, RED_BICG_OMEGA),
+                 fn = fin(h, RED_BICG_NEXT, 0, cond);
+    float* b32 = cycle_rhs(h);
+    int rc;
     L.skip = nullptr;
-    CK(L.bicg_p(N, h->scal, h->r, h->v, h->p, -1, h->rh));
+    CK(L.bicg_p(N, h->scal, h->r, h->v, h->p, h->rh, b32));
     if ((rc = precond_into(h, L, h->p, h->ph))) return rc;
-    CK(L.matvec_ns(h->opns, h->ph, h->v, h->rh, 0, h->partials, np));
-    CK(L.reduce(h->partials, np, h->scal, RED_BICG_ALPHA, 0));
-    CK(L.bicg_s(N, h->scal, h->r, h->v, h->s, h->partials, np));
-    CK(L.reduce_loop(h->partials, np, h->scal, RED_BICG_SS, 0));
+    CK(L.matvec_ns(h->opns, h->ph, h->v, h->rh, 0, fa));
+    CK(L.bicg_s(N, h->scal, h->r, h->v, h->s, b32, fs));
     L.skip = h->scal + S_DONE;
     if ((rc = precond_into(h, L, h->s, h->sh))) return rc;
-    CK(L.matvec_ns(h->opns, h->sh, h->t, h->s, 1, h->partials, np));
-    CK(L.reduce(h->partials, np, h->scal, RED_BICG_OMEGA, 0));
+    CK(L.matvec_ns(h->opns, h->sh, h->t, h->s, 1, fo));
     L.skip = nullptr;
-    CK(L.bicg_xr_loop(N, h->scal, h->x, h->ph, h->sh, h->s, h->t, h->r, h->rh, h->partials, np));
-    CK(L.reduce_loop(h->partials, np, h->scal, RED_BICG_NEXT, cond));
+    CK(L.bicg_xr(N, h->scal, h->x, h->ph, h->sh, h->s, h->t, h->r, h->rh, fn));
     return RHI_OK;
 }
 
@@ -889,6 +905,8 @@ void with_set(rhi_ctx* h, PhysBuffers& B, int b, int set) {
 
 int cell(rhi_ctx* h, const StepParams& P, int mode, PhysBuffers B) {
     const int nb = (int)((h->N + cell_block_size() - 1) / cell_block_size());
+    B.count = nb > CELL_SUM_BLOCKS ? nullptr : h->red_count;
+    B.norm_sq = h->scal + S_TMP;
     Scope s(h->prof, mode == MODE_ITER ? "cell_residual_schur" :
                      mode == MODE_RESID ? "cell_residual" :
                      (mode == MODE_PREP ? "cell_prep_residual_schur" : "cell_prep_predictor"));
@@ -1196,26 +1214,28 @@ int rhi_create(const rhi_grid* grid, const rhi_bc* bc, const rhi_params* params,
                                                  2 * (long long)stream_blocks(N));
     A(&h->partials, (size_t)nparts);
     A(&h->scal, S_NSCAL);
+    if (!rc) rc = dalloc(h, &h->red_count, 1);
     if (!rc) rc = dalloc(h, &h->d_flag, 1);
     if (!rc) rc = dalloc(h, &h->table, (size_t)NBINS * NRATES);
-    if (!rc) rc = mg_build_levels(h);
     if (!rc) {
-        cudaError_t e = cudaMallocHost(&h->h_scal, sizeof(double) * S_NSCAL);
+        cudaError_t e = mg_tail_init(&h->tail_blocks[0], &h->tail_blocks[1]);
+        if (e == cudaSuccess) e = cudaMallocHost(&h->h_scal, sizeof(double) * S_NSCAL);
         if (e == cudaSuccess) e = cudaMallocHost(&h->h_ctl, sizeof(double) * 3);
         if (e == cudaSuccess) e = cudaMallocHost(&h->h_kerr, sizeof(int));
-        if (e != cudaSuccess) rc = fail(h, RHI_ERR_CUDA, "cudaMallocHost");
+        if (e != cudaSuccess) rc = fail(h, RHI_ERR_CUDA, std::string("rhi_create: ") + cudaGetErrorString(e));
         if (!rc) {
             *h->h_kerr = 0;
             e = linear_kernels_init();
-            if (e == cudaSuccess) e = mg_tail_init(&h->tail_blocks[0], &h->tail_blocks[1]);
             if (e != cudaSuccess) rc = fail(h, RHI_ERR_CUDA, std::string("multigrid kernels: ") + cudaGetErrorString(e));
         }
     }
+    if (!rc) rc = mg_build_levels(h);
     if (!rc) {
         std::vector<double2> tab = build_rate_table();
         cudaError_t e = cudaMemcpy(h->table, tab.data(), tab.size() * sizeof(double2), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemset(h->src, 0, N * sizeof(double));
         if (e == cudaSuccess) e = cudaMemset(h->scal, 0, S_NSCAL * sizeof(double));
+        if (e == cudaSuccess) e = cudaMemset(h->red_count, 0, sizeof(unsigned));
         if (e == cudaSuccess) e = cudaEventCreate(&h->ev0);
         if (e == cudaSuccess) e = cudaEventCreate(&h->ev1);
         if (e != cudaSuccess) rc = fail(h, RHI_ERR_CUDA, std::string("rhi_create: ") + cudaGetErrorString(e));
@@ -1495,8 +1515,7 @@ int rhi_precond_apply(rhi_handle h, const double* r, double* z, int on_device) {
     const long long N = h->N;
     CK(cudaMemcpyAsync(h->q, r, N * sizeof(double), on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->st));
     double* zr = nullptr;
-    int np = 0;
-    int rc = precond_apply(h, h->q, &zr, np);
+    int rc = precond_apply(h, h->q, &zr, fin(h, RED_NONE));
     if (rc) return rc;
     CK(cudaMemcpyAsync(z, zr, N * sizeof(double), on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->st));
     CK(bulk_wait_flag_read(h->h_kerr, h->st));

@@ -92,6 +92,14 @@ __device__ __forceinline__ double fast_rcp(double d) {
     return fma(r, fma(e, e, e), r);
 }
 
+// A value the compiler cannot see through.  `for (int go = rare; go; go = opaque(0)) {...}` is an `if`
+// that stays a branch: as predicated instructions, FP64 work of a rare case would take its time on
+// the FP64 pipe in every case.
+__device__ __forceinline__ int opaque(int v) {
+    asm volatile("" : "+r"(v));
+    return v;
+}
+
 // ---------------------------------------------------------------------------------------------
 // grid helpers
 
@@ -131,22 +139,57 @@ __device__ __forceinline__ Nbr neighbours(const StepParams& P, long long c, int 
 }
 
 // ---------------------------------------------------------------------------------------------
-// deterministic block reduction of a double; result valid in thread 0
+// Deterministic block reduction of a double; result valid in thread 0.  One warp adds everything: a
+// warp's FP64 instruction takes its sub-partition's pipe for 64 cycles whatever its lanes hold, so
+// 12 instructions of one warp cost less than 5 of each of eight warps.
 template <int BLOCK>
 __device__ __forceinline__ double block_sum(double v) {
-    __shared__ double warp_part[BLOCK / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (lane == 0) warp_part[w] = v;
+    __shared__ double part[BLOCK];
+    part[threadIdx.x] = v;
     __syncthreads();
     double s = 0.0;
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {
+        s = part[threadIdx.x];
 #pragma unroll
-        for (int q = 0; q < BLOCK / 32; ++q) s += warp_part[q];
+        for (int q = 1; q < BLOCK / 32; ++q) s += part[threadIdx.x + 32 * q];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     }
     __syncthreads();
     return s;
+}
+
+// Grid-wide sum without a second launch: every block writes its partial and takes a ticket; the
+// block with the last one (true) adds the partials in a fixed order, so the result does not depend on
+// the order the blocks ended in.  Returns true in all threads of that block; the sums are valid in
+// its thread 0.  The counter wraps to 0 by itself; launches that share it run one after another.
+template <int BLOCK, bool TWO>
+__device__ __forceinline__ bool grid_sum(double v1, double v2, double* partials, unsigned* count,
+                                         double& s1, double& s2) {
+    __shared__ bool last_block;
+    const int n = (int)gridDim.x;
+    s1 = block_sum<BLOCK>(v1);
+    s2 = TWO ? block_sum<BLOCK>(v2) : 0.0;
+    if (threadIdx.x == 0) {
+        partials[blockIdx.x] = s1;
+        if (TWO) partials[n + blockIdx.x] = s2;
+        last_block = false;
+        if (count) {
+            __threadfence();
+            last_block = atomicInc(count, (unsigned)n - 1u) == (unsigned)n - 1u;
+        }
+    }
+    __syncthreads();
+    if (!last_block) return false;
+    __threadfence();
+    double a1 = 0.0, a2 = 0.0;
+    for (int q = (int)threadIdx.x; q < n; q += BLOCK) {
+        a1 += __ldcg(partials + q);
+        if (TWO) a2 += __ldcg(partials + n + q);
+    }
+    s1 = block_sum<BLOCK>(a1);
+    s2 = TWO ? block_sum<BLOCK>(a2) : 0.0;
+    return true;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -183,6 +226,8 @@ struct PhysBuffers {
     double* MiU;            // (ns + 1) * N   M^-1 U  (scaled)
     double* f_out;          // optional (ns + 2) * N scaled residual
     double* partials;       // per-block sums of the squared scaled residual
+    unsigned* count;        // with it, their sum goes to *norm_sq (null: partials only)
+    double* norm_sq;
     double* U0;             // optional predictor output (ns + 2) * N
 };
 

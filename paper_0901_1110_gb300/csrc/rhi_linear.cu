@@ -1,7 +1,7 @@
 // Scalar Schur-system solve (Sec. 3.2.1, step (ii)): conjugate gradients on the 7-point
 // matrix S, preconditioned by one geometric multigrid V-cycle (FP64, or FP32 for the mixed-
 // precision form) or by Jacobi.  Reductions are deterministic: per-block partial sums are
-// added in a fixed order by a single block.
+// added in a fixed order by the last block to end.
 //
 // Operator of a level: (A x)_c = diag_c x_c - sum_ax (W[ax]_c x_lo + Wp[ax]_hi x_hi),
 // stored per lower face (0 on zero-flux boundary faces): W couples the upper cell's row to the
@@ -21,6 +21,14 @@ __device__ __forceinline__ bool skipped(const double* skip) { return skip && *sk
 int stream_blocks(long long N) {
     const long long want = (N + LIN_BLOCK - 1) / LIN_BLOCK;
     const long long cap = 152LL * 16;                 // 16 resident blocks per SM x 152 SMs
+    return (int)(want < cap ? (want > 0 ? want : 1) : cap);
+}
+
+// blocks of the kernels that end with a sum: one wave of 8 blocks per SM, since every block adds its
+// own partial (a chain of FP64 additions) and takes a ticket
+static int sum_blocks(long long N) {
+    const long long want = (N + LIN_BLOCK - 1) / LIN_BLOCK;
+    const long long cap = 152LL * 8;
     return (int)(want < cap ? (want > 0 ? want : 1) : cap);
 }
 
@@ -88,360 +96,14 @@ __device__ __forceinline__ T jacobi_update(T xc, T b, T wi, T off, T omega) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// CG building blocks (FP64)
-
-__global__ void __launch_bounds__(LIN_BLOCK) k_matvec_dot(const Op<double> A,
-                                                          const double* __restrict__ p,
-                                                          double* __restrict__ q,
-                                                          double* __restrict__ partials) {
-    double acc = 0.0;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < A.N;
-         c += (long long)gridDim.x * LIN_BLOCK) {
-        int i, j, k;
-        coords3(A, c, i, j, k);
-        const double pc = p[c];
-        const double v = apply_row(A, p, c, i, j, k, pc);
-        q[c] = v;
-        acc += pc * v;
-    }
-    const double s = block_sum<LIN_BLOCK>(acc);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
-// x += alpha p; r -= alpha q; partial r.r      (alpha = scal[S_ALPHA])
-__global__ void __launch_bounds__(LIN_BLOCK) k_cg_xr(long long N, const double* __restrict__ scal,
-                                                     double* __restrict__ x, double* __restrict__ r,
-                                                     const double* __restrict__ p,
-                                                     const double* __restrict__ q,
-                                                     double* __restrict__ partials) {
-    const double alpha = scal[S_ALPHA];
-    double acc = 0.0;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK) {
-        x[c] += alpha * p[c];
-        const double rv = r[c] - alpha * q[c];
-        r[c] = rv;
-        acc += rv * rv;
-    }
-    const double s = block_sum<LIN_BLOCK>(acc);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
-// p = z + beta p    (beta = scal[S_BETA]); first: p = z
-__global__ void __launch_bounds__(LIN_BLOCK) k_cg_p(long long N, const double* __restrict__ scal,
-                                                    const double* __restrict__ z,
-                                                    double* __restrict__ p, int first) {
-    const double beta = first ? 0.0 : scal[S_BETA];
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK)
-        p[c] = first ? z[c] : z[c] + beta * p[c];
-}
-
-// z = r / diag; partial r.z
-__global__ void __launch_bounds__(LIN_BLOCK) k_jacobi_dot(long long N, const double* __restrict__ r,
-                                                          const double* __restrict__ diag,
-                                                          double* __restrict__ z,
-                                                          double* __restrict__ partials,
-                                                          const double* skip) {
-    if (skipped(skip)) return;
-    double acc = 0.0;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK) {
-        const double rv = r[c];
-        const double zv = rv / diag[c];
-        z[c] = zv;
-        acc += rv * zv;
-    }
-    const double s = block_sum<LIN_BLOCK>(acc);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
-// partial a.b
-__global__ void __launch_bounds__(LIN_BLOCK) k_dot(long long N, const double* __restrict__ a,
-                                                   const double* __restrict__ b,
-                                                   double* __restrict__ partials) {
-    double acc = 0.0;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK)
-        acc += a[c] * b[c];
-    const double s = block_sum<LIN_BLOCK>(acc);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
-// r = b, x = 0; partial r.r
-__global__ void __launch_bounds__(LIN_BLOCK) k_cg_init(long long N, const double* __restrict__ b,
-                                                       double* __restrict__ r,
-                                                       double* __restrict__ x,
-                                                       double* __restrict__ partials) {
-    double acc = 0.0;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK) {
-        const double v = b[c];
-        r[c] = v;
-        x[c] = 0.0;
-        acc += v * v;
-    }
-    const double s = block_sum<LIN_BLOCK>(acc);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
-// Sum of partials in a fixed order, then a scalar update:
-//   SUM_TO(k):   scal[k] = sum
-//   SUM_ALPHA:   scal[S_PQ] = sum; scal[S_ALPHA] = scal[S_RZ] / sum (breakdown flag if <= 0)
-//   SUM_BETA:    scal[S_BETA] = sum / scal[S_RZ]; scal[S_RZ] = sum
-__global__ void __launch_bounds__(RED_BLOCK) k_reduce(const double* __restrict__ partials, int n,
-                                                      double* __restrict__ scal, int op,
-                                                      int slot, const double* skip) {
-    if (skipped(skip)) return;
-    // the BiCGStab updates carry a second set of partials after the first n
-    const bool two = op == RED_BICG_OMEGA || op == RED_BICG_RHO;
-    if (op == RED_MAX) {                        // max of non-negative partials
-        __shared__ double wmax[RED_BLOCK / 32];
-        double m = 0.0;
-        for (int q = threadIdx.x; q < n; q += RED_BLOCK) m = fmax(m, partials[q]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
-        if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int q = 1; q < RED_BLOCK / 32; ++q) m = fmax(m, wmax[q]);
-            scal[slot] = fmax(m, wmax[0]);
-        }
-        return;
-    }
-    double acc = 0.0, acc2 = 0.0;
-    for (int q = threadIdx.x; q < n; q += RED_BLOCK) {
-        acc += partials[q];
-        if (two) acc2 += partials[n + q];
-    }
-    const double s = block_sum<RED_BLOCK>(acc);
-    const double s2 = two ? block_sum<RED_BLOCK>(acc2) : 0.0;
-    if (threadIdx.x == 0) {
-        if (op == RED_SUM) {
-            scal[slot] = s;
-        } else if (op == RED_ALPHA) {
-            scal[S_PQ] = s;
-            if (!(s > 0.0)) scal[S_BREAK] = 1.0;
-            scal[S_ALPHA] = (s > 0.0) ? scal[S_RZ] / s : 0.0;
-        } else if (op == RED_BETA) {
-            scal[S_BETA] = s / scal[S_RZ];
-            scal[S_RZ] = s;
-        } else if (op == RED_BICG_ALPHA) {          // s = rh.v
-            scal[S_RST] = 0.0;                      // a restart's p and rh are in place
-            scal[S_RV] = s;
-            if (!(s != 0.0)) scal[S_BREAK] = 1.0;
-            scal[S_ALPHA] = (s != 0.0) ? scal[S_RHO] / s : 0.0;
-        } else if (op == RED_BICG_OMEGA) {          // partials: t.s then t.t
-            const double tt = s2;
-            scal[S_TS] = s;
-            scal[S_TT] = tt;
-            scal[S_OMEGA] = (tt > 0.0) ? s / tt : 0.0;
-            if (!(tt > 0.0)) scal[S_BREAK] = 1.0;
-        } else {                                    // RED_BICG_RHO: partials r.r then rh.r
-            const double rho = s2;
-            scal[S_RR] = s;
-            scal[S_BETA] = (rho / scal[S_RHO]) * (scal[S_ALPHA] / scal[S_OMEGA]);
-            scal[S_RHO] = rho;
-            if (!(rho != 0.0)) scal[S_BREAK] = 1.0;
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------------------------
-// BiCGStab building blocks (FP64), right preconditioning
-
-// y = A x with the non-symmetric operator; partials w1.y (and y.y when TWO)
-template <bool TWO>
-__global__ void __launch_bounds__(LIN_BLOCK) k_matvec_ns(const OpNS A, const double* __restrict__ x,
-                                                         double* __restrict__ y,
-                                                         const double* __restrict__ w1,
-                                                         double* __restrict__ partials) {
-    if (skipped(A.skip)) return;
-    double d1 = 0.0, d2 = 0.0;
-    const long long sz = (long long)A.nx * A.ny;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < A.N;
-         c += (long long)gridDim.x * LIN_BLOCK) {
-        int i, j, k;
-        coords_fd(c, A.fd_nx, A.fd_nxy, i, j, k);
-        const int q[3] = {i, j, k};
-        const int n[3] = {A.nx, A.ny, A.nz};
-        const long long s[3] = {1, A.nx, sz};
-        double off = 0.0;
-#pragma unroll
-        for (int ax = 0; ax < 3; ++ax) {
-            const long long lo = q[ax] > 0 ? c - s[ax] : c + (long long)(n[ax] - 1) * s[ax];
-            off += A.Q[ax][c] * x[lo];                // 0 on zero-flux boundary faces
-            long long hi = -1;
-            if (q[ax] < n[ax] - 1) hi = c + s[ax];
-            else if (A.per[ax]) hi = c - (long long)(n[ax] - 1) * s[ax];
-            if (hi >= 0) off += A.P[ax][hi] * x[hi];
-        }
-        const double v = A.diag[c] * x[c] - off;
-        y[c] = v;
-        d1 += w1[c] * v;
-        if (TWO) d2 += v * v;
-    }
-    const double s1 = block_sum<LIN_BLOCK>(d1);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s1;
-    if (TWO) {
-        const double s2 = block_sum<LIN_BLOCK>(d2);
-        if (threadIdx.x == 0) partials[gridDim.x + blockIdx.x] = s2;
-    }
-}
-
-// r = b, rh = b, x = 0; partial r.r
-__global__ void __launch_bounds__(LIN_BLOCK) k_bicg_init(long long N, const double* __restrict__ b,
-                                                         double* __restrict__ r,
-                                                         double* __restrict__ rh,
-                                                         double* __restrict__ x,
-                                                         double* __restrict__ partials) {
-    double acc = 0.0;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK) {
-        const double v = b[c];
-        r[c] = v;
-        rh[c] = v;
-        x[c] = 0.0;
-        acc += v * v;
-    }
-    const double s = block_sum<LIN_BLOCK>(acc);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
-}
-
-// p = r + beta (p - omega v); first: p = r.  first < 0: decided on the device, p = r at the
-// loop's first iteration and after a restart, when also the shadow vector becomes rh = r
-__global__ void __launch_bounds__(LIN_BLOCK) k_bicg_p(long long N, const double* __restrict__ scal,
-                                                      const double* __restrict__ r,
-                                                      const double* __restrict__ v,
-                                                      double* __restrict__ p, int first,
-                                                      double* __restrict__ rh) {
-    const double beta = scal[S_BETA], omega = scal[S_OMEGA];
-    bool restart = false;
-    if (first < 0) {
-        restart = scal[S_RST] != 0.0;
-        first = scal[S_ITS] == 0.0 || restart;
-    }
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK) {
-        const double rc = r[c];
-        p[c] = first ? rc : rc + beta * (p[c] - omega * v[c]);
-        if (restart && rh) rh[c] = rc;
-    }
-}
-
-// s = r - alpha v; partial s.s
-__global__ void __launch_bounds__(LIN_BLOCK) k_bicg_s(long long N, const double* __restrict__ scal,
-                                                      const double* __restrict__ r,
-                                                      const double* __restrict__ v,
-                                                      double* __restrict__ s,
-                                                      double* __restrict__ partials) {
-    const double alpha = scal[S_ALPHA];
-    double acc = 0.0;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK) {
-        const double sv = r[c] - alpha * v[c];
-        s[c] = sv;
-        acc += sv * sv;
-    }
-    const double t = block_sum<LIN_BLOCK>(acc);
-    if (threadIdx.x == 0) partials[blockIdx.x] = t;
-}
-
-// x += alpha ph + omega sh; r = s - omega t; partials r.r then rh.r
-__global__ void __launch_bounds__(LIN_BLOCK) k_bicg_xr(long long N, const double* __restrict__ scal,
-                                                       double* __restrict__ x,
-                                                       const double* __restrict__ ph,
-                                                       const double* __restrict__ sh,
-                                                       const double* __restrict__ s,
-                                                       const double* __restrict__ t,
-                                                       double* __restrict__ r,
-                                                       const double* __restrict__ rh,
-                                                       double* __restrict__ partials) {
-    const double alpha = scal[S_ALPHA], omega = scal[S_OMEGA];
-    double rr = 0.0, rhr = 0.0;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK) {
-        x[c] += alpha * ph[c] + omega * sh[c];
-        const double rv = s[c] - omega * t[c];
-        r[c] = rv;
-        rr += rv * rv;
-        rhr += rh[c] * rv;
-    }
-    const double a1 = block_sum<LIN_BLOCK>(rr);
-    if (threadIdx.x == 0) partials[blockIdx.x] = a1;
-    const double a2 = block_sum<LIN_BLOCK>(rhr);
-    if (threadIdx.x == 0) partials[gridDim.x + blockIdx.x] = a2;
-}
-
-// x += scal[slot] p
-__global__ void __launch_bounds__(LIN_BLOCK) k_axpy(long long N, const double* __restrict__ scal,
-                                                    int slot, const double* __restrict__ p,
-                                                    double* __restrict__ x) {
-    const double a = scal[slot];
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK)
-        x[c] += a * p[c];
-}
-
-// x / r update of the device-controlled loop.  Converged at the middle of the iteration
-// (S_HALF): x += alpha ph, r untouched.  Otherwise, unless a breakdown ended the iteration:
-// x += alpha ph + omega sh, r = s - omega t, partials r.r then rh.r (zeros when skipped)
-__global__ void __launch_bounds__(LIN_BLOCK) k_bicg_xr_loop(long long N,
-                                                            const double* __restrict__ scal,
-                                                            double* __restrict__ x,
-                                                            const double* __restrict__ ph,
-                                                            const double* __restrict__ sh,
-                                                            const double* __restrict__ s,
-                                                            const double* __restrict__ t,
-                                                            double* __restrict__ r,
-                                                            const double* __restrict__ rh,
-                                                            double* __restrict__ partials) {
-    const double alpha = scal[S_ALPHA], omega = scal[S_OMEGA];
-    const bool half = scal[S_HALF] != 0.0;
-    const bool none = !half && scal[S_DONE] != 0.0;
-    double rr = 0.0, rhr = 0.0;
-    if (!none) {
-        for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-             c += (long long)gridDim.x * LIN_BLOCK) {
-            if (half) {
-                x[c] += alpha * ph[c];
-            } else {
-                x[c] += alpha * ph[c] + omega * sh[c];
-                const double rv = s[c] - omega * t[c];
-                r[c] = rv;
-                rr += rv * rv;
-                rhr += rh[c] * rv;
-            }
-        }
-    }
-    const double a1 = block_sum<LIN_BLOCK>(rr);
-    if (threadIdx.x == 0) partials[blockIdx.x] = a1;
-    const double a2 = block_sum<LIN_BLOCK>(rhr);
-    if (threadIdx.x == 0) partials[gridDim.x + blockIdx.x] = a2;
-}
-
-// z = x widened to FP64 (a four-per-thread form measured no faster here: 0.73 of HBM in the
-// step against 0.79)
-__global__ void __launch_bounds__(LIN_BLOCK) k_from_f32(long long N, const float* __restrict__ x,
-                                                        double* __restrict__ z,
-                                                        const double* skip) {
-    if (skipped(skip)) return;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK)
-        z[c] = (double)x[c];
-}
-
-__global__ void __launch_bounds__(LIN_BLOCK) k_copy(long long N, const double* __restrict__ a,
-                                                    double* __restrict__ b, const double* skip) {
-    if (skipped(skip)) return;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK)
-        b[c] = a[c];
-}
-
-// The reductions of the device-controlled BiCGStab loop: a fixed-order sum of the partials
-// (two sets for RED_BICG_NEXT), then the loop's scalar logic, and the continue flag written to
-// S_CONT and, inside a CUDA graph, to the while node's conditional handle.
+// Scalar updates.  A kernel with dot products ends with finish(): its last block adds all blocks'
+// partials in a fixed order and applies the update, so that a Krylov iteration needs no separate
+// reduction launches (about 3.6 us each inside a graph; the last block adds about 2 us).
+//   RED_SUM:        scal[slot] = sum
+//   RED_ALPHA:      S_PQ = sum; S_ALPHA = S_RZ / sum (breakdown flag if <= 0)
+//   RED_BETA:       S_BETA = sum / S_RZ; S_RZ = sum
+//   RED_BICG_ALPHA: sum = rh.v: S_ALPHA = S_RHO / sum
+//   RED_BICG_OMEGA: sums t.s and t.t: S_OMEGA
 //   RED_BICG_START: r.r of r = b: S_RR = S_RHO = r.r, counters cleared; done when
 //                   r.r <= S_THR (or not finite: breakdown).
 //   RED_BICG_SS:    s.s: converged at the middle of the iteration when s.s <= S_THR (S_HALF,
@@ -454,21 +116,51 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_copy(long long N, const double* _
 //                   preconditioner slowly erodes the bi-orthogonality BiCGStab relies on); a
 //                   stagnation past the last restart ends the loop, and the Newton step is
 //                   then that of an inexact Newton iteration.
-// This kernel always runs to its end: it is what ends the loop.
-__global__ void __launch_bounds__(RED_BLOCK) k_reduce_loop(const double* __restrict__ partials,
-                                                           int n, double* __restrict__ scal,
-                                                           int op, unsigned long long cond) {
-    const bool two = op == RED_BICG_NEXT;
-    double acc = 0.0, acc2 = 0.0;
-    for (int q = threadIdx.x; q < n; q += RED_BLOCK) {
-        acc += partials[q];
-        if (two) acc2 += partials[n + q];
-    }
-    const double s = block_sum<RED_BLOCK>(acc);
-    const double s2 = two ? block_sum<RED_BLOCK>(acc2) : 0.0;
-    if (threadIdx.x != 0) return;
+// RED_BICG_START and RED_BICG_NEXT write the continue flag to S_CONT and, inside a CUDA graph, to
+// the while node's conditional handle: these kernels always run to their end.
+template <int OP>
+__device__ __forceinline__ void scalar_update(double* scal, int dyn, int slot, unsigned long long cond,
+                                              double s, double s2) {
+    // (the kernels of the preconditioned residual's dot serve several updates)
+    const int op = OP == RED_NONE ? dyn : OP;
     int cont = 0;
-    if (op == RED_BICG_START) {
+    if (op == RED_SUM) {
+        scal[slot] = s;
+        return;
+    } else if (op == RED_ALPHA) {
+        scal[S_PQ] = s;
+        if (!(s > 0.0)) scal[S_BREAK] = 1.0;
+        scal[S_ALPHA] = (s > 0.0) ? scal[S_RZ] / s : 0.0;
+        return;
+    } else if (op == RED_BETA) {
+        scal[S_BETA] = s / scal[S_RZ];
+        scal[S_RZ] = s;
+        return;
+    } else if (op == RED_BICG_ALPHA) {
+        scal[S_RST] = 0.0;                      // a restart's p and rh are in place
+        scal[S_RV] = s;
+        if (!(s != 0.0)) scal[S_BREAK] = 1.0;
+        scal[S_ALPHA] = (s != 0.0) ? scal[S_RHO] / s : 0.0;
+        return;
+    } else if (op == RED_BICG_OMEGA) {          // t.s, t.t
+        scal[S_TS] = s;
+        scal[S_TT] = s2;
+        scal[S_OMEGA] = (s2 > 0.0) ? s / s2 : 0.0;
+        if (!(s2 > 0.0)) scal[S_BREAK] = 1.0;
+        return;
+    } else if (op == RED_BICG_SS) {
+        scal[S_SS] = s;
+        if (!isfinite(s)) {
+            scal[S_BREAK] = 1.0;
+            scal[S_DONE] = 1.0;
+        } else if (scal[S_BREAK] != 0.0) {
+            scal[S_DONE] = 1.0;
+        } else if (!(s > scal[S_THR])) {
+            scal[S_HALF] = 1.0;
+            scal[S_DONE] = 1.0;
+        }
+        return;                                    // no loop decision here
+    } else if (op == RED_BICG_START) {
         const bool fin = isfinite(s);
         scal[S_RR] = s;
         scal[S_RHO] = s;
@@ -484,18 +176,6 @@ __global__ void __launch_bounds__(RED_BLOCK) k_reduce_loop(const double* __restr
         const bool done = !(s > scal[S_THR]) || !fin || !(scal[S_MAXIT] >= 1.0);
         scal[S_DONE] = done ? 1.0 : 0.0;
         cont = !done;
-    } else if (op == RED_BICG_SS) {
-        scal[S_SS] = s;
-        if (!isfinite(s)) {
-            scal[S_BREAK] = 1.0;
-            scal[S_DONE] = 1.0;
-        } else if (scal[S_BREAK] != 0.0) {
-            scal[S_DONE] = 1.0;
-        } else if (!(s > scal[S_THR])) {
-            scal[S_HALF] = 1.0;
-            scal[S_DONE] = 1.0;
-        }
-        return;                                    // no loop decision here
     } else {                                       // RED_BICG_NEXT
         const double its = scal[S_ITS] + 1.0;
         scal[S_ITS] = its;
@@ -534,8 +214,288 @@ __global__ void __launch_bounds__(RED_BLOCK) k_reduce_loop(const double* __restr
     if (cond) cudaGraphSetConditional((cudaGraphConditionalHandle)cond, cont ? 1u : 0u);
 }
 
+// v1 (and v2): this thread's share of the sums; called by every thread of every block.  OP: the one
+// update the kernel ends with, so that its code holds no other (RED_NONE: F.op, of SUM, BETA, NONE)
+template <bool TWO, int OP>
+__device__ __forceinline__ void finish(const Finish& F, double v1, double v2) {
+    __shared__ double sc[S_NSCAL];
+    double s1, s2;
+    if (!grid_sum<LIN_BLOCK, TWO>(v1, v2, F.partials, F.op == RED_NONE ? nullptr : F.count, s1, s2)) return;
+    // the scalars by way of shared memory: one trip to memory each way
+    if (threadIdx.x < S_NSCAL) sc[threadIdx.x] = __ldcg(F.scal + threadIdx.x);
+    __syncthreads();
+    if (threadIdx.x == 0) scalar_update<OP>(sc, F.op == RED_BETA ? RED_BETA : RED_SUM, F.slot, F.cond, s1, s2);
+    __syncthreads();
+    if (threadIdx.x < S_NSCAL) F.scal[threadIdx.x] = sc[threadIdx.x];
+}
+
+// sum or max of partials in a fixed order by one block (where a kernel has too many blocks for its
+// last one to add them, or none of the above)
+__global__ void __launch_bounds__(RED_BLOCK) k_reduce(const double* __restrict__ partials, int n,
+                                                      double* __restrict__ scal, int op, int slot) {
+    if (op == RED_MAX) {                        // max of non-negative partials
+        __shared__ double wmax[RED_BLOCK / 32];
+        double m = 0.0;
+        for (int q = threadIdx.x; q < n; q += RED_BLOCK) m = fmax(m, partials[q]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_down_sync(0xffffffffu, m, o));
+        if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int q = 1; q < RED_BLOCK / 32; ++q) m = fmax(m, wmax[q]);
+            scal[slot] = fmax(m, wmax[0]);
+        }
+        return;
+    }
+    double acc = 0.0;
+    for (int q = threadIdx.x; q < n; q += RED_BLOCK) acc += partials[q];
+    const double s = block_sum<RED_BLOCK>(acc);
+    if (threadIdx.x == 0) scal[slot] = s;
+}
+
+// ---------------------------------------------------------------------------------------------
+// CG building blocks (FP64)
+
+__global__ void __launch_bounds__(LIN_BLOCK) k_matvec_dot(const Op<double> A,
+                                                          const double* __restrict__ p,
+                                                          double* __restrict__ q, const Finish F) {
+    double acc = 0.0;
+    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < A.N;
+         c += (long long)gridDim.x * LIN_BLOCK) {
+        int i, j, k;
+        coords3(A, c, i, j, k);
+        const double pc = p[c];
+        const double v = apply_row(A, p, c, i, j, k, pc);
+        q[c] = v;
+        acc += pc * v;
+    }
+    finish<false, RED_ALPHA>(F, acc, 0.0);
+}
+
+// x += alpha p; r -= alpha q; r.r      (alpha = scal[S_ALPHA])
+__global__ void __launch_bounds__(LIN_BLOCK) k_cg_xr(long long N, const double* __restrict__ scal,
+                                                     double* __restrict__ x, double* __restrict__ r,
+                                                     const double* __restrict__ p,
+                                                     const double* __restrict__ q, const Finish F) {
+    const double alpha = scal[S_ALPHA];
+    double acc = 0.0;
+    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
+         c += (long long)gridDim.x * LIN_BLOCK) {
+        x[c] += alpha * p[c];
+        const double rv = r[c] - alpha * q[c];
+        r[c] = rv;
+        acc += rv * rv;
+    }
+    finish<false, RED_SUM>(F, acc, 0.0);
+}
+
+// p = z + beta p    (beta = scal[S_BETA]); first: p = z
+__global__ void __launch_bounds__(LIN_BLOCK) k_cg_p(long long N, const double* __restrict__ scal,
+                                                    const double* __restrict__ z,
+                                                    double* __restrict__ p, int first) {
+    const double beta = first ? 0.0 : scal[S_BETA];
+    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
+         c += (long long)gridDim.x * LIN_BLOCK)
+        p[c] = first ? z[c] : z[c] + beta * p[c];
+}
+
+// z = r / diag; r.z
+__global__ void __launch_bounds__(LIN_BLOCK) k_jacobi_dot(long long N, const double* __restrict__ r,
+                                                          const double* __restrict__ diag,
+                                                          double* __restrict__ z, const Finish F,
+                                                          const double* skip) {
+    if (skipped(skip)) return;
+    double acc = 0.0;
+    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
+         c += (long long)gridDim.x * LIN_BLOCK) {
+        const double rv = r[c];
+        const double zv = rv / diag[c];
+        z[c] = zv;
+        acc += rv * zv;
+    }
+    finish<false, RED_NONE>(F, acc, 0.0);
+}
+
+// a.b
+__global__ void __launch_bounds__(LIN_BLOCK) k_dot(long long N, const double* __restrict__ a,
+                                                   const double* __restrict__ b, const Finish F) {
+    double acc = 0.0;
+    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
+         c += (long long)gridDim.x * LIN_BLOCK)
+        acc += a[c] * b[c];
+    finish<false, RED_NONE>(F, acc, 0.0);
+}
+
+// r = b, x = 0; r.r
+__global__ void __launch_bounds__(LIN_BLOCK) k_cg_init(long long N, const double* __restrict__ b,
+                                                       double* __restrict__ r,
+                                                       double* __restrict__ x, const Finish F) {
+    double acc = 0.0;
+    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
+         c += (long long)gridDim.x * LIN_BLOCK) {
+        const double v = b[c];
+        r[c] = v;
+        x[c] = 0.0;
+        acc += v * v;
+    }
+    finish<false, RED_SUM>(F, acc, 0.0);
+}
+
+// ---------------------------------------------------------------------------------------------
+// BiCGStab building blocks (FP64), right preconditioning.  With the FP32 multigrid the vectors
+// p and s are also written in FP32, as the cycle's right-hand side, and the cycle's last sweep writes
+// its result in FP64, so no conversion passes remain.  (The product does not read an FP32 vector
+// itself: a conversion takes an FP64 slot like an FMA, seven of them beside its eight; conversions
+// by integer instructions with a branch for subnormals measured slower still, 449 against 321 us.)
+
+// y = A x with the non-symmetric operator; w1.y (and y.y when TWO).  Every load of a row is issued
+// before its first use; the sum is one chain of FMAs, 8 FP64 instructions a row with one dot.
+// Measured at 256^3: 267 us against 321 us with the products summed apart from the diagonal.
+template <bool TWO>
+__global__ void __launch_bounds__(LIN_BLOCK) k_matvec_ns(const OpNS A, const double* __restrict__ x,
+                                                         double* __restrict__ y,
+                                                         const double* __restrict__ w1,
+                                                         const Finish F) {
+    if (skipped(A.skip)) return;
+    double d1 = 0.0, d2 = 0.0;
+    const long long sz = (long long)A.nx * A.ny;
+    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < A.N;
+         c += (long long)gridDim.x * LIN_BLOCK) {
+        int i, j, k;
+        coords_fd(c, A.fd_nx, A.fd_nxy, i, j, k);
+        const int q[3] = {i, j, k};
+        const int n[3] = {A.nx, A.ny, A.nz};
+        const long long s[3] = {1, A.nx, sz};
+        double w[6], xv[6];
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+            // (the lower entry is 0 on zero-flux boundary faces, where lo is the far side)
+            const long long lo = q[ax] > 0 ? c - s[ax] : c + (long long)(n[ax] - 1) * s[ax];
+            const bool has = q[ax] < n[ax] - 1 || A.per[ax];
+            const long long hi = q[ax] < n[ax] - 1 ? c + s[ax] : (has ? c - (long long)(n[ax] - 1) * s[ax] : c);
+            xv[2 * ax] = __ldg(x + lo);
+            xv[2 * ax + 1] = has ? __ldg(x + hi) : 0.0;
+            w[2 * ax] = __ldg(A.Q[ax] + c);
+            w[2 * ax + 1] = has ? __ldg(A.P[ax] + hi) : 0.0;
+        }
+        double v = __ldg(A.diag + c) * __ldg(x + c);
+        const double w1c = __ldg(w1 + c);
+#pragma unroll
+        for (int f = 0; f < 6; ++f) v = fma(-w[f], xv[f], v);
+        y[c] = v;
+        d1 = fma(w1c, v, d1);
+        if (TWO) d2 = fma(v, v, d2);
+    }
+    finish<TWO, TWO ? RED_BICG_OMEGA : RED_BICG_ALPHA>(F, d1, d2);
+}
+
+// r = b, rh = b, x = 0; r.r
+__global__ void __launch_bounds__(LIN_BLOCK) k_bicg_init(long long N, const double* __restrict__ b,
+                                                         double* __restrict__ r,
+                                                         double* __restrict__ rh,
+                                                         double* __restrict__ x, const Finish F) {
+    double acc = 0.0;
+    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
+         c += (long long)gridDim.x * LIN_BLOCK) {
+        const double v = b[c];
+        r[c] = v;
+        rh[c] = v;
+        x[c] = 0.0;
+        acc += v * v;
+    }
+    finish<false, RED_BICG_START>(F, acc, 0.0);
+}
+
+// p = r + beta (p - omega v); at the loop's first iteration and after a restart p = r, and after a
+// restart also the shadow vector rh = r
+__global__ void __launch_bounds__(LIN_BLOCK) k_bicg_p(long long N, const double* __restrict__ scal,
+                                                      const double* __restrict__ r,
+                                                      const double* __restrict__ v,
+                                                      double* __restrict__ p,
+                                                      double* __restrict__ rh,
+                                                      float* __restrict__ p32) {
+    const double beta = scal[S_BETA], omega = scal[S_OMEGA];
+    const bool restart = scal[S_RST] != 0.0;
+    const bool first = scal[S_ITS] == 0.0 || restart;
+    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
+         c += (long long)gridDim.x * LIN_BLOCK) {
+        const double rc = r[c];
+        const double pv = first ? rc : rc + beta * (p[c] - omega * v[c]);
+        p[c] = pv;
+        if (p32) p32[c] = (float)pv;
+        if (restart) rh[c] = rc;
+    }
+}
+
+// s = r - alpha v; s.s
+__global__ void __launch_bounds__(LIN_BLOCK) k_bicg_s(long long N, const double* __restrict__ scal,
+                                                      const double* __restrict__ r,
+                                                      const double* __restrict__ v,
+                                                      double* __restrict__ s,
+                                                      float* __restrict__ s32, const Finish F) {
+    const double alpha = scal[S_ALPHA];
+    double acc = 0.0;
+    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
+         c += (long long)gridDim.x * LIN_BLOCK) {
+        const double sv = r[c] - alpha * v[c];
+        s[c] = sv;
+        if (s32) s32[c] = (float)sv;
+        acc += sv * sv;
+    }
+    finish<false, RED_BICG_SS>(F, acc, 0.0);
+}
+
+// Converged at the middle of the iteration (S_HALF): x += alpha ph, r untouched.  Otherwise, unless
+// a breakdown ended the iteration: x += alpha ph + omega sh, r = s - omega t, r.r and rh.r (zeros when
+// skipped)
+__global__ void __launch_bounds__(LIN_BLOCK) k_bicg_xr(long long N, const double* __restrict__ scal,
+                                                       double* __restrict__ x,
+                                                       const double* __restrict__ ph,
+                                                       const double* __restrict__ sh,
+                                                       const double* __restrict__ s,
+                                                       const double* __restrict__ t,
+                                                       double* __restrict__ r,
+                                                       const double* __restrict__ rh,
+                                                       const Finish F) {
+    const double alpha = scal[S_ALPHA], omega = scal[S_OMEGA];
+    const bool half = scal[S_HALF] != 0.0;
+    const bool none = !half && scal[S_DONE] != 0.0;
+    double rr = 0.0, rhr = 0.0;
+    if (!none) {
+        for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
+             c += (long long)gridDim.x * LIN_BLOCK) {
+            if (half) {
+                x[c] += alpha * ph[c];
+            } else {
+                x[c] += alpha * ph[c] + omega * sh[c];
+                const double rv = s[c] - omega * t[c];
+                r[c] = rv;
+                rr += rv * rv;
+                rhr += rh[c] * rv;
+            }
+        }
+    }
+    finish<true, RED_BICG_NEXT>(F, rr, rhr);
+}
+
+__global__ void __launch_bounds__(LIN_BLOCK) k_copy(long long N, const double* __restrict__ a,
+                                                    double* __restrict__ b, const double* skip) {
+    if (skipped(skip)) return;
+    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
+         c += (long long)gridDim.x * LIN_BLOCK)
+        b[c] = a[c];
+}
+
 // ---------------------------------------------------------------------------------------------
 // multigrid kernels (templated on the level precision)
+
+// a sweep's result: in the level's precision, or in FP64 where the sweep ends the cycle (out64; the
+// caller's vector, one conversion per cell under the sweep's memory time instead of a pass of its own)
+template <typename T>
+__device__ __forceinline__ void store_sweep(T* xout, double* out64, long long c, T v) {
+    if (out64) out64[c] = (double)v;
+    else xout[c] = v;
+}
 
 // weighted Jacobi with wid = omega / diag: first sweep from x = 0: x_out = wid b; else
 // x_out = x_in + omega (b - A x_in) / diag, written as (1 - omega) x_in + wid (b + off)
@@ -543,7 +503,7 @@ template <typename T>
 __global__ void __launch_bounds__(LIN_BLOCK) k_mg_smooth(const Op<T> A, const T* __restrict__ b,
                                                          const T* __restrict__ xin,
                                                          T* __restrict__ xout, T omega,
-                                                         int first) {
+                                                         int first, double* __restrict__ out64) {
     if (skipped(A.skip)) return;
     for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < A.N;
          c += (long long)gridDim.x * LIN_BLOCK) {
@@ -554,7 +514,7 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_smooth(const Op<T> A, const T*
             int i, j, k;
             coords3(A, c, i, j, k);
             const T off = off_row(A, xin, c, i, j, k);
-            xout[c] = jacobi_update(xin[c], b[c], wi, off, omega);
+            store_sweep(xout, out64, c, jacobi_update(xin[c], b[c], wi, off, omega));
         }
     }
 }
@@ -593,7 +553,8 @@ constexpr int ZM = 2;
 template <typename T>
 __global__ void __launch_bounds__(LIN_BLOCK) k_mg_smooth_zm(const Op<T> A, const T* __restrict__ b,
                                                             const T* __restrict__ xin,
-                                                            T* __restrict__ xout, T omega) {
+                                                            T* __restrict__ xout, T omega,
+                                                            double* __restrict__ out64) {
     if (skipped(A.skip)) return;
     const long long nxy = (long long)A.nx * A.ny;
     const long long col = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x;
@@ -657,7 +618,7 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_smooth_zm(const Op<T> A, const
         if (hhi1) off += w1h[kk] * x1h[kk];
         off += wz[kk] * xz[kk];
         if (hz) off += pz[kk] * xz[kk + 2];
-        xout[c0 + (long long)kk * nxy] = jacobi_update(xz[kk + 1], bb[kk], dd[kk], off, omega);
+        store_sweep(xout, out64, c0 + (long long)kk * nxy, jacobi_update(xz[kk + 1], bb[kk], dd[kk], off, omega));
     }
 }
 
@@ -723,7 +684,8 @@ __global__ void __launch_bounds__(BULK_MAX_NX) k_mg_smooth_bulk(const Op<float> 
                                                                 const float* __restrict__ b,
                                                                 const float* __restrict__ xin,
                                                                 float* __restrict__ xout,
-                                                                float omega, int* err) {
+                                                                float omega, int* err,
+                                                                double* __restrict__ out64) {
     if (skipped(A.skip)) return;
     extern __shared__ __align__(128) float rows[];          // [BULK_STAGES][BULK_ROWS][nx]
     __shared__ __align__(8) unsigned long long bar[BULK_STAGES];
@@ -797,8 +759,8 @@ __global__ void __launch_bounds__(BULK_MAX_NX) k_mg_smooth_bulk(const Op<float> 
             if (hhi1) off += Q1[i] * XP[i];
             off += R2[i] * xlo;
             if (hz) off += Q2[i] * XU[i];
-            xout[(long long)j * nx + (long long)k * nxy + i] =
-                jacobi_update(xcen, BB[i], WD[i], off, omega);
+            store_sweep(xout, out64, (long long)j * nx + (long long)k * nxy + i,
+                        jacobi_update(xcen, BB[i], WD[i], off, omega));
         }
         xlo = xcen;
         __syncthreads();                                    // stage st is free again
@@ -954,15 +916,6 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_prolong(int nx, int ny, int nz
     }
 }
 
-// FP32 to FP64 on the integer pipe (a conversion instruction takes the FP64 pipe for as long as an
-// FMA); zeros, subnormals and non-finite values take the instruction
-__device__ __forceinline__ double widen(float f) {
-    const unsigned u = __float_as_uint(f), m = u & 0x7fffffffu;
-    if (m - 0x00800000u >= 0x7f000000u) return (double)f;
-    return __hiloint2double((int)((u & 0x80000000u) | ((m >> 3) + 0x38000000u)), (int)(u << 29));
-}
-__device__ __forceinline__ double widen(double f) { return f; }
-
 // One coarse level of the hierarchy in one pass: the operator by re-discretisation, and the smoother's
 // omega / diagonal.  Local diagonal = mean of the children's local diagonals (diag - the six
 // couplings of their rows); each face array of the coarse cell's lower face = (mean of that array over
@@ -1013,14 +966,14 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_build(const Op<TF> A, int cnx,
                 const int d[3] = {di, dj, dk};
                 if ((di && !two[0]) || (dj && !two[1]) || (dk && !two[2])) continue;
                 const long long c = c0 + di + dj * s[1] + dk * s[2];
-                dl += widen(__ldg(A.diag + c));
+                dl += (double)(__ldg(A.diag + c));
 #pragma unroll
                 for (int ax = 0; ax < 3; ++ax) {
-                    const double w = widen(__ldg(A.W[ax] + c)), v = widen(__ldg(A.Wp[ax] + c));
+                    const double w = (double)(__ldg(A.W[ax] + c)), v = (double)(__ldg(A.Wp[ax] + c));
                     if (d[ax] == 0) { wl[ax] += w; wp[ax] += v; }      // the parent's lower face
                     else tot += w + v;                                 // a face between children
                     if ((d[ax] == 1 || !two[ax]) && up[ax])            // the parent's upper face
-                        wu[ax] += widen(__ldg(A.Wp[ax] + c + above[ax]));
+                        wu[ax] += (double)(__ldg(A.Wp[ax] + c + above[ax]));
                 }
             }
     double diag = 0.0;
@@ -1112,11 +1065,20 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_to_f32(long long N, const double*
         b[c] = (float)a[c];
 }
 
-// z = x (widened); partial r.z
+// z = x widened to FP64 (a cycle without post-sweeps, whose last sweep would have done it)
+__global__ void __launch_bounds__(LIN_BLOCK) k_from_f32(long long N, const float* __restrict__ x,
+                                                        double* __restrict__ z,
+                                                        const double* skip) {
+    if (skipped(skip)) return;
+    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
+         c += (long long)gridDim.x * LIN_BLOCK)
+        z[c] = (double)x[c];
+}
+
+// z = x (widened); r.z
 __global__ void __launch_bounds__(LIN_BLOCK) k_from_f32_dot(long long N, const float* __restrict__ x,
                                                             const double* __restrict__ r,
-                                                            double* __restrict__ z,
-                                                            double* __restrict__ partials) {
+                                                            double* __restrict__ z, const Finish F) {
     double acc = 0.0;
     for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
          c += (long long)gridDim.x * LIN_BLOCK) {
@@ -1124,8 +1086,7 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_from_f32_dot(long long N, const f
         z[c] = zv;
         acc += r[c] * zv;
     }
-    const double s = block_sum<LIN_BLOCK>(acc);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
+    finish<false, RED_NONE>(F, acc, 0.0);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1140,18 +1101,15 @@ cudaError_t LinLaunch::end() {
     return e;
 }
 
-cudaError_t LinLaunch::matvec_dot(const Op<double>& A, const double* p, double* q, double* part,
-                                  int& nparts) {
-    nparts = stream_blocks(A.N);
+cudaError_t LinLaunch::matvec_dot(const Op<double>& A, const double* p, double* q, const Finish& F) {
     begin("cg_matvec_dot");
-    k_matvec_dot<<<nparts, LIN_BLOCK, 0, st>>>(A, p, q, part);
+    k_matvec_dot<<<sum_blocks(A.N), LIN_BLOCK, 0, st>>>(A, p, q, F);
     return end();
 }
 cudaError_t LinLaunch::cg_xr(long long N, const double* scal, double* x, double* r,
-                             const double* p, const double* q, double* part, int& nparts) {
-    nparts = stream_blocks(N);
+                             const double* p, const double* q, const Finish& F) {
     begin("cg_update_xr");
-    k_cg_xr<<<nparts, LIN_BLOCK, 0, st>>>(N, scal, x, r, p, q, part);
+    k_cg_xr<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, scal, x, r, p, q, F);
     return end();
 }
 cudaError_t LinLaunch::cg_p(long long N, const double* scal, const double* z, double* p, int first) {
@@ -1160,48 +1118,24 @@ cudaError_t LinLaunch::cg_p(long long N, const double* scal, const double* z, do
     return end();
 }
 cudaError_t LinLaunch::jacobi_dot(long long N, const double* r, const double* diag, double* z,
-                                  double* part, int& nparts) {
-    nparts = stream_blocks(N);
+                                  const Finish& F) {
     begin("precond_jacobi");
-    k_jacobi_dot<<<nparts, LIN_BLOCK, 0, st>>>(N, r, diag, z, part, skip);
+    k_jacobi_dot<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, r, diag, z, F, skip);
     return end();
 }
-cudaError_t LinLaunch::dot(long long N, const double* a, const double* b, double* part,
-                           int& nparts) {
-    nparts = stream_blocks(N);
+cudaError_t LinLaunch::dot(long long N, const double* a, const double* b, const Finish& F) {
     begin("dot");
-    k_dot<<<nparts, LIN_BLOCK, 0, st>>>(N, a, b, part);
+    k_dot<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, a, b, F);
     return end();
 }
-cudaError_t LinLaunch::cg_init(long long N, const double* b, double* r, double* x, double* part,
-                               int& nparts) {
-    nparts = stream_blocks(N);
+cudaError_t LinLaunch::cg_init(long long N, const double* b, double* r, double* x, const Finish& F) {
     begin("cg_init");
-    k_cg_init<<<nparts, LIN_BLOCK, 0, st>>>(N, b, r, x, part);
+    k_cg_init<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, b, r, x, F);
     return end();
 }
 cudaError_t LinLaunch::reduce(const double* part, int n, double* scal, int op, int slot) {
     begin("reduce");
-    k_reduce<<<1, RED_BLOCK, 0, st>>>(part, n, scal, op, slot, skip);
-    return end();
-}
-cudaError_t LinLaunch::reduce_loop(const double* part, int n, double* scal, int op,
-                                   unsigned long long cond) {
-    begin("reduce");
-    k_reduce_loop<<<1, RED_BLOCK, 0, st>>>(part, n, scal, op, cond);
-    return end();
-}
-cudaError_t LinLaunch::bicg_xr_loop(long long N, const double* scal, double* x, const double* ph,
-                                    const double* sh, const double* s, const double* t,
-                                    double* r, const double* rh, double* part, int& nparts) {
-    nparts = stream_blocks(N);
-    begin("bicg_update_xr");
-    k_bicg_xr_loop<<<nparts, LIN_BLOCK, 0, st>>>(N, scal, x, ph, sh, s, t, r, rh, part);
-    return end();
-}
-cudaError_t LinLaunch::from_f32(long long N, const float* x, double* z) {
-    begin("mg_from_f32");
-    k_from_f32<<<stream_blocks(N), LIN_BLOCK, 0, st>>>(N, x, z, skip);
+    k_reduce<<<1, RED_BLOCK, 0, st>>>(part, n, scal, op, slot);
     return end();
 }
 cudaError_t LinLaunch::copy(long long N, const double* a, double* b) {
@@ -1211,52 +1145,49 @@ cudaError_t LinLaunch::copy(long long N, const double* a, double* b) {
 }
 
 cudaError_t LinLaunch::matvec_ns(const OpNS& A, const double* x, double* y, const double* w1,
-                                 int two_dots, double* part, int& nparts) {
-    nparts = stream_blocks(A.N);
+                                 int two_dots, const Finish& F) {
     begin("bicg_matvec");
     OpNS B = A;
     B.skip = skip;
-    if (two_dots) k_matvec_ns<true><<<nparts, LIN_BLOCK, 0, st>>>(B, x, y, w1, part);
-    else k_matvec_ns<false><<<nparts, LIN_BLOCK, 0, st>>>(B, x, y, w1, part);
+    const int nb = sum_blocks(A.N);
+    if (two_dots) k_matvec_ns<true><<<nb, LIN_BLOCK, 0, st>>>(B, x, y, w1, F);
+    else k_matvec_ns<false><<<nb, LIN_BLOCK, 0, st>>>(B, x, y, w1, F);
     return end();
 }
 cudaError_t LinLaunch::bicg_init(long long N, const double* b, double* r, double* rh, double* x,
-                                 double* part, int& nparts) {
-    nparts = stream_blocks(N);
+                                 const Finish& F) {
     begin("bicg_init");
-    k_bicg_init<<<nparts, LIN_BLOCK, 0, st>>>(N, b, r, rh, x, part);
+    k_bicg_init<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, b, r, rh, x, F);
     return end();
 }
 cudaError_t LinLaunch::bicg_p(long long N, const double* scal, const double* r, const double* v,
-                              double* p, int first, double* rh) {
-    begin("bicg_update_p");
-    k_bicg_p<<<stream_blocks(N), LIN_BLOCK, 0, st>>>(N, scal, r, v, p, first, rh);
+                              double* p, double* rh, float* p32) {
+    begin(p32 ? "bicg_update_p_f32" : "bicg_update_p");
+    k_bicg_p<<<stream_blocks(N), LIN_BLOCK, 0, st>>>(N, scal, r, v, p, rh, p32);
     return end();
 }
 cudaError_t LinLaunch::bicg_s(long long N, const double* scal, const double* r, const double* v,
-                              double* s, double* part, int& nparts) {
-    nparts = stream_blocks(N);
-    begin("bicg_update_s");
-    k_bicg_s<<<nparts, LIN_BLOCK, 0, st>>>(N, scal, r, v, s, part);
+                              double* s, float* s32, const Finish& F) {
+    begin(s32 ? "bicg_update_s_f32" : "bicg_update_s");
+    k_bicg_s<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, scal, r, v, s, s32, F);
     return end();
 }
 cudaError_t LinLaunch::bicg_xr(long long N, const double* scal, double* x, const double* ph,
                                const double* sh, const double* s, const double* t, double* r,
-                               const double* rh, double* part, int& nparts) {
-    nparts = stream_blocks(N);
+                               const double* rh, const Finish& F) {
     begin("bicg_update_xr");
-    k_bicg_xr<<<nparts, LIN_BLOCK, 0, st>>>(N, scal, x, ph, sh, s, t, r, rh, part);
+    k_bicg_xr<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, scal, x, ph, sh, s, t, r, rh, F);
     return end();
 }
-cudaError_t LinLaunch::axpy(long long N, const double* scal, int slot, const double* p, double* x) {
-    begin("axpy");
-    k_axpy<<<stream_blocks(N), LIN_BLOCK, 0, st>>>(N, scal, slot, p, x);
+cudaError_t LinLaunch::from_f32(long long N, const float* x, double* z) {
+    begin("mg_from_f32");
+    k_from_f32<<<stream_blocks(N), LIN_BLOCK, 0, st>>>(N, x, z, skip);
     return end();
 }
 
 template <typename T>
 cudaError_t LinLaunch::smooth(const Op<T>& A, const T* b, const T* xin, T* xout, T omega,
-                              int first) {
+                              int first, double* out64) {
     // the finest level's sweeps get their own names (the first sweep of a cycle, from x = 0,
     // reads only b and omega / diag)
     if (A.N == fine_N && first) begin(sizeof(T) == 4 ? "mg_smooth_f32_fine_first" : "mg_smooth_f64_fine_first");
@@ -1285,13 +1216,13 @@ cudaError_t LinLaunch::smooth(const Op<T>& A, const T* b, const T* xin, T* xout,
             const size_t smem = (size_t)BULK_STAGES * BULK_ROWS * A.nx * sizeof(float);
             k_mg_smooth_bulk<<<dim3((unsigned)A.ny, (unsigned)(A.nz / BULK_ZB)),
                                (unsigned)((A.nx + 31) / 32 * 32), smem, st>>>(
-                B, b, xin, xout, omega, g_bulk_err_ptr);
+                B, b, xin, xout, omega, g_bulk_err_ptr, out64);
         }
     } else if (sizeof(T) == 4 && !first && A.nz % ZM == 0 && nxy >= 4 * LIN_BLOCK && xin != xout) {
         const dim3 g((unsigned)((nxy + LIN_BLOCK - 1) / LIN_BLOCK), (unsigned)((A.nz + ZM - 1) / ZM));
-        k_mg_smooth_zm<T><<<g, LIN_BLOCK, 0, st>>>(B, b, xin, xout, omega);
+        k_mg_smooth_zm<T><<<g, LIN_BLOCK, 0, st>>>(B, b, xin, xout, omega, out64);
     } else {
-        k_mg_smooth<T><<<stream_blocks(A.N), LIN_BLOCK, 0, st>>>(B, b, xin, xout, omega, first);
+        k_mg_smooth<T><<<stream_blocks(A.N), LIN_BLOCK, 0, st>>>(B, b, xin, xout, omega, first, out64);
     }
     return end();
 }
@@ -1357,17 +1288,16 @@ cudaError_t LinLaunch::to_f32(long long N, const double* a, float* b) {
     return end();
 }
 cudaError_t LinLaunch::from_f32_dot(long long N, const float* x, const double* r, double* z,
-                                    double* part, int& nparts) {
-    nparts = stream_blocks(N);
+                                    const Finish& F) {
     begin("mg_from_f32_dot");
-    k_from_f32_dot<<<nparts, LIN_BLOCK, 0, st>>>(N, x, r, z, part);
+    k_from_f32_dot<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, x, r, z, F);
     return end();
 }
 
 template cudaError_t LinLaunch::smooth<double>(const Op<double>&, const double*, const double*,
-                                               double*, double, int);
+                                               double*, double, int, double*);
 template cudaError_t LinLaunch::smooth<float>(const Op<float>&, const float*, const float*,
-                                              float*, float, int);
+                                              float*, float, int, double*);
 template cudaError_t LinLaunch::restrict_res<double>(const Op<double>&, const double*,
                                                      const double*, int, int, int, double*);
 template cudaError_t LinLaunch::restrict_res<float>(const Op<float>&, const float*, const float*,

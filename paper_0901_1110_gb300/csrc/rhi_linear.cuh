@@ -74,9 +74,19 @@ enum { S_RZ = 0, S_PQ, S_ALPHA, S_BETA, S_RR, S_BREAK, S_TMP, S_RHO, S_OMEGA, S_
        S_STALL, S_RR0, S_NRST, S_RST, S_NSCAL = 32 };
 constexpr int STALL_ITS = 20;
 constexpr int MAX_RESTARTS = 8;
-enum { RED_SUM = 0, RED_ALPHA = 1, RED_BETA = 2, RED_BICG_ALPHA = 3, RED_BICG_OMEGA = 4,
-       RED_BICG_RHO = 5, RED_MAX = 6, RED_BICG_START = 7, RED_BICG_SS = 8,
-       RED_BICG_NEXT = 9 };
+enum { RED_NONE = 0, RED_SUM, RED_ALPHA, RED_BETA, RED_MAX, RED_BICG_ALPHA, RED_BICG_OMEGA,
+       RED_BICG_START, RED_BICG_SS, RED_BICG_NEXT };
+
+// What the last block of a kernel with a dot product does with the sum(s): the scalar update `op` on
+// scal (RED_SUM: to `slot`; RED_NONE: nothing) and, for the loop's updates, the continue flag to the
+// CUDA-graph conditional handle cond (0: none).
+struct Finish {
+    double* partials = nullptr;
+    unsigned* count = nullptr;
+    double* scal = nullptr;
+    int op = RED_NONE, slot = 0;
+    unsigned long long cond = 0;
+};
 
 // number of blocks of the grid-stride streaming kernels (= number of partial sums)
 int stream_blocks(long long N);
@@ -106,46 +116,39 @@ struct LinLaunch {
     void begin(const char* name);
     cudaError_t end();
 
-    cudaError_t matvec_dot(const Op<double>& A, const double* p, double* q, double* part,
-                           int& nparts);
+    cudaError_t matvec_dot(const Op<double>& A, const double* p, double* q, const Finish& F);
     cudaError_t cg_xr(long long N, const double* scal, double* x, double* r, const double* p,
-                      const double* q, double* part, int& nparts);
+                      const double* q, const Finish& F);
     cudaError_t cg_p(long long N, const double* scal, const double* z, double* p, int first);
     cudaError_t jacobi_dot(long long N, const double* r, const double* diag, double* z,
-                           double* part, int& nparts);
-    cudaError_t dot(long long N, const double* a, const double* b, double* part, int& nparts);
-    cudaError_t cg_init(long long N, const double* b, double* r, double* x, double* part,
-                        int& nparts);
+                           const Finish& F);
+    cudaError_t dot(long long N, const double* a, const double* b, const Finish& F);
+    cudaError_t cg_init(long long N, const double* b, double* r, double* x, const Finish& F);
+    // sum (RED_SUM) or max (RED_MAX) of n partials into scal[slot]
     cudaError_t reduce(const double* part, int n, double* scal, int op, int slot);
-    // the reductions of the device-controlled BiCGStab loop (RED_BICG_START / _SS / _NEXT);
-    // cond: the CUDA-graph conditional handle the loop's continue flag is written to (0: none)
-    cudaError_t reduce_loop(const double* part, int n, double* scal, int op,
-                            unsigned long long cond);
     // BiCGStab (right-preconditioned) building blocks
-    cudaError_t matvec_ns(const OpNS& A, const double* x, double* y, const double* w1,
-                          int two_dots, double* part, int& nparts);
+    cudaError_t matvec_ns(const OpNS& A, const double* x, double* y, const double* w1, int two_dots,
+                          const Finish& F);
     cudaError_t bicg_init(long long N, const double* b, double* r, double* rh, double* x,
-                          double* part, int& nparts);
-    // first: 1 p = r; 0 the update; -1 decided on the device (p = r, and rh = r when rh is
-    // given, at S_ITS = 0 or after a restart)
+                          const Finish& F);
+    // p = r at the loop's first iteration and after a restart (then also rh = r), else the update;
+    // p32 (may be null): its FP32 copy
     cudaError_t bicg_p(long long N, const double* scal, const double* r, const double* v,
-                       double* p, int first, double* rh = nullptr);
+                       double* p, double* rh, float* p32);
     cudaError_t bicg_s(long long N, const double* scal, const double* r, const double* v,
-                       double* s, double* part, int& nparts);
+                       double* s, float* s32, const Finish& F);
+    // the x / r update: converged at the middle of the iteration (S_HALF) x += alpha ph only;
+    // after a breakdown nothing
     cudaError_t bicg_xr(long long N, const double* scal, double* x, const double* ph,
-                        const double* sh, const double* s, const double* t, double* r,
-                        const double* rh, double* part, int& nparts);
-    cudaError_t axpy(long long N, const double* scal, int slot, const double* p, double* x);
-    // the x / r update of the device-controlled loop: converged at the middle of the
-    // iteration (S_HALF) x += alpha ph only; after a breakdown nothing
-    cudaError_t bicg_xr_loop(long long N, const double* scal, double* x, const double* ph,
-                             const double* sh, const double* s, const double* t, double* r,
-                             const double* rh, double* part, int& nparts);
-    cudaError_t from_f32(long long N, const float* x, double* z);
+                        const double* sh, const double* s, const double* t, double* r, const double* rh,
+                        const Finish& F);
     cudaError_t copy(long long N, const double* a, double* b);
+    cudaError_t from_f32(long long N, const float* x, double* z);
 
+    // out64 (not for the first sweep): the result goes there in FP64 instead of to xout
     template <typename T>
-    cudaError_t smooth(const Op<T>& A, const T* b, const T* xin, T* xout, T omega, int first);
+    cudaError_t smooth(const Op<T>& A, const T* b, const T* xin, T* xout, T omega, int first,
+                       double* out64 = nullptr);
     template <typename T>
     cudaError_t mg_tail(const MgTail<T>& M);
     template <typename T>
@@ -166,7 +169,7 @@ struct LinLaunch {
     cudaError_t cast_op(const Op<double>& A, float* d, float* const* w);
     cudaError_t to_f32(long long N, const double* a, float* b);
     cudaError_t from_f32_dot(long long N, const float* x, const double* r, double* z,
-                             double* part, int& nparts);
+                             const Finish& F);
 };
 
 }  // namespace rhi

@@ -86,13 +86,7 @@ struct TailCell {
     bool on;                 // the thread has such a cell
 };
 
-// A thread's work on its one cell of a level sits in a loop the compiler cannot see the length of, so
-// that warps without a cell branch around it: predicated FP64 instructions would take their turn on
-// the FP64 pipe (64 cycles each) all the same.
-__device__ __forceinline__ int opaque(int v) {
-    asm volatile("" : "+r"(v));
-    return v;
-}
+// A thread's work on its one cell of a level stays a branch (opaque): warps without a cell go around it.
 #define TAIL_CELL(on) for (int go_ = (on) ? 1 : 0; go_; go_ = M == 1 ? opaque(0) : 0)
 
 template <typename T>

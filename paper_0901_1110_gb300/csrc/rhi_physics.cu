@@ -726,8 +726,9 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_cell(const StepParams P, const P
         }
     }
     if (MODE != MODE_PREP_PREDICT) {
-        const double s = block_sum<CELL_BLOCK>(fsq);
-        if (threadIdx.x == 0) B.partials[blockIdx.x] = s;
+        double s, unused;
+        if (grid_sum<CELL_BLOCK, false>(fsq, 0.0, B.partials, B.count, s, unused) && threadIdx.x == 0)
+            *B.norm_sq = s;
     }
 }
 
