@@ -188,7 +188,7 @@ struct rhi_ctx {
     long long mlp_t = 0;                  // Adam steps taken
     int mlp_skip = 0;                     // steps left that skip the network (mlp_retry)
     struct Scratch { void* p = nullptr; size_t bytes = 0; };
-    Scratch mlp_scr[6];                   // act, del, partials, X, Y, grad staging
+    Scratch mlp_scr[4];                   // block gradients, loss partials, X, Y staging
     ~rhi_ctx() { for (auto& s : mlp_scr) if (s.p) cudaFree(s.p); }
 };
 
@@ -1037,7 +1037,7 @@ int validate_params(const rhi_params* p) {
 
 // ---- learned guess helpers
 
-enum { SCR_ACT = 0, SCR_DEL, SCR_PART, SCR_X, SCR_Y, SCR_G };
+enum { SCR_GRAD = 0, SCR_PART, SCR_X, SCR_Y };
 
 template <typename T>
 int scratch(rhi_ctx* h, int slot, size_t count, T** out) {
@@ -1076,33 +1076,20 @@ MlpArgs mlp_args(const rhi_ctx* h, double dt, double a) {
     return A;
 }
 
-// host copy of the master weights -> BF16 inference copy on the device
-int mlp_repack(rhi_ctx* h) {
-    std::vector<float> w(RHI_MLP_NWEIGHTS);
-    CK(cudaMemcpyAsync(w.data(), h->mlp_w, w.size() * sizeof(float), cudaMemcpyDeviceToHost, h->st));
-    CK(cudaStreamSynchronize(h->st));
-    MlpPacked pk;
-    mlp_pack(w.data(), &pk);
-    CK(cudaMemcpyAsync(h->mlp_pk, &pk, sizeof pk, cudaMemcpyHostToDevice, h->st));
-    CK(cudaStreamSynchronize(h->st));
+// forward + backward of m samples (device X, Y): block gradients into the scratch (*gpart), the
+// blocks' squared-error sums into part (mlp_train_blocks(m) entries)
+int mlp_batch(rhi_ctx* h, const float* X, const float* Y, long long m, double* part, float** gpart) {
+    int rc;
+    if ((rc = scratch(h, SCR_GRAD, (size_t)mlp_train_blocks(m) * mlp_ntrain(), gpart))) return rc;
+    Scope s(h->prof, "mlp_fwd_bwd");
+    CK(launch_mlp_train(h->mlp_w, X, Y, m, *gpart, part, h->st));
     return RHI_OK;
 }
 
-// forward + backward of m samples (device X, Y) into h->mlp_g; squared-error block sums in
-// part (ceil(m / block) entries)
-int mlp_grad(rhi_ctx* h, const float* X, const float* Y, long long m, double* part) {
-    float *act, *del;
-    int rc;
-    if ((rc = scratch(h, SCR_ACT, (size_t)m * ACT_STRIDE, &act))) return rc;
-    if ((rc = scratch(h, SCR_DEL, (size_t)m * DEL_STRIDE, &del))) return rc;
-    {
-        Scope s(h->prof, "mlp_fwd_bwd");
-        CK(launch_mlp_fwd_bwd(h->mlp_w, X, Y, m, act, del, part, h->st));
-    }
-    {
-        Scope s(h->prof, "mlp_wgrad");
-        CK(launch_mlp_wgrad(act, del, m, h->mlp_g, h->st));
-    }
+// FP32 master weights -> BF16 inference copy
+int mlp_repack(rhi_ctx* h) {
+    Scope s(h->prof, "mlp_pack");
+    CK(launch_mlp_pack(h->mlp_w, h->mlp_pk, h->st));
     return RHI_OK;
 }
 
@@ -1869,6 +1856,8 @@ int rhi_mlp_set_weights(rhi_handle h, const float* w, size_t n) {
     h->mlp_t = 0;
     h->mlp_skip = 0;
     if ((rc = mlp_repack(h))) return rc;
+    CK(cudaStreamSynchronize(h->st));
+    h->prof.resolve();
     h->mlp_ready = true;
     return RHI_OK;
 }
@@ -1979,13 +1968,18 @@ int rhi_mlp_loss_grad(rhi_handle h, const float* X, const float* Y, long long n,
         xs = xd;
         ys = yd;
     }
-    const long long nb = (n + mlp_train_block() - 1) / mlp_train_block();
+    const int nb = mlp_train_blocks(n);
     double* part;
+    float* gpart;
     if ((rc = scratch(h, SCR_PART, (size_t)nb, &part))) return rc;
-    CK(cudaMemsetAsync(h->mlp_g, 0, RHI_MLP_NWEIGHTS * sizeof(float), h->st));
-    if ((rc = mlp_grad(h, xs, ys, n, part))) return rc;
+    // (the normalisation's entries of the gradient stay at the 0 rhi_mlp_set_weights gave them)
+    if ((rc = mlp_batch(h, xs, ys, n, part, &gpart))) return rc;
+    {
+        Scope s(h->prof, "mlp_wgrad");
+        CK(launch_mlp_grad(gpart, nb, h->mlp_g, h->st));
+    }
     LinLaunch L(h->st, &h->prof);
-    CK(L.reduce(part, (int)nb, h->scal, RED_SUM, S_TMP));
+    CK(L.reduce(part, nb, h->scal, RED_SUM, S_TMP));
     double se = 0.0;
     if ((rc = read_scalar(h, S_TMP, &se))) return rc;
     if (loss) *loss = se / ((double)n * MLP_OUT);
@@ -2003,28 +1997,27 @@ int rhi_mlp_train(rhi_handle h, const float* X, const float* Y, long long n, int
     if (!h->mlp_ready) return fail(h, RHI_ERR_STATE, "rhi_mlp_train: no weights set");
     if (!X || !Y || n < 1 || epochs < 1 || batch < 1 || !(lr > 0.0))
         return fail(h, RHI_ERR_ARG, "rhi_mlp_train: bad arguments");
-    const long long tb = mlp_train_block();
     const long long nbatch = (n + batch - 1) / batch;
     // block partials of one epoch, one slice per minibatch
-    const long long nparts = nbatch * (((long long)batch + tb - 1) / tb);
+    const long long nparts = nbatch * mlp_train_blocks(batch);
     if (nparts > (1LL << 30)) return fail(h, RHI_ERR_ARG, "rhi_mlp_train: too many samples");
     double* part;
     int rc;
     if ((rc = scratch(h, SCR_PART, (size_t)nparts, &part))) return rc;
-    CK(cudaMemsetAsync(part, 0, (size_t)nparts * sizeof(double), h->st));
-    const int nupd = RHI_MLP_NWEIGHTS - 2 * RHI_MLP_IN;        // normalisation stays fixed
     for (int ep = 0; ep < epochs; ++ep) {
         long long po = 0;
         for (long long b = 0; b < nbatch; ++b) {
             const long long s0 = b * batch;
             const long long m = std::min<long long>(batch, n - s0);
-            if ((rc = mlp_grad(h, X + s0 * MLP_IN, Y + s0 * MLP_OUT, m, part + po))) return rc;
-            po += (m + tb - 1) / tb;
+            float* gpart;
+            if ((rc = mlp_batch(h, X + s0 * MLP_IN, Y + s0 * MLP_OUT, m, part + po, &gpart))) return rc;
+            const int nb = mlp_train_blocks(m);
+            po += nb;
             h->mlp_t += 1;
             const float b1t = (float)std::pow(0.9, (double)h->mlp_t);
             const float b2t = (float)std::pow(0.999, (double)h->mlp_t);
             Scope s(h->prof, "mlp_adam");
-            CK(launch_mlp_adam(h->mlp_w, h->mlp_g, h->mlp_m1, h->mlp_m2, nupd, (float)lr, b1t, b2t, h->st));
+            CK(launch_mlp_adam(gpart, nb, h->mlp_w, h->mlp_m1, h->mlp_m2, (float)lr, b1t, b2t, h->st));
         }
         if (ep == epochs - 1 && loss) {
             LinLaunch L(h->st, &h->prof);
@@ -2035,6 +2028,7 @@ int rhi_mlp_train(rhi_handle h, const float* X, const float* Y, long long n, int
         }
     }
     if ((rc = mlp_repack(h))) return rc;
+    CK(cudaStreamSynchronize(h->st));
     h->prof.resolve();
     return RHI_OK;
 }

@@ -10,9 +10,10 @@
 //   outputs   log10 E'/E, log10 e'/e, logit x_HI', He fraction logits (softmax)
 //
 // Inference runs on the tensor cores (mma.sync m16n8k16, BF16 operands, FP32 accumulation)
-// with the layer activations chained in registers; training runs FP32 on the CUDA cores with
-// one thread per sample, a deterministic weight-gradient reduction and Adam.
+// with the layer activations chained in registers; training runs FP32 on the CUDA cores, tiles of
+// 32 samples per block, with a deterministic gradient reduction and Adam.
 #include <cmath>
+#include <cstddef>
 
 #include "rhi_mlp.cuh"
 
@@ -21,7 +22,7 @@ namespace rhi {
 namespace {
 
 constexpr int INF_WARPS = 4;                  // warps per inference block
-constexpr int TRAIN_BLOCK = 128;
+constexpr int TRAIN_BLOCK = 256;
 
 // ------------------------------------------------------------------------------------------
 // features of one cell (FP32 from the FP64 state)
@@ -273,7 +274,7 @@ __global__ void __launch_bounds__(32 * INF_WARPS) k_mlp_infer(const MlpArgs A,
 }
 
 // ------------------------------------------------------------------------------------------
-// FP32 training: one thread per sample
+// FP32 training
 
 struct TrainW {
     float W1[MLP_HID * MLP_IN], b1[MLP_HID];
@@ -283,135 +284,333 @@ struct TrainW {
     float mean[MLP_IN], scale[MLP_IN];
 };
 static_assert(sizeof(TrainW) == RHI_MLP_NWEIGHTS * sizeof(float), "weight layout");
+// offsets in the weight vector
+constexpr int OW1 = 0, OB1 = OW1 + MLP_HID * MLP_IN, OW2 = OB1 + MLP_HID,
+              OB2 = OW2 + MLP_HID * MLP_HID, OW3 = OB2 + MLP_HID, OB3 = OW3 + MLP_HID * MLP_HID,
+              OW4 = OB3 + MLP_HID, OB4 = OW4 + MLP_OUT * MLP_HID, NTRAIN = OB4 + MLP_OUT;
 
 __device__ __forceinline__ float sig_f(float z) { return 1.0f / (1.0f + expf(-z)); }
 
-// forward + backward of one sample: stores the per-sample deltas d1, d2, d3 (64 each), g4 (6)
-// and the activations h0 (9), h1, h2, h3 (64 each) for the weight-gradient reduction, and the
-// squared error into the block partials
-__global__ void __launch_bounds__(TRAIN_BLOCK) k_mlp_fwd_bwd(const float* __restrict__ w,
-                                                             const float* __restrict__ X,
-                                                             const float* __restrict__ Y,
-                                                             long long m, float inv_norm,
-                                                             float* __restrict__ act,
-                                                             float* __restrict__ del,
-                                                             double* __restrict__ partials) {
-    extern __shared__ float smem[];
-    TrainW& W = *reinterpret_cast<TrainW*>(smem);
-    for (int q = threadIdx.x; q < RHI_MLP_NWEIGHTS; q += blockDim.x) smem[q] = w[q];
-    __syncthreads();
-    const long long s = blockIdx.x * (long long)TRAIN_BLOCK + threadIdx.x;
+// Forward, backward and weight gradient of tiles of 32 samples, one tile at a time per block of 256
+// threads, all in shared memory: the weights (rows padded to 68 floats, so that the eight rows a
+// warp reads at once fall into different banks), the activations and their derivatives, [sample]
+// [feature].  Each matrix product is a 64 x 32 (layers) or 64 x 64 (weight gradients) tile in FP32
+// FMAs, 4 x 2 or 4 x 4 results per thread from 16-byte loads.  A block adds the gradients of its
+// tiles in registers and writes them once; k_mlp_apply adds the blocks' in order, so a result does
+// not depend on timing.
+//
+// Bound by shared-memory loads (four wavefronts per 16-byte load of a warp).  A minibatch of 4096
+// samples: 40 us with its update, against 450 us for one thread per sample with its activations in local memory and a
+// gradient pass that walked the samples in one chain per weight.
+constexpr int TT = 32;                         // samples per tile
+constexpr int PS = MLP_HID + 4;                // padded row
+constexpr int PS0 = MLP_IN + 3;                // padded input row (16 floats)
+struct TrainSmem {
+    float W1[MLP_HID * PS0], W2[MLP_HID * PS], W3[MLP_HID * PS], W4[MLP_OUT * PS];
+    float b1[MLP_HID], b2[MLP_HID], b3[MLP_HID], b4[8];
+    float mean[16], scale[16];                                      // (MLP_IN of each)
+    float h0[TT * PS0], h1[TT * PS], h2[TT * PS], h3[TT * PS];      // activations
+    float p1[TT * PS], p2[TT * PS], p3[TT * PS];                    // SiLU', then the deltas
+    float g4[TT * 8];
+};
+// every row that is read or written in 16-byte pieces starts on a 16-byte boundary
+static_assert(PS % 4 == 0 && PS0 % 4 == 0 && PS0 >= MLP_IN, "row padding");
+static_assert(offsetof(TrainSmem, W1) % 16 == 0 && offsetof(TrainSmem, W2) % 16 == 0 &&
+              offsetof(TrainSmem, W3) % 16 == 0 && offsetof(TrainSmem, W4) % 16 == 0 &&
+              offsetof(TrainSmem, h0) % 16 == 0 && offsetof(TrainSmem, h1) % 16 == 0 &&
+              offsetof(TrainSmem, h2) % 16 == 0 && offsetof(TrainSmem, h3) % 16 == 0 &&
+              offsetof(TrainSmem, p1) % 16 == 0 && offsetof(TrainSmem, p2) % 16 == 0 &&
+              offsetof(TrainSmem, p3) % 16 == 0, "alignment of the tiles");
+
+// acc[4][2] = rows n0.. of W (64 x K, row stride S) times samples s0, s0 + 1 (row stride S)
+template <int K, int S>
+__device__ __forceinline__ void tile_fwd(const float* W, const float* h, int n0, int s0, float (&acc)[4][2]) {
+#pragma unroll 4
+    for (int k = 0; k < K; k += 4) {
+        float4 w[4], x[2];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) w[q] = *reinterpret_cast<const float4*>(W + (n0 + q) * S + k);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) x[q] = *reinterpret_cast<const float4*>(h + (s0 + q) * S + k);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                acc[q][t] = fmaf(w[q].x, x[t].x, acc[q][t]);
+                acc[q][t] = fmaf(w[q].y, x[t].y, acc[q][t]);
+                acc[q][t] = fmaf(w[q].z, x[t].z, acc[q][t]);
+                acc[q][t] = fmaf(w[q].w, x[t].w, acc[q][t]);
+            }
+    }
+}
+// SiLU and its derivative of a tile's pre-activations
+__device__ __forceinline__ void tile_act(const float (&acc)[4][2], int n0, int s0, float* h, float* p) {
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        float4 hv, pv;
+        float* hq = &hv.x;
+        float* pq = &pv.x;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float z = acc[q][t], sg = sig_f(z);
+            hq[q] = z * sg;
+            pq[q] = sg * (1.0f + z * (1.0f - sg));
+        }
+        *reinterpret_cast<float4*>(h + (s0 + t) * PS + n0) = hv;
+        *reinterpret_cast<float4*>(p + (s0 + t) * PS + n0) = pv;
+    }
+}
+// deltas of the layer below: p (SiLU') *= W^T d, columns k0.. of W (64 x 64), samples s0, s0 + 1
+__device__ __forceinline__ void tile_bwd(const float* W, const float* d, int k0, int s0, float* p) {
+    float acc[2][4] = {};
+#pragma unroll 4
+    for (int n = 0; n < MLP_HID; n += 4) {
+        float4 x[2];
+#pragma unroll
+        for (int t = 0; t < 2; ++t) x[t] = *reinterpret_cast<const float4*>(d + (s0 + t) * PS + n);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 w = *reinterpret_cast<const float4*>(W + (n + q) * PS + k0);
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                const float dv = q == 0 ? x[t].x : (q == 1 ? x[t].y : (q == 2 ? x[t].z : x[t].w));
+                acc[t][0] = fmaf(w.x, dv, acc[t][0]);
+                acc[t][1] = fmaf(w.y, dv, acc[t][1]);
+                acc[t][2] = fmaf(w.z, dv, acc[t][2]);
+                acc[t][3] = fmaf(w.w, dv, acc[t][3]);
+            }
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < 2; ++t) {
+        float4* pp = reinterpret_cast<float4*>(p + (s0 + t) * PS + k0);
+        float4 v = *pp;
+        v.x *= acc[t][0]; v.y *= acc[t][1]; v.z *= acc[t][2]; v.w *= acc[t][3];
+        *pp = v;
+    }
+}
+// weight gradient rows n0.., columns k0.. += sum over the tile's samples of d_n h_k
+__device__ __forceinline__ void tile_grad(const float* d, const float* h, int n0, int k0, float (&g)[4][4]) {
+#pragma unroll 4
+    for (int s = 0; s < TT; ++s) {
+        const float4 a = *reinterpret_cast<const float4*>(d + s * PS + n0);
+        const float4 x = *reinterpret_cast<const float4*>(h + s * PS + k0);
+        const float av[4] = {a.x, a.y, a.z, a.w}, xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int t = 0; t < 4; ++t) g[q][t] = fmaf(av[q], xv[t], g[q][t]);
+    }
+}
+
+__global__ void __launch_bounds__(TRAIN_BLOCK) k_mlp_train(const float* __restrict__ w,
+                                                           const float* __restrict__ X,
+                                                           const float* __restrict__ Y,
+                                                           long long m, float inv_norm,
+                                                           float* __restrict__ gpart,
+                                                           double* __restrict__ partials) {
+    extern __shared__ __align__(16) unsigned char train_smem[];
+    TrainSmem& S = *reinterpret_cast<TrainSmem*>(train_smem);
+    const int tid = (int)threadIdx.x;
+    for (int q = tid; q < MLP_HID * MLP_HID; q += TRAIN_BLOCK) {
+        const int n = q >> 6, k = q & 63;
+        S.W2[n * PS + k] = w[OW2 + q];
+        S.W3[n * PS + k] = w[OW3 + q];
+        if (n < MLP_OUT) S.W4[n * PS + k] = w[OW4 + q];
+    }
+    for (int q = tid; q < MLP_HID * PS0; q += TRAIN_BLOCK) {
+        const int n = q / PS0, k = q % PS0;
+        S.W1[q] = k < MLP_IN ? w[OW1 + n * MLP_IN + k] : 0.0f;
+    }
+    if (tid < MLP_HID) {
+        S.b1[tid] = w[OB1 + tid];
+        S.b2[tid] = w[OB2 + tid];
+        S.b3[tid] = w[OB3 + tid];
+        if (tid < MLP_OUT) S.b4[tid] = w[OB4 + tid];
+        if (tid < MLP_IN) { S.mean[tid] = w[NTRAIN + tid]; S.scale[tid] = w[NTRAIN + MLP_IN + tid]; }
+    }
+    // layer tiles: 16 groups of 4 neurons x 16 pairs of samples, 8 x 4 of them per warp; gradient tiles:
+    // 16 x 16 groups of 4 x 4
+    const int lane = tid & 31, warp = tid >> 5;
+    const int n0 = 4 * ((lane & 7) + 8 * (warp & 1)), s0 = 2 * ((lane >> 3) + 4 * (warp >> 1));
+    const int gn = 4 * (tid >> 4), gk = 4 * (tid & 15);
+    float g2[4][4] = {}, g3[4][4] = {}, g1[4] = {}, gw4[2] = {}, gb = 0.0f, gb4 = 0.0f;
     double se = 0.0;
-    if (s < m) {
-        float h0[MLP_IN], z1[MLP_HID], z2[MLP_HID], z3[MLP_HID], h[MLP_HID], out[MLP_OUT];
-        for (int k = 0; k < MLP_IN; ++k) h0[k] = (X[s * MLP_IN + k] - W.mean[k]) / W.scale[k];
-        for (int n = 0; n < MLP_HID; ++n) {
-            float a = W.b1[n];
-            for (int k = 0; k < MLP_IN; ++k) a += W.W1[n * MLP_IN + k] * h0[k];
-            z1[n] = a;
+    const long long tiles = (m + TT - 1) / TT;
+    for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const long long base = tile * TT;
+        const int cnt = (int)(m - base < TT ? m - base : TT);
+        __syncthreads();                                    // the last tile's arrays are free
+        for (int q = tid; q < TT * PS0; q += TRAIN_BLOCK) {
+            const int s = q / PS0, k = q % PS0;
+            float v = 0.0f;
+            if (k < MLP_IN && s < cnt) v = (X[(base + s) * MLP_IN + k] - S.mean[k]) / S.scale[k];
+            S.h0[q] = v;
         }
-        for (int k = 0; k < MLP_HID; ++k) h[k] = z1[k] * sig_f(z1[k]);
-        for (int n = 0; n < MLP_HID; ++n) {
-            float a = W.b2[n];
-            for (int k = 0; k < MLP_HID; ++k) a += W.W2[n * MLP_HID + k] * h[k];
-            z2[n] = a;
+        __syncthreads();
+        float acc[4][2];
+        auto bias = [&](const float* b) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[q][0] = acc[q][1] = b[n0 + q];
+        };
+        bias(S.b1);
+        tile_fwd<PS0, PS0>(S.W1, S.h0, n0, s0, acc);
+        tile_act(acc, n0, s0, S.h1, S.p1);
+        __syncthreads();
+        bias(S.b2);
+        tile_fwd<MLP_HID, PS>(S.W2, S.h1, n0, s0, acc);
+        tile_act(acc, n0, s0, S.h2, S.p2);
+        __syncthreads();
+        bias(S.b3);
+        tile_fwd<MLP_HID, PS>(S.W3, S.h2, n0, s0, acc);
+        tile_act(acc, n0, s0, S.h3, S.p3);
+        __syncthreads();
+        // outputs: thread (sample, n); the delta of a sample beyond the last is 0
+        {
+            const int s = tid >> 3, n = tid & 7;
+            float gv = 0.0f;
+            if (n < MLP_OUT && s < cnt) {
+                float a = S.b4[n];
+#pragma unroll 4
+                for (int k = 0; k < MLP_HID; k += 4) {
+                    const float4 wv = *reinterpret_cast<const float4*>(S.W4 + n * PS + k);
+                    const float4 hv = *reinterpret_cast<const float4*>(S.h3 + s * PS + k);
+                    a = fmaf(wv.x, hv.x, a);
+                    a = fmaf(wv.y, hv.y, a);
+                    a = fmaf(wv.z, hv.z, a);
+                    a = fmaf(wv.w, hv.w, a);
+                }
+                const float d = a - Y[(base + s) * MLP_OUT + n];
+                se += (double)d * d;
+                gv = 2.0f * d * inv_norm;
+            }
+            S.g4[s * 8 + n] = gv;
         }
-        for (int k = 0; k < MLP_HID; ++k) h[k] = z2[k] * sig_f(z2[k]);
-        for (int n = 0; n < MLP_HID; ++n) {
-            float a = W.b3[n];
-            for (int k = 0; k < MLP_HID; ++k) a += W.W3[n * MLP_HID + k] * h[k];
-            z3[n] = a;
-        }
-        for (int k = 0; k < MLP_HID; ++k) h[k] = z3[k] * sig_f(z3[k]);
-        float g4[MLP_OUT];
-        for (int n = 0; n < MLP_OUT; ++n) {
-            float a = W.b4[n];
-            for (int k = 0; k < MLP_HID; ++k) a += W.W4[n * MLP_HID + k] * h[k];
-            out[n] = a;
-            const float d = a - Y[s * MLP_OUT + n];
-            se += (double)d * d;
-            g4[n] = 2.0f * d * inv_norm;
-        }
-        // activations for the weight gradients: h0 | h1 | h2 | h3
-        float* as = act + s * ACT_STRIDE;
-        for (int k = 0; k < MLP_IN; ++k) as[k] = h0[k];
-        for (int k = 0; k < MLP_HID; ++k) {
-            as[MLP_IN + k] = z1[k] * sig_f(z1[k]);
-            as[MLP_IN + MLP_HID + k] = z2[k] * sig_f(z2[k]);
-            as[MLP_IN + 2 * MLP_HID + k] = h[k];
-        }
-        // deltas: d1 | d2 | d3 | g4
-        float* ds = del + s * DEL_STRIDE;
-        for (int n = 0; n < MLP_OUT; ++n) ds[3 * MLP_HID + n] = g4[n];
-        float d3[MLP_HID];
-        for (int k = 0; k < MLP_HID; ++k) {
+        __syncthreads();
+        // deltas d3 (in p3), then d2, d1
+        for (int q = tid; q < TT * MLP_HID; q += TRAIN_BLOCK) {
+            const int s = q >> 6, k = q & 63;
             float a = 0.0f;
-            for (int n = 0; n < MLP_OUT; ++n) a += W.W4[n * MLP_HID + k] * g4[n];
-            const float sg = sig_f(z3[k]);
-            d3[k] = a * sg * (1.0f + z3[k] * (1.0f - sg));
-            ds[2 * MLP_HID + k] = d3[k];
+#pragma unroll
+            for (int n = 0; n < MLP_OUT; ++n) a = fmaf(S.W4[n * PS + k], S.g4[s * 8 + n], a);
+            S.p3[s * PS + k] *= a;
         }
-        float d2[MLP_HID];
-        for (int k = 0; k < MLP_HID; ++k) {
-            float a = 0.0f;
-            for (int n = 0; n < MLP_HID; ++n) a += W.W3[n * MLP_HID + k] * d3[n];
-            const float sg = sig_f(z2[k]);
-            d2[k] = a * sg * (1.0f + z2[k] * (1.0f - sg));
-            ds[MLP_HID + k] = d2[k];
+        __syncthreads();
+        tile_bwd(S.W3, S.p3, n0, s0, S.p2);
+        __syncthreads();
+        tile_bwd(S.W2, S.p2, n0, s0, S.p1);
+        __syncthreads();
+        // gradients: W3 and W2 tiles, W1 (thread: neuron, 4 inputs), W4 (384 entries) and the biases
+        tile_grad(S.p3, S.h2, gn, gk, g3);
+        tile_grad(S.p2, S.h1, gn, gk, g2);
+        {
+            const int n = tid >> 2, k = 4 * (tid & 3);
+#pragma unroll 4
+            for (int s = 0; s < TT; ++s) {
+                const float d = S.p1[s * PS + n];
+                const float4 x = *reinterpret_cast<const float4*>(S.h0 + s * PS0 + k);
+                g1[0] = fmaf(d, x.x, g1[0]);
+                g1[1] = fmaf(d, x.y, g1[1]);
+                g1[2] = fmaf(d, x.z, g1[2]);
+                g1[3] = fmaf(d, x.w, g1[3]);
+            }
+            const int k4 = tid & 63, n4 = tid >> 6;          // W4: rows n4 and, for n4 < 2, n4 + 4
+#pragma unroll 4
+            for (int s = 0; s < TT; ++s) {
+                const float hv = S.h3[s * PS + k4];
+                gw4[0] = fmaf(S.g4[s * 8 + n4], hv, gw4[0]);
+                if (n4 < 2) gw4[1] = fmaf(S.g4[s * 8 + n4 + 4], hv, gw4[1]);
+            }
+            // biases: b1, b2, b3 by threads 0-191, b4 by threads 192-197
+            const float* d = tid < 64 ? S.p1 : (tid < 128 ? S.p2 : S.p3);
+            if (tid < 192) {
+#pragma unroll 4
+                for (int s = 0; s < TT; ++s) gb += d[s * PS + (tid & 63)];
+            } else if (tid < 192 + MLP_OUT) {
+#pragma unroll 4
+                for (int s = 0; s < TT; ++s) gb4 += S.g4[s * 8 + tid - 192];
+            }
         }
-        for (int k = 0; k < MLP_HID; ++k) {
-            float a = 0.0f;
-            for (int n = 0; n < MLP_HID; ++n) a += W.W2[n * MLP_HID + k] * d2[n];
-            const float sg = sig_f(z1[k]);
-            ds[k] = a * sg * (1.0f + z1[k] * (1.0f - sg));
+    }
+    // this block's gradient
+    float* g = gpart + (long long)blockIdx.x * NTRAIN;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            g[OW2 + (gn + q) * MLP_HID + gk + t] = g2[q][t];
+            g[OW3 + (gn + q) * MLP_HID + gk + t] = g3[q][t];
         }
+    {
+        const int n = tid >> 2, k = 4 * (tid & 3);
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+            if (k + t < MLP_IN) g[OW1 + n * MLP_IN + k + t] = g1[t];
+        const int k4 = tid & 63, n4 = tid >> 6;
+        g[OW4 + n4 * MLP_HID + k4] = gw4[0];
+        if (n4 < 2) g[OW4 + (n4 + 4) * MLP_HID + k4] = gw4[1];
+        if (tid < 192) g[(tid < 64 ? OB1 : (tid < 128 ? OB2 : OB3)) + (tid & 63)] = gb;
+        else if (tid < 192 + MLP_OUT) g[OB4 + tid - 192] = gb4;
     }
     const double bs = block_sum<TRAIN_BLOCK>(se);
-    if (threadIdx.x == 0) partials[blockIdx.x] = bs;
+    if (tid == 0) partials[blockIdx.x] = bs;
 }
 
-// weight gradients: one block per weight row (layer, n); thread k sums delta_n h_k over the
-// samples in a fixed order (deterministic); the last thread of a row also sums the bias
-__global__ void __launch_bounds__(MLP_HID) k_mlp_wgrad(const float* __restrict__ act,
-                                                       const float* __restrict__ del, long long m,
-                                                       float* __restrict__ grad) {
-    // rows: layer 1: 64 rows x 9 inputs, layer 2, 3: 64 x 64, layer 4: 6 x 64
-    int row = blockIdx.x, layer, n;
-    if (row < MLP_HID) { layer = 0; n = row; }
-    else if (row < 2 * MLP_HID) { layer = 1; n = row - MLP_HID; }
-    else if (row < 3 * MLP_HID) { layer = 2; n = row - 2 * MLP_HID; }
-    else { layer = 3; n = row - 3 * MLP_HID; }
-    const int K = layer == 0 ? MLP_IN : MLP_HID;
-    const int aoff = layer == 0 ? 0 : MLP_IN + (layer - 1) * MLP_HID;
-    const int doff = layer == 3 ? 3 * MLP_HID + n : layer * MLP_HID + n;
-    const int k = threadIdx.x;
-    float acc = 0.0f, bacc = 0.0f;
-    for (long long s = 0; s < m; ++s) {
-        const float d = del[s * DEL_STRIDE + doff];
-        if (k < K) acc += d * act[s * ACT_STRIDE + aoff + k];
-        bacc += d;
+// Sum of the blocks' gradients in a fixed order, then the Adam update (ADAM) or the gradient itself.
+// 32 weights per block, 8 threads for each.
+template <bool ADAM>
+__global__ void __launch_bounds__(256) k_mlp_apply(const float* __restrict__ gpart, int nb,
+                                                   float* __restrict__ w, float* __restrict__ g,
+                                                   float* __restrict__ m1, float* __restrict__ m2,
+                                                   float lr, float b1t, float b2t) {
+    __shared__ float part[8][32];
+    const int q = blockIdx.x * 32 + (threadIdx.x & 31), grp = threadIdx.x >> 5;
+    float a = 0.0f;
+    if (q < NTRAIN) {
+#pragma unroll 4
+        for (int b = grp; b < nb; b += 8) a += gpart[(long long)b * NTRAIN + q];
     }
-    // weight vector offsets
-    const int wofs[4] = {0, MLP_HID * MLP_IN + MLP_HID,
-                         MLP_HID * MLP_IN + MLP_HID + MLP_HID * MLP_HID + MLP_HID,
-                         MLP_HID * MLP_IN + MLP_HID + 2 * (MLP_HID * MLP_HID + MLP_HID)};
-    const int nrows = layer == 3 ? MLP_OUT : MLP_HID;
-    if (k < K) grad[wofs[layer] + n * K + k] = acc;
-    if (k == 0) grad[wofs[layer] + nrows * K + n] = bacc;
+    part[grp][threadIdx.x & 31] = a;
+    __syncthreads();
+    if (grp != 0 || q >= NTRAIN) return;
+    float gv = a;
+#pragma unroll
+    for (int t = 1; t < 8; ++t) gv += part[t][threadIdx.x];
+    if (!ADAM) {
+        g[q] = gv;
+        return;
+    }
+    const float b1 = 0.9f, b2 = 0.999f;
+    const float u = b1 * m1[q] + (1.0f - b1) * gv;
+    const float v = b2 * m2[q] + (1.0f - b2) * gv * gv;
+    m1[q] = u;
+    m2[q] = v;
+    w[q] -= lr * (u / (1.0f - b1t)) / (sqrtf(v / (1.0f - b2t)) + 1e-8f);
 }
 
-__global__ void k_mlp_adam(float* __restrict__ w, const float* __restrict__ g,
-                           float* __restrict__ m1, float* __restrict__ m2, int n, float lr,
-                           float b1t, float b2t) {
-    const int q = blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= n) return;
-    const float b1 = 0.9f, b2 = 0.999f;
-    const float gv = g[q];
-    const float a = b1 * m1[q] + (1.0f - b1) * gv;
-    const float b = b2 * m2[q] + (1.0f - b2) * gv * gv;
-    m1[q] = a;
-    m2[q] = b;
-    w[q] -= lr * (a / (1.0f - b1t)) / (sqrtf(b / (1.0f - b2t)) + 1e-8f);
+// FP32 master weights to the padded BF16 inference layout (one block)
+__global__ void __launch_bounds__(1024) k_mlp_pack(const float* __restrict__ w, MlpPacked* __restrict__ out) {
+    const int tid = (int)threadIdx.x;
+    for (int q = tid; q < MLP_HID * RS1; q += 1024) {
+        const int n = q / RS1, k = q % RS1;
+        out->W1[q] = __float2bfloat16_rn(k < MLP_IN ? w[OW1 + n * MLP_IN + k] : 0.0f);
+    }
+    for (int q = tid; q < MLP_HID * RS2; q += 1024) {
+        const int n = q / RS2, k = q % RS2;
+        out->W2[q] = __float2bfloat16_rn(k < MLP_HID ? w[OW2 + n * MLP_HID + k] : 0.0f);
+        out->W3[q] = __float2bfloat16_rn(k < MLP_HID ? w[OW3 + n * MLP_HID + k] : 0.0f);
+        if (n < 8) out->W4[q] = __float2bfloat16_rn(n < MLP_OUT && k < MLP_HID ? w[OW4 + n * MLP_HID + k] : 0.0f);
+    }
+    if (tid < MLP_HID) {
+        out->b1[tid] = w[OB1 + tid];
+        out->b2[tid] = w[OB2 + tid];
+        out->b3[tid] = w[OB3 + tid];
+    }
+    if (tid < 8) out->b4[tid] = tid < MLP_OUT ? w[OB4 + tid] : 0.0f;
+    if (tid < MLP_IN) {
+        out->mean[tid] = w[NTRAIN + tid];
+        out->iscale[tid] = 1.0f / w[NTRAIN + MLP_IN + tid];
+    }
 }
 
 }  // namespace
@@ -442,61 +641,37 @@ cudaError_t launch_mlp_infer(const MlpArgs& A, const MlpPacked* pk, const float*
     return cudaGetLastError();
 }
 
-int mlp_train_block() { return TRAIN_BLOCK; }
+// two blocks per SM hold a tile each; more tiles go round
+int mlp_train_blocks(long long m) {
+    const long long tiles = (m + TT - 1) / TT;
+    return (int)(tiles < 304 ? tiles : 304);
+}
+int mlp_ntrain() { return NTRAIN; }
 
-cudaError_t launch_mlp_fwd_bwd(const float* w, const float* X, const float* Y, long long m,
-                               float* act, float* del, double* partials, cudaStream_t st) {
-    const unsigned blocks = (unsigned)((m + TRAIN_BLOCK - 1) / TRAIN_BLOCK);
-    const size_t sm = RHI_MLP_NWEIGHTS * sizeof(float);
-    cudaFuncSetAttribute(k_mlp_fwd_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_mlp_fwd_bwd<<<blocks, TRAIN_BLOCK, sm, st>>>(w, X, Y, m, 1.0f / (float)(m * MLP_OUT), act,
-                                                   del, partials);
+cudaError_t launch_mlp_train(const float* w, const float* X, const float* Y, long long m, float* gpart,
+                             double* partials, cudaStream_t st) {
+    const size_t sm = sizeof(TrainSmem);
+    cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    k_mlp_train<<<mlp_train_blocks(m), TRAIN_BLOCK, sm, st>>>(w, X, Y, m, 1.0f / (float)(m * MLP_OUT),
+                                                            gpart, partials);
     return cudaGetLastError();
 }
 
-cudaError_t launch_mlp_wgrad(const float* act, const float* del, long long m, float* grad,
-                             cudaStream_t st) {
-    k_mlp_wgrad<<<3 * MLP_HID + MLP_OUT, MLP_HID, 0, st>>>(act, del, m, grad);
+cudaError_t launch_mlp_grad(const float* gpart, int nb, float* grad, cudaStream_t st) {
+    k_mlp_apply<false><<<(NTRAIN + 31) / 32, 256, 0, st>>>(gpart, nb, nullptr, grad, nullptr, nullptr, 0.0f,
+                                                          0.0f, 0.0f);
     return cudaGetLastError();
 }
 
-cudaError_t launch_mlp_adam(float* w, const float* g, float* m1, float* m2, int n, float lr,
+cudaError_t launch_mlp_adam(const float* gpart, int nb, float* w, float* m1, float* m2, float lr,
                             float b1t, float b2t, cudaStream_t st) {
-    k_mlp_adam<<<(n + 255) / 256, 256, 0, st>>>(w, g, m1, m2, n, lr, b1t, b2t);
+    k_mlp_apply<true><<<(NTRAIN + 31) / 32, 256, 0, st>>>(gpart, nb, w, nullptr, m1, m2, lr, b1t, b2t);
     return cudaGetLastError();
 }
 
-// pack FP32 master weights into the padded BF16 inference layout
-void mlp_pack(const float* w, MlpPacked* out) {
-    std::memset(out, 0, sizeof(MlpPacked));
-    const float* W1 = w;
-    const float* b1 = W1 + MLP_HID * MLP_IN;
-    const float* W2 = b1 + MLP_HID;
-    const float* b2 = W2 + MLP_HID * MLP_HID;
-    const float* W3 = b2 + MLP_HID;
-    const float* b3 = W3 + MLP_HID * MLP_HID;
-    const float* W4 = b3 + MLP_HID;
-    const float* b4 = W4 + MLP_OUT * MLP_HID;
-    const float* mean = b4 + MLP_OUT;
-    const float* scale = mean + MLP_IN;
-    for (int n = 0; n < MLP_HID; ++n) {
-        for (int k = 0; k < MLP_IN; ++k) out->W1[n * RS1 + k] = __float2bfloat16(W1[n * MLP_IN + k]);
-        for (int k = 0; k < MLP_HID; ++k) {
-            out->W2[n * RS2 + k] = __float2bfloat16(W2[n * MLP_HID + k]);
-            out->W3[n * RS2 + k] = __float2bfloat16(W3[n * MLP_HID + k]);
-        }
-        out->b1[n] = b1[n];
-        out->b2[n] = b2[n];
-        out->b3[n] = b3[n];
-    }
-    for (int n = 0; n < MLP_OUT; ++n) {
-        for (int k = 0; k < MLP_HID; ++k) out->W4[n * RS2 + k] = __float2bfloat16(W4[n * MLP_HID + k]);
-        out->b4[n] = b4[n];
-    }
-    for (int k = 0; k < MLP_IN; ++k) {
-        out->mean[k] = mean[k];
-        out->iscale[k] = 1.0f / scale[k];
-    }
+cudaError_t launch_mlp_pack(const float* w, MlpPacked* out, cudaStream_t st) {
+    k_mlp_pack<<<1, 1024, 0, st>>>(w, out);
+    return cudaGetLastError();
 }
 
 }  // namespace rhi

@@ -12,8 +12,6 @@ namespace rhi {
 constexpr int MLP_IN = RHI_MLP_IN, MLP_HID = RHI_MLP_HID, MLP_OUT = RHI_MLP_OUT;
 constexpr int RS1 = 24;                       // padded row strides (bf16) of the packed weights
 constexpr int RS2 = 72;
-constexpr int ACT_STRIDE = MLP_IN + 3 * MLP_HID;     // per-sample activations h0 | h1 | h2 | h3
-constexpr int DEL_STRIDE = 3 * MLP_HID + MLP_OUT;    // per-sample deltas d1 | d2 | d3 | g4
 
 // inference weights: BF16 rows padded for conflict-free fragment loads, FP32 biases and
 // the input normalisation (mean, 1 / scale)
@@ -46,18 +44,20 @@ struct MlpArgs {
     double* U0;                               // guess (e_c | n | E), MODE 1
 };
 
-void mlp_pack(const float* w, MlpPacked* out);
+cudaError_t launch_mlp_pack(const float* w, MlpPacked* out, cudaStream_t st);
 cudaError_t launch_mlp_features(const MlpArgs& A, float* X, cudaStream_t st);
 cudaError_t launch_mlp_targets(const MlpArgs& A, const double* E0, const double* e0,
                                const double* n0, float* Y, cudaStream_t st);
 cudaError_t launch_mlp_infer(const MlpArgs& A, const MlpPacked* pk, const float* X, float* Y,
                              long long n_rows, int guess, cudaStream_t st);
-int mlp_train_block();
-cudaError_t launch_mlp_fwd_bwd(const float* w, const float* X, const float* Y, long long m,
-                               float* act, float* del, double* partials, cudaStream_t st);
-cudaError_t launch_mlp_wgrad(const float* act, const float* del, long long m, float* grad,
-                             cudaStream_t st);
-cudaError_t launch_mlp_adam(float* w, const float* g, float* m1, float* m2, int n, float lr,
+// Forward and backward of m samples: the gradients (mlp_ntrain() floats) of mlp_train_blocks(m)
+// blocks into gpart, their squared errors into partials; then their sum (grad) or the Adam update
+int mlp_train_blocks(long long m);
+int mlp_ntrain();
+cudaError_t launch_mlp_train(const float* w, const float* X, const float* Y, long long m, float* gpart,
+                             double* partials, cudaStream_t st);
+cudaError_t launch_mlp_grad(const float* gpart, int nb, float* grad, cudaStream_t st);
+cudaError_t launch_mlp_adam(const float* gpart, int nb, float* w, float* m1, float* m2, float lr,
                             float b1t, float b2t, cudaStream_t st);
 
 }  // namespace rhi
