@@ -104,9 +104,10 @@ typedef struct {
     int mg_pre, mg_post;    /* weighted-Jacobi sweeps before / after the coarse correction   */
     int mg_coarse_sweeps;   /* weighted-Jacobi sweeps on the coarsest level                  */
     double mg_omega;        /* Jacobi weight                                                 */
-    int vcycle_graph;       /* 1: the FP32 V-cycle is captured once as a CUDA graph and
-                               replayed (on a library-owned stream ordered by events)       */
-    int krylov_graph;       /* 1: each BiCGStab solve runs as one CUDA graph launch, its loop a
+    int vcycle_graph;       /* 1: an FP32 V-cycle outside such a solve's graph is captured once
+                               as a CUDA graph and replayed (on a library-owned stream
+                               ordered by events)                                           */
+    int krylov_graph;       /* 1: each BiCGStab or CG solve runs as one CUDA graph launch, its loop a
                                while node whose iterations decide on the device whether to
                                continue (no host round trip per iteration); 0: the same
                                kernels launched from the host, one read per iteration       */

@@ -164,11 +164,13 @@ struct rhi_ctx {
         bool failed = false;
     } vg;
 
-    // the BiCGStab solve as one CUDA graph (a while node whose body is one iteration); the
-    // assembled system and the hierarchy live in fixed buffers and hold dt theta, so one capture
-    // serves every solve of the handle, whatever the step size (two with the lagged-D hierarchy)
+    // a Krylov solve as one CUDA graph (a while node whose body is one iteration).  The assembled
+    // system and the hierarchy live in fixed buffers and hold dt theta, so one capture serves every
+    // BiCGStab solve of the handle, whatever the step size; CG works on the face arrays and Schur set
+    // of the iterate, of which there are a few (key: W, diagonal, right-hand side)
     struct KGraph {
-        bool nonsym = false;
+        bool cg = false, nonsym = false;
+        const void* key[3] = {nullptr, nullptr, nullptr};
         cudaGraphExec_t exec = nullptr;
         int k_init = 0, k_body = 0;
     };
@@ -600,76 +602,6 @@ Finish fin(const rhi_ctx* h, int op, int slot = 0, unsigned long long cond = 0) 
     return F;
 }
 
-// z = M^-1 r, and the scalar update of r.z
-int precond_apply(rhi_ctx* h, const double* r, double** zout, const Finish& F) {
-    LinLaunch L(h->st, &h->prof);
-    const long long N = h->N;
-    if (h->prm.precond == RHI_PRECOND_JACOBI) {
-        CK(L.jacobi_dot(N, r, h->pc0.diag, h->z, F));
-        *zout = h->z;
-    } else if (h->prm.precond == RHI_PRECOND_MG_FP64) {
-        auto& lv = h->mg64;
-        lv[0].b = const_cast<double*>(r);
-        lv[0].x = h->z;
-        int rc = vcycle<double>(h, lv, 0, h->pc0);
-        if (rc) return rc;
-        // the result may sit in either level-0 buffer
-        double* R = lv[0].x;
-        if (R != h->z) { lv[0].xt = h->z; h->z = R; }
-        *zout = h->z;
-        lv[0].x = nullptr;
-        CK(L.dot(N, r, h->z, F));
-    } else {
-        auto& lv = h->mg32;
-        Op<float> A0 = level_op(h, lv[0]);
-        if (tail_at(h, lv, 0)) {                         // the whole cycle and its conversions
-            CK(L.mg_tail<float>(tail_from<float>(h, lv, 0, A0, nullptr, r, nullptr, h->z)));
-            CK(L.dot(N, r, h->z, F));
-            *zout = h->z;
-            h->stats.vcycles += 1;
-            return RHI_OK;
-        }
-        CK(L.to_f32(N, r, lv[0].b));
-        int rc = vcycle_graph_usable(h) ? vcycle_graph(h, A0) : vcycle<float>(h, lv, 0, A0);
-        if (rc) return rc;
-        CK(L.from_f32_dot(N, lv[0].x, r, h->z, F));
-        *zout = h->z;
-    }
-    h->stats.vcycles += 1;
-    return RHI_OK;
-}
-
-// CG on S sE = rhs to ||r||_RMS <= tol; solution in h->x
-int pcg(rhi_ctx* h, const double* rhs, double tol, int* its_out) {
-    LinLaunch L(h->st, &h->prof);
-    const long long N = h->N;
-    const double norm = 1.0 / ((double)N * h->nv);
-    CK(cudaMemsetAsync(h->scal + S_BREAK, 0, sizeof(double), h->st));     // clear an old breakdown
-    CK(L.cg_init(N, rhs, h->r, h->x, fin(h, RED_SUM, S_RR)));
-    double rr;
-    int rc = read_scalar(h, S_RR, &rr);
-    if (rc) return rc;
-    int its = 0;
-    if (std::sqrt(rr * norm) > tol) {
-        double* z = nullptr;
-        if ((rc = precond_apply(h, h->r, &z, fin(h, RED_SUM, S_RZ)))) return rc;
-        CK(L.cg_p(N, h->scal, z, h->p, 1));
-        for (its = 1; its <= h->prm.max_pcg; ++its) {
-            CK(L.matvec_dot(h->op0, h->p, h->q, fin(h, RED_ALPHA)));
-            CK(L.cg_xr(N, h->scal, h->x, h->r, h->p, h->q, fin(h, RED_SUM, S_RR)));
-            if ((rc = read_scalar(h, S_RR, &rr))) return rc;
-            if (h->h_scal[S_BREAK] != 0.0 || !std::isfinite(rr))
-                return fail(h, RHI_ERR_NONPHYSICAL, "CG breakdown: p.Sp <= 0 or non-finite residual");
-            if (std::sqrt(rr * norm) <= tol) break;
-            if ((rc = precond_apply(h, h->r, &z, fin(h, RED_BETA)))) return rc;
-            CK(L.cg_p(N, h->scal, z, h->p, 0));
-        }
-        if (its > h->prm.max_pcg) its = h->prm.max_pcg;
-    }
-    *its_out = its;
-    return RHI_OK;
-}
-
 // the FP32 copy of a vector the FP32 cycle takes as its right-hand side (null: none; a cycle that is
 // one launch reads the FP64 vector)
 float* cycle_rhs(const rhi_ctx* h) {
@@ -677,12 +609,15 @@ float* cycle_rhs(const rhi_ctx* h) {
     return h->mg32[0].b;
 }
 
-// M^-1 r into dest with the launcher's stream, hook and skip flag (an iteration of BiCGStab; the
-// FP32 copy of r is in place where cycle_rhs names one); the V-cycle's kernels are launched one by one (also while a graph is being captured)
-int precond_into(rhi_ctx* h, LinLaunch& L, const double* r, double* dest) {
+// M^-1 r into dest with the launcher's stream, hook and skip flag (the FP32 copy of r is in place
+// where cycle_rhs names one).  The V-cycle's kernels are launched one by one, also while a graph is
+// being captured; outside of one (vg), an FP32 cycle may run as a graph of its own.
+int precond_into(rhi_ctx* h, LinLaunch& L, const double* r, double* dest, bool vg = false) {
     const long long N = h->N;
     if (h->prm.precond == RHI_PRECOND_JACOBI) {
-        CK(L.jacobi_dot(N, r, h->pc0.diag, dest, fin(h, RED_NONE)));
+        Finish none = fin(h, RED_NONE);
+        none.count = nullptr;
+        CK(L.jacobi_dot(N, r, h->pc0.diag, dest, none));
     } else if (h->prm.precond == RHI_PRECOND_MG_FP64) {
         auto& lv = h->mg64;
         double* xt0 = lv[0].xt;
@@ -697,6 +632,12 @@ int precond_into(rhi_ctx* h, LinLaunch& L, const double* r, double* dest) {
         auto& lv = h->mg32;
         if (!cycle_rhs(h)) {
             CK(L.mg_tail<float>(tail_from<float>(h, lv, 0, level_op(h, lv[0]), nullptr, r, nullptr, dest)));
+            return RHI_OK;
+        }
+        if (vg && vcycle_graph_usable(h)) {
+            int rc = vcycle_graph(h, level_op(h, lv[0]));
+            if (rc) return rc;
+            CK(L.from_f32(N, lv[0].x, dest));
             return RHI_OK;
         }
         float *x0 = lv[0].x, *xt0 = lv[0].xt;
@@ -738,14 +679,37 @@ int bicg_iteration(rhi_ctx* h, LinLaunch& L, unsigned long long cond) {
     return RHI_OK;
 }
 
+// CG on the lagged-D matrix h->op0 with the control on the device, likewise: r = b, x = 0; then per
+// iteration z = M^-1 r and beta, p, q = S p and alpha, the x / r update and the continue flag
+int cg_start(rhi_ctx* h, LinLaunch& L, const double* rhs, unsigned long long cond) {
+    L.skip = nullptr;
+    CK(L.cg_init(h->N, rhs, h->r, h->x, cycle_rhs(h), fin(h, RED_CG_START, 0, cond)));
+    return RHI_OK;
+}
+int cg_iteration(rhi_ctx* h, LinLaunch& L, unsigned long long cond, bool vg) {
+    const long long N = h->N;
+    int rc;
+    L.skip = nullptr;
+    if (h->prm.precond == RHI_PRECOND_JACOBI) {
+        CK(L.jacobi_dot(N, h->r, h->pc0.diag, h->z, fin(h, RED_CG_BETA)));
+    } else {
+        if ((rc = precond_into(h, L, h->r, h->z, vg))) return rc;
+        CK(L.dot(N, h->r, h->z, fin(h, RED_CG_BETA)));
+    }
+    CK(L.cg_p(N, h->scal, h->z, h->p));
+    CK(L.matvec_dot(h->op0, h->p, h->q, fin(h, RED_CG_ALPHA)));
+    CK(L.cg_xr(N, h->scal, h->x, h->r, h->p, h->q, cycle_rhs(h), fin(h, RED_CG_NEXT, 0, cond)));
+    return RHI_OK;
+}
+
 // the solve's graph is used unless per-launch timing of one of its kernels is requested
 bool krylov_graph_usable(const rhi_ctx* h) {
     if (!h->prm.krylov_graph || h->kg_failed) return false;
     if (!h->prof.on) return true;
     if (h->prof.only.empty()) return false;
     for (const auto& nm : h->prof.only)
-        if (nm.compare(0, 3, "mg_") == 0 || nm.compare(0, 5, "bicg_") == 0 || nm == "reduce" ||
-            nm == "copy" || nm == "precond_jacobi")
+        if (nm.compare(0, 3, "mg_") == 0 || nm.compare(0, 5, "bicg_") == 0 || nm.compare(0, 3, "cg_") == 0 ||
+            nm == "dot" || nm == "copy" || nm == "precond_jacobi")
             return false;
     return true;
 }
@@ -754,6 +718,8 @@ bool krylov_graph_usable(const rhi_ctx* h) {
 // launch) whose body is one iteration; the last kernel of the start and of each iteration
 // writes the node's condition.  The body graph is filled by a second capture.
 int krylov_graph_build(rhi_ctx* h, const double* rhs, rhi_ctx::KGraph& g) {
+    const auto start = [&](LinLaunch& L, unsigned long long c) { return g.cg ? cg_start(h, L, rhs, c) : bicg_start(h, L, rhs, c); };
+    const auto iteration = [&](LinLaunch& L, unsigned long long c) { return g.cg ? cg_iteration(h, L, c, false) : bicg_iteration(h, L, c); };
     if (!h->kst) CK(cudaStreamCreateWithFlags(&h->kst, cudaStreamNonBlocking));
     Counter cnt;
     LinLaunch L(h->kst, &cnt);
@@ -779,7 +745,7 @@ int krylov_graph_build(rhi_ctx* h, const double* rhs, rhi_ctx::KGraph& g) {
     e = cudaStreamGetCaptureInfo(h->kst, &stt, nullptr, &graph, &deps, nullptr, &nd);
     if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&hc, graph, 1, cudaGraphCondAssignDefault);
     if (e != cudaSuccess) return abort_capture("conditional handle", e);
-    int rc = bicg_start(h, L, rhs, (unsigned long long)hc);
+    int rc = start(L, (unsigned long long)hc);
     if (rc) { abort_capture("start kernels", cudaGetLastError()); return rc; }
     e = cudaStreamGetCaptureInfo(h->kst, &stt, nullptr, &graph, &deps, nullptr, &nd);
     cudaGraphNodeParams cp = {};
@@ -798,7 +764,7 @@ int krylov_graph_build(rhi_ctx* h, const double* rhs, rhi_ctx::KGraph& g) {
     body = cp.conditional.phGraph_out[0];
     e = cudaStreamBeginCaptureToGraph(h->kst, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return abort_capture("begin body capture", e);
-    rc = bicg_iteration(h, L, (unsigned long long)hc);
+    rc = iteration(L, (unsigned long long)hc);
     if (rc) { abort_capture("body kernels", cudaGetLastError()); return rc; }
     e = cudaStreamEndCapture(h->kst, &body);
     if (e != cudaSuccess) return abort_capture("end body capture", e);
@@ -811,14 +777,20 @@ int krylov_graph_build(rhi_ctx* h, const double* rhs, rhi_ctx::KGraph& g) {
     return RHI_OK;
 }
 
-// the outcome of the last BiCGStab solve from the host copy of the scalars (h->h_scal, filled
-// by the read that followed the solve): iterations, multigrid cycles, breakdown
-int bicg_outcome(rhi_ctx* h, int* its_out) {
+// the outcome of the last solve from the host copy of the scalars (h->h_scal, filled by the read that
+// followed it): iterations, multigrid cycles, breakdown
+int krylov_outcome(rhi_ctx* h, bool cg, int* its_out) {
     const int its = (int)h->h_scal[S_ITS];
     *its_out = its;
-    h->stats.krylov_stalls += h->h_scal[S_STALL] != 0.0 ? 1 : 0;
     h->prof.launches += its * h->kg_body_kernels;
     h->kg_body_kernels = 0;
+    if (cg) {
+        if (h->prm.precond != RHI_PRECOND_JACOBI) h->stats.vcycles += its;
+        if (h->h_scal[S_BREAK] != 0.0)
+            return fail(h, RHI_ERR_NONPHYSICAL, "CG breakdown: p.Sp <= 0 or non-finite residual");
+        return RHI_OK;
+    }
+    h->stats.krylov_stalls += h->h_scal[S_STALL] != 0.0 ? 1 : 0;
     if (h->prm.precond != RHI_PRECOND_JACOBI)
         h->stats.vcycles += 2 * its - (h->h_scal[S_HALF] != 0.0 ? 1 : 0);
     if (h->h_scal[S_BREAK] != 0.0 || !std::isfinite(h->h_scal[S_RR]))
@@ -826,14 +798,15 @@ int bicg_outcome(rhi_ctx* h, int* its_out) {
     return RHI_OK;
 }
 
-// Right-preconditioned BiCGStab on the assembled Newton matrix and right-hand side (dD/dE kept), to
-// ||r||_RMS <= tol (counted over the N (N_s + 2) unknowns of eq. rmsnorm); solution in h->x.
+// A Krylov solve to ||r||_RMS <= tol (counted over the N (N_s + 2) unknowns of eq. rmsnorm); solution
+// in h->x.  cg: conjugate gradients on the lagged-D matrix h->op0; else right-preconditioned BiCGStab
+// on the assembled Newton matrix and right-hand side (dD/dE kept).
 // The iteration's control runs on the device: as one CUDA graph launch per solve, or, while
 // per-launch timing is on, as direct launches with one host read per iteration.  With
 // `deferred` and the graph, the call only enqueues the solve (*its_out = -1): the next host
-// read of the scalars brings its outcome back for bicg_outcome.  Otherwise the outcome is read
+// read of the scalars brings its outcome back for krylov_outcome.  Otherwise the outcome is read
 // here; RHI_ERR_NONPHYSICAL on a breakdown.
-int bicgstab(rhi_ctx* h, double tol, int* its_out, bool deferred = false) {
+int krylov(rhi_ctx* h, bool cg, const double* rhs, double tol, int* its_out, bool deferred) {
     const long long N = h->N;
     h->h_ctl[0] = tol * tol * (double)N * h->nv;                   // S_THR: bound on r.r
     h->h_ctl[1] = (double)h->prm.max_pcg;                           // S_MAXIT
@@ -846,13 +819,15 @@ int bicgstab(rhi_ctx* h, double tol, int* its_out, bool deferred = false) {
     CK(cudaMemcpyAsync(h->scal + S_THR, h->h_ctl, 3 * sizeof(double), cudaMemcpyHostToDevice, h->st));
     int rc = RHI_OK;
     if (krylov_graph_usable(h)) {
+        rhi_ctx::KGraph ng;
+        ng.cg = cg;
+        ng.nonsym = h->pc_nonsym;
+        if (cg) { ng.key[0] = h->op0.W[0]; ng.key[1] = h->op0.diag; ng.key[2] = rhs; }
         rhi_ctx::KGraph* g = nullptr;
         for (auto& c : h->kg)
-            if (c.nonsym == h->pc_nonsym) g = &c;
+            if (c.cg == ng.cg && c.nonsym == ng.nonsym && std::equal(c.key, c.key + 3, ng.key)) g = &c;
         if (!g) {
-            rhi_ctx::KGraph ng;
-            ng.nonsym = h->pc_nonsym;
-            if ((rc = krylov_graph_build(h, h->sysrhs, ng))) return rc;
+            if ((rc = krylov_graph_build(h, rhs, ng))) return rc;
             h->kg.push_back(ng);
             g = &h->kg.back();
         }
@@ -873,15 +848,15 @@ int bicgstab(rhi_ctx* h, double tol, int* its_out, bool deferred = false) {
         h->kg_body_kernels = 0;                         // direct launches count themselves
         LinLaunch L(h->st, &h->prof);
         L.fine_N = N;
-        if ((rc = bicg_start(h, L, h->sysrhs, 0))) return rc;
+        if ((rc = cg ? cg_start(h, L, rhs, 0) : bicg_start(h, L, rhs, 0))) return rc;
         double cont = 0.0;
         if ((rc = read_scalar(h, S_CONT, &cont))) return rc;
         while (cont != 0.0) {
-            if ((rc = bicg_iteration(h, L, 0))) return rc;
+            if ((rc = cg ? cg_iteration(h, L, 0, true) : bicg_iteration(h, L, 0))) return rc;
             if ((rc = read_scalar(h, S_CONT, &cont))) return rc;
         }
     }
-    return bicg_outcome(h, its_out);
+    return krylov_outcome(h, cg, its_out);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1501,10 +1476,12 @@ int rhi_precond_apply(rhi_handle h, const double* r, double* z, int on_device) {
     if (!h->have_linear) return fail(h, RHI_ERR_STATE, "rhi_precond_apply: call rhi_linearize first");
     const long long N = h->N;
     CK(cudaMemcpyAsync(h->q, r, N * sizeof(double), on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->st));
-    double* zr = nullptr;
-    int rc = precond_apply(h, h->q, &zr, fin(h, RED_NONE));
+    LinLaunch L(h->st, &h->prof);
+    L.fine_N = N;
+    if (float* b32 = cycle_rhs(h)) CK(L.to_f32(N, h->q, b32));
+    int rc = precond_into(h, L, h->q, h->z, true);
     if (rc) return rc;
-    CK(cudaMemcpyAsync(z, zr, N * sizeof(double), on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->st));
+    CK(cudaMemcpyAsync(z, h->z, N * sizeof(double), on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, h->st));
     CK(bulk_wait_flag_read(h->h_kerr, h->st));
     CK(cudaStreamSynchronize(h->st));
     h->prof.resolve();
@@ -1639,18 +1616,13 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
             if (cur < 0 && (r2 = kappa(h, P, h->n_s, h->kap[0]))) return r2;
             if ((r2 = lagged_system(h, P, Ek, h->kap[fb], set))) return r2;
             if (h->pc_nonsym && (r2 = precond_setup(h, h->op0, false))) return r2;
-            return pcg(h, h->sysrhs, lin_tol * res, &its);
+            return krylov(h, true, h->sysrhs, lin_tol * res, &its, false);
         };
-        bool deferred = false;
-        if (h->prm.limiter_jacobian) {
-            rc = bicgstab(h, lin_tol * res, &its, true);
-            deferred = rc == RHI_OK && its < 0;
-            if (rc == RHI_ERR_NONPHYSICAL) rc = krylov_fallback();
-            if (rc) { S.status = rc; return rc; }
-        } else if ((rc = pcg(h, h->rhs[set], lin_tol * res, &its))) {
-            S.status = rc;
-            return rc;
-        }
+        const bool cg = h->prm.limiter_jacobian == 0;
+        rc = krylov(h, cg, cg ? h->rhs[set] : h->sysrhs, lin_tol * res, &its, true);
+        const bool deferred = rc == RHI_OK && its < 0;
+        if (rc == RHI_ERR_NONPHYSICAL && !cg) rc = krylov_fallback();
+        if (rc) { S.status = rc; return rc; }
         const int t = (cur == 0) ? 1 : 0;
         const double* ec0 = cur < 0 ? nullptr : U_ec(h, cur);
         const double* n0 = cur < 0 ? h->n_s : U_n(h, cur);
@@ -1694,8 +1666,8 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
         if ((rc = trial(1.0, &rt, resid_only))) return rc;
         if (deferred) {
             // the full step's residual read also brought the Krylov solve's outcome back
-            rc = bicg_outcome(h, &its);
-            if (rc == RHI_ERR_NONPHYSICAL) {
+            rc = krylov_outcome(h, cg, &its);
+            if (rc == RHI_ERR_NONPHYSICAL && !cg) {
                 if ((rc = krylov_fallback())) { S.status = rc; return rc; }
                 if ((rc = trial(1.0, &rt))) return rc;        // in full
                 resid_only = false;

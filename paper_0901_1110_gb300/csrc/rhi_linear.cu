@@ -100,8 +100,10 @@ __device__ __forceinline__ T jacobi_update(T xc, T b, T wi, T off, T omega) {
 // partials in a fixed order and applies the update, so that a Krylov iteration needs no separate
 // reduction launches (about 3.6 us each inside a graph; the last block adds about 2 us).
 //   RED_SUM:        scal[slot] = sum
-//   RED_ALPHA:      S_PQ = sum; S_ALPHA = S_RZ / sum (breakdown flag if <= 0)
-//   RED_BETA:       S_BETA = sum / S_RZ; S_RZ = sum
+//   RED_CG_START:   r.r of r = b: S_RR, counters cleared; done when r.r <= S_THR
+//   RED_CG_BETA:    r.z: S_BETA = sum / S_RZ; S_RZ = sum
+//   RED_CG_ALPHA:   p.Sp: S_PQ = sum; S_ALPHA = S_RZ / sum (breakdown flag if <= 0)
+//   RED_CG_NEXT:    r.r: S_RR, S_ITS += 1; ends when converged, on a breakdown, or at S_MAXIT
 //   RED_BICG_ALPHA: sum = rh.v: S_ALPHA = S_RHO / sum
 //   RED_BICG_OMEGA: sums t.s and t.t: S_OMEGA
 //   RED_BICG_START: r.r of r = b: S_RR = S_RHO = r.r, counters cleared; done when
@@ -116,26 +118,35 @@ __device__ __forceinline__ T jacobi_update(T xc, T b, T wi, T off, T omega) {
 //                   preconditioner slowly erodes the bi-orthogonality BiCGStab relies on); a
 //                   stagnation past the last restart ends the loop, and the Newton step is
 //                   then that of an inexact Newton iteration.
-// RED_BICG_START and RED_BICG_NEXT write the continue flag to S_CONT and, inside a CUDA graph, to
-// the while node's conditional handle: these kernels always run to their end.
-template <int OP>
-__device__ __forceinline__ void scalar_update(double* scal, int dyn, int slot, unsigned long long cond,
+// The START and NEXT updates write the continue flag to S_CONT and, inside a CUDA graph, to the
+// while node's conditional handle: these kernels always run to their end.
+template <int op>
+__device__ __forceinline__ void scalar_update(double* scal, int slot, unsigned long long cond,
                                               double s, double s2) {
-    // (the kernels of the preconditioned residual's dot serve several updates)
-    const int op = OP == RED_NONE ? dyn : OP;
     int cont = 0;
     if (op == RED_SUM) {
         scal[slot] = s;
         return;
-    } else if (op == RED_ALPHA) {
+    } else if (op == RED_CG_START) {
+        scal[S_RR] = s;
+        scal[S_ITS] = 0.0;
+        scal[S_BREAK] = 0.0;
+        cont = s > scal[S_THR] && scal[S_MAXIT] >= 1.0;
+    } else if (op == RED_CG_BETA) {
+        scal[S_BETA] = s / scal[S_RZ];          // (not read in the first iteration)
+        scal[S_RZ] = s;
+        return;
+    } else if (op == RED_CG_ALPHA) {
         scal[S_PQ] = s;
         if (!(s > 0.0)) scal[S_BREAK] = 1.0;
         scal[S_ALPHA] = (s > 0.0) ? scal[S_RZ] / s : 0.0;
         return;
-    } else if (op == RED_BETA) {
-        scal[S_BETA] = s / scal[S_RZ];
-        scal[S_RZ] = s;
-        return;
+    } else if (op == RED_CG_NEXT) {
+        const double its = scal[S_ITS] + 1.0;
+        scal[S_ITS] = its;
+        scal[S_RR] = s;
+        if (!isfinite(s)) scal[S_BREAK] = 1.0;
+        cont = scal[S_BREAK] == 0.0 && s > scal[S_THR] && its < scal[S_MAXIT] && its < 1e6;
     } else if (op == RED_BICG_ALPHA) {
         scal[S_RST] = 0.0;                      // a restart's p and rh are in place
         scal[S_RV] = s;
@@ -214,17 +225,17 @@ __device__ __forceinline__ void scalar_update(double* scal, int dyn, int slot, u
     if (cond) cudaGraphSetConditional((cudaGraphConditionalHandle)cond, cont ? 1u : 0u);
 }
 
-// v1 (and v2): this thread's share of the sums; called by every thread of every block.  OP: the one
-// update the kernel ends with, so that its code holds no other (RED_NONE: F.op, of SUM, BETA, NONE)
+// v1 (and v2): this thread's share of the sums; called by every thread of every block.  OP: the
+// update the kernel ends with, so that its code holds no other
 template <bool TWO, int OP>
 __device__ __forceinline__ void finish(const Finish& F, double v1, double v2) {
     __shared__ double sc[S_NSCAL];
     double s1, s2;
-    if (!grid_sum<LIN_BLOCK, TWO>(v1, v2, F.partials, F.op == RED_NONE ? nullptr : F.count, s1, s2)) return;
+    if (!grid_sum<LIN_BLOCK, TWO>(v1, v2, F.partials, F.count, s1, s2)) return;
     // the scalars by way of shared memory: one trip to memory each way
     if (threadIdx.x < S_NSCAL) sc[threadIdx.x] = __ldcg(F.scal + threadIdx.x);
     __syncthreads();
-    if (threadIdx.x == 0) scalar_update<OP>(sc, F.op == RED_BETA ? RED_BETA : RED_SUM, F.slot, F.cond, s1, s2);
+    if (threadIdx.x == 0) scalar_update<OP>(sc, F.slot, F.cond, s1, s2);
     __syncthreads();
     if (threadIdx.x < S_NSCAL) F.scal[threadIdx.x] = sc[threadIdx.x];
 }
@@ -269,14 +280,15 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_matvec_dot(const Op<double> A,
         q[c] = v;
         acc += pc * v;
     }
-    finish<false, RED_ALPHA>(F, acc, 0.0);
+    finish<false, RED_CG_ALPHA>(F, acc, 0.0);
 }
 
 // x += alpha p; r -= alpha q; r.r      (alpha = scal[S_ALPHA])
 __global__ void __launch_bounds__(LIN_BLOCK) k_cg_xr(long long N, const double* __restrict__ scal,
                                                      double* __restrict__ x, double* __restrict__ r,
                                                      const double* __restrict__ p,
-                                                     const double* __restrict__ q, const Finish F) {
+                                                     const double* __restrict__ q,
+                                                     float* __restrict__ r32, const Finish F) {
     const double alpha = scal[S_ALPHA];
     double acc = 0.0;
     for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
@@ -284,15 +296,17 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_cg_xr(long long N, const double* 
         x[c] += alpha * p[c];
         const double rv = r[c] - alpha * q[c];
         r[c] = rv;
+        if (r32) r32[c] = (float)rv;
         acc += rv * rv;
     }
-    finish<false, RED_SUM>(F, acc, 0.0);
+    finish<false, RED_CG_NEXT>(F, acc, 0.0);
 }
 
-// p = z + beta p    (beta = scal[S_BETA]); first: p = z
+// p = z + beta p    (beta = scal[S_BETA]); at the loop's first iteration p = z
 __global__ void __launch_bounds__(LIN_BLOCK) k_cg_p(long long N, const double* __restrict__ scal,
                                                     const double* __restrict__ z,
-                                                    double* __restrict__ p, int first) {
+                                                    double* __restrict__ p) {
+    const bool first = scal[S_ITS] == 0.0;
     const double beta = first ? 0.0 : scal[S_BETA];
     for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
          c += (long long)gridDim.x * LIN_BLOCK)
@@ -313,7 +327,7 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_jacobi_dot(long long N, const dou
         z[c] = zv;
         acc += rv * zv;
     }
-    finish<false, RED_NONE>(F, acc, 0.0);
+    finish<false, RED_CG_BETA>(F, acc, 0.0);
 }
 
 // a.b
@@ -323,22 +337,24 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_dot(long long N, const double* __
     for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
          c += (long long)gridDim.x * LIN_BLOCK)
         acc += a[c] * b[c];
-    finish<false, RED_NONE>(F, acc, 0.0);
+    finish<false, RED_CG_BETA>(F, acc, 0.0);
 }
 
 // r = b, x = 0; r.r
 __global__ void __launch_bounds__(LIN_BLOCK) k_cg_init(long long N, const double* __restrict__ b,
                                                        double* __restrict__ r,
-                                                       double* __restrict__ x, const Finish F) {
+                                                       double* __restrict__ x,
+                                                       float* __restrict__ r32, const Finish F) {
     double acc = 0.0;
     for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
          c += (long long)gridDim.x * LIN_BLOCK) {
         const double v = b[c];
         r[c] = v;
         x[c] = 0.0;
+        if (r32) r32[c] = (float)v;
         acc += v * v;
     }
-    finish<false, RED_SUM>(F, acc, 0.0);
+    finish<false, RED_CG_START>(F, acc, 0.0);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1075,20 +1091,6 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_from_f32(long long N, const float
         z[c] = (double)x[c];
 }
 
-// z = x (widened); r.z
-__global__ void __launch_bounds__(LIN_BLOCK) k_from_f32_dot(long long N, const float* __restrict__ x,
-                                                            const double* __restrict__ r,
-                                                            double* __restrict__ z, const Finish F) {
-    double acc = 0.0;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK) {
-        const double zv = (double)x[c];
-        z[c] = zv;
-        acc += r[c] * zv;
-    }
-    finish<false, RED_NONE>(F, acc, 0.0);
-}
-
 // ---------------------------------------------------------------------------------------------
 // host-side launchers
 
@@ -1107,14 +1109,14 @@ cudaError_t LinLaunch::matvec_dot(const Op<double>& A, const double* p, double* 
     return end();
 }
 cudaError_t LinLaunch::cg_xr(long long N, const double* scal, double* x, double* r,
-                             const double* p, const double* q, const Finish& F) {
+                             const double* p, const double* q, float* r32, const Finish& F) {
     begin("cg_update_xr");
-    k_cg_xr<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, scal, x, r, p, q, F);
+    k_cg_xr<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, scal, x, r, p, q, r32, F);
     return end();
 }
-cudaError_t LinLaunch::cg_p(long long N, const double* scal, const double* z, double* p, int first) {
+cudaError_t LinLaunch::cg_p(long long N, const double* scal, const double* z, double* p) {
     begin("cg_update_p");
-    k_cg_p<<<stream_blocks(N), LIN_BLOCK, 0, st>>>(N, scal, z, p, first);
+    k_cg_p<<<stream_blocks(N), LIN_BLOCK, 0, st>>>(N, scal, z, p);
     return end();
 }
 cudaError_t LinLaunch::jacobi_dot(long long N, const double* r, const double* diag, double* z,
@@ -1128,9 +1130,10 @@ cudaError_t LinLaunch::dot(long long N, const double* a, const double* b, const 
     k_dot<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, a, b, F);
     return end();
 }
-cudaError_t LinLaunch::cg_init(long long N, const double* b, double* r, double* x, const Finish& F) {
+cudaError_t LinLaunch::cg_init(long long N, const double* b, double* r, double* x, float* r32,
+                               const Finish& F) {
     begin("cg_init");
-    k_cg_init<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, b, r, x, F);
+    k_cg_init<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, b, r, x, r32, F);
     return end();
 }
 cudaError_t LinLaunch::reduce(const double* part, int n, double* scal, int op, int slot) {
@@ -1287,13 +1290,6 @@ cudaError_t LinLaunch::to_f32(long long N, const double* a, float* b) {
         k_to_f32<false><<<stream_blocks(N), LIN_BLOCK, 0, st>>>(N, a, b, skip);
     return end();
 }
-cudaError_t LinLaunch::from_f32_dot(long long N, const float* x, const double* r, double* z,
-                                    const Finish& F) {
-    begin("mg_from_f32_dot");
-    k_from_f32_dot<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, x, r, z, F);
-    return end();
-}
-
 template cudaError_t LinLaunch::smooth<double>(const Op<double>&, const double*, const double*,
                                                double*, double, int, double*);
 template cudaError_t LinLaunch::smooth<float>(const Op<float>&, const float*, const float*,

@@ -59,7 +59,7 @@ struct MgTail {
 };
 cudaError_t mg_tail_init(int* blocks32, int* blocks64);
 
-// device scalar slots of the Krylov iterations.  The BiCGStab loop keeps its control state
+// device scalar slots of the Krylov iterations.  The BiCGStab and CG loops keep their control state
 // on the device: S_THR (converged when r.r <= S_THR), S_MAXIT, the iteration count S_ITS, S_DONE
 // (nothing left to do in this iteration), S_HALF (converged at the middle of an iteration:
 // x += alpha M^-1 p only) and S_CONT (1 while another iteration follows).
@@ -74,7 +74,7 @@ enum { S_RZ = 0, S_PQ, S_ALPHA, S_BETA, S_RR, S_BREAK, S_TMP, S_RHO, S_OMEGA, S_
        S_STALL, S_RR0, S_NRST, S_RST, S_NSCAL = 32 };
 constexpr int STALL_ITS = 20;
 constexpr int MAX_RESTARTS = 8;
-enum { RED_NONE = 0, RED_SUM, RED_ALPHA, RED_BETA, RED_MAX, RED_BICG_ALPHA, RED_BICG_OMEGA,
+enum { RED_NONE = 0, RED_SUM, RED_MAX, RED_CG_START, RED_CG_BETA, RED_CG_ALPHA, RED_CG_NEXT, RED_BICG_ALPHA, RED_BICG_OMEGA,
        RED_BICG_START, RED_BICG_SS, RED_BICG_NEXT };
 
 // What the last block of a kernel with a dot product does with the sum(s): the scalar update `op` on
@@ -118,12 +118,15 @@ struct LinLaunch {
 
     cudaError_t matvec_dot(const Op<double>& A, const double* p, double* q, const Finish& F);
     cudaError_t cg_xr(long long N, const double* scal, double* x, double* r, const double* p,
-                      const double* q, const Finish& F);
-    cudaError_t cg_p(long long N, const double* scal, const double* z, double* p, int first);
+                      const double* q, float* r32, const Finish& F);
+    // p = z at the loop's first iteration, else z + beta p
+    cudaError_t cg_p(long long N, const double* scal, const double* z, double* p);
     cudaError_t jacobi_dot(long long N, const double* r, const double* diag, double* z,
                            const Finish& F);
     cudaError_t dot(long long N, const double* a, const double* b, const Finish& F);
-    cudaError_t cg_init(long long N, const double* b, double* r, double* x, const Finish& F);
+    // r32 (may be null), here and above: the FP32 copy of r
+    cudaError_t cg_init(long long N, const double* b, double* r, double* x, float* r32,
+                        const Finish& F);
     // sum (RED_SUM) or max (RED_MAX) of n partials into scal[slot]
     cudaError_t reduce(const double* part, int n, double* scal, int op, int slot);
     // BiCGStab (right-preconditioned) building blocks
@@ -168,8 +171,6 @@ struct LinLaunch {
     // FP32 copy of a symmetric FP64 operator
     cudaError_t cast_op(const Op<double>& A, float* d, float* const* w);
     cudaError_t to_f32(long long N, const double* a, float* b);
-    cudaError_t from_f32_dot(long long N, const float* x, const double* r, double* z,
-                             const Finish& F);
 };
 
 }  // namespace rhi
