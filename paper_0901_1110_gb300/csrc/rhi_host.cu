@@ -101,6 +101,8 @@ struct rhi_ctx {
     bool have_linear = false;
 
     std::vector<void*> allocs;
+    char* slab = nullptr;                 // the rest of the slab small buffers come from
+    size_t slab_left = 0;
 
     // state U^n
     double *E_s = nullptr, *e_s = nullptr, *n_s = nullptr, *nH = nullptr, *src = nullptr,
@@ -208,13 +210,29 @@ int fail(rhi_ctx* h, int code, const std::string& msg) {
             return fail(h, RHI_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
+// Small buffers share slabs: a handle has about a hundred of them, and on a small grid their cudaMalloc
+// calls would be most of rhi_create.
+constexpr size_t SLAB_BYTES = 4u << 20, SLAB_SHARE = 512u << 10;
+
 template <typename T>
 int dalloc(rhi_ctx* h, T** p, size_t count) {
+    const size_t bytes = (std::max<size_t>(count, 1) * sizeof(T) + 255) & ~(size_t)255;
+    if (bytes <= SLAB_SHARE && bytes <= h->slab_left) {
+        *p = (T*)h->slab;
+        h->slab += bytes;
+        h->slab_left -= bytes;
+        return RHI_OK;
+    }
     void* v = nullptr;
-    cudaError_t e = cudaMalloc(&v, std::max<size_t>(count, 1) * sizeof(T));
+    const bool share = bytes <= SLAB_SHARE;
+    cudaError_t e = cudaMalloc(&v, share ? SLAB_BYTES : bytes);
     if (e != cudaSuccess) return fail(h, RHI_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
     h->allocs.push_back(v);
     *p = (T*)v;
+    if (share) {
+        h->slab = (char*)v + bytes;
+        h->slab_left = SLAB_BYTES - bytes;
+    }
     return RHI_OK;
 }
 
@@ -1291,10 +1309,16 @@ int rhi_set_sources(rhi_handle h, int nsrc, const int* ijk, const double* rate) 
             return fail(h, RHI_ERR_ARG, "rhi_set_sources: source outside the grid");
         if (!(rate[s] >= 0.0)) return fail(h, RHI_ERR_ARG, "rhi_set_sources: negative rate");
     }
-    for (int s = 0; s < nsrc; ++s) {
-        const long long c = ijk[3 * s] + (long long)h->grid.nx * (ijk[3 * s + 1] + (long long)h->grid.ny * ijk[3 * s + 2]);
+    for (int s0 = 0; s0 < nsrc; s0 += SOURCE_BATCH) {
+        SourceBatch S;
+        S.n = std::min(SOURCE_BATCH, nsrc - s0);
+        for (int q = 0; q < S.n; ++q) {
+            const int* c = ijk + 3 * (s0 + q);
+            S.cell[q] = c[0] + (long long)h->grid.nx * (c[1] + (long long)h->grid.ny * c[2]);
+            S.value[q] = rate[s0 + q] * h->prm.photon_energy / vol;
+        }
         Scope sc(h->prof, "deposit_source");
-        CK(launch_deposit(c, rate[s] * h->prm.photon_energy / vol, h->src, h->st));
+        CK(launch_deposit(S, h->src, h->st));
     }
     CK(cudaStreamSynchronize(h->st));
     h->prof.resolve();

@@ -274,7 +274,14 @@ cudaError_t launch_temperature(const StepParams& P, int ns, const double* e, con
                                const double* nH, double* T, cudaStream_t st);
 cudaError_t launch_check_state(const StepParams& P, int ns, const double* E, const double* e,
                                const double* n, const double* nH, int* bad, cudaStream_t st);
-cudaError_t launch_deposit(long long cell, double value, double* src, cudaStream_t st);
+// emissivity of up to SOURCE_BATCH point sources added to src, in their order
+constexpr int SOURCE_BATCH = 128;
+struct SourceBatch {
+    int n;
+    long long cell[SOURCE_BATCH];
+    double value[SOURCE_BATCH];
+};
+cudaError_t launch_deposit(const SourceBatch& S, double* src, cudaStream_t st);
 // block partials (nblocks of 256 threads) of the step's error estimate against the predictor
 // Up: sum of q^pn, or max q when pn < 0
 cudaError_t launch_time_error(const StepParams& P, int ns, const double* ec, const double* n,

@@ -930,10 +930,22 @@ cudaError_t launch_check_state(const StepParams& P, int ns, const double* E, con
     return cudaGetLastError();
 }
 
-__global__ void k_deposit(long long cell, double value, double* src) { src[cell] += value; }
+// Point sources, a batch per launch (one block, a thread per source; the batch rides in the kernel's
+// parameters).  Several sources in one cell are added by the first of them, in their order.
+__global__ void __launch_bounds__(SOURCE_BATCH) k_deposit(const SourceBatch S, double* src) {
+    const int t = (int)threadIdx.x;
+    if (t >= S.n) return;
+    const long long c = S.cell[t];
+    for (int q = 0; q < t; ++q)
+        if (S.cell[q] == c) return;
+    double v = src[c];
+    for (int q = t; q < S.n; ++q)
+        if (S.cell[q] == c) v += S.value[q];
+    src[c] = v;
+}
 
-cudaError_t launch_deposit(long long cell, double value, double* src, cudaStream_t st) {
-    k_deposit<<<1, 1, 0, st>>>(cell, value, src);
+cudaError_t launch_deposit(const SourceBatch& S, double* src, cudaStream_t st) {
+    k_deposit<<<1, SOURCE_BATCH, 0, st>>>(S, src);
     return cudaGetLastError();
 }
 
