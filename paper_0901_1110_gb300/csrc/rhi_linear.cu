@@ -405,20 +405,53 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_matvec_ns(const OpNS A, const dou
     finish<TWO, TWO ? RED_BICG_OMEGA : RED_BICG_ALPHA>(F, d1, d2);
 }
 
+// The vector updates below take two elements per thread and turn (16-byte accesses: twice the bytes in
+// flight of one; the library's vectors start on 256-byte boundaries) and the odd last one alone:
+// f(i, n) works on the n elements from i on.
+template <typename F>
+__device__ __forceinline__ void for_pairs(long long N, F f) {
+    const long long pairs = N / 2;
+    for (long long q = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; q < pairs;
+         q += (long long)gridDim.x * LIN_BLOCK)
+        f(2 * q, std::integral_constant<int, 2>());
+    if ((N & 1) && blockIdx.x == 0 && threadIdx.x == 0) f(N - 1, std::integral_constant<int, 1>());
+}
+template <int n>
+__device__ __forceinline__ void ld_pair(const double* p, double (&v)[n]) {
+    if constexpr (n == 2) {
+        const double2 t = *reinterpret_cast<const double2*>(p);
+        v[0] = t.x; v[1] = t.y;
+    } else {
+        v[0] = *p;
+    }
+}
+template <int n>
+__device__ __forceinline__ void st_pair(double* p, const double (&v)[n]) {
+    if constexpr (n == 2) *reinterpret_cast<double2*>(p) = make_double2(v[0], v[1]);
+    else *p = v[0];
+}
+template <int n>
+__device__ __forceinline__ void st_pair(float* p, const double (&v)[n]) {
+    if constexpr (n == 2) *reinterpret_cast<float2*>(p) = make_float2((float)v[0], (float)v[1]);
+    else *p = (float)v[0];
+}
+
 // r = b, rh = b, x = 0; r.r
 __global__ void __launch_bounds__(LIN_BLOCK) k_bicg_init(long long N, const double* __restrict__ b,
                                                          double* __restrict__ r,
                                                          double* __restrict__ rh,
                                                          double* __restrict__ x, const Finish F) {
     double acc = 0.0;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK) {
-        const double v = b[c];
-        r[c] = v;
-        rh[c] = v;
-        x[c] = 0.0;
-        acc += v * v;
-    }
+    for_pairs(N, [&](long long i, auto cnt) {
+        constexpr int n = decltype(cnt)::value;
+        double v[n], z[n] = {};
+        ld_pair(b + i, v);
+        st_pair(r + i, v);
+        st_pair(rh + i, v);
+        st_pair(x + i, z);
+#pragma unroll
+        for (int q = 0; q < n; ++q) acc = fma(v[q], v[q], acc);
+    });
     finish<false, RED_BICG_START>(F, acc, 0.0);
 }
 
@@ -433,14 +466,23 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_bicg_p(long long N, const double*
     const double beta = scal[S_BETA], omega = scal[S_OMEGA];
     const bool restart = scal[S_RST] != 0.0;
     const bool first = scal[S_ITS] == 0.0 || restart;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK) {
-        const double rc = r[c];
-        const double pv = first ? rc : rc + beta * (p[c] - omega * v[c]);
-        p[c] = pv;
-        if (p32) p32[c] = (float)pv;
-        if (restart) rh[c] = rc;
-    }
+    for_pairs(N, [&](long long i, auto cnt) {
+        constexpr int n = decltype(cnt)::value;
+        double rv[n], pv[n], vv[n];
+        ld_pair(r + i, rv);
+        if (first) {
+#pragma unroll
+            for (int q = 0; q < n; ++q) pv[q] = rv[q];
+        } else {
+            ld_pair(p + i, pv);
+            ld_pair(v + i, vv);
+#pragma unroll
+            for (int q = 0; q < n; ++q) pv[q] = fma(beta, fma(-omega, vv[q], pv[q]), rv[q]);
+        }
+        st_pair(p + i, pv);
+        if (p32) st_pair(p32 + i, pv);
+        if (restart) st_pair(rh + i, rv);
+    });
 }
 
 // s = r - alpha v; s.s
@@ -451,13 +493,19 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_bicg_s(long long N, const double*
                                                       float* __restrict__ s32, const Finish F) {
     const double alpha = scal[S_ALPHA];
     double acc = 0.0;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK) {
-        const double sv = r[c] - alpha * v[c];
-        s[c] = sv;
-        if (s32) s32[c] = (float)sv;
-        acc += sv * sv;
-    }
+    for_pairs(N, [&](long long i, auto cnt) {
+        constexpr int n = decltype(cnt)::value;
+        double rv[n], vv[n];
+        ld_pair(r + i, rv);
+        ld_pair(v + i, vv);
+#pragma unroll
+        for (int q = 0; q < n; ++q) {
+            rv[q] = fma(-alpha, vv[q], rv[q]);
+            acc = fma(rv[q], rv[q], acc);
+        }
+        st_pair(s + i, rv);
+        if (s32) st_pair(s32 + i, rv);
+    });
     finish<false, RED_BICG_SS>(F, acc, 0.0);
 }
 
@@ -477,19 +525,36 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_bicg_xr(long long N, const double
     const bool half = scal[S_HALF] != 0.0;
     const bool none = !half && scal[S_DONE] != 0.0;
     double rr = 0.0, rhr = 0.0;
-    if (!none) {
-        for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-             c += (long long)gridDim.x * LIN_BLOCK) {
-            if (half) {
-                x[c] += alpha * ph[c];
-            } else {
-                x[c] += alpha * ph[c] + omega * sh[c];
-                const double rv = s[c] - omega * t[c];
-                r[c] = rv;
-                rr += rv * rv;
-                rhr += rh[c] * rv;
+    if (half) {
+        for_pairs(N, [&](long long i, auto cnt) {
+            constexpr int n = decltype(cnt)::value;
+            double xv[n], pv[n];
+            ld_pair(x + i, xv);
+            ld_pair(ph + i, pv);
+#pragma unroll
+            for (int q = 0; q < n; ++q) xv[q] = fma(alpha, pv[q], xv[q]);
+            st_pair(x + i, xv);
+        });
+    } else if (!none) {
+        for_pairs(N, [&](long long i, auto cnt) {
+            constexpr int n = decltype(cnt)::value;
+            double xv[n], pv[n], qv[n], sv[n], tv[n], hv[n];
+            ld_pair(x + i, xv);
+            ld_pair(ph + i, pv);
+            ld_pair(sh + i, qv);
+            ld_pair(s + i, sv);
+            ld_pair(t + i, tv);
+            ld_pair(rh + i, hv);
+#pragma unroll
+            for (int q = 0; q < n; ++q) {
+                xv[q] = fma(alpha, pv[q], fma(omega, qv[q], xv[q]));
+                sv[q] = fma(-omega, tv[q], sv[q]);
+                rr = fma(sv[q], sv[q], rr);
+                rhr = fma(hv[q], sv[q], rhr);
             }
-        }
+            st_pair(x + i, xv);
+            st_pair(r + i, sv);
+        });
     }
     finish<true, RED_BICG_NEXT>(F, rr, rhr);
 }

@@ -243,14 +243,14 @@ __global__ void __launch_bounds__(256) k_schur_assemble(const StepParams P, cons
         O.PQ[ax * N + c] = p;
         O.PQ[(3 + ax) * N + c] = q;
         if (PC == 1) {
-            O.W32[ax][c] = (float)q;
-            O.Wp32[ax][c] = (float)p;
+            O.W32[ax][c] = (float)(q);
+            O.Wp32[ax][c] = (float)(p);
         }
     }
     O.diag[c] = diag;
     O.rhs[c] = __ldg(I.rhs + c) + dr;
     if (PC == 1) {
-        O.d32[c] = (float)diag;
+        O.d32[c] = (float)(diag);
         O.wid32[c] = (float)(O.omega * fast_rcp(diag));
     }
     if (PC == 2) O.wid64[c] = O.omega * fast_rcp(diag);
@@ -476,13 +476,13 @@ __device__ __forceinline__ void local_model(const StepParams& P, double ec,
         o.zU[0] = 0.0;
     } else {
         const double x0 = ne3 * dCdT;
-        const double q0 = fma(x0, dT_dne, P.i3 * C);
         const double ir = irho * P.r_ne;
+        const double q0 = ir * fma(x0, dT_dne, P.i3 * C), en = -(ir * Ed), ni = ir * ne3;
         o.M[0][0] = fma(x0, P.cTR * intot, P.one_adot2);    // cTR intot = dT_dec / rho
-        o.M[0][1] = ir * (fma(ne3, k[R_COOL_HI] - k[R_COOL_HII], -(Ed * P.ph[0])) - q0);
+        o.M[0][1] = fma(ni, k[R_COOL_HI] - k[R_COOL_HII], fma(en, P.ph[0], -q0));
         if constexpr (NS == 3) {
-            o.M[0][2] = ir * fma(-2.0, q0, fma(ne3, k[R_COOL_HEI] - k[R_COOL_HEIII], -(Ed * P.ph[1])));
-            o.M[0][3] = ir * (fma(ne3, k[R_COOL_HEII] - k[R_COOL_HEIII], -(Ed * P.ph[2])) - q0);
+            o.M[0][2] = fma(ni, k[R_COOL_HEI] - k[R_COOL_HEIII], fma(en, P.ph[1], -2.0 * q0));
+            o.M[0][3] = fma(ni, k[R_COOL_HEII] - k[R_COOL_HEIII], fma(en, P.ph[2], -q0));
         }
         o.zU[0] = P.cz0 * heat * irho;
     }
@@ -715,7 +715,9 @@ __global__ void __launch_bounds__(CELL_BLOCK) k_cell(const StepParams P, const P
                     B.phi[c] = phi;
                 }
             }
-            B.diag[c] = (1.0 + lo.dLEE) - LMU + Wsum;
+            double dg = (1.0 + lo.dLEE) - LMU;
+            for (int go = !FLUX || P.dir_mask; go; go = opaque(0)) dg += Wsum;
+            B.diag[c] = dg;
             B.rhs[c] = LMf - fs[NV - 1];
 #pragma unroll
             for (int r = 0; r < NM; ++r) {
@@ -766,18 +768,20 @@ cudaError_t launch_cell(const StepParams& P, int ns, int mode, const PhysBuffers
 // its quantities, which few cells do, so all cells form tau (q + tiny) (one FMA each; of x and
 // total - x only the decreasing one) and compare bit patterns on the integer pipe, and only
 // the cells with a bound in force take the smallest fraction.  Measured over the launches
-// of four 256^3 steps, H + He: 1.60 ms each against 2.27 ms with every bound in FP64.
+// of four 256^3 steps, H + He: 1.35 ms each against 2.27 ms with every bound in FP64.
 
-// the smallest fraction min(1, tau (q + tiny) / (-dq)) over the decreasing quantities
+// the smallest fraction min(1, tau (q + tiny) / (-dq)) over the quantities with a bound in force;
+// warps without one go around, and non-negative numbers compare as integers
 struct CapFraction {
     double num = 1.0, den = 1.0;
-    __device__ __forceinline__ void bound(double tau, double q, double dq, double tiny) {
-        if (dq < 0.0) {
-            const double v = fmax(tau * (q + tiny), 0.0);
-            if (v * den < num * (-dq)) { num = v; den = -dq; }
+    __device__ __forceinline__ void bound(bool force, double tau, double q, double dq, double tiny) {
+        for (int go = force; go; go = opaque(0)) {
+            const long long vb = __double_as_longlong(tau * (q + tiny));
+            const double v = (vb >= 0 && vb <= 0x7FF0000000000000LL) ? __longlong_as_double(vb) : 0.0;
+            const long long lhs = __double_as_longlong(v * den), rhs = __double_as_longlong(num * -dq);
+            if (lhs < rhs && rhs <= 0x7FF0000000000000LL) { num = v; den = -dq; }
         }
     }
-    __device__ __forceinline__ double value() const { return den == 1.0 ? num : num / den; }
 };
 
 template <int NS>
@@ -813,36 +817,36 @@ __global__ void __launch_bounds__(256) k_update(const StepParams P, double lam,
         const long long d = __double_as_longlong(dq);
         return d < 0 && __double_as_longlong(v) < (d & 0x7FFFFFFFFFFFFFFFLL);
     };
-    bool act = in_force(s[0], P.tau * e) || in_force(sEp, P.tau * E);
-    double nHe = 0.0, nHeIII = 0.0, sIII = 0.0;
+    const bool fe = in_force(s[0], P.tau * e), fE = in_force(sEp, P.tau * E);
+    bool fx = false, f1 = false, f2 = false, f3 = false;
+    double qx = 0.0, nHe = 0.0, nHeIII = 0.0, sIII = 0.0;
     if constexpr (NS >= 1) {
         // x decreases or total - x does, by the same amount
-        const double q = __double_as_longlong(s[1]) < 0 ? n[0] : nH - n[0];
-        act = act || in_force(-fabs(s[1]), fma(P.tau, q, P.tau_tiny * nH));
+        qx = __double_as_longlong(s[1]) < 0 ? n[0] : nH - n[0];
+        fx = in_force(-fabs(s[1]), fma(P.tau, qx, P.tau_tiny * nH));
     }
     if constexpr (NS == 3) {
         nHe = P.y_he * nH;
         nHeIII = nHe - n[1] - n[2];
         sIII = -(s[2] + s[3]);
         const double tiny = P.tau_tiny * nHe;
-        act = act || in_force(s[2], fma(P.tau, n[1], tiny)) || in_force(s[3], fma(P.tau, n[2], tiny)) ||
-              in_force(sIII, fma(P.tau, nHeIII, tiny));
+        f1 = in_force(s[2], fma(P.tau, n[1], tiny));
+        f2 = in_force(s[3], fma(P.tau, n[2], tiny));
+        f3 = in_force(sIII, fma(P.tau, nHeIII, tiny));
     }
     double fr = lam;
-    if (act) {
+    for (int go = fe || fE || fx || f1 || f2 || f3; go; go = opaque(0)) {
         CapFraction cap;
-        cap.bound(P.tau, e, s[0], 0.0);
-        cap.bound(P.tau, E, sEp, 0.0);
-        if constexpr (NS >= 1) {
-            cap.bound(P.tau, n[0], s[1], 1e-13 * nH);
-            cap.bound(P.tau, nH - n[0], -s[1], 1e-13 * nH);
-        }
+        cap.bound(fe, P.tau, e, s[0], 0.0);
+        cap.bound(fE, P.tau, E, sEp, 0.0);
+        if constexpr (NS >= 1) cap.bound(fx, P.tau, qx, -fabs(s[1]), 1e-13 * nH);
         if constexpr (NS == 3) {
-            cap.bound(P.tau, n[1], s[2], 1e-13 * nHe);
-            cap.bound(P.tau, n[2], s[3], 1e-13 * nHe);
-            cap.bound(P.tau, nHeIII, sIII, 1e-13 * nHe);
+            cap.bound(f1, P.tau, n[1], s[2], 1e-13 * nHe);
+            cap.bound(f2, P.tau, n[2], s[3], 1e-13 * nHe);
+            cap.bound(f3, P.tau, nHeIII, sIII, 1e-13 * nHe);
         }
-        fr = fmin(lam, cap.value());
+        const double f = cap.num / cap.den;
+        fr = __double_as_longlong(f) < __double_as_longlong(lam) ? f : lam;
     }
     ec1[c] = fma(fr, s[0], ec);
     double ksum = 0.0;
