@@ -118,7 +118,20 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-__device__ __forceinline__ float silu_f(float z) { return z / (1.0f + __expf(-z)); }
+// z / (1 + exp(-z)).  Two special-function results each (192 a row bound the forward pass); FAST: the
+// quotient from the reciprocal approximation and one residual correction, q + (z - q d) r, which rounds as
+// the IEEE division does but for a last bit now and then, in 5 instructions instead of a division's 15
+// or so.  (The denominator's bound keeps a zero times infinity out of the correction.)  The guess keeps the
+// division: its FP64 results are held to the bit, and its time is its FP64 logarithms'.
+template <bool FAST>
+__device__ __forceinline__ float silu_f(float z) {
+    if constexpr (!FAST) return z / (1.0f + __expf(-z));
+    const float d = fminf(1.0f + __expf(-z), 3e38f);
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(d));
+    const float q = z * r;
+    return fmaf(fmaf(-q, d, z), r, q);
+}
 
 // one hidden layer on a 16-row tile: in = A fragments over KS k-steps, out = 8 n-tiles
 template <int KS, int RS>
@@ -130,21 +143,21 @@ __device__ __forceinline__ void hidden_layer(const uint32_t (&a)[4][4], const __
         acc[j][0] = b0; acc[j][1] = b1; acc[j][2] = b0; acc[j][3] = b1;
 #pragma unroll
         for (int s = 0; s < KS; ++s) {
-            const __nv_bfloat16* w = W + (8 * j + g) * RS + 16 * s + 2 * t;
-            mma_bf16(acc[j], a[s], *reinterpret_cast<const uint32_t*>(w),
-                     *reinterpret_cast<const uint32_t*>(w + 8));
+            const uint2 w = *reinterpret_cast<const uint2*>(W + (8 * j + g) * RS + 16 * s + 4 * t);
+            mma_bf16(acc[j], a[s], w.x, w.y);
         }
     }
 }
 
 // SiLU of 8 n-tiles into the A fragments of the next layer's 4 k-steps
+template <bool FAST>
 __device__ __forceinline__ void to_fragments(const float (&acc)[8][4], uint32_t (&a)[4][4]) {
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
-        a[s][0] = pack_bf16(silu_f(acc[2 * s][0]), silu_f(acc[2 * s][1]));
-        a[s][1] = pack_bf16(silu_f(acc[2 * s][2]), silu_f(acc[2 * s][3]));
-        a[s][2] = pack_bf16(silu_f(acc[2 * s + 1][0]), silu_f(acc[2 * s + 1][1]));
-        a[s][3] = pack_bf16(silu_f(acc[2 * s + 1][2]), silu_f(acc[2 * s + 1][3]));
+        a[s][0] = pack_bf16(silu_f<FAST>(acc[2 * s][0]), silu_f<FAST>(acc[2 * s][1]));
+        a[s][1] = pack_bf16(silu_f<FAST>(acc[2 * s][2]), silu_f<FAST>(acc[2 * s][3]));
+        a[s][2] = pack_bf16(silu_f<FAST>(acc[2 * s + 1][0]), silu_f<FAST>(acc[2 * s + 1][1]));
+        a[s][3] = pack_bf16(silu_f<FAST>(acc[2 * s + 1][2]), silu_f<FAST>(acc[2 * s + 1][3]));
     }
 }
 
@@ -156,7 +169,7 @@ __global__ void __launch_bounds__(32 * INF_WARPS) k_mlp_infer(const MlpArgs A,
                                                               const float* __restrict__ X,
                                                               float* __restrict__ Y,
                                                               long long n_rows) {
-    __shared__ MlpPacked sw;
+    __shared__ __align__(16) MlpPacked sw;
     __shared__ __nv_bfloat16 xs[INF_WARPS][32][24];
     __shared__ float os[INF_WARPS][32][8];
     // stage the packed weights
@@ -193,7 +206,9 @@ __global__ void __launch_bounds__(32 * INF_WARPS) k_mlp_infer(const MlpArgs A,
             xs[warp][lane][q] = __float2bfloat16_rn(xn);
         }
         __syncwarp();
-#pragma unroll
+        // (not unrolled, like the two middle layers: the code then fits the instruction cache, whose misses
+        // were a third of the stalls)
+#pragma unroll 1
         for (int half = 0; half < 2; ++half) {
             const int r0 = 16 * half + g;
             uint32_t a[4][4];
@@ -203,17 +218,17 @@ __global__ void __launch_bounds__(32 * INF_WARPS) k_mlp_infer(const MlpArgs A,
             a[0][3] = *reinterpret_cast<const uint32_t*>(&xs[warp][r0 + 8][2 * t + 8]);
             float acc[8][4];
             hidden_layer<1, RS1>(a, sw.W1, sw.b1, acc, g, t);
-            to_fragments(acc, a);
-            hidden_layer<4, RS2>(a, sw.W2, sw.b2, acc, g, t);
-            to_fragments(acc, a);
-            hidden_layer<4, RS2>(a, sw.W3, sw.b3, acc, g, t);
-            to_fragments(acc, a);
+            to_fragments<MODE == 0>(acc, a);
+#pragma unroll 1
+            for (int layer = 0; layer < 2; ++layer) {
+                hidden_layer<4, RS2>(a, layer ? sw.W3 : sw.W2, layer ? sw.b3 : sw.b2, acc, g, t);
+                to_fragments<MODE == 0>(acc, a);
+            }
             float o[4] = {sw.b4[2 * t], sw.b4[2 * t + 1], sw.b4[2 * t], sw.b4[2 * t + 1]};
 #pragma unroll
             for (int s = 0; s < 4; ++s) {
-                const __nv_bfloat16* w = sw.W4 + g * RS2 + 16 * s + 2 * t;
-                mma_bf16(o, a[s], *reinterpret_cast<const uint32_t*>(w),
-                         *reinterpret_cast<const uint32_t*>(w + 8));
+                const uint2 w = *reinterpret_cast<const uint2*>(sw.W4 + g * RS2 + 16 * s + 4 * t);
+                mma_bf16(o, a[s], w.x, w.y);
             }
             os[warp][r0][2 * t] = o[0];
             os[warp][r0][2 * t + 1] = o[1];
@@ -591,15 +606,16 @@ __global__ void __launch_bounds__(256) k_mlp_apply(const float* __restrict__ gpa
 // FP32 master weights to the padded BF16 inference layout (one block)
 __global__ void __launch_bounds__(1024) k_mlp_pack(const float* __restrict__ w, MlpPacked* __restrict__ out) {
     const int tid = (int)threadIdx.x;
+    const __nv_bfloat16 zero = __float2bfloat16_rn(0.0f);
     for (int q = tid; q < MLP_HID * RS1; q += 1024) {
         const int n = q / RS1, k = q % RS1;
-        out->W1[q] = __float2bfloat16_rn(k < MLP_IN ? w[OW1 + n * MLP_IN + k] : 0.0f);
+        out->W1[n * RS1 + packed_k(k)] = k < MLP_IN ? __float2bfloat16_rn(w[OW1 + n * MLP_IN + k]) : zero;
     }
     for (int q = tid; q < MLP_HID * RS2; q += 1024) {
-        const int n = q / RS2, k = q % RS2;
-        out->W2[q] = __float2bfloat16_rn(k < MLP_HID ? w[OW2 + n * MLP_HID + k] : 0.0f);
-        out->W3[q] = __float2bfloat16_rn(k < MLP_HID ? w[OW3 + n * MLP_HID + k] : 0.0f);
-        if (n < 8) out->W4[q] = __float2bfloat16_rn(n < MLP_OUT && k < MLP_HID ? w[OW4 + n * MLP_HID + k] : 0.0f);
+        const int n = q / RS2, k = q % RS2, at = n * RS2 + packed_k(k);
+        out->W2[at] = k < MLP_HID ? __float2bfloat16_rn(w[OW2 + n * MLP_HID + k]) : zero;
+        out->W3[at] = k < MLP_HID ? __float2bfloat16_rn(w[OW3 + n * MLP_HID + k]) : zero;
+        if (n < 8) out->W4[at] = n < MLP_OUT && k < MLP_HID ? __float2bfloat16_rn(w[OW4 + n * MLP_HID + k]) : zero;
     }
     if (tid < MLP_HID) {
         out->b1[tid] = w[OB1 + tid];
@@ -634,7 +650,9 @@ cudaError_t launch_mlp_infer(const MlpArgs& A, const MlpPacked* pk, const float*
     const long long rows = guess ? A.N : n_rows;
     const long long tiles = (rows + 31) / 32;
     long long blocks = (tiles + INF_WARPS - 1) / INF_WARPS;
-    if (blocks > 152LL * 8) blocks = 152LL * 8;
+    // one wave of the 6 blocks an SM holds (their shared memory): with more, the few that start late
+    // would take as long as the first ones
+    if (blocks > 152LL * 6) blocks = 152LL * 6;
     if (blocks < 1) blocks = 1;
     if (guess) k_mlp_infer<1><<<(unsigned)blocks, 32 * INF_WARPS, 0, st>>>(A, pk, X, Y, n_rows);
     else k_mlp_infer<0><<<(unsigned)blocks, 32 * INF_WARPS, 0, st>>>(A, pk, X, Y, n_rows);

@@ -10,10 +10,17 @@
 namespace rhi {
 
 constexpr int MLP_IN = RHI_MLP_IN, MLP_HID = RHI_MLP_HID, MLP_OUT = RHI_MLP_OUT;
-constexpr int RS1 = 24;                       // padded row strides (bf16) of the packed weights
-constexpr int RS2 = 72;
+// Row strides (bf16) of the packed weights: 8 words more than a multiple of 32 (or 8), so that the
+// eight-byte fragment loads of a half-warp (4 rows x 4 pieces) fall into different banks
+constexpr int RS1 = 16;
+constexpr int RS2 = 80;
+// place of input k in a packed row: within each 16, a thread's four values of an m16n8k16 B
+// fragment (k = 2t, 2t + 1, 2t + 8, 2t + 9) side by side
+__host__ __device__ constexpr int packed_k(int k) {
+    return (k & ~15) + 4 * ((k & 7) >> 1) + 2 * ((k >> 3) & 1) + (k & 1);
+}
 
-// inference weights: BF16 rows padded for conflict-free fragment loads, FP32 biases and
+// inference weights: BF16 rows in fragment order, padded for conflict-free loads, FP32 biases and
 // the input normalisation (mean, 1 / scale)
 struct MlpPacked {
     __nv_bfloat16 W1[MLP_HID * RS1];
