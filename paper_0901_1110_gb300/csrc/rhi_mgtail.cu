@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(TailTraits<T>::THREADS) k_mg_tail(const __grid
     TailCell<T> r1[1], rn[1];                         // another level, and the next one on the way
     if (mine > 0) B.cells(lv[0], r0);
     if (mine > 1) B.cells(lv[1], r1);
-    if (wide > 0) cl.sync();                          // every block has started
+    // (a block reads another's memory only after a barrier of all, so after all have started)
     // down
     if (mine > 0) B.down(0, wide > 0, n == 1 ? A.coarse : A.pre, n == 1, 0, r0);
     for (int l = 1; l < mine; ++l) {
@@ -298,6 +298,8 @@ __global__ void __launch_bounds__(TailTraits<T>::THREADS) k_mg_tail(const __grid
         if (wide == 1) cl.sync();
         B.up(0, wide > 0, pre, n == 2 ? after(A.coarse) : done, true, r0);
     }
+    // no block leaves while its memory may be read: all have arrived here, their last reads done
+    if (wide > 0) cl.barrier_arrive();
     if (mine > 0) {
 #pragma unroll
         for (int u = 0; u < TailTraits<T>::CELLS; ++u)
@@ -307,7 +309,7 @@ __global__ void __launch_bounds__(TailTraits<T>::THREADS) k_mg_tail(const __grid
                 if (A.x64) A.x64[c] = (double)r0[u].x;
             }
     }
-    if (wide > 0) cl.sync();                          // no block leaves while its memory is read
+    if (wide > 0) cl.barrier_wait();
 }
 
 // blocks of the cluster on the current device: 16 where such a cluster (a non-portable size) fits,
