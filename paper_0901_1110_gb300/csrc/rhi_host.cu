@@ -416,6 +416,35 @@ Op<double> newton_op(const rhi_ctx* h) {
     return A;
 }
 
+// the coarse levels of the finest operator h->pc0, one launch each down to a level small enough for the
+// rest to take one launch together
+template <typename T>
+int build_hierarchy(rhi_ctx* h, std::vector<Level<T>>& lv, bool nonsym) {
+    LinLaunch L(h->st, &h->prof);
+    const double om = h->prm.mg_omega;
+    std::vector<MgLevel<T>> c(lv.size());
+    for (size_t l = 1; l < lv.size(); ++l) {
+        Level<T>& v = lv[l];
+        c[l] = MgLevel<T>{v.nx, v.ny, v.nz, v.N, v.diag, v.wid, nonsym ? nullptr : v.loc,
+                          {v.W[0], v.W[1], v.W[2]}, {nullptr, nullptr, nullptr}};
+        if (nonsym) for (int a = 0; a < 3; ++a) c[l].wp[a] = v.Wp[a];
+    }
+    for (size_t l = 0; l + 1 < lv.size(); ++l) {
+        const int n = (int)(lv.size() - 1 - l);
+        const bool rest = n > 1 && c[l + 1].N <= MG_BUILD_TAIL && n <= MG_TAIL_LEVELS;
+        const int blocks = h->tail_blocks[sizeof(T) == 8];
+        if (l == 0) {
+            if (rest) CK((L.build_levels<double, T>(h->pc0, &c[1], n, om, blocks)));
+            else CK((L.build_level<double, T>(h->pc0, c[1], om)));
+        } else {
+            if (rest) CK((L.build_levels<T, T>(level_op(h, lv[l]), &c[l + 1], n, om, blocks)));
+            else CK((L.build_level<T, T>(level_op(h, lv[l]), c[l + 1], om)));
+        }
+        if (rest) break;
+    }
+    return RHI_OK;
+}
+
 // coarse operators for the finest operator A0 (the lagged-D matrix h->op0, or the Newton matrix
 // when nonsym, whose finest level the assembly has written); A0 becomes the preconditioner's
 // finest operator h->pc0
@@ -431,12 +460,7 @@ int precond_setup(rhi_ctx* h, const Op<double>& A0, bool nonsym) {
         h->pc0.wid = lv[0].wid;
         h->pc0.loc = lv[0].loc;
         if (!nonsym) CK((L.level_prep<double, double>(h->pc0, om, lv[0].wid, lv[0].loc)));
-        for (size_t l = 0; l + 1 < lv.size(); ++l) {
-            Op<double> A = (l == 0) ? h->pc0 : level_op(h, lv[l]);
-            auto& c = lv[l + 1];
-            CK((L.build_level<double, double>(A, c.nx, c.ny, c.nz, om, c.diag, c.wid, nonsym ? nullptr : c.loc,
-                                              c.W, nonsym ? c.Wp : nullptr)));
-        }
+        return build_hierarchy<double>(h, lv, nonsym);
     } else if (h->prm.precond == RHI_PRECOND_MG_FP32) {
         auto& lv = h->mg32;
         if (nonsym && !lv[0].Wp[0])
@@ -447,14 +471,7 @@ int precond_setup(rhi_ctx* h, const Op<double>& A0, bool nonsym) {
             // each child's full row and needs no local part)
             CK((L.level_prep<double, float>(h->pc0, om, lv[0].wid, nullptr)));
         }
-        for (size_t l = 0; l + 1 < lv.size(); ++l) {
-            auto& c = lv[l + 1];
-            float* const* wp = nonsym ? c.Wp : nullptr;
-            if (l == 0)
-                CK((L.build_level<double, float>(h->pc0, c.nx, c.ny, c.nz, om, c.diag, c.wid, nullptr, c.W, wp)));
-            else
-                CK((L.build_level<float, float>(level_op(h, lv[l]), c.nx, c.ny, c.nz, om, c.diag, c.wid, nullptr, c.W, wp)));
-        }
+        return build_hierarchy<float>(h, lv, nonsym);
     }
     return RHI_OK;
 }
@@ -1199,6 +1216,7 @@ int rhi_create(const rhi_grid* grid, const rhi_bc* bc, const rhi_params* params,
     if (!rc) rc = dalloc(h, &h->table, (size_t)NBINS * NRATES);
     if (!rc) {
         cudaError_t e = mg_tail_init(&h->tail_blocks[0], &h->tail_blocks[1]);
+        if (e == cudaSuccess) e = mg_build_init();
         if (e == cudaSuccess) e = cudaMallocHost(&h->h_scal, sizeof(double) * S_NSCAL);
         if (e == cudaSuccess) e = cudaMallocHost(&h->h_ctl, sizeof(double) * 3);
         if (e == cudaSuccess) e = cudaMallocHost(&h->h_kerr, sizeof(int));

@@ -6,9 +6,11 @@
 // Operator of a level: (A x)_c = diag_c x_c - sum_ax (W[ax]_c x_lo + Wp[ax]_hi x_hi),
 // stored per lower face (0 on zero-flux boundary faces): W couples the upper cell's row to the
 // lower cell, Wp the lower cell's row to the upper cell.  Symmetric levels pass Wp = W.
-#include "rhi_linear.cuh"
+#include <cooperative_groups.h>
 
 #include <type_traits>
+
+#include "rhi_linear.cuh"
 
 namespace rhi {
 
@@ -997,33 +999,34 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_prolong(int nx, int ny, int nz
     }
 }
 
-// One coarse level of the hierarchy in one pass: the operator by re-discretisation, and the smoother's
-// omega / diagonal.  Local diagonal = mean of the children's local diagonals (diag - the six
-// couplings of their rows); each face array of the coarse cell's lower face = (mean of that array over
-// the existing fine lower faces of its first-layer children) / 4, W from W and, for a
-// non-symmetric operator, Wp from Wp; diagonal = local diagonal + the row's six couplings, of which the
-// upper ones are the Wp of the faces above, formed here from the same fine entries as the cells
-// above form them.  (Counts of children are powers of two, so the means are exact products.)
+// FP32 to FP64 on the integer pipe, exact for every value: a conversion instruction takes the FP64 pipe
+// as long as an FMA (64 cycles a warp), which is most of a small level's build.  No branch; subnormals
+// are scaled up in FP32 first.
+__device__ __forceinline__ double widen(float f) {
+    const bool small = (__float_as_uint(f) & 0x7fffffffu) < 0x00800000u;
+    const unsigned u = __float_as_uint(small ? f * 18446744073709551616.0f : f), m = u & 0x7fffffffu;
+    unsigned hi = (m >> 3) + (small ? (896u - 64u) << 20 : 896u << 20);
+    hi = m == 0u ? 0u : hi;
+    hi = m >= 0x7f800000u ? 0x7ff00000u | (m >> 3 & 0xfffffu) : hi;
+    return __hiloint2double((int)((u & 0x80000000u) | hi), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double f) { return f; }
+
+// One coarse cell of the hierarchy: the operator by re-discretisation, and the smoother's omega /
+// diagonal.  Local diagonal = mean of the children's local diagonals (diag - the six couplings of their
+// rows); each face array of the coarse cell's lower face = (mean of that array over the existing fine
+// lower faces of its first-layer children) / 4, W from W and, for a non-symmetric operator, Wp from Wp;
+// diagonal = local diagonal + the row's six couplings, of which the upper ones are the Wp of the faces
+// above, formed here from the same fine entries as the cells above form them.  (Counts of children are
+// powers of two, so the means are exact products.)
 //
 // Sums of couplings are shared between the faces and the local diagonal: 8.5 loads and about 8 FP64
 // additions per fine cell.  Measured for all five coarse levels of a 256^3 FP32 hierarchy, both
 // couplings per face: 0.63 ms in 5 launches, against 1.04 ms in 15 for separate passes (operator, diagonal,
 // omega / diagonal) with a 64-bit division and dependent loads per child.
 template <typename TF, typename TC>
-__global__ void __launch_bounds__(LIN_BLOCK) k_mg_build(const Op<TF> A, int cnx, int cny, int cnz,
-                                                        FastDiv fcx, FastDiv fcxy, double omega,
-                                                        TC* __restrict__ dc, TC* __restrict__ wid,
-                                                        TC* __restrict__ loc,
-                                                        TC* __restrict__ wcx, TC* __restrict__ wcy,
-                                                        TC* __restrict__ wcz,
-                                                        TC* __restrict__ wpcx,
-                                                        TC* __restrict__ wpcy,
-                                                        TC* __restrict__ wpcz) {
-    const long long Nc = (long long)cnx * cny * cnz;
-    const long long cc = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x;
-    if (cc >= Nc) return;
-    int I, J, K;
-    coords_fd(cc, fcx, fcxy, I, J, K);
+__device__ __forceinline__ void build_cell(const Op<TF>& A, const MgLevel<TC>& c, int I, int J, int K,
+                                           long long cc, double omega) {
     const long long s[3] = {1, A.nx, (long long)A.nx * A.ny};
     const int n[3] = {A.nx, A.ny, A.nz}, q0[3] = {2 * I, 2 * J, 2 * K};
     const long long c0 = q0[0] + s[1] * q0[1] + s[2] * q0[2];
@@ -1046,40 +1049,79 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_build(const Op<TF> A, int cnx,
             for (int di = 0; di < 2; ++di) {
                 const int d[3] = {di, dj, dk};
                 if ((di && !two[0]) || (dj && !two[1]) || (dk && !two[2])) continue;
-                const long long c = c0 + di + dj * s[1] + dk * s[2];
-                dl += (double)(__ldg(A.diag + c));
+                const long long f = c0 + di + dj * s[1] + dk * s[2];
+                dl += widen(A.diag[f]);
 #pragma unroll
                 for (int ax = 0; ax < 3; ++ax) {
-                    const double w = (double)(__ldg(A.W[ax] + c)), v = (double)(__ldg(A.Wp[ax] + c));
+                    const double w = widen(A.W[ax][f]), v = widen(A.Wp[ax][f]);
                     if (d[ax] == 0) { wl[ax] += w; wp[ax] += v; }      // the parent's lower face
                     else tot += w + v;                                 // a face between children
                     if ((d[ax] == 1 || !two[ax]) && up[ax])            // the parent's upper face
-                        wu[ax] += (double)(__ldg(A.Wp[ax] + c + above[ax]));
+                        wu[ax] += widen(A.Wp[ax][f + above[ax]]);
                 }
             }
     double diag = 0.0;
     const double half[3] = {two[0] ? 0.5 : 1.0, two[1] ? 0.5 : 1.0, two[2] ? 0.5 : 1.0};
-    double wlc[3], wpc[3];
 #pragma unroll
     for (int ax = 0; ax < 3; ++ax) {
         tot += wl[ax] + wu[ax];
         const double mean = 0.25 * half[(ax + 1) % 3] * half[(ax + 2) % 3];
-        wlc[ax] = mean * wl[ax];
-        wpc[ax] = mean * wp[ax];
-        diag += wlc[ax] + mean * wu[ax];
+        const double wlc = mean * wl[ax];
+        diag += wlc + mean * wu[ax];
+        c.w[ax][cc] = (TC)wlc;
+        if (c.wp[0]) c.wp[ax][cc] = (TC)(mean * wp[ax]);
     }
     const double local = (dl - tot) * (half[0] * half[1] * half[2]);
     diag += local;
-    dc[cc] = (TC)diag;
-    if (loc) loc[cc] = (TC)local;
-    wid[cc] = (TC)omega / (TC)diag;
-    wcx[cc] = (TC)wlc[0];
-    wcy[cc] = (TC)wlc[1];
-    wcz[cc] = (TC)wlc[2];
-    if (wpcx) {
-        wpcx[cc] = (TC)wpc[0];
-        wpcy[cc] = (TC)wpc[1];
-        wpcz[cc] = (TC)wpc[2];
+    c.diag[cc] = (TC)diag;
+    if (c.loc) c.loc[cc] = (TC)local;
+    c.wid[cc] = (TC)omega / (TC)diag;
+}
+
+template <typename TF, typename TC>
+__global__ void __launch_bounds__(LIN_BLOCK) k_mg_build(const Op<TF> A, const MgLevel<TC> c, FastDiv fcx,
+                                                        FastDiv fcxy, double omega) {
+    const long long cc = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (cc >= c.N) return;
+    int I, J, K;
+    coords_fd(cc, fcx, fcxy, I, J, K);
+    build_cell<TF, TC>(A, c, I, J, K, cc, omega);
+}
+
+// Small levels, each from the one before, by one cluster with its barrier between them.  The levels are
+// read and written in global memory (plain loads: the barrier orders them).
+template <typename TC>
+struct BuildArgs {
+    MgLevel<TC> c[MG_TAIL_LEVELS];
+    int n;
+    double omega;
+};
+template <typename TF, typename TC>
+__global__ void __launch_bounds__(LIN_BLOCK) k_mg_build_tail(const __grid_constant__ Op<TF> A,
+                                                             const __grid_constant__ BuildArgs<TC> B) {
+    const int me = (int)(blockIdx.x * LIN_BLOCK + threadIdx.x), all = (int)(gridDim.x * LIN_BLOCK);
+    for (int l = 0; l < B.n; ++l) {
+        const MgLevel<TC> c = B.c[l];
+        const int nxy = c.nx * c.ny;
+        for (int cc = me; cc < (int)c.N; cc += all) {
+            const int K = cc / nxy, J = (cc - K * nxy) / c.nx, I = cc - K * nxy - J * c.nx;
+            if (l == 0) {
+                build_cell<TF, TC>(A, c, I, J, K, cc, B.omega);
+            } else {
+                const MgLevel<TC>& f = B.c[l - 1];
+                Op<TC> o{};
+                o.nx = f.nx; o.ny = f.ny; o.nz = f.nz;
+                o.diag = f.diag;
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    o.per[a] = A.per[a];
+                    o.W[a] = f.w[a];
+                    o.Wp[a] = f.wp[0] ? f.wp[a] : f.w[a];
+                }
+                build_cell<TC, TC>(o, c, I, J, K, cc, B.omega);
+            }
+        }
+        if (l + 1 < B.n) cooperative_groups::this_cluster().sync();
     }
 }
 
@@ -1326,15 +1368,44 @@ cudaError_t LinLaunch::prolong(int nx, int ny, int nz, int cnx, int cny, const T
     return end();
 }
 template <typename TF, typename TC>
-cudaError_t LinLaunch::build_level(const Op<TF>& A, int cnx, int cny, int cnz, double omega, TC* dc,
-                                   TC* wid, TC* loc, TC* const* wc, TC* const* wpc) {
+cudaError_t LinLaunch::build_level(const Op<TF>& A, const MgLevel<TC>& c, double omega) {
     begin("mg_build");
-    const long long Nc = (long long)cnx * cny * cnz;
-    k_mg_build<TF, TC><<<(unsigned)((Nc + LIN_BLOCK - 1) / LIN_BLOCK), LIN_BLOCK, 0, st>>>(
-        A, cnx, cny, cnz, make_fastdiv((unsigned)cnx), make_fastdiv((unsigned)cnx * cny), omega, dc,
-        wid, loc, wc[0], wc[1], wc[2], wpc ? wpc[0] : nullptr, wpc ? wpc[1] : nullptr,
-        wpc ? wpc[2] : nullptr);
+    // a cell's chain of FP64 additions (64 cycles each) is the time of a small level: small blocks spread its
+    // warps over all SMs
+    const int block = c.N < 152LL * LIN_BLOCK ? 64 : LIN_BLOCK;
+    k_mg_build<TF, TC><<<(unsigned)((c.N + block - 1) / block), block, 0, st>>>(
+        A, c, make_fastdiv((unsigned)c.nx), make_fastdiv((unsigned)c.nx * c.ny), omega);
     return end();
+}
+template <typename TF, typename TC>
+cudaError_t LinLaunch::build_levels(const Op<TF>& A, const MgLevel<TC>* c, int n, double omega,
+                                    int blocks) {
+    begin("mg_build_tail");
+    BuildArgs<TC> B{};
+    B.n = n;
+    B.omega = omega;
+    for (int l = 0; l < n; ++l) B.c[l] = c[l];
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = blocks;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(LIN_BLOCK);
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_mg_build_tail<TF, TC>, A, B);
+    const cudaError_t e2 = end();
+    return e != cudaSuccess ? e : e2;
+}
+// the cluster of the coarse-end kernel (16 blocks, a non-portable size) for the build too; called for
+// every handle
+cudaError_t mg_build_init() {
+    cudaError_t e = cudaFuncSetAttribute(k_mg_build_tail<double, double>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mg_build_tail<double, float>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mg_build_tail<float, float>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    return e;
 }
 template <typename TF, typename TO>
 cudaError_t LinLaunch::level_prep(const Op<TF>& A, double omega, TO* wid, TO* loc) {
@@ -1365,15 +1436,12 @@ template cudaError_t LinLaunch::restrict_res<float>(const Op<float>&, const floa
                                                     int, int, int, float*);
 template cudaError_t LinLaunch::prolong<double>(int, int, int, int, int, const double*, double*);
 template cudaError_t LinLaunch::prolong<float>(int, int, int, int, int, const float*, float*);
-template cudaError_t LinLaunch::build_level<double, double>(const Op<double>&, int, int, int, double,
-                                                            double*, double*, double*,
-                                                            double* const*, double* const*);
-template cudaError_t LinLaunch::build_level<double, float>(const Op<double>&, int, int, int, double,
-                                                           float*, float*, float*, float* const*,
-                                                           float* const*);
-template cudaError_t LinLaunch::build_level<float, float>(const Op<float>&, int, int, int, double,
-                                                          float*, float*, float*, float* const*,
-                                                          float* const*);
+template cudaError_t LinLaunch::build_level<double, double>(const Op<double>&, const MgLevel<double>&, double);
+template cudaError_t LinLaunch::build_level<double, float>(const Op<double>&, const MgLevel<float>&, double);
+template cudaError_t LinLaunch::build_level<float, float>(const Op<float>&, const MgLevel<float>&, double);
+template cudaError_t LinLaunch::build_levels<double, double>(const Op<double>&, const MgLevel<double>*, int, double, int);
+template cudaError_t LinLaunch::build_levels<double, float>(const Op<double>&, const MgLevel<float>*, int, double, int);
+template cudaError_t LinLaunch::build_levels<float, float>(const Op<float>&, const MgLevel<float>*, int, double, int);
 template cudaError_t LinLaunch::level_prep<double, double>(const Op<double>&, double, double*,
                                                            double*);
 template cudaError_t LinLaunch::level_prep<double, float>(const Op<double>&, double, float*, float*);

@@ -46,6 +46,16 @@ struct OpNS {
 constexpr int MG_TAIL_LEVELS = 18;
 constexpr int MG_TAIL_SMEM = 128 * 1024;
 template <typename T> bool mg_tail_fits(long long N, long long N_next, int blocks);
+// one coarse level of the hierarchy build (rhi_linear.cu): its size and arrays (loc, wp: may be null)
+template <typename T>
+struct MgLevel {
+    int nx, ny, nz;
+    long long N;
+    T *diag, *wid, *loc, *w[3], *wp[3];
+};
+// levels of at most this many cells (one warp per sub-partition of the cluster's SMs) are built by one
+// cluster launch together
+constexpr long long MG_BUILD_TAIL = 2048;
 template <typename T>
 struct MgTail {
     Op<T> op[MG_TAIL_LEVELS];
@@ -58,6 +68,7 @@ struct MgTail {
     double* x64;
 };
 cudaError_t mg_tail_init(int* blocks32, int* blocks64);
+cudaError_t mg_build_init();
 
 // device scalar slots of the Krylov iterations.  The BiCGStab and CG loops keep their control state
 // on the device: S_THR (converged when r.r <= S_THR), S_MAXIT, the iteration count S_ITS, S_DONE
@@ -159,11 +170,13 @@ struct LinLaunch {
                              T* bc);
     template <typename T>
     cudaError_t prolong(int nx, int ny, int nz, int cnx, int cny, const T* xc, T* xf);
-    // coarse level of A: diagonal dc, wid = omega / diagonal, loc (may be null) the diagonal's local
-    // part, W-type face arrays wc[3] and, for a non-symmetric A, Wp-type face arrays wpc[3] (else null)
+    // coarse level c of A
     template <typename TF, typename TC>
-    cudaError_t build_level(const Op<TF>& A, int cnx, int cny, int cnz, double omega, TC* dc, TC* wid,
-                            TC* loc, TC* const* wc, TC* const* wpc);
+    cudaError_t build_level(const Op<TF>& A, const MgLevel<TC>& c, double omega);
+    // the n coarse levels c of A, each from the one before, in one launch of `blocks` blocks; the first has
+    // at most MG_BUILD_TAIL cells
+    template <typename TF, typename TC>
+    cudaError_t build_levels(const Op<TF>& A, const MgLevel<TC>* c, int n, double omega, int blocks);
     // finest level of a symmetric operator: wid = omega / diag (smoothers) and, if loc is not null,
     // loc = diag - (six faces) (FP64 restriction), evaluated in TF and rounded to TO
     template <typename TF, typename TO>
