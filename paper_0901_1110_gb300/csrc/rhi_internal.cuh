@@ -175,13 +175,16 @@ __device__ __forceinline__ bool grid_sum(double v1, double v2, double* partials,
         if (TWO) partials[n + blockIdx.x] = s2;
         last_block = false;
         if (count) {
-            __threadfence();
-            last_block = atomicInc(count, (unsigned)n - 1u) == (unsigned)n - 1u;
+            // the ticket releases this thread's partials and, with the last one, acquires all others'
+            // (for the block by way of its barrier)
+            unsigned t;
+            asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;"
+                         : "=r"(t) : "l"(count), "r"((unsigned)n - 1u) : "memory");
+            last_block = t == (unsigned)n - 1u;
         }
     }
     __syncthreads();
     if (!last_block) return false;
-    __threadfence();
     double a1 = 0.0, a2 = 0.0;
     for (int q = (int)threadIdx.x; q < n; q += BLOCK) {
         a1 += __ldcg(partials + q);

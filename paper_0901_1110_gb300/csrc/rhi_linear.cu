@@ -233,10 +233,10 @@ template <bool TWO, int OP>
 __device__ __forceinline__ void finish(const Finish& F, double v1, double v2) {
     __shared__ double sc[S_NSCAL];
     double s1, s2;
+    // the scalars by way of shared memory, fetched by every block under its own sum (only the last
+    // one, which alone writes them, after every block has its ticket, uses them)
+    if (threadIdx.x < S_NSCAL && F.count) sc[threadIdx.x] = __ldcg(F.scal + threadIdx.x);
     if (!grid_sum<LIN_BLOCK, TWO>(v1, v2, F.partials, F.count, s1, s2)) return;
-    // the scalars by way of shared memory: one trip to memory each way
-    if (threadIdx.x < S_NSCAL) sc[threadIdx.x] = __ldcg(F.scal + threadIdx.x);
-    __syncthreads();
     if (threadIdx.x == 0) scalar_update<OP>(sc, F.slot, F.cond, s1, s2);
     __syncthreads();
     if (threadIdx.x < S_NSCAL) F.scal[threadIdx.x] = sc[threadIdx.x];
