@@ -159,6 +159,29 @@ __device__ __forceinline__ double block_sum(double v) {
     return s;
 }
 
+// two sums at once, by two warps; valid in thread 0
+template <int BLOCK>
+__device__ __forceinline__ void block_sum2(double& v1, double& v2) {
+    static_assert(BLOCK >= 64, "two warps");
+    __shared__ double part[2][BLOCK];
+    part[0][threadIdx.x] = v1;
+    part[1][threadIdx.x] = v2;
+    __syncthreads();
+    if (threadIdx.x < 64) {
+        const double* p = part[threadIdx.x >> 5] + (threadIdx.x & 31);
+        double s = p[0];
+#pragma unroll
+        for (int q = 1; q < BLOCK / 32; ++q) s += p[32 * q];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        v1 = s;
+        if (threadIdx.x == 32) part[1][0] = s;
+    }
+    __syncthreads();
+    v2 = part[1][0];
+    __syncthreads();
+}
+
 // Grid-wide sum without a second launch: every block writes its partial and takes a ticket; the
 // block with the last one (true) adds the partials in a fixed order, so the result does not depend on
 // the order the blocks ended in.  Returns true in all threads of that block; the sums are valid in
@@ -168,8 +191,10 @@ __device__ __forceinline__ bool grid_sum(double v1, double v2, double* partials,
                                          double& s1, double& s2) {
     __shared__ bool last_block;
     const int n = (int)gridDim.x;
-    s1 = block_sum<BLOCK>(v1);
-    s2 = TWO ? block_sum<BLOCK>(v2) : 0.0;
+    s1 = v1;
+    s2 = v2;
+    if constexpr (TWO) block_sum2<BLOCK>(s1, s2);
+    else s1 = block_sum<BLOCK>(v1);
     if (threadIdx.x == 0) {
         partials[blockIdx.x] = s1;
         if (TWO) partials[n + blockIdx.x] = s2;
@@ -190,8 +215,10 @@ __device__ __forceinline__ bool grid_sum(double v1, double v2, double* partials,
         a1 += __ldcg(partials + q);
         if (TWO) a2 += __ldcg(partials + n + q);
     }
-    s1 = block_sum<BLOCK>(a1);
-    s2 = TWO ? block_sum<BLOCK>(a2) : 0.0;
+    s1 = a1;
+    s2 = a2;
+    if constexpr (TWO) block_sum2<BLOCK>(s1, s2);
+    else s1 = block_sum<BLOCK>(a1);
     return true;
 }
 
