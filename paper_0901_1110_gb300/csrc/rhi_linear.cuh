@@ -56,14 +56,20 @@ struct MgLevel {
 // levels of at most this many cells (one warp per sub-partition of the cluster's SMs) are built by one
 // cluster launch together
 constexpr long long MG_BUILD_TAIL = 2048;
+// BiCGStab's p = r + beta (p - omega v) with the scalars of scal, and rh = r after a restart (k_bicg_p)
+struct BicgP {
+    const double *scal = nullptr, *r = nullptr, *v = nullptr;
+    double *p = nullptr, *rh = nullptr;
+};
 template <typename T>
 struct MgTail {
     Op<T> op[MG_TAIL_LEVELS];
     int n, blocks;
     int pre, post, coarse;      // sweeps
     T omega;
-    const T* b;                 // right-hand side of the first level, or in FP64 (b64)
+    const T* b;                 // right-hand side of the first level, or in FP64 (b64), or of up
     const double* b64;
+    BicgP up;
     T* x;                       // result, in T and / or FP64
     double* x64;
 };

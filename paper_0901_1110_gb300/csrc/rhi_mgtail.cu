@@ -62,6 +62,7 @@ struct TailArgs {
     T* x;                    // result in T (may be null) and FP64 (may be null)
     double* x64;
     const double* skip;
+    BicgP up;                // with up.scal, the right-hand side is the p this launch updates
 };
 
 // shared memory of a block of the cluster by its address in the cluster's window (the block's own too:
@@ -155,10 +156,46 @@ struct TailBlock {
         if (wide) cg::this_cluster().sync();
         else __syncthreads();
     }
-    // right-hand side of the first level (given) or of a coarse cell (the children's residuals, which
-    // sit in buffer `rb` of the level above)
+    // The first level's right-hand side: given, or BiCGStab's p, updated here (k_bicg_p's formulas; the
+    // thread that owns a cell is the only one to read or write its p).
+    template <int M>
+    __device__ __forceinline__ void given(TailCell<T> (&r)[M]) const {
+        const BicgP& P = A.up;
+        if (!P.scal) {
+#pragma unroll
+            for (int u = 0; u < M; ++u)
+                if (r[u].on) {
+                    const int c = cell(lv[0], u);
+                    r[u].b = A.b64 ? (T)A.b64[c] : A.b[c];
+                }
+            return;
+        }
+        const double beta = P.scal[S_BETA], omega = P.scal[S_OMEGA];
+        const bool restart = P.scal[S_RST] != 0.0;
+        const bool first = P.scal[S_ITS] == 0.0 || restart;
+        double rv[M], pv[M], vv[M];
+#pragma unroll
+        for (int u = 0; u < M; ++u)
+            if (r[u].on) {
+                const int c = cell(lv[0], u);
+                rv[u] = P.r[c];
+                if (!first) {
+                    pv[u] = P.p[c];
+                    vv[u] = P.v[c];
+                }
+            }
+#pragma unroll
+        for (int u = 0; u < M; ++u)
+            TAIL_CELL(r[u].on) {
+                const int c = cell(lv[0], u);
+                const double p = first ? rv[u] : fma(beta, fma(-omega, vv[u], pv[u]), rv[u]);
+                P.p[c] = p;
+                if (restart) P.rh[c] = rv[u];
+                r[u].b = (T)p;
+            }
+    }
+    // right-hand side of a coarse cell: the children's residuals, which sit in buffer `rb` of the level above
     __device__ __forceinline__ T rhs(int l, int rb, int c) const {
-        if (l == 0) return A.b64 ? (T)A.b64[c] : A.b[c];
         const TailLevel<T>& f = lv[l - 1];
         int I, J, K;
         coords(lv[l], c, I, J, K);
@@ -200,10 +237,11 @@ struct TailBlock {
     __device__ __forceinline__ void down(int l, bool w, int sweeps, bool last, int rb, TailCell<T> (&r)[M]) const {
         const TailLevel<T>& v = lv[l];
         T dg[M];
+        if (l == 0) given(r);
 #pragma unroll
         for (int u = 0; u < M; ++u)
             TAIL_CELL(r[u].on) {
-                r[u].b = rhs(l, rb, cell(v, u));
+                if (l > 0) r[u].b = rhs(l, rb, cell(v, u));
                 if (!last) dg[u] = __ldg(v.diag + cell(v, u));
                 r[u].x = r[u].wid * r[u].b;
                 if (M == 1) sm[v.b + at(u)] = r[u].b;       // (the first level's b stays in its registers)
@@ -380,6 +418,7 @@ cudaError_t LinLaunch::mg_tail(const MgTail<T>& M) {
     if (at * sizeof(T) > (size_t)MG_TAIL_SMEM) return cudaErrorInvalidValue;
     A.pre = M.pre; A.post = M.post; A.coarse = M.coarse;
     A.om1 = T(1) - M.omega;
+    A.up = M.up;
     A.b = M.b; A.b64 = M.b64; A.x = M.x; A.x64 = M.x64;
     A.skip = skip;
     begin(sizeof(T) == 4 ? "mg_tail_f32" : "mg_tail_f64");
