@@ -127,11 +127,14 @@ def alg_bytes(nonsym):
         "bicg_update_s_f32": 8 * 2 + 8 + 4,
         "kappa": 8 * 3 + 8,
         # weighted-Jacobi sweep on the finest level: x, b, omega / diag and the face arrays
-        # read, x written; the first sweep of a cycle starts from x = 0: b, omega / diag read
+        # read, x written; the first sweep of a cycle starts from x = 0: b, omega / diag read, or,
+        # the first two in one, these and the face arrays
         "mg_smooth_f32_fine": 4 * (3 + f) + 4,
         "mg_smooth_f32_fine_first": 4 * 2 + 4,
+        "mg_smooth_f32_fine_two": 4 * (2 + f) + 4,
         "mg_smooth_f64_fine": 8 * (3 + f) + 8,
         "mg_smooth_f64_fine_first": 8 * 2 + 8,
+        "mg_smooth_f64_fine_two": 8 * (2 + f) + 8,
         # residual restriction from the finest level: b, x, diag and the face arrays of each
         # fine cell read, one coarse value per 8 fine cells written
         "mg_restrict_f32_fine": 4 * (3 + f) + 4 / 8,
@@ -152,7 +155,8 @@ def alg_bytes(nonsym):
 LINEAR_KERNELS = ("cg_matvec_dot", "cg_update_xr", "cg_update_p", "bicg_matvec",
                   "bicg_update_xr", "bicg_update_p", "bicg_update_s", "bicg_update_p_f32",
                   "bicg_update_s_f32", "mg_smooth_f32_fine",
-                  "mg_smooth_f32_fine_first", "mg_smooth_f64_fine", "mg_smooth_f64_fine_first",
+                  "mg_smooth_f32_fine_first", "mg_smooth_f32_fine_two", "mg_smooth_f64_fine",
+                  "mg_smooth_f64_fine_first", "mg_smooth_f64_fine_two",
                   "mg_restrict_f32_fine", "mg_restrict_f64_fine", "mg_prolong_f32_fine",
                   "mg_prolong_f64_fine", "mg_to_f32", "mg_from_f32", "mg_from_f32_dot")
 

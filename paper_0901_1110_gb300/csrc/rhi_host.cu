@@ -530,25 +530,27 @@ int vcycle(rhi_ctx* h, std::vector<Level<T>>& lv, size_t l, const Op<T>& A0,
         CK(L.mg_tail<T>(M));
         return RHI_OK;
     }
-    if (l + 1 == lv.size()) {
-        CK(L.smooth<T>(A, v.b, v.x, v.x, om, 1));
-        for (int s = 1; s < h->prm.mg_coarse_sweeps; ++s) {
+    // the level's sweeps from x = 0, result in v.x
+    const auto sweeps = [&](int n) {
+        int s = mg_first_sweeps<T>(v.N, n);
+        CK(L.smooth<T>(A, v.b, nullptr, v.x, om, s));
+        for (; s < n; ++s) {
             CK(L.smooth<T>(A, v.b, v.x, v.xt, om, 0));
             std::swap(v.x, v.xt);
         }
+        return (int)RHI_OK;
+    };
+    int rc;
+    if (l + 1 == lv.size()) {
+        if ((rc = sweeps(h->prm.mg_coarse_sweeps))) return rc;
         if constexpr (sizeof(T) == 4)
             if (out64) CK(L.from_f32(v.N, v.x, out64));
         return RHI_OK;
     }
-    CK(L.smooth<T>(A, v.b, v.x, v.x, om, 1));
-    for (int s = 1; s < h->prm.mg_pre; ++s) {
-        CK(L.smooth<T>(A, v.b, v.x, v.xt, om, 0));
-        std::swap(v.x, v.xt);
-    }
+    if ((rc = sweeps(h->prm.mg_pre))) return rc;
     Level<T>& c = lv[l + 1];
     CK(L.restrict_res<T>(A, v.b, v.x, c.nx, c.ny, c.nz, c.b));
-    int rc = vcycle<T>(h, lv, l + 1, A0, st, hook, skip);
-    if (rc) return rc;
+    if ((rc = vcycle<T>(h, lv, l + 1, A0, st, hook, skip))) return rc;
     // (a sweep that reads the coarse correction on the fly measured 3.6x slower than the
     // separate prolongation and sweep at 256^3, so the two stay separate)
     CK(L.prolong<T>(v.nx, v.ny, v.nz, c.nx, c.ny, c.x, v.x));
@@ -666,12 +668,18 @@ int precond_into(rhi_ctx* h, LinLaunch& L, const double* r, double* dest, bool v
         auto& lv = h->mg64;
         double* xt0 = lv[0].xt;
         lv[0].b = const_cast<double*>(r);
-        lv[0].x = dest;
+        // each sweep beyond the first launch swaps the two vectors: start so that the last is dest
+        int swaps = 0;
+        if (!tail_at(h, lv, 0)) {
+            const int down = lv.size() == 1 ? h->prm.mg_coarse_sweeps : h->prm.mg_pre;
+            swaps = down - mg_first_sweeps<double>(lv[0].N, down) + (lv.size() == 1 ? 0 : h->prm.mg_post);
+        }
+        lv[0].x = swaps & 1 ? xt0 : dest;
+        lv[0].xt = swaps & 1 ? dest : xt0;
         int rc = vcycle<double>(h, lv, 0, h->pc0, L.st, L.hook, L.skip, nullptr, up);
-        if (rc) return rc;
-        if (lv[0].x != dest) CK(L.copy(N, lv[0].x, dest));     // odd number of swaps
         lv[0].x = nullptr;
         lv[0].xt = xt0;
+        if (rc) return rc;
     } else {
         auto& lv = h->mg32;
         if (!cycle_rhs(h)) {

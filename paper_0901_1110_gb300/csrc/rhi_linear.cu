@@ -57,9 +57,17 @@ __device__ __forceinline__ void coords_fd(long long c, const FastDiv& fx, const 
     i = (int)(r - jj * fx.d);
 }
 
+// x after a cycle's first sweep, from x = 0, without that sweep's launch: omega / diag times b
+template <typename T>
+struct FirstSweep {
+    const T* __restrict__ wid;
+    const T* __restrict__ b;
+    __device__ __forceinline__ T operator[](long long c) const { return wid[c] * b[c]; }
+};
+
 // sum over the six neighbours of c of W_face x_neighbour (the off-diagonal part of row c)
-template <typename T, typename TX>
-__device__ __forceinline__ T off_row(const Op<T>& A, const TX* __restrict__ x, long long c,
+template <typename T, typename X>
+__device__ __forceinline__ T off_row(const Op<T>& A, const X& x, long long c,
                                      int i, int j, int k) {
     const long long sx = 1, sy = A.nx, sz = (long long)A.nx * A.ny;
     const int n[3] = {A.nx, A.ny, A.nz};
@@ -561,14 +569,6 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_bicg_xr(long long N, const double
     finish<true, RED_BICG_NEXT>(F, rr, rhr);
 }
 
-__global__ void __launch_bounds__(LIN_BLOCK) k_copy(long long N, const double* __restrict__ a,
-                                                    double* __restrict__ b, const double* skip) {
-    if (skipped(skip)) return;
-    for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
-         c += (long long)gridDim.x * LIN_BLOCK)
-        b[c] = a[c];
-}
-
 // ---------------------------------------------------------------------------------------------
 // multigrid kernels (templated on the level precision)
 
@@ -581,7 +581,9 @@ __device__ __forceinline__ void store_sweep(T* xout, double* out64, long long c,
 }
 
 // weighted Jacobi with wid = omega / diag: first sweep from x = 0: x_out = wid b; else
-// x_out = x_in + omega (b - A x_in) / diag, written as (1 - omega) x_in + wid (b + off)
+// x_out = x_in + omega (b - A x_in) / diag, written as (1 - omega) x_in + wid (b + off).  first: 0: a
+// sweep from x_in; 1: the first; 2: the first two in one pass, the first one's x made where it
+// is read (the same numbers; no launch and no trip to memory for it)
 template <typename T>
 __global__ void __launch_bounds__(LIN_BLOCK) k_mg_smooth(const Op<T> A, const T* __restrict__ b,
                                                          const T* __restrict__ xin,
@@ -591,13 +593,17 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_smooth(const Op<T> A, const T*
     for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < A.N;
          c += (long long)gridDim.x * LIN_BLOCK) {
         const T wi = A.wid[c];
-        if (first) {
+        if (first == 1) {
             xout[c] = wi * b[c];
+            continue;
+        }
+        int i, j, k;
+        coords3(A, c, i, j, k);
+        if (first == 2) {
+            const FirstSweep<T> x1{A.wid, b};
+            xout[c] = jacobi_update(x1[c], b[c], wi, off_row(A, x1, c, i, j, k), omega);
         } else {
-            int i, j, k;
-            coords3(A, c, i, j, k);
-            const T off = off_row(A, xin, c, i, j, k);
-            store_sweep(xout, out64, c, jacobi_update(xin[c], b[c], wi, off, omega));
+            store_sweep(xout, out64, c, jacobi_update(xin[c], b[c], wi, off_row(A, xin, c, i, j, k), omega));
         }
     }
 }
@@ -633,7 +639,7 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_smooth_first_vec(long long N,
 // per face), 0.91 of the HBM copy bandwidth against 0.61 for ZM = 8 (whose 104 loads do not fit
 // the register budget and were issued in dependent groups) and 0.78 for one cell per thread.
 constexpr int ZM = 2;
-template <typename T>
+template <typename T, bool TWO>
 __global__ void __launch_bounds__(LIN_BLOCK) k_mg_smooth_zm(const Op<T> A, const T* __restrict__ b,
                                                             const T* __restrict__ xin,
                                                             T* __restrict__ xout, T omega,
@@ -662,6 +668,7 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_smooth_zm(const Op<T> A, const
     const T* __restrict__ P1 = A.Wp[1];
     const T* __restrict__ P2 = A.Wp[2];
     const T* __restrict__ wd = A.wid;
+    const auto X = [&](long long c) { return TWO ? __ldg(wd + c) * __ldg(b + c) : __ldg(xin + c); };
     // z: plane below k0 (the far side when k0 = 0: W = 0 there unless periodic).  All loads of
     // the ZM planes are issued first (registers), then the planes are computed in order;
     // the launcher uses this kernel only when ZM divides nz.
@@ -671,25 +678,26 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_smooth_zm(const Op<T> A, const
     // the plane above (Wp of the face above; the same numbers as wz[kk + 1] when symmetric)
     T xz[ZM + 2], wz[ZM], pz[ZM], w0l[ZM], w0h[ZM], w1l[ZM], w1h[ZM], x0l[ZM], x0h[ZM], x1l[ZM],
         x1h[ZM], dd[ZM], bb[ZM];
-    xz[0] = __ldg(xin + (k0 > 0 ? c0 - nxy : col + (long long)(nz - 1) * nxy));
-    xz[ZM + 1] = __ldg(xin + ctop);
+    xz[0] = X(k0 > 0 ? c0 - nxy : col + (long long)(nz - 1) * nxy);
+    xz[ZM + 1] = X(ctop);
 #pragma unroll
     for (int kk = 0; kk < ZM; ++kk) {
         const long long c = c0 + (long long)kk * nxy;
         const long long cu = kk + 1 < ZM ? c + nxy : ctop;
-        xz[kk + 1] = __ldg(xin + c);
+        if (!TWO) xz[kk + 1] = __ldg(xin + c);
         wz[kk] = __ldg(W2 + c);
         pz[kk] = __ldg(P2 + cu);
         w0l[kk] = __ldg(W0 + c);
-        x0l[kk] = __ldg(xin + c + dlo0);
+        x0l[kk] = X(c + dlo0);
         w0h[kk] = hhi0 ? __ldg(P0 + c + dhi0) : T(0);
-        x0h[kk] = hhi0 ? __ldg(xin + c + dhi0) : T(0);
+        x0h[kk] = hhi0 ? X(c + dhi0) : T(0);
         w1l[kk] = __ldg(W1 + c);
-        x1l[kk] = __ldg(xin + c + dlo1);
+        x1l[kk] = X(c + dlo1);
         w1h[kk] = hhi1 ? __ldg(P1 + c + dhi1) : T(0);
-        x1h[kk] = hhi1 ? __ldg(xin + c + dhi1) : T(0);
+        x1h[kk] = hhi1 ? X(c + dhi1) : T(0);
         dd[kk] = __ldg(wd + c);
         bb[kk] = __ldg(b + c);
+        if (TWO) xz[kk + 1] = dd[kk] * bb[kk];
     }
 #pragma unroll
     for (int kk = 0; kk < ZM; ++kk) {
@@ -709,7 +717,8 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_smooth_zm(const Op<T> A, const
 // CTA owns one grid row (j) of every plane of a z-slab of ZB planes, one thread per x cell.
 // For each plane it needs 12 contiguous rows of nx floats: x at (j, k), (j-1, k), (j+1, k),
 // (j, k+1); b, omega / diag and the lower-face couplings W0, W1, W2 and P0 at (j, k); P1 at
-// (j+1, k); P2 at (j, k+1).  One elected thread issues them as cp.async.bulk copies into a
+// (j+1, k); P2 at (j, k+1).  For the first two sweeps in one (TWO) it is 14: b and omega / diag take
+// the place of x.  One elected thread issues them as cp.async.bulk copies into a
 // ring of BS stages, each completing on its stage's mbarrier; the CTA computes plane k from
 // shared memory while the copies of the next planes are in flight.  Rows whose neighbour
 // does not exist (zero-flux faces) are fetched from a valid row and not used, as in
@@ -718,7 +727,7 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_smooth_zm(const Op<T> A, const
 // arrays, nz a multiple of ZB.  Each wait on a stage is bounded: after BULK_SPIN tries the
 // kernel records the plane in *err, waits (bounded) for its own copies once more, and
 // returns.
-constexpr int BULK_ROWS = 12;
+constexpr int BULK_ROWS = 12, BULK_ROWS_TWO = 14;
 constexpr int BULK_STAGES = 3;
 constexpr int BULK_ZB = 16;
 constexpr int BULK_MAX_NX = 512;
@@ -763,6 +772,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
     return false;
 }
 
+template <bool TWO>
 __global__ void __launch_bounds__(BULK_MAX_NX) k_mg_smooth_bulk(const Op<float> A,
                                                                 const float* __restrict__ b,
                                                                 const float* __restrict__ xin,
@@ -770,7 +780,8 @@ __global__ void __launch_bounds__(BULK_MAX_NX) k_mg_smooth_bulk(const Op<float> 
                                                                 float omega, int* err,
                                                                 double* __restrict__ out64) {
     if (skipped(A.skip)) return;
-    extern __shared__ __align__(128) float rows[];          // [BULK_STAGES][BULK_ROWS][nx]
+    constexpr int ROWS = TWO ? BULK_ROWS_TWO : BULK_ROWS;
+    extern __shared__ __align__(128) float rows[];          // [BULK_STAGES][ROWS][nx]
     __shared__ __align__(8) unsigned long long bar[BULK_STAGES];
     const int nx = A.nx, ny = A.ny, nz = A.nz;
     const int i = threadIdx.x;
@@ -782,7 +793,7 @@ __global__ void __launch_bounds__(BULK_MAX_NX) k_mg_smooth_bulk(const Op<float> 
     const bool hhi0 = i < nx - 1 || A.per[0];
     const bool hhi1 = j < ny - 1 || A.per[1];
     const unsigned row_bytes = (unsigned)nx * 4u;
-    auto stage_row = [&](int st, int r) { return rows + ((long long)st * BULK_ROWS + r) * nx; };
+    auto stage_row = [&](int st, int r) { return rows + ((long long)st * ROWS + r) * nx; };
     // the copies of plane k into stage st (one elected thread)
     auto issue = [&](int k, int st) {
         const int ku = k + 1 < nz ? k + 1 : 0;
@@ -790,12 +801,19 @@ __global__ void __launch_bounds__(BULK_MAX_NX) k_mg_smooth_bulk(const Op<float> 
         const long long cm = (long long)jm * nx + (long long)k * nxy;
         const long long cp = (long long)jp * nx + (long long)k * nxy;
         const long long cu = (long long)j * nx + (long long)ku * nxy;
-        const float* src[BULK_ROWS] = {xin + c, xin + cm, xin + cp, xin + cu, b + c, A.wid + c,
-                                       A.W[0] + c, A.W[1] + c, A.W[2] + c, A.Wp[0] + c,
-                                       A.Wp[1] + cp, A.Wp[2] + cu};
-        mbar_expect_tx(&bar[st], row_bytes * BULK_ROWS);
+        const float* const x = TWO ? b : xin;
+        const float* src[ROWS] = {x + c, x + cm, x + cp, x + cu, A.W[0] + c, A.W[1] + c, A.W[2] + c,
+                                  A.Wp[0] + c, A.Wp[1] + cp, A.Wp[2] + cu, A.wid + c};
+        if constexpr (TWO) {
+            src[11] = A.wid + cm;
+            src[12] = A.wid + cp;
+            src[13] = A.wid + cu;
+        } else {
+            src[11] = b + c;
+        }
+        mbar_expect_tx(&bar[st], row_bytes * ROWS);
 #pragma unroll
-        for (int r = 0; r < BULK_ROWS; ++r) bulk_g2s(stage_row(st, r), src[r], row_bytes, &bar[st]);
+        for (int r = 0; r < ROWS; ++r) bulk_g2s(stage_row(st, r), src[r], row_bytes, &bar[st]);
     };
     if (i == 0) {
 #pragma unroll
@@ -809,8 +827,11 @@ __global__ void __launch_bounds__(BULK_MAX_NX) k_mg_smooth_bulk(const Op<float> 
             if (st < BULK_ZB) issue(k0 + st, st);
     }
     // x of the plane below the first one (the far side when k0 = 0: W = 0 there unless periodic)
-    float xlo = i < nx ? __ldg(xin + (long long)j * nx + (long long)(k0 > 0 ? k0 - 1 : nz - 1) * nxy + i)
-                       : 0.f;
+    float xlo = 0.f;
+    if (i < nx) {
+        const long long c = (long long)j * nx + (long long)(k0 > 0 ? k0 - 1 : nz - 1) * nxy + i;
+        xlo = TWO ? __ldg(A.wid + c) * __ldg(b + c) : __ldg(xin + c);
+    }
     bool ok = true;
     for (int kk = 0; kk < BULK_ZB; ++kk) {
         const int st = kk % BULK_STAGES;
@@ -819,29 +840,32 @@ __global__ void __launch_bounds__(BULK_MAX_NX) k_mg_smooth_bulk(const Op<float> 
         const int k = k0 + kk;
         float xcen = 0.f;
         if (i < nx) {
-            const float* XC = stage_row(st, 0);
+            const float* XC = stage_row(st, 0);                 // (TWO: b, to be multiplied by wid)
             const float* XM = stage_row(st, 1);
             const float* XP = stage_row(st, 2);
             const float* XU = stage_row(st, 3);
-            const float* BB = stage_row(st, 4);
-            const float* WD = stage_row(st, 5);
-            const float* R0 = stage_row(st, 6);
-            const float* R1 = stage_row(st, 7);
-            const float* R2 = stage_row(st, 8);
-            const float* Q0 = stage_row(st, 9);
-            const float* Q1 = stage_row(st, 10);
-            const float* Q2 = stage_row(st, 11);
+            const float* R0 = stage_row(st, 4);
+            const float* R1 = stage_row(st, 5);
+            const float* R2 = stage_row(st, 6);
+            const float* Q0 = stage_row(st, 7);
+            const float* Q1 = stage_row(st, 8);
+            const float* Q2 = stage_row(st, 9);
+            const float* WD = stage_row(st, 10);
+            const float* BB = TWO ? XC : stage_row(st, 11);
+            const auto x = [&](const float* row, int w, int at) {   // w: its row of wid
+                return TWO ? stage_row(st, w)[at] * row[at] : row[at];
+            };
             const int il = i > 0 ? i - 1 : nx - 1;
             const int ih = i < nx - 1 ? i + 1 : 0;
             const bool hz = k < nz - 1 || A.per[2];
-            xcen = XC[i];
+            xcen = x(XC, 10, i);
             float off = 0.f;
-            off += R0[i] * XC[il];
-            if (hhi0) off += Q0[ih] * XC[ih];
-            off += R1[i] * XM[i];
-            if (hhi1) off += Q1[i] * XP[i];
+            off += R0[i] * x(XC, 10, il);
+            if (hhi0) off += Q0[ih] * x(XC, 10, ih);
+            off += R1[i] * x(XM, 11, i);
+            if (hhi1) off += Q1[i] * x(XP, 12, i);
             off += R2[i] * xlo;
-            if (hz) off += Q2[i] * XU[i];
+            if (hz) off += Q2[i] * x(XU, 13, i);
             store_sweep(xout, out64, (long long)j * nx + (long long)k * nxy + i,
                         jacobi_update(xcen, BB[i], WD[i], off, omega));
         }
@@ -858,8 +882,11 @@ __global__ void __launch_bounds__(BULK_MAX_NX) k_mg_smooth_bulk(const Op<float> 
 
 cudaError_t linear_kernels_init() {
     if (g_bulk_err_ptr) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_mg_smooth_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_mg_smooth_bulk<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          BULK_STAGES * BULK_ROWS * BULK_MAX_NX * (int)sizeof(float));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_mg_smooth_bulk<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 BULK_STAGES * BULK_ROWS_TWO * BULK_MAX_NX * (int)sizeof(float));
     void* p = nullptr;
     if (e == cudaSuccess) e = cudaGetSymbolAddress(&p, g_bulk_wait_error);
     if (e == cudaSuccess) g_bulk_err_ptr = static_cast<int*>(p);
@@ -1248,11 +1275,6 @@ cudaError_t LinLaunch::reduce(const double* part, int n, double* scal, int op, i
     k_reduce<<<1, RED_BLOCK, 0, st>>>(part, n, scal, op, slot);
     return end();
 }
-cudaError_t LinLaunch::copy(long long N, const double* a, double* b) {
-    begin("copy");
-    k_copy<<<stream_blocks(N), LIN_BLOCK, 0, st>>>(N, a, b, skip);
-    return end();
-}
 
 cudaError_t LinLaunch::matvec_ns(const OpNS& A, const double* x, double* y, const double* w1,
                                  int two_dots, const Finish& F) {
@@ -1300,7 +1322,8 @@ cudaError_t LinLaunch::smooth(const Op<T>& A, const T* b, const T* xin, T* xout,
                               int first, double* out64) {
     // the finest level's sweeps get their own names (the first sweep of a cycle, from x = 0,
     // reads only b and omega / diag)
-    if (A.N == fine_N && first) begin(sizeof(T) == 4 ? "mg_smooth_f32_fine_first" : "mg_smooth_f64_fine_first");
+    if (A.N == fine_N && first == 2) begin(sizeof(T) == 4 ? "mg_smooth_f32_fine_two" : "mg_smooth_f64_fine_two");
+    else if (A.N == fine_N && first) begin(sizeof(T) == 4 ? "mg_smooth_f32_fine_first" : "mg_smooth_f64_fine_first");
     else if (A.N == fine_N) begin(sizeof(T) == 4 ? "mg_smooth_f32_fine" : "mg_smooth_f64_fine");
     else begin(sizeof(T) == 4 ? "mg_smooth_f32" : "mg_smooth_f64");
     const long long nxy = (long long)A.nx * A.ny;
@@ -1313,24 +1336,26 @@ cudaError_t LinLaunch::smooth(const Op<T>& A, const T* b, const T* xin, T* xout,
     // 256^3, even at 192^3, and slower on rows of 128 whose level fits in L2)
     bool bulk_ok = false;
     if constexpr (sizeof(T) == 4) {
-        bulk_ok = !first && xin != xout && g_bulk_err_ptr && A.nx % 4 == 0 && A.nx >= 256 &&
-                  A.nx <= BULK_MAX_NX && A.nz % BULK_ZB == 0 && al16(xin) && al16(b) &&
+        bulk_ok = first != 1 && xin != xout && g_bulk_err_ptr && A.nx % 4 == 0 && A.nx >= 256 &&
+                  A.nx <= BULK_MAX_NX && A.nz % BULK_ZB == 0 && (first || al16(xin)) && al16(b) &&
                   al16(A.wid) && al16(A.W[0]) && al16(A.W[1]) && al16(A.W[2]) &&
                   al16(A.Wp[0]) && al16(A.Wp[1]) && al16(A.Wp[2]);
     }
-    if (first && (A.N * (long long)sizeof(T)) % 16 == 0 && al16(A.wid) && al16(b) && al16(xout)) {
+    if (first == 1 && (A.N * (long long)sizeof(T)) % 16 == 0 && al16(A.wid) && al16(b) && al16(xout)) {
         k_mg_smooth_first_vec<T><<<stream_blocks(A.N * (long long)sizeof(T) / 16), LIN_BLOCK, 0, st>>>(
             A.N, A.wid, b, xout, skip);
     } else if (bulk_ok) {
         if constexpr (sizeof(T) == 4) {
-            const size_t smem = (size_t)BULK_STAGES * BULK_ROWS * A.nx * sizeof(float);
-            k_mg_smooth_bulk<<<dim3((unsigned)A.ny, (unsigned)(A.nz / BULK_ZB)),
-                               (unsigned)((A.nx + 31) / 32 * 32), smem, st>>>(
-                B, b, xin, xout, omega, g_bulk_err_ptr, out64);
+            const size_t smem = (size_t)BULK_STAGES * (first ? BULK_ROWS_TWO : BULK_ROWS) * A.nx * sizeof(float);
+            const dim3 g((unsigned)A.ny, (unsigned)(A.nz / BULK_ZB));
+            const unsigned nt = (unsigned)((A.nx + 31) / 32 * 32);
+            if (first) k_mg_smooth_bulk<true><<<g, nt, smem, st>>>(B, b, xin, xout, omega, g_bulk_err_ptr, out64);
+            else k_mg_smooth_bulk<false><<<g, nt, smem, st>>>(B, b, xin, xout, omega, g_bulk_err_ptr, out64);
         }
-    } else if (sizeof(T) == 4 && !first && A.nz % ZM == 0 && nxy >= 4 * LIN_BLOCK && xin != xout) {
+    } else if (sizeof(T) == 4 && first != 1 && A.nz % ZM == 0 && nxy >= 4 * LIN_BLOCK && xin != xout) {
         const dim3 g((unsigned)((nxy + LIN_BLOCK - 1) / LIN_BLOCK), (unsigned)((A.nz + ZM - 1) / ZM));
-        k_mg_smooth_zm<T><<<g, LIN_BLOCK, 0, st>>>(B, b, xin, xout, omega, out64);
+        if (first) k_mg_smooth_zm<T, true><<<g, LIN_BLOCK, 0, st>>>(B, b, xin, xout, omega, out64);
+        else k_mg_smooth_zm<T, false><<<g, LIN_BLOCK, 0, st>>>(B, b, xin, xout, omega, out64);
     } else {
         k_mg_smooth<T><<<stream_blocks(A.N), LIN_BLOCK, 0, st>>>(B, b, xin, xout, omega, first, out64);
     }

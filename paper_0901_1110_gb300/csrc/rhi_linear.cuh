@@ -75,6 +75,15 @@ struct MgTail {
 };
 cudaError_t mg_tail_init(int* blocks32, int* blocks64);
 cudaError_t mg_build_init();
+// A cycle's first two sweeps of a level of N cells as one kernel, which multiplies omega / diag by b where
+// the second sweep reads x: one launch and, in memory, the first sweep's x less.  Measured, FP32: 256^3
+// 131 -> 99 us, 128^3 24.4 -> 22.1 us, 64^3 about 12.5 -> 7.5 us.  FP64 pays its seven
+// multiplications on the FP64 pipe: 32^3 13.1 -> 7.6 us, 64^3 5 us less, but 128^3 51 -> 64 us.
+// Returns how many of n sweeps the first launch makes.
+template <typename T>
+constexpr int mg_first_sweeps(long long N, int n) {
+    return n >= 2 && (sizeof(T) == 4 || N <= 1LL << 18) ? 2 : 1;
+}
 
 // device scalar slots of the Krylov iterations.  The BiCGStab and CG loops keep their control state
 // on the device: S_THR (converged when r.r <= S_THR), S_MAXIT, the iteration count S_ITS, S_DONE
@@ -162,7 +171,6 @@ struct LinLaunch {
     cudaError_t bicg_xr(long long N, const double* scal, double* x, const double* ph,
                         const double* sh, const double* s, const double* t, double* r, const double* rh,
                         const Finish& F);
-    cudaError_t copy(long long N, const double* a, double* b);
     cudaError_t from_f32(long long N, const float* x, double* z);
 
     // out64 (not for the first sweep): the result goes there in FP64 instead of to xout
