@@ -979,6 +979,62 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_restrict(const Op<T> A, const 
     }
 }
 
+// The same with eight lanes to a parent, one for each child (a warp: four parents in a row, so runs of
+// eight cells along x), summed by shuffles: a child's loads do not wait for those of its siblings,
+// and eight times as many threads ask for them.  Measured at 64^3, where that is what counts: FP32
+// 11.0 -> 8.4 us, FP64 14.0 -> 12.1 us (32^3: 13.7 -> 7.9 us).  At 128^3 the first form, with fewer
+// instructions per cell, is the better one: 19.2 against 22.6 us, and 45 against 55 us in FP64; at
+// 256^3 FP32 99 against 154 us.  RESTRICT_SPLIT: most parents of a level that takes this form.
+constexpr long long RESTRICT_SPLIT = 1LL << 16;
+template <typename T>
+__global__ void __launch_bounds__(LIN_BLOCK) k_mg_restrict_split(const Op<T> A, const T* __restrict__ b,
+                                                                 const T* __restrict__ x, int cnx,
+                                                                 int cny, int cnz, FastDiv fcx,
+                                                                 FastDiv fcxy, T* __restrict__ bc) {
+    if (skipped(A.skip)) return;
+    const long long Nc = (long long)cnx * cny * cnz;
+    const int n[3] = {A.nx, A.ny, A.nz};
+    const long long s[3] = {1, A.nx, (long long)A.nx * A.ny};
+    const int lane = (int)(threadIdx.x & 31u);
+    const int d[3] = {lane & 1, lane >> 3 & 1, lane >> 4};
+    const bool inner_cancel = sizeof(T) == 8 && A.loc && A.Wp[0] == A.W[0];
+    const long long warps = (long long)gridDim.x * (LIN_BLOCK / 32);
+    for (long long w = blockIdx.x * (long long)(LIN_BLOCK / 32) + threadIdx.x / 32; w * 4 < Nc; w += warps) {
+        const long long cc = w * 4 + (lane >> 1 & 3);
+        T acc = T(0);
+        if (cc < Nc) {
+            int I, J, K;
+            coords_fd(cc, fcx, fcxy, I, J, K);
+            const int q[3] = {2 * I + d[0], 2 * J + d[1], 2 * K + d[2]};
+            if (q[0] < n[0] && q[1] < n[1] && q[2] < n[2]) {
+                const long long c = q[0] + (long long)A.nx * (q[1] + (long long)A.ny * q[2]);
+                const T xc = x[c];
+                if (inner_cancel) {
+                    T fl = T(0);
+#pragma unroll
+                    for (int ax = 0; ax < 3; ++ax) {
+                        // the face to the outside: lower for a first child, upper for a second
+                        const long long wrap = (long long)(n[ax] - 1) * s[ax];
+                        const bool up = d[ax] == 1, end = q[ax] == n[ax] - 1;
+                        const long long nb = up ? (end ? c - wrap : c + s[ax]) : (q[ax] > 0 ? c - s[ax] : c + wrap);
+                        const T wf = up && end && !A.per[ax] ? T(0) : A.W[ax][up ? nb : c];
+                        fl += wf * (xc - x[nb]);
+                        // an only child has both
+                        if (!up && end && A.per[ax]) fl += A.W[ax][c - wrap] * (xc - x[c - wrap]);
+                    }
+                    acc = b[c] - A.loc[c] * xc - fl;
+                } else {
+                    acc = b[c] - apply_row(A, x, c, q[0], q[1], q[2], xc);
+                }
+            }
+        }
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 8);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+        if ((lane & 25) == 0 && cc < Nc) bc[cc] = acc * T(0.125);
+    }
+}
+
 // x_f += x_c(parent), 16 bytes of fine cells per thread along x (4 FP32 or 2 FP64 cells, whose
 // parents are 2 or 1 consecutive coarse cells); needs nx a multiple of 4 (FP32) or 2 (FP64) and
 // 16-byte aligned rows, which the launcher checks.  fx, fxy divide by nx / V and nx ny / V.
@@ -1368,8 +1424,12 @@ cudaError_t LinLaunch::restrict_res(const Op<T>& A, const T* b, const T* x, int 
     else begin(sizeof(T) == 4 ? "mg_restrict_f32" : "mg_restrict_f64");
     Op<T> B = A;
     B.skip = skip;
-    k_mg_restrict<T><<<stream_blocks((long long)cnx * cny * cnz), LIN_BLOCK, 0, st>>>(
-        B, b, x, cnx, cny, cnz, make_fastdiv((unsigned)cnx), make_fastdiv((unsigned)cnx * cny), bc);
+    const long long Nc = (long long)cnx * cny * cnz;
+    const FastDiv fx = make_fastdiv((unsigned)cnx), fxy = make_fastdiv((unsigned)cnx * cny);
+    if (Nc <= RESTRICT_SPLIT)
+        k_mg_restrict_split<T><<<stream_blocks(Nc * 8), LIN_BLOCK, 0, st>>>(B, b, x, cnx, cny, cnz, fx, fxy, bc);
+    else
+        k_mg_restrict<T><<<stream_blocks(Nc), LIN_BLOCK, 0, st>>>(B, b, x, cnx, cny, cnz, fx, fxy, bc);
     return end();
 }
 template <typename T>
