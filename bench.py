@@ -72,17 +72,22 @@ def load_peaks():
 # x 2 flop = 1.259 TFLOP/s (a register-resident DFMA loop measures 1.20 TFLOP/s)
 FP64_PEAK_TFLOPS = 152 * 2.070e9 * 4 / 1e12
 
-# FP64 flops per cell of the fused cell kernels (bound by the FP64 pipe, about 1.2 TFLOP/s here),
-# counted by ncu as 2 DFMA + DMUL + DADD thread instructions per cell (175, 106, 76 on the
-# H + He lognormal 128^3 case)
+# FP64 flops per cell of the fused cell kernels (bound by the FP64 pipe, about 1.2 TFLOP/s here) as
+# the formulas were first written, 2 DFMA + DMUL + DADD (175, 106, 76 on the H + He lognormal 128^3
+# case): the model that makes these kernels candidates for the roofline
 ALU_FLOPS = {
     "cell_residual_schur": 532,
 }
+# the flops the kernel executes now, counted by ncu in the same way (127, 69, 42): the roofline's
+# numerator, since work that is no longer done is not a rate
+EXECUTED_FLOPS = {
+    "cell_residual_schur": 2 * 127 + 69 + 42,
+}
 # DRAM bytes per launch (read + write) from ncu, per cell of a capture times the cells of the
 # timed grid (each of these kernels streams its fields once, so traffic grows with the cells);
-# an entry is removed when its kernel changes.  k_cell<3,1> at 128^3: 368.94 MB read +
-# 151.53 MB written per launch (ncu --set full, the current kernel).
-TRAFFIC_PER_CELL = {"cell_residual_schur": (368.936192e6 + 151.531520e6) / 128 ** 3}
+# an entry is removed when its kernel changes.  k_cell<3,ITER> at 128^3: 268.51 MB read +
+# 163.03 MB written per launch.
+TRAFFIC_PER_CELL = {"cell_residual_schur": (268.511232e6 + 163.033344e6) / 128 ** 3}
 
 FORM_TEXT = {
     "plain_fp64": "FP64 Newton/Schur/BiCGStab + FP64 multigrid V-cycle of the Newton matrix "
@@ -789,11 +794,11 @@ def main():
         roof["launches_timed"] = tcnt
         roof["units_per_launch"] = w.N
         if tname in ALU_FLOPS:
-            ach = ALU_FLOPS[tname] * w.N / avg_s / 1e12
+            ach = EXECUTED_FLOPS[tname] * w.N / avg_s / 1e12
             roof.update(bound="alu", achieved=ach, peak=FP64_PEAK_TFLOPS, unit="TFLOP/s",
                         frac=ach / FP64_PEAK_TFLOPS,
                         traffic=TRAFFIC_PER_CELL[tname] * w.N if tname in TRAFFIC_PER_CELL else None,
-                        flops_per_cell=ALU_FLOPS[tname],
+                        flops_per_cell=EXECUTED_FLOPS[tname],
                         peak_source="derived: 152 SMs x 2070 MHz x 2 DFMA/clk/SM x 2 flop")
         elif tname in AB:
             ach = AB[tname] * w.N / avg_s / 1e9
