@@ -54,12 +54,14 @@ __device__ __forceinline__ void cell_features(const MlpArgs& A, long long c, flo
     f[8] = log10_clamped(A.dt * 1e-12);
     if (A.E_p) {
         // the previous step's change: ratios in FP64, the logit difference in FP64 (neutral
-        // cells sit within 1e-16 of x_HI = 1), rounded to FP32
+        // cells sit within 1e-16 of x_HI = 1), rounded to FP32.  One logarithm of the quotient (at most
+        // 1e46 either way) instead of four: an FP64 logarithm is some 30 instructions of the FP64
+        // pipe, which bounds this kernel, and the sum of four rounded worse (2e-14 against 7e-15)
         f[9] = log10_clamped(E / A.E_p[c]);
         f[10] = log10_clamped(e / A.e_p[c]);
         const double x1 = fmin(fmax(A.n[c] * inH, 1e-30), 1.0 - 1e-16);
         const double x0 = fmin(fmax(A.n_p[c] * inH, 1e-30), 1.0 - 1e-16);
-        f[11] = (float)((log(x1) - log1p(-x1)) - (log(x0) - log1p(-x0)));
+        f[11] = (float)log((x1 * (1.0 - x0)) / ((1.0 - x1) * x0));
         f[12] = A.ldt_ratio;
     } else {
         f[9] = f[10] = f[11] = f[12] = 0.0f;
@@ -248,7 +250,7 @@ __global__ void __launch_bounds__(32 * INF_WARPS) k_mlp_infer(const MlpArgs A,
                 const double E0 = A.E[c], e0 = A.e[c], nH = A.nH[c];
                 const double x0 = fmin(fmax(A.n[c] / nH, 1e-30), 1.0 - 1e-16);
                 float change = fmaxf(fabsf(o[0]), fabsf(o[1]));
-                change = fmaxf(change, fabsf(o[2] - (float)(log(x0) - log1p(-x0))));
+                change = fmaxf(change, fabsf(o[2] - (float)log(x0 / (1.0 - x0))));
                 const double xHI = 1.0 / (1.0 + (double)expf(-o[2]));
                 double nHeI = 0.0, nHeII = 0.0;
                 if (A.ns == 3) {
