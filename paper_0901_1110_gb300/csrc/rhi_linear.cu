@@ -1397,6 +1397,7 @@ cudaError_t LinLaunch::smooth(const Op<T>& A, const T* b, const T* xin, T* xout,
                   al16(A.wid) && al16(A.W[0]) && al16(A.W[1]) && al16(A.W[2]) &&
                   al16(A.Wp[0]) && al16(A.Wp[1]) && al16(A.Wp[2]);
     }
+    const bool zm_ok = sizeof(T) == 4 && first != 1 && A.nz % ZM == 0 && nxy >= 4 * LIN_BLOCK && xin != xout;
     if (first == 1 && (A.N * (long long)sizeof(T)) % 16 == 0 && al16(A.wid) && al16(b) && al16(xout)) {
         k_mg_smooth_first_vec<T><<<stream_blocks(A.N * (long long)sizeof(T) / 16), LIN_BLOCK, 0, st>>>(
             A.N, A.wid, b, xout, skip);
@@ -1408,10 +1409,12 @@ cudaError_t LinLaunch::smooth(const Op<T>& A, const T* b, const T* xin, T* xout,
             if (first) k_mg_smooth_bulk<true><<<g, nt, smem, st>>>(B, b, xin, xout, omega, g_bulk_err_ptr, out64);
             else k_mg_smooth_bulk<false><<<g, nt, smem, st>>>(B, b, xin, xout, omega, g_bulk_err_ptr, out64);
         }
-    } else if (sizeof(T) == 4 && first != 1 && A.nz % ZM == 0 && nxy >= 4 * LIN_BLOCK && xin != xout) {
-        const dim3 g((unsigned)((nxy + LIN_BLOCK - 1) / LIN_BLOCK), (unsigned)((A.nz + ZM - 1) / ZM));
-        if (first) k_mg_smooth_zm<T, true><<<g, LIN_BLOCK, 0, st>>>(B, b, xin, xout, omega, out64);
-        else k_mg_smooth_zm<T, false><<<g, LIN_BLOCK, 0, st>>>(B, b, xin, xout, omega, out64);
+    } else if (zm_ok) {
+        if constexpr (sizeof(T) == 4) {
+            const dim3 g((unsigned)((nxy + LIN_BLOCK - 1) / LIN_BLOCK), (unsigned)(A.nz / ZM));
+            if (first) k_mg_smooth_zm<T, true><<<g, LIN_BLOCK, 0, st>>>(B, b, xin, xout, omega, out64);
+            else k_mg_smooth_zm<T, false><<<g, LIN_BLOCK, 0, st>>>(B, b, xin, xout, omega, out64);
+        }
     } else {
         k_mg_smooth<T><<<stream_blocks(A.N), LIN_BLOCK, 0, st>>>(B, b, xin, xout, omega, first, out64);
     }

@@ -21,6 +21,9 @@
 // latency: about 0.4 us for a cluster barrier, and in FP64 64 cycles for each instruction of a warp.
 // Larger levels stay with the level kernels, which use all SMs: at 64^3 FP32 a sweep moves 10 MB.
 //
+// Where the whole cycle is one such launch, BiCGStab's p is updated as it is read (given): a launch and
+// the gap before it less per iteration, 37.3 -> 36.7 ms for 377 iterations on 32^3.
+//
 // The arithmetic of a sweep, the residual, the restriction (sum of the children's residuals / 8) and
 // the injection is that of the level kernels in rhi_linear.cu.  Sweeps alternate between the two
 // buffers with a barrier between, so no buffer is written while it is read.
