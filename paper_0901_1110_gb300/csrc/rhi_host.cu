@@ -845,7 +845,7 @@ int krylov_outcome(rhi_ctx* h, bool cg, int* its_out) {
     h->prof.launches += its * h->kg_body_kernels;
     h->kg_body_kernels = 0;
     if (cg) {
-        if (h->prm.precond != RHI_PRECOND_JACOBI) h->stats.vcycles += its;
+        h->stats.vcycles += its;                // one preconditioner application each, Jacobi's too
         if (h->h_scal[S_BREAK] != 0.0)
             return fail(h, RHI_ERR_NONPHYSICAL, "CG breakdown: p.Sp <= 0 or non-finite residual");
         return RHI_OK;
