@@ -12,6 +12,7 @@
 // Inference runs on the tensor cores (mma.sync m16n8k16, BF16 operands, FP32 accumulation)
 // with the layer activations chained in registers; training runs FP32 on the CUDA cores, tiles of
 // 32 samples per block, with a deterministic gradient reduction and Adam.
+#include <cfloat>
 #include <cmath>
 #include <cstddef>
 
@@ -122,17 +123,19 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 
 // z / (1 + exp(-z)).  Two special-function results each (192 a row bound the forward pass); FAST: the
 // quotient from the reciprocal approximation and one residual correction, q + (z - q d) r, which rounds as
-// the IEEE division does but for a last bit now and then, in 5 instructions instead of a division's 15
-// or so.  (The denominator's bound keeps a zero times infinity out of the correction.)  The guess keeps the
-// division: its FP64 results are held to the bit, and its time is its FP64 logarithms'.
+// the IEEE division does but for a last bit now and then, in 7 instructions instead of a division's 15
+// or so.  The correction alone takes q and d held finite: where exp(-z) overflows r is 0 and the
+// result the division's -0, and z = inf gives inf (a bound on the d that r comes from would leave
+// z / 3e38 there, -0.1 for z = -3e38).  The guess keeps the division: its FP64 results are held to the
+// bit, and its time is its FP64 logarithms'.
 template <bool FAST>
 __device__ __forceinline__ float silu_f(float z) {
     if constexpr (!FAST) return z / (1.0f + __expf(-z));
-    const float d = fminf(1.0f + __expf(-z), 3e38f);
+    const float d = 1.0f + __expf(-z);
     float r;
     asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(d));
     const float q = z * r;
-    return fmaf(fmaf(-q, d, z), r, q);
+    return fmaf(fmaf(-fminf(q, FLT_MAX), fminf(d, FLT_MAX), z), r, q);
 }
 
 // one hidden layer on a 16-row tile: in = A fragments over KS k-steps, out = 8 n-tiles
