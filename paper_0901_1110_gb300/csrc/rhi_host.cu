@@ -125,10 +125,8 @@ struct rhi_ctx {
     // Schur sets: the diagonal (limiter_jacobian 0) or its local part, right-hand side, opacity
     // responses (exact matrix), elimination
     double *rho[2] = {nullptr, nullptr}, *phi[2] = {nullptr, nullptr};
-    // the assembled Newton matrix and right-hand side of the current system (dD/dE kept), and the
-    // lagged-D matrix's W and diagonal where such a solver needs them (allocated on first use)
+    // the assembled Newton matrix and right-hand side of the current system (dD/dE kept)
     double *sysPQ = nullptr, *sysdiag = nullptr, *sysrhs = nullptr;
-    double *lagW = nullptr, *lagdiag = nullptr;
     double *diag[2] = {nullptr, nullptr}, *rhs[2] = {nullptr, nullptr};
     double *fMt[2] = {nullptr, nullptr}, *MiU[2] = {nullptr, nullptr};
     double* f_tmp = nullptr;
@@ -977,18 +975,19 @@ void set_op0(rhi_ctx* h, const double* W, const double* diag) {
     A.diag = diag;
 }
 
-// the lagged-D matrix of an iterate of a solver that keeps dD/dE
-int lagged_system(rhi_ctx* h, const StepParams& P, const double* E, const double* kap, int set) {
-    int rc;
-    if (!h->lagW && (rc = dalloc(h, &h->lagW, 3 * (size_t)h->N))) return rc;
-    if (!h->lagdiag && (rc = dalloc(h, &h->lagdiag, (size_t)h->N))) return rc;
+// The lagged-D matrix of an iterate of a solver that keeps dD/dE (Schur set `set`, at E and kap): W and the
+// diagonal in PQ[0], which nothing reads from the assembly of a system until the next trial's faces
+// (a trial that wrote its own there before a breakdown showed is evaluated again after the fallback).
+// Always the same buffer: the captured BiCGStab graph holds the preconditioner's pointers.
+int lagged_system(rhi_ctx* h, const StepParams& P, int set, const double* E, const double* kap) {
+    double *W = h->PQ[0], *diag = h->PQ[0] + 3 * h->N;
     {
         Scope s(h->prof, "faces_lagged");
-        CK(launch_faces(P, 0, 0, E, kap, h->lagW, nullptr, nullptr, h->st));
+        CK(launch_faces(P, 0, 0, E, kap, W, nullptr, nullptr, h->st));
     }
     Scope s(h->prof, "lagged_diag");
-    CK(launch_lagged_diag(P, h->lagW, h->diag[set], E, kap, h->lagdiag, h->st));
-    set_op0(h, h->lagW, h->lagdiag);
+    CK(launch_lagged_diag(P, W, h->diag[set], E, kap, diag, h->st));
+    set_op0(h, W, diag);
     return RHI_OK;
 }
 
@@ -1030,7 +1029,7 @@ int build_system(rhi_ctx* h, const StepParams& P, int b, int set, const double* 
     }
     A.diag = h->sysdiag;
     // the hierarchy of the lagged-D matrix, or its diagonal for Jacobi
-    if (!newton_hierarchy(h)) return lagged_system(h, P, E, kap, set);
+    if (!newton_hierarchy(h)) return lagged_system(h, P, set, E, kap);
     return RHI_OK;
 }
 
@@ -1681,7 +1680,7 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
             int r2;
             // (from U^n, a trial evaluated meanwhile has overwritten the opacity in kap[0])
             if (cur < 0 && (r2 = kappa(h, P, h->n_s, h->kap[0]))) return r2;
-            if ((r2 = lagged_system(h, P, Ek, h->kap[fb], set))) return r2;
+            if ((r2 = lagged_system(h, P, set, Ek, h->kap[fb]))) return r2;
             if (h->pc_nonsym && (r2 = precond_setup(h, h->op0, false))) return r2;
             return krylov(h, true, h->sysrhs, lin_tol * res, &its, false);
         };
