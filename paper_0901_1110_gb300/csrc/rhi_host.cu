@@ -112,11 +112,16 @@ struct rhi_ctx {
     double *E_p = nullptr, *e_p = nullptr, *n_p = nullptr;
     double dt_prev = 0.0;
     bool have_prev = false;
-    // two work iterates, contiguous (e_c | n_1 .. | E), their opacity and face arrays (times
-    // dt theta): W (limiter_jacobian 0) or the fluxes W (E_c - E_lower), and with dD/dE kept the
-    // Newton-matrix entries PQ and the exact matrix's opacity terms Kf
+    // two work iterates, contiguous (e_c | n_1 .. | E), and their opacity
     double* U[2] = {nullptr, nullptr};
     double* kap[2] = {nullptr, nullptr};
+    // face arrays (times dt theta): W (limiter_jacobian 0) or the fluxes W (E_c - E_lower), and with
+    // dD/dE kept the Newton-matrix entries PQ and the exact matrix's opacity terms Kf.  One set (0)
+    // serves every iterate: fluxes are read by the cell kernel right after, PQ and Kf by the assembly, and
+    // the W of a CG solve until it ends, all before the next iterate's faces.  Set 1 is for U^n alone
+    // where a learned guess is evaluated beside it.  With dD/dE kept it lies in the Krylov vectors, which
+    // nothing uses before the assembly has read it; with limiter_jacobian 0 the solve reads W, and a
+    // solver with a learned guess has a second one
     double* W[2] = {nullptr, nullptr};
     double* PQ[2] = {nullptr, nullptr};
     double* Kf[2] = {nullptr, nullptr};
@@ -1211,26 +1216,42 @@ int rhi_create(const rhi_grid* grid, const rhi_bc* bc, const rhi_params* params,
 
     int rc = RHI_OK;
     auto A = [&](double** p, size_t n) { if (!rc) rc = dalloc(h, p, n); };
+    // several vectors in one block, which also serves as that many times N values in a row: each starts on
+    // a 256-byte boundary, as the kernels' wide accesses need
+    auto block = [&](std::initializer_list<double**> vs) {
+        const size_t Np = ((size_t)N + 31) & ~(size_t)31;
+        double* b = nullptr;
+        A(&b, vs.size() * Np);
+        for (double** v : vs) {
+            if (b) { *v = b; b += Np; }
+        }
+    };
     A(&h->E_s, N); A(&h->e_s, N); A(&h->n_s, (size_t)h->ns * N); A(&h->nH, N); A(&h->src, N);
     A(&h->Tiso, N);
     if (h->ns > 0) { A(&h->E_p, N); A(&h->e_p, N); A(&h->n_p, (size_t)h->ns * N); }
+    // (with a constant opacity, n_species = 0, the exact matrix has no opacity terms)
+    const bool exact = params->limiter_jacobian == 2 && h->ns > 0;
     for (int b = 0; b < 2; ++b) {
-        A(&h->U[b], (size_t)h->nv * N); A(&h->kap[b], N); A(&h->W[b], 3 * (size_t)N);
+        A(&h->U[b], (size_t)h->nv * N); A(&h->kap[b], N);
         A(&h->diag[b], N); A(&h->rhs[b], N); A(&h->fMt[b], (size_t)h->nm * N);
         A(&h->MiU[b], (size_t)h->nm * N);
-        if (params->limiter_jacobian) A(&h->PQ[b], 6 * (size_t)N);
-        // (with a constant opacity, n_species = 0, the exact matrix has no opacity terms)
-        if (params->limiter_jacobian == 2 && h->ns > 0) {
-            A(&h->Kf[b], 3 * (size_t)N); A(&h->rho[b], N); A(&h->phi[b], N);
-        }
+        if (exact) { A(&h->rho[b], N); A(&h->phi[b], N); }
     }
+    block({&h->x, &h->r, &h->p});
+    A(&h->W[0], 3 * (size_t)N);
     if (params->limiter_jacobian) {
+        A(&h->PQ[0], 6 * (size_t)N);
+        if (exact) A(&h->Kf[0], 3 * (size_t)N);
         A(&h->sysPQ, 6 * (size_t)N); A(&h->sysdiag, N); A(&h->sysrhs, N);
-        A(&h->rh, N); A(&h->v, N); A(&h->s, N); A(&h->t, N); A(&h->ph, N); A(&h->sh, N);
+        block({&h->rh, &h->v, &h->s, &h->t, &h->ph, &h->sh});
+        h->z = h->ph; h->q = h->v;              // CG's, which runs after a BiCGStab breakdown only
+        h->W[1] = h->W[0]; h->PQ[1] = h->rh; h->Kf[1] = exact ? h->x : nullptr;
+    } else {
+        A(&h->z, N); A(&h->q, N);
+        if (params->guess == RHI_GUESS_LEARNED) A(&h->W[1], 3 * (size_t)N);
     }
     A(&h->g, (size_t)h->nv * N);
     if (params->dt_norm) A(&h->Upred, (size_t)h->nv * N);
-    A(&h->x, N); A(&h->r, N); A(&h->z, N); A(&h->p, N); A(&h->q, N);
     const long long nparts = std::max<long long>((N + cell_block_size() - 1) / cell_block_size(),
                                                  2 * (long long)stream_blocks(N));
     A(&h->partials, (size_t)nparts);
@@ -1449,8 +1470,8 @@ int rhi_linearize(rhi_handle h, double dt, double a, double adot, double* f, dou
     if (S_diag) CK(cudaMemcpyAsync(S_diag, nonsym ? h->sysdiag : h->diag[0], N * sizeof(double), kind, h->st));
     if (rhs) CK(cudaMemcpyAsync(rhs, nonsym ? h->sysrhs : h->rhs[0], N * sizeof(double), kind, h->st));
     if (S_lo || S_hi) {
-        // face entries of the Newton matrix: straight to a device destination, or by way of the
-        // face arrays of the second work iterate and g^n, which every call writes anew
+        // face entries of the Newton matrix: straight to a device destination, or by way of the CG
+        // vectors x, r, p, which every solve writes anew
         const double* Q = nonsym ? h->opns.Q[0] : h->W[0];
         const double* Pf = nonsym ? h->opns.P[0] : h->W[0];
         if (on_device) {
@@ -1462,9 +1483,9 @@ int rhi_linearize(rhi_handle h, double dt, double a, double adot, double* f, dou
                 if (!dst) continue;
                 {
                     Scope s(h->prof, "export_faces");
-                    CK(launch_export_faces(P, Q, Pf, q ? nullptr : h->W[1], q ? h->W[1] : nullptr, h->st));
+                    CK(launch_export_faces(P, Q, Pf, q ? nullptr : h->x, q ? h->x : nullptr, h->st));
                 }
-                CK(cudaMemcpyAsync(dst, h->W[1], 3 * N * sizeof(double), kind, h->st));
+                CK(cudaMemcpyAsync(dst, h->x, 3 * N * sizeof(double), kind, h->st));
             }
         }
     }
@@ -1492,10 +1513,10 @@ int rhi_residual(rhi_handle h, double dt, double a, double adot, const double* U
     if ((rc = cell(h, P, MODE_PREP, B))) return rc;
     CK(cudaMemcpyAsync(h->U[1], U, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->st));
     if ((rc = kappa(h, P, U_n(h, 1), h->kap[1]))) return rc;
-    if ((rc = faces(h, P, U_E(h, 1), h->kap[1], 1))) return rc;
+    if ((rc = faces(h, P, U_E(h, 1), h->kap[1], 0))) return rc;
     PhysBuffers C = state_buffers(h);
     C.ec = U_ec(h, 1); C.n = U_n(h, 1); C.E = U_E(h, 1);
-    with_set(h, C, 1, 1);
+    with_set(h, C, 0, 1);
     if (f) C.f_out = on_device ? f : h->U[0];
     if ((rc = cell(h, P, MODE_ITER, C))) return rc;
     double r = 0.0;
@@ -1577,9 +1598,11 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
 
     // ---- g^n and the initial iterate U_0
     if ((rc = kappa(h, P, h->n_s, h->kap[0]))) return rc;
-    if ((rc = faces(h, P, h->E_s, h->kap[0], 0))) return rc;
+    // face arrays of U_k: set 1 for U^n where a guess is evaluated beside it, else 0
+    int fb = h->prm.guess == RHI_GUESS_LEARNED && h->mlp_skip == 0 ? 1 : 0;
+    if ((rc = faces(h, P, h->E_s, h->kap[0], fb))) return rc;
     PhysBuffers B = state_buffers(h);
-    with_set(h, B, 0, 0);
+    with_set(h, B, fb, 0);
     int cur = -1;            // -1: U_k is the state U^n (e_c = 0); 0 / 1: work buffer
     int set = 0;             // Schur set of U_k
     double res = 0.0;
@@ -1602,10 +1625,10 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
                 CK(launch_mlp_infer(A, h->mlp_pk, nullptr, nullptr, 0, 1, h->st));
             }
             if ((rc = kappa(h, P, U_n(h, 1), h->kap[1]))) return rc;
-            if ((rc = faces(h, P, U_E(h, 1), h->kap[1], 1))) return rc;
+            if ((rc = faces(h, P, U_E(h, 1), h->kap[1], 0))) return rc;
             PhysBuffers C = state_buffers(h);
             C.ec = U_ec(h, 1); C.n = U_n(h, 1); C.E = U_E(h, 1);
-            with_set(h, C, 1, 1);
+            with_set(h, C, 0, 1);
             if ((rc = cell(h, P, MODE_ITER, C))) return rc;
             double rg = 0.0;
             if ((rc = residual_norm(h, ncell_blocks(h), &rg))) return rc;
@@ -1613,6 +1636,7 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
             if (rg < res) {
                 cur = 1;
                 set = 1;
+                fb = 0;
                 res = rg;
             } else {
                 S.guess_used = RHI_GUESS_PREVIOUS;
@@ -1658,6 +1682,7 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
             if ((rc = residual_norm(h, ncell_blocks(h), &res))) return rc;
             cur = -1;
             set = 0;
+            fb = 0;
             r_best = res;
             bad = 0;
             k_start = k;
@@ -1666,9 +1691,9 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
             S.guess_restarts = 1;
             if (res < newton_tol) break;
         }
-        const int fb = cur < 0 ? 0 : cur;
+        const int kb = cur < 0 ? 0 : cur;                   // opacity of U_k
         const double* Ek = cur < 0 ? h->E_s : U_E(h, cur);
-        if ((rc = build_system(h, P, fb, set, Ek, h->kap[fb]))) return rc;
+        if ((rc = build_system(h, P, fb, set, Ek, h->kap[kb]))) return rc;
         if ((rc = precond_setup_newton(h))) return rc;
         int its = 0;
         // BiCGStab broke down (where free streaming makes the advective part of the matrix
@@ -1680,7 +1705,7 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
             int r2;
             // (from U^n, a trial evaluated meanwhile has overwritten the opacity in kap[0])
             if (cur < 0 && (r2 = kappa(h, P, h->n_s, h->kap[0]))) return r2;
-            if ((r2 = lagged_system(h, P, set, Ek, h->kap[fb]))) return r2;
+            if ((r2 = lagged_system(h, P, set, Ek, h->kap[kb]))) return r2;
             if (h->pc_nonsym && (r2 = precond_setup(h, h->op0, false))) return r2;
             return krylov(h, true, h->sysrhs, lin_tol * res, &its, false);
         };
@@ -1697,13 +1722,13 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
         auto evaluate = [&](double* rt, bool resid_only) -> int {
             int r2;
             if (resid_only) {
-                if ((r2 = faces_w(h, P, U_E(h, t), h->kap[t], t))) return r2;
-            } else if ((r2 = faces(h, P, U_E(h, t), h->kap[t], t))) {
+                if ((r2 = faces_w(h, P, U_E(h, t), h->kap[t], 0))) return r2;
+            } else if ((r2 = faces(h, P, U_E(h, t), h->kap[t], 0))) {
                 return r2;
             }
             PhysBuffers C = state_buffers(h);
             C.ec = U_ec(h, t); C.n = U_n(h, t); C.E = U_E(h, t);
-            with_set(h, C, t, 1 - set);
+            with_set(h, C, 0, 1 - set);
             if ((r2 = cell(h, P, resid_only ? MODE_RESID : MODE_ITER, C))) return r2;
             return residual_norm(h, ncell_blocks(h), rt);
         };
@@ -1770,6 +1795,7 @@ int rhi_implicit_step(rhi_handle h, double dt, double a, double adot, double new
         }
         cur = t;
         set = 1 - set;
+        fb = 0;
         res_prev = res;
         res = rt;
         ++k;
