@@ -214,8 +214,9 @@ int fail(rhi_ctx* h, int code, const std::string& msg) {
     } while (0)
 
 // Small buffers share slabs: a handle has about a hundred of them, and on a small grid their cudaMalloc
-// calls would be most of rhi_create.
-constexpr size_t SLAB_BYTES = 4u << 20, SLAB_SHARE = 512u << 10;
+// calls would be most of rhi_create.  A slab holds about what the handle needs (a hundred fields of its
+// grid), within these bounds: many small handles can be alive at once.
+constexpr size_t SLAB_MIN = 512u << 10, SLAB_MAX = 4u << 20, SLAB_SHARE = 512u << 10;
 
 template <typename T>
 int dalloc(rhi_ctx* h, T** p, size_t count) {
@@ -228,13 +229,14 @@ int dalloc(rhi_ctx* h, T** p, size_t count) {
     }
     void* v = nullptr;
     const bool share = bytes <= SLAB_SHARE;
-    cudaError_t e = cudaMalloc(&v, share ? SLAB_BYTES : bytes);
+    const size_t slab = std::min(SLAB_MAX, std::max(SLAB_MIN, 100 * sizeof(double) * (size_t)h->N));
+    cudaError_t e = cudaMalloc(&v, share ? slab : bytes);
     if (e != cudaSuccess) return fail(h, RHI_ERR_CUDA, std::string("cudaMalloc: ") + cudaGetErrorString(e));
     h->allocs.push_back(v);
     *p = (T*)v;
     if (share) {
         h->slab = (char*)v + bytes;
-        h->slab_left = SLAB_BYTES - bytes;
+        h->slab_left = slab - bytes;
     }
     return RHI_OK;
 }

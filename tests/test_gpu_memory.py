@@ -63,3 +63,19 @@ def test_lost_guess_leaves_the_step_of_the_previous_state(shape, ljac, graph, pr
         s.close()
     for k in ("E", "e", "n"):
         assert np.array_equal(out[0][k], out[1][k]), k
+
+
+def test_small_handles_stay_small():
+    """A 4^3 handle's buffers are 0.4 MB (most of it the rate table): 20 of them within 1 MB each."""
+    import torch
+
+    import paper_0901_1110_gb300 as rhi
+    p = rhi.rhi_params_default(1)
+    rhi.Solver(4, 4, 4, 1e22, p).close()
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    handles = [rhi.Solver(4, 4, 4, 1e22, p) for _ in range(20)]
+    taken = before - torch.cuda.mem_get_info()[0]
+    for s in handles:
+        s.close()
+    assert taken <= 20 * 2 ** 20, taken / 20
