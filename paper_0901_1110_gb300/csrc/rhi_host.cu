@@ -253,23 +253,20 @@ StepParams make_params(const rhi_ctx* h, double dt, double a, double adot) {
         P.Eb[d] = h->bc.value[d];
         if (h->bc.kind[d] == RHI_BC_DIRICHLET) P.dir_mask |= 1 << d;
     }
-    P.dx = h->grid.dx;
-    P.a = a; P.ia3 = 1.0 / (a * a * a); P.adot_a = adot / a;
-    P.dt = dt; P.dth = dt * h->prm.theta; P.dtm1 = dt * (h->prm.theta - 1.0);
-    P.inv_adx = 1.0 / (a * h->grid.dx);
+    P.ia3 = 1.0 / (a * a * a); P.adot_a = adot / a;
+    P.dth = dt * h->prm.theta;
+    const double inv_adx = 1.0 / (a * h->grid.dx);
     P.half_adx = 0.5 * a * h->grid.dx;
-    P.inv_a2dx2 = P.inv_adx * P.inv_adx;
     const int nmax = std::max(h->grid.nx, std::max(h->grid.ny, h->grid.nz));
     P.R_min = 1.0 / (a * nmax * h->grid.dx);
     P.quart_adx = 0.5 * P.half_adx;
     P.R_min2 = 2.0 * P.R_min;
-    const double d = C_LIGHT * P.dth * P.inv_a2dx2;
+    const double d = C_LIGHT * P.dth * (inv_adx * inv_adx);
     P.cF = 2.0 * d;
     P.cK = -0.5 / d;
     P.cV = d * P.half_adx;
     P.cD = d / 3.0;
     P.kappa_floor = h->prm.kappa_floor;
-    P.m_grey = (double)h->prm.m_grey;
     P.isothermal = h->prm.isothermal; P.limiter = h->prm.limiter;
     P.limiter_newton = h->prm.limiter_jacobian;
     P.y_he = h->prm.y_he;
@@ -283,7 +280,7 @@ StepParams make_params(const rhi_ctx* h, double dt, double a, double adot) {
     P.i3 = P.dth * P.ia3;
     P.cdth = C_LIGHT * P.dth;
     P.cE3 = P.cdth * P.ia3;
-    P.madot_dth = P.m_grey * P.adot_a * P.dth;
+    P.madot_dth = (double)h->prm.m_grey * P.adot_a * P.dth;
     P.adot2_dth = 2.0 * P.adot_a * P.dth;
     P.one_adot2 = 1.0 + P.adot2_dth;
     P.r_ne = P.u_n * P.iu_e;
@@ -638,11 +635,11 @@ int vcycle_graph(rhi_ctx* h, const Op<float>& A0) {
     return RHI_OK;
 }
 
-// what the last block of a kernel with a sum does with it
-Finish fin(const rhi_ctx* h, int op, int slot = 0, unsigned long long cond = 0) {
+// the partials, tickets and scalars of the kernels that end with a sum
+Finish fin(const rhi_ctx* h, unsigned long long cond = 0) {
     Finish F;
     F.partials = h->partials; F.count = h->red_count; F.scal = h->scal;
-    F.op = op; F.slot = slot; F.cond = cond;
+    F.cond = cond;
     return F;
 }
 
@@ -666,7 +663,7 @@ int precond_into(rhi_ctx* h, LinLaunch& L, const double* r, double* dest, bool v
                  const BicgP& up = BicgP()) {
     const long long N = h->N;
     if (h->prm.precond == RHI_PRECOND_JACOBI) {
-        Finish none = fin(h, RED_NONE);
+        Finish none = fin(h);
         none.count = nullptr;
         CK(L.jacobi_dot(N, r, h->pc0.diag, dest, none));
     } else if (h->prm.precond == RHI_PRECOND_MG_FP64) {
@@ -711,7 +708,7 @@ int precond_into(rhi_ctx* h, LinLaunch& L, const double* r, double* dest, bool v
 // r = b, rh = b, x = 0 and the loop's start (S_RR = S_RHO = r.r, counters cleared)
 int bicg_start(rhi_ctx* h, LinLaunch& L, const double* rhs, unsigned long long cond) {
     L.skip = nullptr;
-    CK(L.bicg_init(h->N, rhs, h->r, h->rh, h->x, fin(h, RED_BICG_START, 0, cond)));
+    CK(L.bicg_init(h->N, rhs, h->r, h->rh, h->x, fin(h, cond)));
     return RHI_OK;
 }
 
@@ -721,8 +718,7 @@ int bicg_start(rhi_ctx* h, LinLaunch& L, const double* rhs, unsigned long long c
 // r update; the next rho, beta and the continue flag (cond: the graph's while handle, or 0).
 int bicg_iteration(rhi_ctx* h, LinLaunch& L, unsigned long long cond) {
     const long long N = h->N;
-    const Finish fa = fin(h, RED_BICG_ALPHA), fs = fin(h, RED_BICG_SS), fo = fin(h, RED_BICG_OMEGA),
-                 fn = fin(h, RED_BICG_NEXT, 0, cond);
+    const Finish f = fin(h), fn = fin(h, cond);
     float* b32 = cycle_rhs(h);
     int rc;
     L.skip = nullptr;
@@ -734,11 +730,11 @@ int bicg_iteration(rhi_ctx* h, LinLaunch& L, unsigned long long cond) {
         CK(L.bicg_p(N, h->scal, h->r, h->v, h->p, h->rh, b32));
     }
     if ((rc = precond_into(h, L, h->p, h->ph, false, up))) return rc;
-    CK(L.matvec_ns(h->opns, h->ph, h->v, h->rh, 0, fa));
-    CK(L.bicg_s(N, h->scal, h->r, h->v, h->s, b32, fs));
+    CK(L.matvec_ns(h->opns, h->ph, h->v, h->rh, 0, f));
+    CK(L.bicg_s(N, h->scal, h->r, h->v, h->s, b32, f));
     L.skip = h->scal + S_DONE;
     if ((rc = precond_into(h, L, h->s, h->sh))) return rc;
-    CK(L.matvec_ns(h->opns, h->sh, h->t, h->s, 1, fo));
+    CK(L.matvec_ns(h->opns, h->sh, h->t, h->s, 1, f));
     L.skip = nullptr;
     CK(L.bicg_xr(N, h->scal, h->x, h->ph, h->sh, h->s, h->t, h->r, h->rh, fn));
     return RHI_OK;
@@ -748,7 +744,7 @@ int bicg_iteration(rhi_ctx* h, LinLaunch& L, unsigned long long cond) {
 // iteration z = M^-1 r and beta, p, q = S p and alpha, the x / r update and the continue flag
 int cg_start(rhi_ctx* h, LinLaunch& L, const double* rhs, unsigned long long cond) {
     L.skip = nullptr;
-    CK(L.cg_init(h->N, rhs, h->r, h->x, cycle_rhs(h), fin(h, RED_CG_START, 0, cond)));
+    CK(L.cg_init(h->N, rhs, h->r, h->x, cycle_rhs(h), fin(h, cond)));
     return RHI_OK;
 }
 int cg_iteration(rhi_ctx* h, LinLaunch& L, unsigned long long cond, bool vg) {
@@ -756,14 +752,14 @@ int cg_iteration(rhi_ctx* h, LinLaunch& L, unsigned long long cond, bool vg) {
     int rc;
     L.skip = nullptr;
     if (h->prm.precond == RHI_PRECOND_JACOBI) {
-        CK(L.jacobi_dot(N, h->r, h->pc0.diag, h->z, fin(h, RED_CG_BETA)));
+        CK(L.jacobi_dot(N, h->r, h->pc0.diag, h->z, fin(h)));
     } else {
         if ((rc = precond_into(h, L, h->r, h->z, vg))) return rc;
-        CK(L.dot(N, h->r, h->z, fin(h, RED_CG_BETA)));
+        CK(L.cg_beta(N, h->r, h->z, fin(h)));
     }
     CK(L.cg_p(N, h->scal, h->z, h->p));
-    CK(L.matvec_dot(h->op0, h->p, h->q, fin(h, RED_CG_ALPHA)));
-    CK(L.cg_xr(N, h->scal, h->x, h->r, h->p, h->q, cycle_rhs(h), fin(h, RED_CG_NEXT, 0, cond)));
+    CK(L.matvec_dot(h->op0, h->p, h->q, fin(h)));
+    CK(L.cg_xr(N, h->scal, h->x, h->r, h->p, h->q, cycle_rhs(h), fin(h, cond)));
     return RHI_OK;
 }
 
@@ -774,7 +770,7 @@ bool krylov_graph_usable(const rhi_ctx* h) {
     if (h->prof.only.empty()) return false;
     for (const auto& nm : h->prof.only)
         if (nm.compare(0, 3, "mg_") == 0 || nm.compare(0, 5, "bicg_") == 0 || nm.compare(0, 3, "cg_") == 0 ||
-            nm == "dot" || nm == "copy" || nm == "precond_jacobi")
+            nm == "dot" || nm == "precond_jacobi")
             return false;
     return true;
 }

@@ -46,18 +46,14 @@ struct StepParams {
     int per_x, per_y, per_z;          // periodic axes
     int dir_mask;                     // bit d: face d (x-, x+, y-, y+, z-, z+) is Dirichlet
     double Eb[6];                     // E on the Dirichlet faces
-    double dx;
-    double a, ia3, adot_a;            // a, 1/a^3, adot / a
-    double dt, dth, dtm1;             // dt, dt theta, dt (theta - 1)
-    double inv_a2dx2;                 // 1 / (a dx)^2
-    double inv_adx;                   // 1 / (a dx)
+    double ia3, adot_a;               // 1/a^3, adot / a
+    double dth;                       // dt theta
     double half_adx;                  // a dx / 2
     double R_min;                     // limiter floor 1 / (a L)
     // face formulas, whose results come multiplied by dt theta: a dx / 4, 2 R_min, and with
     // d = c dth / (a dx)^2: 2 d, -1 / (2 d), d a dx / 2, d (a dx)^2 / 3 (no limiter) over (a dx)^2
     double quart_adx, R_min2, cF, cK, cV, cD;
     double kappa_floor;
-    double m_grey;
     int isothermal, limiter;
     int limiter_newton;               // 1: keep dD/dE in the Newton matrix (non-symmetric S)
     double y_he;

@@ -107,9 +107,8 @@ __device__ __forceinline__ T jacobi_update(T xc, T b, T wi, T off, T omega) {
 
 // ---------------------------------------------------------------------------------------------
 // Scalar updates.  A kernel with dot products ends with finish(): its last block adds all blocks'
-// partials in a fixed order and applies the update, so that a Krylov iteration needs no separate
+// partials in a fixed order and applies the kernel's update, so that a Krylov iteration needs no separate
 // reduction launches (about 3.6 us each inside a graph; the last block adds about 2 us).
-//   RED_SUM:        scal[slot] = sum
 //   RED_CG_START:   r.r of r = b: S_RR, counters cleared; done when r.r <= S_THR
 //   RED_CG_BETA:    r.z: S_BETA = sum / S_RZ; S_RZ = sum
 //   RED_CG_ALPHA:   p.Sp: S_PQ = sum; S_ALPHA = S_RZ / sum (breakdown flag if <= 0)
@@ -130,14 +129,12 @@ __device__ __forceinline__ T jacobi_update(T xc, T b, T wi, T off, T omega) {
 //                   then that of an inexact Newton iteration.
 // The START and NEXT updates write the continue flag to S_CONT and, inside a CUDA graph, to the
 // while node's conditional handle: these kernels always run to their end.
+enum { RED_CG_START, RED_CG_BETA, RED_CG_ALPHA, RED_CG_NEXT, RED_BICG_START, RED_BICG_ALPHA, RED_BICG_SS,
+       RED_BICG_OMEGA, RED_BICG_NEXT };
 template <int op>
-__device__ __forceinline__ void scalar_update(double* scal, int slot, unsigned long long cond,
-                                              double s, double s2) {
+__device__ __forceinline__ void scalar_update(double* scal, unsigned long long cond, double s, double s2) {
     int cont = 0;
-    if (op == RED_SUM) {
-        scal[slot] = s;
-        return;
-    } else if (op == RED_CG_START) {
+    if (op == RED_CG_START) {
         scal[S_RR] = s;
         scal[S_ITS] = 0.0;
         scal[S_BREAK] = 0.0;
@@ -245,13 +242,13 @@ __device__ __forceinline__ void finish(const Finish& F, double v1, double v2) {
     // one, which alone writes them, after every block has its ticket, uses them)
     if (threadIdx.x < S_NSCAL && F.count) sc[threadIdx.x] = __ldcg(F.scal + threadIdx.x);
     if (!grid_sum<LIN_BLOCK, TWO>(v1, v2, F.partials, F.count, s1, s2)) return;
-    if (threadIdx.x == 0) scalar_update<OP>(sc, F.slot, F.cond, s1, s2);
+    if (threadIdx.x == 0) scalar_update<OP>(sc, F.cond, s1, s2);
     __syncthreads();
     if (threadIdx.x < S_NSCAL) F.scal[threadIdx.x] = sc[threadIdx.x];
 }
 
 // sum or max of partials in a fixed order by one block (where a kernel has too many blocks for its
-// last one to add them, or none of the above)
+// last one to add them, or its sum goes to a slot without an update)
 __global__ void __launch_bounds__(RED_BLOCK) k_reduce(const double* __restrict__ partials, int n,
                                                       double* __restrict__ scal, int op, int slot) {
     if (op == RED_MAX) {                        // max of non-negative partials
@@ -340,13 +337,13 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_jacobi_dot(long long N, const dou
     finish<false, RED_CG_BETA>(F, acc, 0.0);
 }
 
-// a.b
-__global__ void __launch_bounds__(LIN_BLOCK) k_dot(long long N, const double* __restrict__ a,
-                                                   const double* __restrict__ b, const Finish F) {
+// r.z
+__global__ void __launch_bounds__(LIN_BLOCK) k_cg_beta(long long N, const double* __restrict__ r,
+                                                       const double* __restrict__ z, const Finish F) {
     double acc = 0.0;
     for (long long c = blockIdx.x * (long long)LIN_BLOCK + threadIdx.x; c < N;
          c += (long long)gridDim.x * LIN_BLOCK)
-        acc += a[c] * b[c];
+        acc += r[c] * z[c];
     finish<false, RED_CG_BETA>(F, acc, 0.0);
 }
 
@@ -1315,9 +1312,9 @@ cudaError_t LinLaunch::jacobi_dot(long long N, const double* r, const double* di
     k_jacobi_dot<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, r, diag, z, F, skip);
     return end();
 }
-cudaError_t LinLaunch::dot(long long N, const double* a, const double* b, const Finish& F) {
+cudaError_t LinLaunch::cg_beta(long long N, const double* r, const double* z, const Finish& F) {
     begin("dot");
-    k_dot<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, a, b, F);
+    k_cg_beta<<<sum_blocks(N), LIN_BLOCK, 0, st>>>(N, r, z, F);
     return end();
 }
 cudaError_t LinLaunch::cg_init(long long N, const double* b, double* r, double* x, float* r32,

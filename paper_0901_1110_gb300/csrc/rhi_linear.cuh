@@ -100,17 +100,16 @@ enum { S_RZ = 0, S_PQ, S_ALPHA, S_BETA, S_RR, S_BREAK, S_TMP, S_RHO, S_OMEGA, S_
        S_STALL, S_RR0, S_NRST, S_RST, S_NSCAL = 32 };
 constexpr int STALL_ITS = 20;
 constexpr int MAX_RESTARTS = 8;
-enum { RED_NONE = 0, RED_SUM, RED_MAX, RED_CG_START, RED_CG_BETA, RED_CG_ALPHA, RED_CG_NEXT, RED_BICG_ALPHA, RED_BICG_OMEGA,
-       RED_BICG_START, RED_BICG_SS, RED_BICG_NEXT };
+// k_reduce's two forms
+enum { RED_SUM = 0, RED_MAX };
 
-// What the last block of a kernel with a dot product does with the sum(s): the scalar update `op` on
-// scal (RED_SUM: to `slot`; RED_NONE: nothing) and, for the loop's updates, the continue flag to the
-// CUDA-graph conditional handle cond (0: none).
+// Where the last block of a kernel with a dot product takes the partials from and puts the outcome: each
+// such kernel has one scalar update on scal (rhi_linear.cu), and those that decide on the loop also set the
+// CUDA-graph conditional handle cond (0: none).  count null: partials only, no update.
 struct Finish {
     double* partials = nullptr;
     unsigned* count = nullptr;
     double* scal = nullptr;
-    int op = RED_NONE, slot = 0;
     unsigned long long cond = 0;
 };
 
@@ -145,11 +144,12 @@ struct LinLaunch {
     cudaError_t matvec_dot(const Op<double>& A, const double* p, double* q, const Finish& F);
     cudaError_t cg_xr(long long N, const double* scal, double* x, double* r, const double* p,
                       const double* q, float* r32, const Finish& F);
-    // p = z at the loop's first iteration, else z + beta p
+    // p = z at the loop's first iteration, else z + beta p.  jacobi_dot: z = r / diag, and CG's beta
     cudaError_t cg_p(long long N, const double* scal, const double* z, double* p);
     cudaError_t jacobi_dot(long long N, const double* r, const double* diag, double* z,
                            const Finish& F);
-    cudaError_t dot(long long N, const double* a, const double* b, const Finish& F);
+    // CG's r.z and beta
+    cudaError_t cg_beta(long long N, const double* r, const double* z, const Finish& F);
     // r32 (may be null), here and above: the FP32 copy of r
     cudaError_t cg_init(long long N, const double* b, double* r, double* x, float* r32,
                         const Finish& F);
