@@ -151,7 +151,6 @@ def alg_bytes(nonsym):
         # FP64 Krylov vector to the FP32 right-hand side, and the FP32 result back to FP64
         "mg_to_f32": 8 + 4,
         "mg_from_f32": 4 + 8,
-        "mg_from_f32_dot": 4 + 8 + 8,
     }
 
 
@@ -163,7 +162,7 @@ LINEAR_KERNELS = ("cg_matvec_dot", "cg_update_xr", "cg_update_p", "bicg_matvec",
                   "mg_smooth_f32_fine_first", "mg_smooth_f32_fine_two", "mg_smooth_f64_fine",
                   "mg_smooth_f64_fine_first", "mg_smooth_f64_fine_two",
                   "mg_restrict_f32_fine", "mg_restrict_f64_fine", "mg_prolong_f32_fine",
-                  "mg_prolong_f64_fine", "mg_to_f32", "mg_from_f32", "mg_from_f32_dot")
+                  "mg_prolong_f64_fine", "mg_to_f32", "mg_from_f32")
 
 
 class ClockSampler:

@@ -320,9 +320,9 @@ int rhi_mlp_train(rhi_handle h, const float* X, const float* Y, long long n, int
    eq. rmsnorm when v holds the scaled residual and count = N (N_s + 2).
    v (n doubles) and out (1 double) are device pointers owned by the caller; stream is a
    cudaStream_t (NULL: legacy default stream); the call only enqueues work and returns.
-   Scratch: a static device array of RHI_NOALLOC_MAX_COUNT / 256 doubles (1 MiB) that every
-   GPU loading the library holds until the process exits; nothing is allocated.  n above
-   RHI_NOALLOC_MAX_COUNT is rejected with RHI_ERR_ARG before any launch.  The first call on a
+   Scratch: a static device array of a few kB, one double per block of a launch that fills the
+   GPU, that every GPU loading the library holds until the process exits; nothing is allocated.  n
+   above RHI_NOALLOC_MAX_COUNT is rejected with RHI_ERR_ARG before any launch.  The first call on a
    device looks up the scratch address for that device (make it before any stream capture).
    Every call overwrites the whole scratch it uses and nothing in it needs to start at zero,
    but calls that overlap on the GPU (different streams or host threads) race on it.  The call

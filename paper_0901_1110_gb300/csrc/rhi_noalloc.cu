@@ -13,11 +13,10 @@
 namespace {
 
 constexpr int NA_BLOCK = 256;
-constexpr long long NA_MAX_PARTIALS = RHI_NOALLOC_MAX_COUNT / NA_BLOCK;
 constexpr int NA_BLOCKS = 152 * 4;             // blocks of a large input, 4 per SM
 
 // one partial sum per block of the first kernel (the result goes to the caller's `out`)
-static __device__ __align__(256) double na_scratch[NA_MAX_PARTIALS];
+static __device__ __align__(256) double na_scratch[NA_BLOCKS];
 
 // Sum of squares of this block's share: four independent 16-byte loads per thread and turn, then single
 // values.  Bound by HBM and the FP64 pipe alike (one FMA per 8 bytes): 2^25 values 72 us, against 478 us
@@ -79,7 +78,7 @@ std::mutex na_mutex;
 extern "C" int rhi_rms_norm_noalloc(const double* v, long long n, long long count,
                                     double* out, void* stream) {
     if (!v || !out || n < 1 || count < 1) return RHI_ERR_ARG;
-    if (n > RHI_NOALLOC_MAX_COUNT) return RHI_ERR_ARG;       // scratch holds n / 256 partials
+    if (n > RHI_NOALLOC_MAX_COUNT) return RHI_ERR_ARG;       // the documented limit
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= NA_MAX_DEVICES) return RHI_ERR_CUDA;
     double* part = nullptr;
@@ -93,7 +92,7 @@ extern "C" int rhi_rms_norm_noalloc(const double* v, long long n, long long coun
         part = na_addr[dev];
     }
     const cudaStream_t st = (cudaStream_t)stream;
-    // four values per thread at least, and no more blocks than fill the GPU (<= NA_MAX_PARTIALS)
+    // four values per thread at least, and no more blocks than fill the GPU, which is what the scratch holds
     const long long want = (n + 4 * NA_BLOCK - 1) / (4 * NA_BLOCK);
     const long long nb = want < NA_BLOCKS ? want : NA_BLOCKS;
     const bool aligned = ((unsigned long long)v & 15ull) == 0;
