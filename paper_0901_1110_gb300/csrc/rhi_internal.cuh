@@ -1,6 +1,7 @@
 // Internal declarations shared by the CUDA translation units of librhi.
 #pragma once
 
+#include <cfloat>
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -80,12 +81,44 @@ struct StepParams {
 // Reciprocal to within one unit in the last place: the hardware's reciprocal seed (PTX
 // rcp.approx.ftz.f64, about 20 bits) and one third-order Householder step r (1 + e + e^2) with
 // e = 1 - d r, whose error is e^3 < 2^-55: three FP64 instructions where the IEEE division takes
-// about ten.  For normal d with a normal reciprocal.
+// about ten.  For normal d below 2^1021 in size (a seed under 2^-1022 is flushed to 0); NaN for d = 0 or
+// subnormal.
 __device__ __forceinline__ double fast_rcp(double d) {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
     const double e = fma(-d, r, 1.0);
     return fma(r, fma(e, e, e), r);
+}
+
+// FP32 to FP64 on the integer pipe, exact for every value: a conversion instruction takes the FP64 pipe
+// as long as an FMA (64 cycles a warp), which is most of a small level's build.  No branch; subnormals
+// are scaled up in FP32 first.
+__device__ __forceinline__ double widen(float f) {
+    const bool small = (__float_as_uint(f) & 0x7fffffffu) < 0x00800000u;
+    const unsigned u = __float_as_uint(small ? f * 18446744073709551616.0f : f), m = u & 0x7fffffffu;
+    unsigned hi = (m >> 3) + (small ? (896u - 64u) << 20 : 896u << 20);
+    hi = m == 0u ? 0u : hi;
+    hi = m >= 0x7f800000u ? 0x7ff00000u | (m >> 3 & 0xfffffu) : hi;
+    return __hiloint2double((int)((u & 0x80000000u) | hi), (int)(u << 29));
+}
+__device__ __forceinline__ double widen(double f) { return f; }
+
+// z / (1 + exp(-z)).  Two special-function results each (192 a row bound the forward pass); FAST: the
+// quotient from the reciprocal approximation and one residual correction, q + (z - q d) r, which rounds as
+// the IEEE division does but for a last bit now and then, in 6 instructions instead of a division's 15
+// or so.  The residual is not a number where exp(-z) overflows (r = 0, q = -0) and at z = inf: fmaxf then
+// gives its other operand, and the results are the division's -0 and inf.  (A bound on d, from which r
+// came too, left z / 3e38 and NaN there; bounds on q and d cost 304 against 288 us for 128^3 rows.)
+// The guess keeps the division: its FP64 results are held to the bit, and its time is its FP64
+// logarithms'.
+template <bool FAST>
+__device__ __forceinline__ float silu_f(float z) {
+    if constexpr (!FAST) return z / (1.0f + __expf(-z));
+    const float d = 1.0f + __expf(-z);
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(d));
+    const float q = z * r;
+    return fmaf(fmaxf(fmaf(-q, d, z), -FLT_MAX), r, q);
 }
 
 // A value the compiler cannot see through.  `for (int go = rare; go; go = opaque(0)) {...}` is an `if`

@@ -1079,19 +1079,6 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_prolong(int nx, int ny, int nz
     }
 }
 
-// FP32 to FP64 on the integer pipe, exact for every value: a conversion instruction takes the FP64 pipe
-// as long as an FMA (64 cycles a warp), which is most of a small level's build.  No branch; subnormals
-// are scaled up in FP32 first.
-__device__ __forceinline__ double widen(float f) {
-    const bool small = (__float_as_uint(f) & 0x7fffffffu) < 0x00800000u;
-    const unsigned u = __float_as_uint(small ? f * 18446744073709551616.0f : f), m = u & 0x7fffffffu;
-    unsigned hi = (m >> 3) + (small ? (896u - 64u) << 20 : 896u << 20);
-    hi = m == 0u ? 0u : hi;
-    hi = m >= 0x7f800000u ? 0x7ff00000u | (m >> 3 & 0xfffffu) : hi;
-    return __hiloint2double((int)((u & 0x80000000u) | hi), (int)(u << 29));
-}
-__device__ __forceinline__ double widen(double f) { return f; }
-
 // One coarse cell of the hierarchy: the operator by re-discretisation, and the smoother's omega /
 // diagonal.  Local diagonal = mean of the children's local diagonals (diag - the six couplings of their
 // rows); each face array of the coarse cell's lower face = (mean of that array over the existing fine

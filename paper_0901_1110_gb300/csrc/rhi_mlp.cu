@@ -12,7 +12,6 @@
 // Inference runs on the tensor cores (mma.sync m16n8k16, BF16 operands, FP32 accumulation)
 // with the layer activations chained in registers; training runs FP32 on the CUDA cores, tiles of
 // 32 samples per block, with a deterministic gradient reduction and Adam.
-#include <cfloat>
 #include <cmath>
 #include <cstddef>
 
@@ -119,24 +118,6 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&v);
-}
-
-// z / (1 + exp(-z)).  Two special-function results each (192 a row bound the forward pass); FAST: the
-// quotient from the reciprocal approximation and one residual correction, q + (z - q d) r, which rounds as
-// the IEEE division does but for a last bit now and then, in 6 instructions instead of a division's 15
-// or so.  The residual is not a number where exp(-z) overflows (r = 0, q = -0) and at z = inf: fmaxf then
-// gives its other operand, and the results are the division's -0 and inf.  (A bound on d, from which r
-// came too, left z / 3e38 and NaN there; bounds on q and d cost 304 against 288 us for 128^3 rows.)
-// The guess keeps the division: its FP64 results are held to the bit, and its time is its FP64
-// logarithms'.
-template <bool FAST>
-__device__ __forceinline__ float silu_f(float z) {
-    if constexpr (!FAST) return z / (1.0f + __expf(-z));
-    const float d = 1.0f + __expf(-z);
-    float r;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(d));
-    const float q = z * r;
-    return fmaf(fmaxf(fmaf(-q, d, z), -FLT_MAX), r, q);
 }
 
 // one hidden layer on a 16-row tile: in = A fragments over KS k-steps, out = 8 n-tiles
