@@ -978,11 +978,15 @@ __global__ void __launch_bounds__(LIN_BLOCK) k_mg_restrict(const Op<T> A, const 
 
 // The same with eight lanes to a parent, one for each child (a warp: four parents in a row, so runs of
 // eight cells along x), summed by shuffles: a child's loads do not wait for those of its siblings,
-// and eight times as many threads ask for them.  Measured at 64^3, where that is what counts: FP32
-// 11.0 -> 8.4 us, FP64 14.0 -> 12.1 us (32^3: 13.7 -> 7.9 us).  At 128^3 the first form, with fewer
-// instructions per cell, is the better one: 19.2 against 22.6 us, and 45 against 55 us in FP64; at
-// 256^3 FP32 99 against 154 us.  RESTRICT_SPLIT: most parents of a level that takes this form.
-constexpr long long RESTRICT_SPLIT = 1LL << 16;
+// and eight times as many threads ask for them.  On large levels the first form, with fewer
+// instructions per cell, is the better one.  Measured, this form / the first, us:
+//   FP32                  64^3 8.4 / 10.0   88^3 11.6 / 12.1   96^3 13.5 / 12.8   128^3 24.0 / 20.5
+//   FP64, non-symmetric   64^3 12.8 / 14.0   88^3 23.2 / 24.0   96^3 29.0 / 24.7   128^3 60.0 / 49.5
+//   FP64, symmetric       48^3 10.0 / 14.3   56^3 12.7 / 14.5   64^3 15.5 / 13.9   80^3 24.6 / 18.1
+// (in the last one the first form leaves out the faces between children, half the arithmetic that
+// bounds it).  RESTRICT_SPLIT and, for that one, RESTRICT_SPLIT_SYM: most parents of a level that
+// takes this form, 80^3 and 58^3 cells, a size below the crossing.
+constexpr long long RESTRICT_SPLIT = 1LL << 16, RESTRICT_SPLIT_SYM = 3LL << 13;
 template <typename T>
 __global__ void __launch_bounds__(LIN_BLOCK) k_mg_restrict_split(const Op<T> A, const T* __restrict__ b,
                                                                  const T* __restrict__ x, int cnx,
@@ -1413,7 +1417,8 @@ cudaError_t LinLaunch::restrict_res(const Op<T>& A, const T* b, const T* x, int 
     B.skip = skip;
     const long long Nc = (long long)cnx * cny * cnz;
     const FastDiv fx = make_fastdiv((unsigned)cnx), fxy = make_fastdiv((unsigned)cnx * cny);
-    if (Nc <= RESTRICT_SPLIT)
+    const bool sym64 = sizeof(T) == 8 && A.loc && A.Wp[0] == A.W[0];
+    if (Nc <= (sym64 ? RESTRICT_SPLIT_SYM : RESTRICT_SPLIT))
         k_mg_restrict_split<T><<<stream_blocks(Nc * 8), LIN_BLOCK, 0, st>>>(B, b, x, cnx, cny, cnz, fx, fxy, bc);
     else
         k_mg_restrict<T><<<stream_blocks(Nc), LIN_BLOCK, 0, st>>>(B, b, x, cnx, cny, cnz, fx, fxy, bc);
