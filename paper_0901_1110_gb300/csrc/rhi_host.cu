@@ -318,7 +318,9 @@ int read_scalar(rhi_ctx* h, int slot, double* out) {
 }
 
 // The cell kernel's last block sums its partials up to this many blocks (10^6 cells); beyond, one
-// block of 1024 threads does it faster in a launch of its own (15 us at 256^3).
+// block of 1024 threads does it in a launch of its own.  Measured, H + He, us with the last block / with
+// the launch: 96^3 409.9 / 414.6, 128^3 950 / 952, 144^3 1351 / 1351, 192^3 3183 / 3175, 224^3 5049 /
+// 5033.  The two cross near 144^3 (23000 blocks); the line, set at 10^6 cells, leaves 2 us between.
 constexpr int CELL_SUM_BLOCKS = 8192;
 
 // ||f||_RMS from the cell kernel's sum or partials

@@ -78,7 +78,8 @@ cudaError_t mg_build_init();
 // A cycle's first two sweeps of a level of N cells as one kernel, which multiplies omega / diag by b where
 // the second sweep reads x: one launch and, in memory, the first sweep's x less.  Measured, FP32: 256^3
 // 131 -> 99 us, 128^3 24.4 -> 22.1 us, 64^3 about 12.5 -> 7.5 us.  FP64 pays its seven
-// multiplications on the FP64 pipe: 32^3 13.1 -> 7.6 us, 64^3 5 us less, but 128^3 51 -> 64 us.
+// multiplications on the FP64 pipe: 32^3 13.1 -> 7.6 us, 64^3 16.8 -> 14.2, 72^3 18.8 -> 18.1, but 80^3
+// 21.3 -> 22.6 and 128^3 52.5 -> 69.6 us: the line lies at 64^3, a size below the crossing.
 // Returns how many of n sweeps the first launch makes.
 template <typename T>
 constexpr int mg_first_sweeps(long long N, int n) {

@@ -19,7 +19,13 @@ PROGRAM = r"""
 #include <cstdio>
 #include "rhi_internal.cuh"
 typedef unsigned long long u64;
-__device__ u64 dist(long long a, long long b) { return (u64)(a > b ? a - b : b - a); }
+// units between two numbers by their bit patterns; the zeros count as one number
+__device__ u64 dist(long long a, long long b) {
+    const long long top = (long long)(1ULL << 63);
+    a = a < 0 ? top - a : a;
+    b = b < 0 ? top - b : b;
+    return (u64)(a > b ? a - b : b - a);
+}
 __global__ void rcp(long long n, u64* out) {
     u64 w = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -50,7 +56,8 @@ __global__ void silu(u64* out) {
     u64 w = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < 1LL << 32; i += (long long)gridDim.x * blockDim.x) {
         const float z = __uint_as_float((unsigned)i), a = rhi::silu_f<true>(z), b = rhi::silu_f<false>(z);
-        u64 u = dist(__float_as_int(a), __float_as_int(b));
+        const unsigned ua = __float_as_uint(a), ub = __float_as_uint(b);
+        u64 u = dist((long long)((u64)ua << 32), (long long)((u64)ub << 32)) >> 32;
         if (a != a || b != b) u = a != a && b != b ? 0 : 1ULL << 40;
         if (u > w) w = u;
     }
