@@ -18,7 +18,8 @@
 //
 // Measured: a whole cycle of a 32^3 FP32 grid (4 levels) 24.6 us, against about 75 us for its 20
 // launches inside a CUDA graph; a 16^3 FP64 cycle (5 levels) 34.8 us against about 90 us.  What is left is
-// latency: about 0.4 us for a cluster barrier, and in FP64 64 cycles for each instruction of a warp.
+// latency: about 0.4 us for each of about twelve cluster barriers (5 of the 25 us; the rest is not attributed),
+// and in FP64 64 cycles for each instruction of a warp.
 // Larger levels stay with the level kernels, which use all SMs: at 64^3 FP32 a sweep moves 10 MB.
 //
 // Where the whole cycle is one such launch, BiCGStab's p is updated as it is read (given): a launch and
